@@ -4,8 +4,9 @@
 // representatives, and attends over the chosen blocks only; the first block and the query's own
 // block (cut at the query's position) are always among them and count inside the budget.
 //
-//   moba_means_kernel    per (head, block): the mean of the block's stored keys, fp32
-//   moba_route_kernel    per (head, 16 consecutive queries), a warp per query: scores q . mean of the
+//   rq_moba_route.cu     bf16 caches: the blocks' mean keys and every query's choice of blocks (a bit mask)
+//   moba_means_kernel    fp32 caches.  Per (head, block): the mean of the block's stored keys
+//   moba_route_kernel    fp32 caches.  Per (head, 16 consecutive queries), a warp per query: scores q . mean of the
 //                        complete blocks before the query's own (a lane per block; the head's
 //                        representatives staged in shared memory once per CTA when they fit), then the
 //                        budget's best (equal scores to the lower block) by a bit-wise search for the
@@ -38,7 +39,6 @@ constexpr int kMobaChunk = 64;                 // positions that pass through sh
 constexpr int kMobaQueries = 16;               // queries (warps) of one attention CTA
 constexpr int kMobaRouteWarps = 16;            // warps of one routing CTA
 constexpr int kMobaRouteQ = 2;                 // consecutive queries of one routing warp when the representatives are staged (they share the reads)
-constexpr int kMobaMaxBlocks = 2048;           // blocks of a prompt at most
 constexpr unsigned FULLMASK = 0xffffffffu;
 
 // floats of shared memory one routing warp needs: query, scores, mask words; a multiple of 4 so that
@@ -473,8 +473,8 @@ __device__ __forceinline__ int moba_walk_next(MobaWalk &w, const uint32_t *chose
 
 template <int D>
 __global__ void __launch_bounds__(kMobaMmaThreads) moba_mma_kernel(const __grid_constant__ CUtensorMap tmap, int64_t page_cap, int S,
-                                                                  int64_t len, const bf16 *q, int H, int block, int nb, int K,
-                                                                  const int32_t *sel, float scale_log2, bf16 *o, int32_t *status)
+                                                                  int64_t len, const bf16 *q, int H, int block, int nb,
+                                                                  const uint32_t *masks, float scale_log2, bf16 *o, int32_t *status)
 {
     using G = MobaMmaGeom<D>;
     constexpr int NST = kMobaMmaStages;
@@ -527,16 +527,12 @@ __global__ void __launch_bounds__(kMobaMmaThreads) moba_mma_kernel(const __grid_
         *reinterpret_cast<uint4 *>(qs + (c >> 3) * (128 * 128) + umma_sw128_offset(r, c & 7)) = v;
     }
     __syncthreads();
-    if (tid < kMobaMmaQueries && t0 + tid < len) {
-        const int32_t *list = sel + ((int64_t)bh * len + t0 + tid) * K;
-        for (int i = 0; i < K; ++i) {
-            const int j = list[i];
-            if (j >= 0 && j < nb) {
-                qmask[tid * words + (j >> 5)] |= 1u << (j & 31);
-                atomicOr(&umask[j >> 5], 1u << (j & 31));
-            }
+    if (t0 + tid < len && tid < kMobaMmaQueries)
+        for (int w = 0; w < words; ++w) {
+            const uint32_t m = masks[((int64_t)bh * len + t0 + tid) * words + w];
+            qmask[tid * words + w] = m;
+            if (m) atomicOr(&umask[w], m);
         }
-    }
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // the queries, written with ordinary stores, are read by the tensor core
     tcgen05_before_sync();
     __syncthreads();
@@ -810,18 +806,45 @@ __global__ void __launch_bounds__(kMobaMmaThreads) moba_mma_kernel(const __grid_
 
 size_t round256(size_t x) { return (x + 255) & ~(size_t)255; }
 
-template <typename T, int D>
-cudaError_t moba_run(const MobaArgs &a, cudaStream_t s)
+// bf16 caches: representatives and routing (rq_moba_route.cu), attention on the tensor cores.
+template <int D>
+cudaError_t moba_run_bf16(const MobaArgs &a, cudaStream_t s)
+{
+    using G = MobaMmaGeom<D>;
+    const int BH = a.B * a.H, nb = (int)((a.len + a.block - 1) / a.block), words = (nb + 31) / 32;
+    static bool ready[64];
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
+    if (!ready[dev]) {
+        e = cudaFuncSetAttribute(moba_mma_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)((size_t)G::FIXED_BYTES + (size_t)(kMobaMaxBlocks / 32) * (kMobaMmaQueries + 1) * sizeof(uint32_t)));
+        if (e != cudaSuccess) return e;
+        ready[dev] = true;
+    }
+    alignas(64) CUtensorMap tmap;
+    e = cache_tensor_map(&tmap, a.kv, D, a.S, (int64_t)BH * a.page_cap, kMobaChunk);
+    if (e != cudaSuccess) return e;
+    e = launch_moba_route_bf16(a, s);
+    if (e != cudaSuccess) return e;
+    const size_t ms = (size_t)G::FIXED_BYTES + (size_t)words * (kMobaMmaQueries + 1) * sizeof(uint32_t);
+    moba_mma_kernel<D><<<dim3((unsigned)BH, (unsigned)((a.len + kMobaMmaQueries - 1) / kMobaMmaQueries)), kMobaMmaThreads, ms, s>>>(
+        tmap, a.page_cap, a.S, a.len, (const bf16 *)a.q, a.H, a.block, nb, a.masks, a.scale * 1.4426950408889634f, (bf16 *)a.o, a.status);
+    return cudaGetLastError();
+}
+
+// fp32 caches: everything on plain fp32 FMAs (tf32 products would round the operands).
+template <int D>
+cudaError_t moba_run_f32(const MobaArgs &a, cudaStream_t s)
 {
     const int BH = a.B * a.H;
     const int nb = (int)((a.len + a.block - 1) / a.block);
     const int words = (nb + 31) / 32;
-    moba_means_kernel<T><<<dim3((unsigned)nb, (unsigned)BH), D, 0, s>>>((const T *)a.kv, a.page_cap, a.S, D, a.len, a.block,
-                                                                      a.means, nb);
     const bool staged = nb <= kMobaStagedBlocks;
     const int rq = staged ? kMobaRouteQ : 1;         // queries of a routing warp
     const size_t rs = (size_t)kMobaRouteWarps * rq * moba_route_floats(D, nb) * sizeof(float) + (staged ? (size_t)nb * (D + 4) * sizeof(float) : 0);
-    constexpr int CHUNK_BYTES = 2 * kMobaChunk * D * (int)sizeof(T);
+    constexpr int CHUNK_BYTES = 2 * kMobaChunk * D * (int)sizeof(float);
     const size_t as = 2 * (size_t)CHUNK_BYTES + (size_t)words * (kMobaQueries + 1) * sizeof(uint32_t);
     static bool ready[64];
     int dev = 0;
@@ -829,60 +852,54 @@ cudaError_t moba_run(const MobaArgs &a, cudaStream_t s)
     if (e != cudaSuccess) return e;
     if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
     if (!ready[dev]) {
-        e = cudaFuncSetAttribute(moba_route_kernel<T, D, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        e = cudaFuncSetAttribute(moba_route_kernel<float, D, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)((size_t)kMobaRouteWarps * moba_route_floats(D, kMobaMaxBlocks) * sizeof(float)));
         if (e != cudaSuccess) return e;
-        e = cudaFuncSetAttribute(moba_route_kernel<T, D, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        e = cudaFuncSetAttribute(moba_route_kernel<float, D, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)((size_t)kMobaRouteWarps * kMobaRouteQ * moba_route_floats(D, kMobaStagedBlocks) * sizeof(float) +
                                        (size_t)kMobaStagedBlocks * (D + 4) * sizeof(float)));
         if (e != cudaSuccess) return e;
-        e = cudaFuncSetAttribute(moba_attend_kernel<T, D>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        e = cudaFuncSetAttribute(moba_attend_kernel<float, D>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)(2 * (size_t)CHUNK_BYTES + (size_t)(kMobaMaxBlocks / 32) * (kMobaQueries + 1) * sizeof(uint32_t)));
         if (e != cudaSuccess) return e;
         ready[dev] = true;
     }
+    moba_means_kernel<float><<<dim3((unsigned)nb, (unsigned)BH), D, 0, s>>>((const float *)a.kv, a.page_cap, a.S, D, a.len, a.block,
+                                                                          a.means, nb);
     const dim3 rgrid((unsigned)((a.len + kMobaRouteWarps * rq - 1) / (kMobaRouteWarps * rq)), (unsigned)BH);
     if (staged)
-        moba_route_kernel<T, D, true><<<rgrid, kMobaRouteWarps * 32, rs, s>>>((const T *)a.q, a.means, a.len, a.H, a.block, nb, a.K, a.sel);
+        moba_route_kernel<float, D, true><<<rgrid, kMobaRouteWarps * 32, rs, s>>>((const float *)a.q, a.means, a.len, a.H, a.block, nb, a.K, a.sel);
     else
-        moba_route_kernel<T, D, false><<<rgrid, kMobaRouteWarps * 32, rs, s>>>((const T *)a.q, a.means, a.len, a.H, a.block, nb, a.K, a.sel);
-    const float sl2 = a.scale * 1.4426950408889634f;
-    if constexpr (sizeof(T) == 2) {
-        // bf16 caches: the attention on the tensor cores
-        using G = MobaMmaGeom<D>;
-        const size_t ms = (size_t)G::FIXED_BYTES + (size_t)words * (kMobaMmaQueries + 1) * sizeof(uint32_t);
-        static bool mready[64];
-        if (!mready[dev]) {
-            e = cudaFuncSetAttribute(moba_mma_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)((size_t)G::FIXED_BYTES + (size_t)(kMobaMaxBlocks / 32) * (kMobaMmaQueries + 1) * sizeof(uint32_t)));
-            if (e != cudaSuccess) return e;
-            mready[dev] = true;
-        }
-        alignas(64) CUtensorMap tmap;
-        e = cache_tensor_map(&tmap, a.kv, D, a.S, (int64_t)BH * a.page_cap, kMobaChunk);
-        if (e != cudaSuccess) return e;
-        moba_mma_kernel<D><<<dim3((unsigned)BH, (unsigned)((a.len + kMobaMmaQueries - 1) / kMobaMmaQueries)), kMobaMmaThreads, ms, s>>>(
-            tmap, a.page_cap, a.S, a.len, (const bf16 *)a.q, a.H, a.block, nb, a.K, a.sel, sl2, (bf16 *)a.o, a.status);
-    } else {
-        moba_attend_kernel<T, D><<<dim3((unsigned)((a.len + kMobaQueries - 1) / kMobaQueries), (unsigned)BH), kMobaQueries * 32, as, s>>>(
-            (const T *)a.kv, a.page_cap, a.S, a.len, (const T *)a.q, a.H, a.block, nb, a.K, a.sel, sl2, (T *)a.o);
-    }
+        moba_route_kernel<float, D, false><<<rgrid, kMobaRouteWarps * 32, rs, s>>>((const float *)a.q, a.means, a.len, a.H, a.block, nb, a.K, a.sel);
+    moba_attend_kernel<float, D><<<dim3((unsigned)((a.len + kMobaQueries - 1) / kMobaQueries), (unsigned)BH), kMobaQueries * 32, as, s>>>(
+        (const float *)a.kv, a.page_cap, a.S, a.len, (const float *)a.q, a.H, a.block, nb, a.K, a.sel, a.scale * 1.4426950408889634f,
+        (float *)a.o);
     return cudaGetLastError();
 }
 
 }  // namespace
 
-size_t moba_scratch_bytes(int BH, int64_t len, int D, int block, int K)
+size_t moba_scratch_bytes(int BH, int64_t len, int D, int block, int K, int dtype)
 {
-    const size_t nb = (size_t)((len + block - 1) / block);
-    return round256((size_t)BH * nb * D * sizeof(float)) + round256((size_t)BH * (size_t)len * K * sizeof(int32_t));
+    const size_t nb = (size_t)((len + block - 1) / block), means = round256((size_t)BH * nb * D * sizeof(float));
+    if (dtype != RQ_BF16) return means + round256((size_t)BH * (size_t)len * K * sizeof(int32_t));
+    return means + round256(moba_plane_bytes(BH, (int)nb, D)) + round256((size_t)BH * (size_t)len * ((nb + 31) / 32) * sizeof(uint32_t));
 }
 
-void moba_carve(void *scratch, int BH, int64_t len, int D, int block, float **means, int32_t **sel)
+void moba_carve(void *scratch, int BH, int64_t len, int D, int block, int dtype, MobaArgs &a)
 {
     const size_t nb = (size_t)((len + block - 1) / block);
-    *means = (float *)scratch;
-    *sel = (int32_t *)((char *)scratch + round256((size_t)BH * nb * D * sizeof(float)));
+    a.means = (float *)scratch;
+    a.sel = nullptr;
+    a.planes = nullptr;
+    a.masks = nullptr;
+    char *p = (char *)scratch + round256((size_t)BH * nb * D * sizeof(float));
+    if (dtype != RQ_BF16) {
+        a.sel = (int32_t *)p;
+    } else {
+        a.planes = (unsigned char *)p;
+        a.masks = (uint32_t *)(p + round256(moba_plane_bytes(BH, (int)nb, D)));
+    }
 }
 
 cudaError_t launch_moba(const MobaArgs &a, cudaStream_t s)
@@ -891,11 +908,11 @@ cudaError_t launch_moba(const MobaArgs &a, cudaStream_t s)
     if ((a.len + a.block - 1) / a.block > kMobaMaxBlocks || a.B * a.H > 65535 || (a.len + kMobaMmaQueries - 1) / kMobaMmaQueries > 65535)
         return cudaErrorInvalidValue;
     if (a.dtype == RQ_BF16) {
-        if (a.D == 128) return moba_run<bf16, 128>(a, s);
-        if (a.D == 64) return moba_run<bf16, 64>(a, s);
+        if (a.D == 128) return moba_run_bf16<128>(a, s);
+        if (a.D == 64) return moba_run_bf16<64>(a, s);
     } else {
-        if (a.D == 128) return moba_run<float, 128>(a, s);
-        if (a.D == 64) return moba_run<float, 64>(a, s);
+        if (a.D == 128) return moba_run_f32<128>(a, s);
+        if (a.D == 64) return moba_run_f32<64>(a, s);
     }
     return cudaErrorInvalidValue;
 }

@@ -1,0 +1,514 @@
+// MoBA routing for bf16 caches (Sec. 2.2, Eq. 3; App. A.1, MoBA paragraph) on the tensor cores: block
+// representatives, the scores of every query against the representatives of the blocks before it, and the
+// budget's best blocks of every query as a bit mask.
+//
+//   moba_means_bf16_kernel   per (head, block): the mean of the block's stored keys in fp32, and the same numbers
+//                            cut into three bf16 terms (hi + mid + lo: 24 significand bits, nothing of the fp32
+//                            mean is lost) laid out as the tensor core reads them
+//   moba_route_mma_kernel    per (head, 128 consecutive queries): scores = Q (hi + mid + lo)^T in tensor memory,
+//                            then per query the threshold of the budget by value buckets, the mask and, if asked
+//                            for, the ascending list
+#include <limits.h>
+#include <math_constants.h>
+
+#include "rq_async.cuh"
+#include "rq_device.cuh"
+#include "rq_internal.h"
+#include "rq_umma.cuh"
+
+namespace rq {
+
+namespace {
+
+constexpr unsigned FULL = 0xffffffffu;
+constexpr int kRouteQueries = 128;             // queries of a CTA: the lanes of the accumulator
+constexpr int kRouteThreads = 512;             // four threads per query, each a quarter of the score words
+constexpr int kRouteGroup = 64;                // blocks of one product (N), and of one copy of representatives
+constexpr int kPanelGroups = 8;                // groups whose scores fit in tensor memory at once (512 columns)
+constexpr int kRouteBins = 64;                 // value buckets of the threshold search
+constexpr int kRouteCap = 16;                  // blocks of the threshold's bucket that are ranked directly
+
+// ---------------------------------------------------------------- block representatives
+// Grid (ceil(blocks / R), heads), R = 256 / (D / 2) blocks per CTA, a thread per two channels of a block.  The sum
+// runs over the block's valid positions in order.
+// planes: [head][group of 64 blocks][hi, mid, lo][half of 64 channels][64 rows x 128 bytes, 128-byte swizzle]
+__global__ void __launch_bounds__(256) moba_means_bf16_kernel(const bf16 *kv, int64_t page_cap, int S, int D, int64_t len, int block,
+                                                             float *means, unsigned char *planes, int nb)
+{
+    const int per = D / 2, r = threadIdx.x / per, c = 2 * (threadIdx.x % per);
+    const int j = blockIdx.x * (256 / per) + r, bh = blockIdx.y;
+    if (j >= nb) return;
+    const int64_t lo = (int64_t)j * block, hi = min(lo + block, len);
+    float s0 = 0.0f, s1 = 0.0f;
+    int64_t p = lo;
+    // sixteen loads in flight at a time (a page holds a multiple of 16 positions and lo is a multiple of 64, so a run
+    // of 16 stays inside one page); the additions keep the order of the positions
+    for (; p + 16 <= hi; p += 16) {
+        const bf16 *src = kv + ((((int64_t)bh * page_cap + p / S) * 2) * S + p % S) * D + c;
+        uint32_t x[16];
+#pragma unroll
+        for (int i = 0; i < 16; ++i) x[i] = __ldg(reinterpret_cast<const uint32_t *>(src + (int64_t)i * D));
+#pragma unroll
+        for (int i = 0; i < 16; ++i) { s0 += bf16lo(x[i]); s1 += bf16hi(x[i]); }
+    }
+    for (; p < hi; ++p) {
+        const uint32_t x = *reinterpret_cast<const uint32_t *>(kv + ((((int64_t)bh * page_cap + p / S) * 2) * S + p % S) * D + c);
+        s0 += bf16lo(x);
+        s1 += bf16hi(x);
+    }
+    const float n = (float)(hi - lo), m0 = s0 / n, m1 = s1 / n;
+    *reinterpret_cast<float2 *>(means + ((int64_t)bh * nb + j) * D + c) = make_float2(m0, m1);
+    const int groups = (nb + kRouteGroup - 1) / kRouteGroup, plane_bytes = kRouteGroup * D * 2;
+    unsigned char *dst = planes + ((int64_t)bh * groups + j / kRouteGroup) * 3 * plane_bytes + (c >> 6) * (kRouteGroup * 128) +
+                         umma_sw128_offset(j % kRouteGroup, (c & 63) >> 3) + (c & 7) * 2;
+    float a = m0, b = m1;
+#pragma unroll
+    for (int t = 0; t < 3; ++t) {                       // the remainders are exact: each term takes the next 8 bits
+        const uint32_t w = pack_bf16(a, b);
+        *reinterpret_cast<uint32_t *>(dst + t * plane_bytes) = w;
+        a -= bf16lo(w);
+        b -= bf16hi(w);
+    }
+}
+
+// ---------------------------------------------------------------- routing
+template <int D> struct RouteGeom {
+    static constexpr int HALVES = D / 64;
+    static constexpr int Q_BYTES = HALVES * kRouteQueries * 128;
+    static constexpr int PLANE_BYTES = HALVES * kRouteGroup * 128;
+    static constexpr int GROUP_BYTES = 3 * PLANE_BYTES;
+    static constexpr int WORK_BYTES = kRouteBins * kRouteQueries * 4 + kRouteCap * kRouteQueries * 6;   // buckets, ranked blocks
+    static constexpr int SMALL_BYTES = (12 + 6) * kRouteQueries * 4;
+    // `stages` copies of representatives; a prompt of one panel is done with queries and representatives when the
+    // buckets are needed, so these share the space
+    static __host__ __device__ int front_bytes(int stages, bool one_panel)
+    {
+        const int qb = Q_BYTES + stages * GROUP_BYTES;
+        return one_panel ? (qb > WORK_BYTES ? qb : WORK_BYTES) : qb + WORK_BYTES;
+    }
+    static int smem_bytes(int stages, bool one_panel, int words)
+    {
+        return 1024 + front_bytes(stages, one_panel) + 2 * words * kRouteQueries * 4 + SMALL_BYTES;
+    }
+};
+
+// order-preserving image of a score; -0 counts as +0
+__device__ __forceinline__ uint32_t score_key(float v)
+{
+    const uint32_t b = __float_as_uint(v + 0.0f);
+    return b ^ ((b >> 31) ? 0xffffffffu : 0x80000000u);
+}
+// Value bucket of a score between the query's smallest and largest: monotone in v, 0 .. kRouteBins - 1.
+__device__ __forceinline__ uint32_t score_bin(float v, float lo, float inv)
+{
+    return min(__float_as_uint(fmaf(v - lo, inv, 8388609.0f)) - 0x4B000000u, (uint32_t)(kRouteBins - 1));
+}
+
+// Grid (heads, tiles of 128 queries; the tiles of the last queries first: their work is the largest).  Bound by the
+// instructions of the three passes over the scores (smallest and largest, buckets, mask; about a dozen per score and
+// 32 queries), which is why a pass that ranks every candidate, or one that takes one block per round, is so much
+// slower.  Per query:
+//   1. smallest and largest score of its candidates (the complete blocks between the first and the query's own);
+//   2. 64 value buckets between them: the bucket that holds the last block taken, and how many of it are wanted;
+//   3. blocks of higher buckets into the mask; those of the threshold's bucket are ranked against each other by
+//      (score, lower block first).
+// A threshold bucket of more than 16 blocks is cut further by buckets on the scores' integer images until at most 16
+// are left or all left are equal (equal scores: the lowest blocks).  More than 512 blocks are taken in panels of 512,
+// whose scores are computed again for each pass (the tensor cores have nothing else to do here).
+// Measured, 32 heads x 128 channels: 4096 queries, 16 of 64 blocks each, 158 -> 58 us; 30011 queries, 30 of 469 blocks
+// each, 28.9 -> 1.35 ms (before: fp32 FMA scores, a lane per block, then a bit-wise vote search up to 128 blocks and one
+// round per taken block beyond).
+template <int D>
+__global__ void __launch_bounds__(kRouteThreads) moba_route_mma_kernel(const bf16 *q, const unsigned char *planes, int64_t len, int H,
+                                                                      int block, int nb, int K, int words, uint32_t *masks,
+                                                                      int32_t *list, int stages, int32_t *status)
+{
+    using G = RouteGeom<D>;
+    constexpr int NQ = kRouteQueries, NB = kRouteBins, CAP = kRouteCap;
+    extern __shared__ __align__(1024) unsigned char rsm_raw[];
+    __shared__ __align__(8) uint64_t full[2], done[2], panel_done;
+    __shared__ uint32_t tbase;
+    unsigned char *sm = rsm_raw + ((1024u - (smem_addr(rsm_raw) & 1023u)) & 1023u);
+    const int groups_all = (nb + kRouteGroup - 1) / kRouteGroup;
+    const bool one_panel_launch = groups_all <= kPanelGroups;
+    unsigned char *qs = sm, *bs = sm + G::Q_BYTES;
+    uint32_t *hist = reinterpret_cast<uint32_t *>(one_panel_launch ? sm : sm + G::Q_BYTES + stages * G::GROUP_BYTES);   // [NB][NQ]
+    uint32_t *ckey = hist + NB * NQ;                                           // [CAP][NQ]
+    uint16_t *cidx = reinterpret_cast<uint16_t *>(ckey + CAP * NQ);            // [CAP][NQ]
+    uint32_t *mk = reinterpret_cast<uint32_t *>(sm + G::front_bytes(stages, one_panel_launch));   // [words][NQ] chosen blocks
+    uint32_t *tie = mk + words * NQ;                                           // [words][NQ] equal scores at the threshold
+    uint32_t *part_a = tie + words * NQ, *part_b = part_a + 4 * NQ, *part_c = part_b + 4 * NQ;    // [4][NQ] each
+    int32_t *s_tb = reinterpret_cast<int32_t *>(part_c + 4 * NQ), *s_need = s_tb + NQ, *s_cnt = s_need + NQ;
+    uint32_t *s_klo = reinterpret_cast<uint32_t *>(s_cnt + NQ), *s_khi = s_klo + NQ, *s_n = s_khi + NQ;
+
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int ql = (warp & 3) * 32 + lane, part = warp >> 2;                   // this thread's query and quarter of the words
+    const int bh = blockIdx.x, b = bh / H, h = bh % H;
+    const int64_t t0 = (int64_t)(gridDim.y - 1 - blockIdx.y) * NQ, t = t0 + ql;
+    const int own = (int)(t / block), own_last = (int)((min(t0 + NQ, len) - 1) / block), own_first = (int)(t0 / block);
+    const int want = K - 2;                                                    // beside the first block and the query's own
+    const bool active = t < len && K < own + 1;                                // otherwise everything up to the query is taken
+    const int c_hi = active ? own : 0;                                         // candidates: blocks 1 .. c_hi - 1
+    const bool any = K < own_last + 1;                                         // some query of the CTA has to choose
+    const int groups = any ? (own_last + kRouteGroup - 1) / kRouteGroup : 0;   // groups that hold blocks 0 .. own_last - 1
+    const int panels = (groups + kPanelGroups - 1) / kPanelGroups;
+    const int words_cta = any ? (own_last + 31) / 32 : 0;
+    uint32_t tcols = kRouteGroup;
+    while ((int)tcols < min(groups, kPanelGroups) * kRouteGroup) tcols *= 2;
+
+    for (int i = tid; i < 2 * words * NQ; i += kRouteThreads) mk[i] = 0u;      // mk and tie
+    if (part == 0) {
+        s_tb[ql] = NB; s_need[ql] = 0; s_cnt[ql] = 0;
+        s_klo[ql] = 0u; s_khi[ql] = 0xffffffffu; s_n[ql] = 0u;
+    }
+    bool ok = true;
+    if (any) {
+        if (tid == 0) {
+            for (int s = 0; s < 2; ++s) { mbar_init(&full[s], 1); mbar_init(&done[s], 1); }
+            mbar_init(&panel_done, 1);
+            mbar_init_fence();
+        }
+        if (warp == 0) tmem_alloc(&tbase, tcols);
+        // the queries (q is [B][T][H][D]) as the K-major operand; rows past the prompt are zero
+        for (int i = tid; i < NQ * (D / 8); i += kRouteThreads) {
+            const int r = i / (D / 8), c = i % (D / 8);
+            uint4 v = make_uint4(0u, 0u, 0u, 0u);
+            if (t0 + r < len) v = *reinterpret_cast<const uint4 *>(q + (((int64_t)b * len + t0 + r) * H + h) * D + c * 8);
+            *reinterpret_cast<uint4 *>(qs + (c >> 3) * (NQ * 128) + umma_sw128_offset(r, c & 7)) = v;
+        }
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");           // ordinary stores, read by the tensor core
+        tcgen05_before_sync();
+        __syncthreads();
+        tcgen05_after_sync();
+        const uint32_t tb = tbase, tl = tb + ((uint32_t)((warp & 3) * 32) << 16);
+        const unsigned char *src = planes + (int64_t)bh * groups_all * G::GROUP_BYTES;
+        int issued = 0, used = 0;                                              // thread 0: copies started, copies multiplied
+        uint32_t panel_phase = 0u;
+
+        // the scores of panel p into tensor memory; thread 0 starts copies and products
+        auto panel = [&](int p) {
+            if (tid == 0 && ok) {
+                const int g0 = p * kPanelGroups, gn = min(kPanelGroups, groups - g0);
+                auto issue = [&](int g) {
+                    const int st = issued % stages;
+                    mbar_arrive_expect_tx(&full[st], G::GROUP_BYTES);
+                    bulk_g2s(bs + (size_t)st * G::GROUP_BYTES, src + (int64_t)g * G::GROUP_BYTES, G::GROUP_BYTES, &full[st]);
+                    ++issued;
+                };
+                constexpr uint32_t idesc = umma_idesc_bf16(NQ, kRouteGroup);
+                const uint32_t qa = smem_addr(qs);
+                tcgen05_after_sync();
+                for (int g = 0; g < gn && g < stages; ++g) issue(g0 + g);
+#pragma unroll 1
+                for (int g = 0; g < gn; ++g) {
+                    const int st = used % stages;
+                    const uint32_t phase = (uint32_t)((used / stages) & 1);
+                    ok = mbar_wait(&full[st], phase);
+                    if (!ok) break;
+                    ++used;
+                    const uint32_t ba = smem_addr(bs + (size_t)st * G::GROUP_BYTES);
+#pragma unroll
+                    for (int pl = 2; pl >= 0; --pl)                            // the smallest terms first
+#pragma unroll
+                        for (int k = 0; k < D / 16; ++k)
+                            umma_bf16(tb + (uint32_t)g * kRouteGroup, umma_desc_sw128(qa + (k >> 2) * (NQ * 128) + (k & 3) * 32),
+                                      umma_desc_sw128(ba + pl * G::PLANE_BYTES + (k >> 2) * (kRouteGroup * 128) + (k & 3) * 32), idesc,
+                                      !(pl == 2 && k == 0));
+                    umma_commit(&done[st]);
+                    if (g + stages < gn) {
+                        ok = mbar_wait(&done[st], phase);
+                        if (!ok) break;
+                        issue(g0 + g + stages);
+                    }
+                }
+                umma_commit(&panel_done);
+            }
+            __syncwarp();
+            if (!mbar_wait(&panel_done, panel_phase)) ok = false;
+            panel_phase ^= 1u;
+            ok = __syncthreads_and(ok);
+            tcgen05_after_sync();
+        };
+        // body(word, scores, candidates among them as bits) for this thread's words of every panel
+        auto for_scores = [&](bool first, auto body) {
+            for (int p = 0; p < panels && ok; ++p) {
+                if (first || panels > 1) panel(p);
+                if (!ok) break;
+#pragma unroll 1
+                for (int wl = part; wl < 2 * kPanelGroups; wl += 4) {
+                    const int w = p * 2 * kPanelGroups + wl;
+                    if (w >= words_cta) break;
+                    float v[32];
+                    __syncwarp();
+                    tmem_ld32(tl + (uint32_t)wl * 32u, v);
+                    const int hi = c_hi - 32 * w;
+                    uint32_t cand = hi >= 32 ? 0xffffffffu : hi <= 0 ? 0u : (1u << hi) - 1u;
+                    if (w == 0) cand &= ~1u;
+                    body(w, v, cand);
+                }
+                tcgen05_before_sync();
+                if (panels > 1) __syncthreads();                               // the scores may be overwritten
+            }
+        };
+        // the bucket that holds the want-th largest of a query's counted scores: thread `part` of the query adds up a
+        // quarter of the buckets, the one whose quarter holds the threshold walks it
+        auto find_bin = [&](bool mine, int wanted, int &bin, int &need, int &cnt) -> bool {
+            uint32_t s = 0u;
+#pragma unroll
+            for (int i = 0; i < NB / 4; ++i) s += hist[(part * (NB / 4) + i) * NQ + ql];
+            part_c[part * NQ + ql] = s;
+            __syncthreads();
+            int cum = 0, pt = 3;
+            for (; pt > 0; --pt) {
+                const int c = (int)part_c[pt * NQ + ql];
+                if (cum + c >= wanted) break;
+                cum += c;
+            }
+            if (!mine || part != pt) return false;
+            int i = NB / 4 - 1;
+            for (; i > 0; --i) {
+                const int c = (int)hist[(pt * (NB / 4) + i) * NQ + ql];
+                if (cum + c >= wanted) break;
+                cum += c;
+            }
+            bin = pt * (NB / 4) + i;
+            cnt = (int)hist[bin * NQ + ql];
+            need = wanted - cum;
+            return true;
+        };
+
+        // ---- 1. smallest and largest
+        float mn = CUDART_INF_F, mx = -CUDART_INF_F;
+        for_scores(true, [&](int w, float (&v)[32], uint32_t cand) {
+            if (w > 0 && 32 * w + 32 <= own_first && own_first >= K) {         // every score is a candidate of every query
+#pragma unroll
+                for (int c = 0; c < 32; ++c) { mn = fminf(mn, v[c]); mx = fmaxf(mx, v[c]); }
+            } else {
+#pragma unroll
+                for (int c = 0; c < 32; ++c)
+                    if ((cand >> c) & 1u) { mn = fminf(mn, v[c]); mx = fmaxf(mx, v[c]); }
+            }
+        });
+        if (ok) {
+            part_a[part * NQ + ql] = __float_as_uint(mn);
+            part_b[part * NQ + ql] = __float_as_uint(mx);
+            for (int i = tid; i < NB * NQ; i += kRouteThreads) hist[i] = 0u;
+            __syncthreads();
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                mn = fminf(mn, __uint_as_float(part_a[i * NQ + ql]));
+                mx = fmaxf(mx, __uint_as_float(part_b[i * NQ + ql]));
+            }
+        }
+        const float range = mx - mn;
+        const float inv = range > 0.0f ? fminf((float)(NB - 3) / range, 3.0e38f) : 0.0f;
+
+        // ---- 2. buckets
+        for_scores(false, [&](int w, float (&v)[32], uint32_t cand) {
+#pragma unroll
+            for (int c = 0; c < 32; ++c)
+                if ((cand >> c) & 1u) atomicAdd(&hist[score_bin(v[c], mn, inv) * NQ + ql], 1u);
+        });
+        if (ok) {
+            __syncthreads();
+            int bin, need, cnt;
+            if (find_bin(active, want, bin, need, cnt)) {
+                if (need == cnt) { bin -= 1; need = 0; }                       // the whole bucket
+                s_tb[ql] = bin; s_need[ql] = need; s_cnt[ql] = cnt;
+            }
+            __syncthreads();
+        }
+        // ---- 2b. (rare) a threshold bucket with too many blocks: buckets on the integer images of its scores
+        bool tied = false;
+        while (ok) {
+            const int tbin = s_tb[ql];
+            const uint32_t klo = s_klo[ql], khi = s_khi[ql];
+            bool over = active && s_need[ql] > 0 && s_cnt[ql] > CAP && !tied;
+            if (over && klo == khi) { tied = true; over = false; }             // all equal: the lowest blocks are taken below
+            if (!__syncthreads_or(over)) break;
+            uint32_t kmin = 0xffffffffu, kmax = 0u;
+            for_scores(false, [&](int w, float (&v)[32], uint32_t cand) {
+#pragma unroll
+                for (int c = 0; c < 32; ++c) {
+                    const uint32_t k = score_key(v[c]);
+                    if (over && ((cand >> c) & 1u) && (int)score_bin(v[c], mn, inv) == tbin && k >= klo && k <= khi) {
+                        kmin = min(kmin, k);
+                        kmax = max(kmax, k);
+                    }
+                }
+            });
+            if (!ok) break;
+            part_a[part * NQ + ql] = kmin;
+            part_b[part * NQ + ql] = kmax;
+            for (int i = tid; i < NB * NQ; i += kRouteThreads) hist[i] = 0u;
+            __syncthreads();
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                kmin = min(kmin, part_a[i * NQ + ql]);
+                kmax = max(kmax, part_b[i * NQ + ql]);
+            }
+            const uint32_t span = over ? kmax - kmin : 0u;
+            const int sh = max(0, 26 - __clz((int)span));                      // (span >> sh) < 64
+            for_scores(false, [&](int w, float (&v)[32], uint32_t cand) {
+#pragma unroll
+                for (int c = 0; c < 32; ++c) {
+                    const uint32_t k = score_key(v[c]);
+                    if (over && ((cand >> c) & 1u) && (int)score_bin(v[c], mn, inv) == tbin && k >= kmin && k <= kmax)
+                        atomicAdd(&hist[((k - kmin) >> sh) * NQ + ql], 1u);
+                }
+            });
+            if (!ok) break;
+            __syncthreads();
+            int bin, need, cnt;
+            const bool got = find_bin(over, over ? s_need[ql] : 1, bin, need, cnt);
+            __syncthreads();
+            if (got) {
+                const uint32_t lo = kmin + ((uint32_t)bin << sh), hi = lo + min(kmax - lo, (1u << sh) - 1u);
+                if (need == cnt) { s_khi[ql] = lo - 1u; need = 0; }            // everything from lo upwards
+                else { s_klo[ql] = lo; s_khi[ql] = hi; }
+                s_need[ql] = need; s_cnt[ql] = cnt;
+            }
+            __syncthreads();
+        }
+        // ---- 3. the mask
+        if (ok) {
+            const int tbin = s_tb[ql], need = s_need[ql];
+            const uint32_t klo = s_klo[ql], khi = s_khi[ql];
+            for_scores(false, [&](int w, float (&v)[32], uint32_t cand) {
+                uint32_t bits = 0u, eq = 0u;
+#pragma unroll
+                for (int c = 0; c < 32; ++c) {
+                    const int bin = (int)score_bin(v[c], mn, inv);
+                    if (bin > tbin) bits |= 1u << c;
+                    if (bin == tbin && ((cand >> c) & 1u)) {
+                        const uint32_t k = score_key(v[c]);
+                        if (k > khi) {
+                            bits |= 1u << c;
+                        } else if (k >= klo && need > 0) {
+                            if (tied) {
+                                eq |= 1u << c;
+                            } else {
+                                const uint32_t at = atomicAdd(&s_n[ql], 1u);
+                                if (at < (uint32_t)CAP) {
+                                    ckey[at * NQ + ql] = k;
+                                    cidx[at * NQ + ql] = (uint16_t)(32 * w + c);
+                                }
+                            }
+                        }
+                    }
+                }
+                mk[w * NQ + ql] = bits & cand;
+                if (tied) tie[w * NQ + ql] = eq;
+            });
+            __syncthreads();
+            if (active && need > 0) {
+                if (tied) {
+                    if (part == 0) {
+                        int left = need;
+                        for (int w = 0; w < words_cta && left > 0; ++w) {
+                            uint32_t e = tie[w * NQ + ql], take = 0u;
+                            while (e && left > 0) { take |= e & (0u - e); e &= e - 1u; --left; }
+                            mk[w * NQ + ql] |= take;
+                        }
+                    }
+                } else {
+                    const int n = min((int)s_n[ql], CAP);
+                    for (int i = part; i < n; i += 4) {
+                        const uint32_t k = ckey[i * NQ + ql];
+                        const int j = cidx[i * NQ + ql];
+                        int rank = 0;
+                        for (int u = 0; u < n; ++u) {
+                            const uint32_t ku = ckey[u * NQ + ql];
+                            rank += (ku > k || (ku == k && (int)cidx[u * NQ + ql] < j)) ? 1 : 0;
+                        }
+                        if (rank < need) atomicOr(&mk[(j >> 5) * NQ + ql], 1u << (j & 31));
+                    }
+                }
+            }
+        }
+        if (tid == 0)                                                          // after a wait that ran out: no copy may still be on its way
+            for (int k = used; k < issued; ++k) mbar_wait(&full[k % stages], (uint32_t)((k / stages) & 1));
+        tcgen05_before_sync();
+        __syncthreads();
+        if (warp == 0) tmem_dealloc(tbase, tcols);
+    }
+    if (!ok && tid == 0) atomicCAS(status, RQ_OK, RQ_ERR_TIMEOUT);
+    __syncthreads();
+    // the masks go out, with the first block and the query's own
+    for (int i = tid; i < NQ * words; i += kRouteThreads) {
+        const int r = i / words, w = i % words;
+        const int64_t tq = t0 + r;
+        if (tq >= len) continue;
+        const int o = (int)(tq / block), hi = o + 1 - 32 * w;
+        uint32_t m;
+        if (K >= o + 1) m = hi >= 32 ? 0xffffffffu : hi <= 0 ? 0u : (1u << hi) - 1u;
+        else m = mk[w * NQ + r] | (w == 0 ? 1u : 0u) | (w == (o >> 5) ? 1u << (o & 31) : 0u);
+        masks[((int64_t)bh * len + t0) * words + i] = m;
+        if (list) mk[w * NQ + r] = m;
+    }
+    if (!list) return;
+    __syncthreads();
+    // the ascending lists for the caller, a warp per query
+    for (int r = warp; r < NQ && t0 + r < len; r += kRouteThreads / 32) {
+        int32_t *out = list + ((int64_t)bh * len + t0 + r) * K;
+        int base = 0;
+        for (int w0 = 0; w0 < words; w0 += 32) {
+            const uint32_t m = w0 + lane < words ? mk[(w0 + lane) * NQ + r] : 0u;
+            const int cnt = __popc(m);
+            int inc = cnt;
+#pragma unroll
+            for (int off = 1; off < 32; off <<= 1) {
+                const int o = __shfl_up_sync(FULL, inc, off);
+                if (lane >= off) inc += o;
+            }
+            int pos = base + inc - cnt;
+            for (uint32_t bits = m; bits; bits &= bits - 1u, ++pos)
+                if (pos < K) out[pos] = (w0 + lane) * 32 + __ffs(bits) - 1;
+            base += __shfl_sync(FULL, inc, 31);
+        }
+        for (int i = base + lane; i < K; i += 32) out[i] = -1;
+    }
+}
+
+template <int D> cudaError_t route_run(const MobaArgs &a, cudaStream_t s)
+{
+    using G = RouteGeom<D>;
+    const int BH = a.B * a.H, nb = (int)((a.len + a.block - 1) / a.block), words = (nb + 31) / 32;
+    const int groups = (nb + kRouteGroup - 1) / kRouteGroup;
+    const bool one_panel = groups <= kPanelGroups;
+    // more than 256 blocks: tensor memory leaves room for one CTA per SM, which then takes the shared memory of a second
+    // stage; up to 256, a second CTA is worth more than a second stage
+    const int stages = one_panel && groups * kRouteGroup > 256 ? 2 : 1;
+    static bool ready[64];
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
+    if (!ready[dev]) {
+        const int one = G::smem_bytes(2, true, kPanelGroups * kRouteGroup / 32), more = G::smem_bytes(1, false, kMobaMaxBlocks / 32);
+        e = cudaFuncSetAttribute(moba_route_mma_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, one > more ? one : more);
+        if (e != cudaSuccess) return e;
+        ready[dev] = true;
+    }
+    const int per = 256 / (D / 2);
+    moba_means_bf16_kernel<<<dim3((unsigned)((nb + per - 1) / per), (unsigned)BH), 256, 0, s>>>(
+        (const bf16 *)a.kv, a.page_cap, a.S, D, a.len, a.block, a.means, a.planes, nb);
+    moba_route_mma_kernel<D><<<dim3((unsigned)BH, (unsigned)((a.len + kRouteQueries - 1) / kRouteQueries)), kRouteThreads,
+                               G::smem_bytes(stages, one_panel, words), s>>>((const bf16 *)a.q, a.planes, a.len, a.H, a.block, nb, a.K,
+                                                                            words, a.masks, a.blocks_out, stages, a.status);
+    return cudaGetLastError();
+}
+
+}  // namespace
+
+size_t moba_plane_bytes(int BH, int nb, int D)
+{
+    return (size_t)BH * ((nb + kRouteGroup - 1) / kRouteGroup) * 3 * kRouteGroup * D * 2;
+}
+
+cudaError_t launch_moba_route_bf16(const MobaArgs &a, cudaStream_t s)
+{
+    return a.D == 128 ? route_run<128>(a, s) : a.D == 64 ? route_run<64>(a, s) : cudaErrorInvalidValue;
+}
+
+}  // namespace rq
