@@ -183,6 +183,8 @@ cudaError_t launch_moba(const MobaArgs &a, cudaStream_t s);
 // bf16 caches: representatives and routing (rq_moba_route.cu)
 size_t moba_plane_bytes(int BH, int nb, int D);
 cudaError_t launch_moba_route_bf16(const MobaArgs &a, cudaStream_t s);
+// bf16 caches: the attention (rq_moba_attend.cu)
+cudaError_t launch_moba_attend_bf16(const MobaArgs &a, cudaStream_t s);
 
 // Grid of a streaming kernel for a number of work units spread evenly over `heads` heads: at
 // most what the device holds at once, at least two units per warp, and a whole number of CTAs per

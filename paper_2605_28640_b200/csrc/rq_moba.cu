@@ -12,10 +12,7 @@
 //                        budget's best (equal scores to the lower block) by a bit-wise search for the
 //                        threshold score, or by repeated arg-max when the budget is small or the candidates many;
 //                        the list written ascending
-//   moba_mma_kernel      bf16 caches.  Per (head, 128 consecutive queries): both contractions on the
-//                        tensor cores (tcgen05.mma, accumulators and the weights in tensor memory),
-//                        the chunks of the blocks any of the 128 queries chose walked twice (row
-//                        maxima, then weights and O += P V); see the comment above the kernel
+//   rq_moba_attend.cu    bf16 caches: the attention on the tensor cores
 //   moba_attend_kernel   fp32 caches.  Per (head, 16 consecutive queries), a warp per query: the blocks
 //                        any of the 16 queries chose pass through shared memory once, 64 positions at a
 //                        time (cp.async, two buffers); a warp folds a chunk into its online softmax
@@ -28,8 +25,6 @@
 #include "rq_device.cuh"
 #include "rq_internal.h"
 #include "rq_stream.cuh"
-#include "rq_tmap.h"
-#include "rq_umma.cuh"
 
 namespace rq {
 
@@ -403,436 +398,7 @@ __global__ void __launch_bounds__(kMobaQueries * 32) moba_attend_kernel(const T 
     }
 }
 
-// ---------------------------------------------------------------- attention on the tensor cores (bf16 caches)
-// Grid (ceil(T / 128), heads).  A CTA owns 128 consecutive queries of a head: they are the 128 lanes of the
-// accumulators, so everything per query (mask, running maximum, sum, weights) is per thread.  The chunks
-// (64 positions) of the blocks ANY of the 128 queries chose are walked twice:
-//   pass 1   S = Q K^T for two chunks at a time (tcgen05.mma, 128 x 128, fp32 in tensor memory, two accumulators);
-//            a thread masks its chunk for its query (block not chosen / positions after the query) and keeps the
-//            running maximum
-//   pass 2   S again; the thread turns its row into weights relative to the query's maximum (summed in fp32 for
-//            the final division), rounds them to bf16 and writes them
-//            into tensor memory (tcgen05.st) as the A operand of the second product, O += P V (128 x D, the values
-//            as an MN-major operand straight from the cache's rows), accumulated in tensor memory over all chunks
-// One thread of a ninth warp starts the tensor-map copies (keys and values of a chunk, two stages each) and the
-// products; the eight other warps read the accumulators (two per query, half of a chunk's positions each).  They meet only through mbarriers; every wait is bounded.
-constexpr int kMobaMmaQueries = 128;
-constexpr int kMobaMmaWarps = 8;               // warps that read the accumulators: two per 32 lanes, half of the columns each
-constexpr int kMobaMmaThreads = (kMobaMmaWarps + 1) * 32;
-constexpr int kMobaMmaStages = 2;
-
-template <int D>
-struct MobaMmaGeom {
-    static constexpr int HALVES = D / 64;
-    static constexpr int Q_BYTES = HALVES * 128 * 128;             // 128 queries
-    static constexpr int KC_BYTES = HALVES * kMobaChunk * 128;     // the keys (or the values) of a chunk
-    static constexpr int OFF_K = Q_BYTES;
-    static constexpr int OFF_V = OFF_K + kMobaMmaStages * KC_BYTES;
-    static constexpr int OFF_MASK = OFF_V + kMobaMmaStages * KC_BYTES;
-    static constexpr int FIXED_BYTES = OFF_MASK + 1024;            // + room to align the base to 1024 bytes
-};
-
-__device__ __forceinline__ uint64_t umma_desc_sw128_mn(uint32_t saddr, uint32_t lbo_bytes)
-{
-    return (uint64_t)((saddr & 0x3FFFFu) >> 4) | ((uint64_t)(lbo_bytes >> 4) << 16) | ((uint64_t)(1024u >> 4) << 32) | (1ull << 46) |
-           (2ull << 61);
-}
-__device__ __forceinline__ float exp2_fast(float x)
-{
-    float y;
-    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-    return y;
-}
-__device__ __forceinline__ uint32_t pack2_bf16(float a, float b)
-{
-    const __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
-    return *reinterpret_cast<const uint32_t *>(&h);
-}
-
-// Walk over the 64-position chunks of the chosen blocks in ascending order: (block, chunk inside the block).
-// A block holds cpb chunks; the walk ends (returns n_chunks) after the last chosen block or at chunk n_chunks.
-struct MobaWalk {
-    int j = -1, r = 0;
-};
-__device__ __forceinline__ int moba_walk_next(MobaWalk &w, const uint32_t *chosen, int nb, int cpb, int n_chunks)
-{
-    if (w.j >= 0 && w.r + 1 < cpb && w.j * cpb + w.r + 1 < n_chunks) return w.j * cpb + ++w.r;
-    int jj = w.j + 1;
-    while (jj < nb) {
-        const uint32_t bits = chosen[jj >> 5] >> (jj & 31);
-        if (bits) {
-            jj += __ffs(bits) - 1;
-            break;
-        }
-        jj = (jj | 31) + 1;
-    }
-    w.j = jj;
-    w.r = 0;
-    return jj < nb ? min(jj * cpb, n_chunks) : n_chunks;
-}
-
-template <int D>
-__global__ void __launch_bounds__(kMobaMmaThreads) moba_mma_kernel(const __grid_constant__ CUtensorMap tmap, int64_t page_cap, int S,
-                                                                  int64_t len, const bf16 *q, int H, int block, int nb,
-                                                                  const uint32_t *masks, float scale_log2, bf16 *o, int32_t *status)
-{
-    using G = MobaMmaGeom<D>;
-    constexpr int NST = kMobaMmaStages;
-    static_assert(NST == 2, "pass 1 uses the key region and the value region as its two stages of two chunks each");
-    // tensor memory, 256 columns.  Pass 1: two score accumulators of 128 columns.  Pass 2: one score accumulator of 64
-    // columns, the output (D columns), two weight buffers of 32 columns (64 positions as bf16 pairs).  With two key and
-    // two value stages a CTA needs 97 KB of shared memory, so that TWO CTAs share an SM: each CTA's chunk is a chain of
-    // dependent steps, and the two chains overlap
-    constexpr uint32_t OFF_O = 64, OFF_P = 64 + D, P_COLS = 32, TCOLS = 256;
-    extern __shared__ __align__(1024) unsigned char msm_raw[];
-    __shared__ __align__(8) uint64_t full_k[NST], full_v[NST], s_ready[2], s_free[2], p_ready[2], pv_done[2], stat_ready;
-    __shared__ __align__(8) uint64_t full1[2], s1_ready[2], s1_free[2];    // pass 1: stage landed, scores ready, scores read
-    __shared__ float2 stat[2][kMobaMmaQueries];                          // pass 1: a query's statistics from its two threads
-    __shared__ uint32_t tbase;
-    unsigned char *msm = msm_raw + ((1024u - (smem_addr(msm_raw) & 1023u)) & 1023u);
-    unsigned char *qs = msm, *kst = msm + G::OFF_K, *vst = msm + G::OFF_V;
-    const int words = (nb + 31) / 32;
-    uint32_t *umask = reinterpret_cast<uint32_t *>(msm + G::OFF_MASK);   // blocks chosen by any query of the CTA
-    uint32_t *qmask = umask + words;                                     // [128][words] blocks chosen by each query
-
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    // the work of a CTA grows with the position of its queries (the blocks before them): the CTAs of the last
-    // queries of every head start first, so that the short ones fill the end of the launch
-    const int bh = blockIdx.x, b = bh / H, h = bh % H;
-    const int64_t t0 = (int64_t)(gridDim.y - 1 - blockIdx.y) * kMobaMmaQueries;
-    // chunks of 64 positions up to the CTA's last query; chunk c belongs to block c * 64 / block
-    const int n_chunks_all = (int)((min(t0 + kMobaMmaQueries, len) + kMobaChunk - 1) / kMobaChunk);
-
-    if (tid == 0) {
-        for (int s = 0; s < NST; ++s) { mbar_init(&full_k[s], 1); mbar_init(&full_v[s], 1); }
-        for (int s = 0; s < 2; ++s) {
-            mbar_init(&s_ready[s], 1);
-            mbar_init(&pv_done[s], 1);
-            mbar_init(&s_free[s], kMobaMmaWarps * 32);
-            mbar_init(&p_ready[s], kMobaMmaWarps * 32);
-            mbar_init(&full1[s], 1);
-            mbar_init(&s1_ready[s], 1);
-            mbar_init(&s1_free[s], kMobaMmaWarps * 32);
-        }
-        mbar_init(&stat_ready, kMobaMmaWarps * 32);
-        mbar_init_fence();
-    }
-    if (warp == 0) tmem_alloc(&tbase, TCOLS);
-    for (int i = tid; i < words * (kMobaMmaQueries + 1); i += kMobaMmaThreads) umask[i] = 0u;
-    // the queries (q is [B][T][H][D]) as the K-major operand; rows past the prompt are zero
-    for (int i = tid; i < 128 * (D / 8); i += kMobaMmaThreads) {
-        const int r = i / (D / 8), c = i % (D / 8);
-        uint4 v = make_uint4(0u, 0u, 0u, 0u);
-        if (t0 + r < len) v = *reinterpret_cast<const uint4 *>(q + (((int64_t)b * len + t0 + r) * H + h) * D + c * 8);
-        *reinterpret_cast<uint4 *>(qs + (c >> 3) * (128 * 128) + umma_sw128_offset(r, c & 7)) = v;
-    }
-    __syncthreads();
-    if (t0 + tid < len && tid < kMobaMmaQueries)
-        for (int w = 0; w < words; ++w) {
-            const uint32_t m = masks[((int64_t)bh * len + t0 + tid) * words + w];
-            qmask[tid * words + w] = m;
-            if (m) atomicOr(&umask[w], m);
-        }
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // the queries, written with ordinary stores, are read by the tensor core
-    tcgen05_before_sync();
-    __syncthreads();
-    tcgen05_after_sync();
-    const uint32_t tb = tbase;
-    // number of chunks the CTA walks in one pass: the chunks of the chosen blocks, below the CTA's last chunk
-    const int cpb = block / kMobaChunk;
-    const int ppc = kMobaChunk / S;                  // pages of a chunk (a page holds 16 or 64 positions)
-    int n = 0;
-    for (int wd = 0; wd < words; ++wd) {
-        uint32_t bits = umask[wd];
-        while (bits) {
-            const int j = wd * 32 + __ffs(bits) - 1;
-            bits &= bits - 1;
-            n += max(0, min(cpb, n_chunks_all - j * cpb));
-        }
-    }
-    // the next chunk of a walk (both roles walk the same chunks in the same order)
-    auto next_chunk = [&](MobaWalk &w) { return moba_walk_next(w, umask, nb, cpb, n_chunks_all); };
-    bool ok = true;
-
-    if (warp == kMobaMmaWarps) {
-        if (lane == 0) {
-            // ---- copies and products; hh counts the chunks of pass 2
-            MobaWalk wk, wv, w1;                     // chunk walks of pass 2's key copies and value copies, and of pass 1
-            int gk_issued = 0, hv_issued = 0, gk_landed = 0, hv_landed = 0;
-            auto issue_k = [&]() {                   // keys of the next chunk of the walk into stage gk_issued % NST
-                const int ck_issue = next_chunk(wk);
-                const int st = gk_issued % NST;
-                const int page = (int)((int64_t)bh * page_cap + ck_issue * ppc);
-                mbar_arrive_expect_tx(&full_k[st], G::KC_BYTES);
-#pragma unroll
-                for (int hf = 0; hf < G::HALVES; ++hf)
-                    tma_load_4d(kst + (size_t)st * G::KC_BYTES + hf * (kMobaChunk * 128), &tmap, hf * 64, 0, 0, page, &full_k[st]);
-                ++gk_issued;
-            };
-            auto issue_v = [&]() {
-                const int cv_issue = next_chunk(wv);
-                const int st = hv_issued % NST;
-                const int page = (int)((int64_t)bh * page_cap + cv_issue * ppc);
-                mbar_arrive_expect_tx(&full_v[st], G::KC_BYTES);
-#pragma unroll
-                for (int hf = 0; hf < G::HALVES; ++hf)
-                    tma_load_4d(vst + (size_t)st * G::KC_BYTES + hf * (kMobaChunk * 128), &tmap, hf * 64, 0, 1, page, &full_v[st]);
-                ++hv_issued;
-            };
-            auto product_pv = [&](int hh) -> bool {  // O += P(hh) V(hh)
-                if (!mbar_wait(&p_ready[hh & 1], (uint32_t)((hh >> 1) & 1))) return false;
-                if (!mbar_wait(&full_v[hh % NST], (uint32_t)((hh / NST) & 1))) return false;
-                hv_landed = hh + 1;
-                tcgen05_after_sync();
-                constexpr uint32_t idesc = umma_idesc_bf16(128, D) | (1u << 16);       // the values are MN-major
-                const uint32_t pa = tb + OFF_P + (uint32_t)(hh & 1) * P_COLS, va = smem_addr(vst + (size_t)(hh % NST) * G::KC_BYTES);
-#pragma unroll
-                for (int k = 0; k < kMobaChunk / 16; ++k)
-                    umma_bf16_ta(tb + OFF_O, pa + k * 8, umma_desc_sw128_mn(va + k * 2048, kMobaChunk * 128), idesc,
-                                 (hh > 0 || k > 0) ? 1u : 0u);
-                umma_commit(&pv_done[hh & 1]);
-                return true;
-            };
-            // ---- pass 1: the queries' maxima.  Two chunks (128 keys) per product; the key region and the value region
-            // are its two stages; two accumulators of 128 columns (the columns pass 2 uses for scores, output and weights)
-            const uint32_t qa = smem_addr(qs);
-            const int n1 = (n + 1) / 2;
-            int issued1 = 0, landed1 = 0;
-            auto issue1 = [&](int it) {
-                unsigned char *dst = (it & 1) ? vst : kst;
-                const int cnt = min(2, n - 2 * it);
-                mbar_arrive_expect_tx(&full1[it & 1], (uint32_t)cnt * G::KC_BYTES);
-                for (int u = 0; u < cnt; ++u) {
-                    const int c1 = next_chunk(w1);
-                    const int page = (int)((int64_t)bh * page_cap + c1 * ppc);
-#pragma unroll
-                    for (int hf = 0; hf < G::HALVES; ++hf)
-                        tma_load_4d(dst + hf * (128 * 128) + u * (kMobaChunk * 128), &tmap, hf * 64, 0, 0, page, &full1[it & 1]);
-                }
-                issued1 = it + 1;
-            };
-            issue1(0);
-            if (n1 > 1) issue1(1);
-            constexpr uint32_t idesc_1 = umma_idesc_bf16(128, 2 * kMobaChunk);
-#pragma unroll 1
-            for (int it = 0; it < n1 && ok; ++it) {
-                if (it >= 2) ok = mbar_wait(&s1_free[it & 1], (uint32_t)(((it >> 1) - 1) & 1));
-                ok = ok && mbar_wait(&full1[it & 1], (uint32_t)((it >> 1) & 1));
-                if (!ok) break;
-                landed1 = it + 1;
-                tcgen05_after_sync();
-                const uint32_t sa = smem_addr((it & 1) ? vst : kst);
-#pragma unroll
-                for (int k = 0; k < D / 16; ++k)
-                    umma_bf16(tb + (uint32_t)(it & 1) * 128u, umma_desc_sw128(qa + (k >> 2) * (128 * 128) + (k & 3) * 32),
-                              umma_desc_sw128(sa + (k >> 2) * (128 * 128) + (k & 3) * 32), idesc_1, k > 0);
-                umma_commit(&s1_ready[it & 1]);
-                if (it >= 1 && it + 1 < n1) {        // the stage of product it - 1 takes the chunks of product it + 1
-                    ok = mbar_wait(&s1_ready[(it - 1) & 1], (uint32_t)(((it - 1) >> 1) & 1));
-                    if (ok) issue1(it + 1);
-                }
-            }
-            // pass 2 reuses the stages and the tensor memory: the last products are complete and their scores read
-            for (int it = max(0, n1 - 2); it < n1 && ok; ++it)
-                ok = mbar_wait(&s1_ready[it & 1], (uint32_t)((it >> 1) & 1)) && mbar_wait(&s1_free[it & 1], (uint32_t)((it >> 1) & 1));
-            for (int k = landed1; k < issued1; ++k) mbar_wait(&full1[k & 1], (uint32_t)((k >> 1) & 1));
-
-            // ---- pass 2: weights and output, a chunk per step
-            if (ok) {
-                for (int s = 0; s < NST && s < n; ++s) issue_k();
-                for (int s = 0; s < NST && s < n; ++s) issue_v();
-            }
-            constexpr uint32_t idesc_s = umma_idesc_bf16(128, kMobaChunk);
-#pragma unroll 1
-            for (int hh = 0; hh < n && ok; ++hh) {
-                if (hh >= 1) ok = mbar_wait(&s_free[0], (uint32_t)((hh - 1) & 1));
-                ok = ok && mbar_wait(&full_k[hh % NST], (uint32_t)((hh / NST) & 1));
-                if (!ok) break;
-                gk_landed = hh + 1;
-                tcgen05_after_sync();
-                const uint32_t ka = smem_addr(kst + (size_t)(hh % NST) * G::KC_BYTES);
-#pragma unroll
-                for (int k = 0; k < D / 16; ++k)
-                    umma_bf16(tb, umma_desc_sw128(qa + (k >> 2) * (128 * 128) + (k & 3) * 32),
-                              umma_desc_sw128(ka + (k >> 2) * (kMobaChunk * 128) + (k & 3) * 32), idesc_s, k > 0);
-                umma_commit(&s_ready[0]);
-                if (hh >= 1) ok = product_pv(hh - 1);
-                // refills: the key stage of chunk hh - 1 (its scores have been read), the value stage of chunk hh - 2 once
-                // the second product of that chunk is complete
-                if (ok && hh >= 1 && hh - 1 + NST < n) issue_k();
-                if (ok && hh >= 2 && hh - 2 + NST < n) {
-                    ok = mbar_wait(&pv_done[(hh - 2) & 1], (uint32_t)(((hh - 2) >> 1) & 1));
-                    if (ok) issue_v();
-                }
-            }
-            if (ok) ok = product_pv(n - 1);
-            // after a wait that ran out: no copy may still be on its way into this CTA's shared memory when it exits
-            for (int k = gk_landed; k < gk_issued; ++k) mbar_wait(&full_k[k % NST], (uint32_t)((k / NST) & 1));
-            for (int k = hv_landed; k < hv_issued; ++k) mbar_wait(&full_v[k % NST], (uint32_t)((k / NST) & 1));
-        }
-    } else {
-        // ---- the eight warps that read the accumulators: warps w and w + 4 share the 32 lanes (queries) of tensor-memory
-        // subpartition w; the first takes the chunk's first 32 positions, the second the other 32
-        const int lq = (warp & 3) * 32 + lane;       // this thread's query inside the CTA
-        const int ch = warp >> 2;                    // which half of a chunk's positions
-        const int64_t tq = t0 + lq;
-        const uint32_t tl = tb + ((uint32_t)((warp & 3) * 32) << 16);
-        const uint32_t *mymask = qmask + lq * words;
-        float m = -CUDART_INF_F, l = 0.0f, inv_l = 0.0f;
-        MobaWalk wr;
-        // ---- pass 1: the maximum of the scores this query attends.  A product covers two chunks; of a query's two
-        // threads the first takes the first chunk, the second the other one.
-        const int n1 = (n + 1) / 2;
-#pragma unroll 1
-        for (int it = 0; it < n1; ++it) {
-            const int ca = next_chunk(wr), ja = wr.j;
-            const int cb2 = 2 * it + 1 < n ? next_chunk(wr) : -1;
-            const int cm = ch == 0 ? ca : cb2;       // this thread's chunk (none: -1)
-            int nv = 0;
-            if (cm >= 0 && tq < len) {
-                const int j = ch == 0 ? ja : wr.j;
-                if ((mymask[j >> 5] >> (j & 31)) & 1u) nv = (int)max((int64_t)0, min((int64_t)kMobaChunk, tq - (int64_t)cm * kMobaChunk + 1));
-            }
-            ok = mbar_wait(&s1_ready[it & 1], (uint32_t)((it >> 1) & 1));
-            if (!__all_sync(FULLMASK, ok)) break;
-            tcgen05_after_sync();
-#pragma unroll 1
-            for (int cb = 0; cb < kMobaChunk; cb += 32) {
-                float v[32];
-                tmem_ld32(tl + (uint32_t)(it & 1) * 128u + (uint32_t)(ch * kMobaChunk + cb), v);
-                if (cb < nv) {
-                    float tm = -CUDART_INF_F;
-#pragma unroll
-                    for (int i = 0; i < 32; ++i) tm = fmaxf(tm, cb + i < nv ? v[i] : -CUDART_INF_F);
-                    m = fmaxf(m, tm * scale_log2);
-                }
-            }
-            tcgen05_before_sync();
-            mbar_arrive(&s1_free[it & 1]);
-        }
-        // the query's maximum over everything it attends: its two threads exchange theirs
-        if (__all_sync(FULLMASK, ok)) {
-            stat[ch][lq] = make_float2(m, 0.0f);
-            mbar_arrive(&stat_ready);
-            ok = mbar_wait(&stat_ready, 0u);
-            if (__all_sync(FULLMASK, ok)) m = fmaxf(m, stat[ch ^ 1][lq].x);
-        }
-        // ---- pass 2: the same chunks one by one; of a query's two threads each takes 32 of a chunk's positions
-        wr = MobaWalk();
-#pragma unroll 1
-        for (int hh = 0; hh < n; ++hh) {
-            if (!__all_sync(FULLMASK, ok)) break;
-            const int c = next_chunk(wr), j = wr.j;
-            const int64_t p0 = (int64_t)c * kMobaChunk + ch * 32;    // first of this thread's 32 positions
-            // positions this query attends among them: none if it did not choose the block, else those up to its own
-            int nv = 0;
-            if (tq < len && ((mymask[j >> 5] >> (j & 31)) & 1u)) nv = (int)max((int64_t)0, min((int64_t)32, tq - p0 + 1));
-            ok = mbar_wait(&s_ready[0], (uint32_t)(hh & 1));
-            if (!__all_sync(FULLMASK, ok)) break;
-            tcgen05_after_sync();
-            if (hh >= 2) {                           // the weights buffer hh & 1 was read by the product of chunk hh - 2
-                ok = mbar_wait(&pv_done[hh & 1], (uint32_t)(((hh - 2) >> 1) & 1));
-                if (!__all_sync(FULLMASK, ok)) break;
-            }
-            float v[32];
-            tmem_ld32(tl + (uint32_t)(ch * 32), v);
-            {
-                // weights of 32 positions relative to the query's maximum (at most 1), rounded to bf16: 16 columns of
-                // this query's lane; their sum is kept in fp32 and divides the output at the end
-                uint32_t w[16];
-#pragma unroll
-                for (int i = 0; i < 32; i += 2) {
-                    const float a = i < nv ? exp2_fast(fmaf(v[i], scale_log2, -m)) : 0.0f;
-                    const float bq = i + 1 < nv ? exp2_fast(fmaf(v[i + 1], scale_log2, -m)) : 0.0f;
-                    l += a + bq;
-                    w[i >> 1] = pack2_bf16(a, bq);
-                }
-                tmem_st16(tl + OFF_P + (uint32_t)(hh & 1) * P_COLS + (uint32_t)(ch * 16), w);
-            }
-            tcgen05_before_sync();
-            mbar_arrive(&s_free[0]);                 // this thread has read the scores
-            if ((int64_t)c * kMobaChunk + kMobaChunk > len) {
-                // the prompt ends inside this chunk: the value rows past its end hold whatever the cache's memory held;
-                // a weight of zero would not stop a NaN there, so those rows are cleared once they have landed
-                ok = mbar_wait(&full_v[hh % NST], (uint32_t)((hh / NST) & 1));
-                if (!__all_sync(FULLMASK, ok)) break;
-                const int r = tid & (kMobaChunk - 1), hf = tid >> 6;
-                if (hf < G::HALVES && (int64_t)c * kMobaChunk + r >= len) {
-                    uint4 *row = reinterpret_cast<uint4 *>(vst + (size_t)(hh % NST) * G::KC_BYTES + hf * (kMobaChunk * 128) + (r >> 3) * 1024 +
-                                                           (r & 7) * 128);
-#pragma unroll
-                    for (int i = 0; i < 8; ++i) row[i] = make_uint4(0u, 0u, 0u, 0u);
-                }
-                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // ordinary stores, read by the tensor core
-            }
-            tmem_st_wait();                          // the weights are in tensor memory
-            tcgen05_before_sync();
-            mbar_arrive(&p_ready[hh & 1]);
-        }
-        // the output once the last product is complete: each of a query's two threads writes half of the channels,
-        // divided by the sum of the query's weights (the two threads' sums, exchanged through shared memory)
-        if (__all_sync(FULLMASK, ok)) {
-            stat[ch][lq] = make_float2(l, 0.0f);
-            mbar_arrive(&stat_ready);
-            ok = mbar_wait(&stat_ready, 1u);
-        }
-        if (__all_sync(FULLMASK, ok)) {
-            l += stat[ch ^ 1][lq].x;
-            inv_l = l > 0.0f ? 1.0f / l : 0.0f;
-            ok = mbar_wait(&pv_done[(n - 1) & 1], (uint32_t)(((n - 1) >> 1) & 1));
-            if (__all_sync(FULLMASK, ok)) {
-                tcgen05_after_sync();
-#pragma unroll 1
-                for (int cb = ch * (D / 2); cb < (ch + 1) * (D / 2); cb += 32) {
-                    float v[32];
-                    tmem_ld32(tl + OFF_O + (uint32_t)cb, v);
-                    if (tq < len) {
-                        bf16 *orow = o + (((int64_t)b * len + tq) * H + h) * D + cb;
-#pragma unroll
-                        for (int i = 0; i < 32; i += 8)
-                            *reinterpret_cast<uint4 *>(orow + i) =
-                                make_uint4(pack2_bf16(v[i] * inv_l, v[i + 1] * inv_l), pack2_bf16(v[i + 2] * inv_l, v[i + 3] * inv_l),
-                                           pack2_bf16(v[i + 4] * inv_l, v[i + 5] * inv_l), pack2_bf16(v[i + 6] * inv_l, v[i + 7] * inv_l));
-                    }
-                }
-            }
-        }
-    }
-    if (__any_sync(FULLMASK, !ok) && lane == 0) atomicCAS(status, RQ_OK, RQ_ERR_TIMEOUT);
-    tcgen05_before_sync();
-    __syncthreads();
-    if (warp == 0) tmem_dealloc(tbase, TCOLS);
-}
-
 size_t round256(size_t x) { return (x + 255) & ~(size_t)255; }
-
-// bf16 caches: representatives and routing (rq_moba_route.cu), attention on the tensor cores.
-template <int D>
-cudaError_t moba_run_bf16(const MobaArgs &a, cudaStream_t s)
-{
-    using G = MobaMmaGeom<D>;
-    const int BH = a.B * a.H, nb = (int)((a.len + a.block - 1) / a.block), words = (nb + 31) / 32;
-    static bool ready[64];
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return e;
-    if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
-    if (!ready[dev]) {
-        e = cudaFuncSetAttribute(moba_mma_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)((size_t)G::FIXED_BYTES + (size_t)(kMobaMaxBlocks / 32) * (kMobaMmaQueries + 1) * sizeof(uint32_t)));
-        if (e != cudaSuccess) return e;
-        ready[dev] = true;
-    }
-    alignas(64) CUtensorMap tmap;
-    e = cache_tensor_map(&tmap, a.kv, D, a.S, (int64_t)BH * a.page_cap, kMobaChunk);
-    if (e != cudaSuccess) return e;
-    e = launch_moba_route_bf16(a, s);
-    if (e != cudaSuccess) return e;
-    const size_t ms = (size_t)G::FIXED_BYTES + (size_t)words * (kMobaMmaQueries + 1) * sizeof(uint32_t);
-    moba_mma_kernel<D><<<dim3((unsigned)BH, (unsigned)((a.len + kMobaMmaQueries - 1) / kMobaMmaQueries)), kMobaMmaThreads, ms, s>>>(
-        tmap, a.page_cap, a.S, a.len, (const bf16 *)a.q, a.H, a.block, nb, a.masks, a.scale * 1.4426950408889634f, (bf16 *)a.o, a.status);
-    return cudaGetLastError();
-}
 
 // fp32 caches: everything on plain fp32 FMAs (tf32 products would round the operands).
 template <int D>
@@ -905,11 +471,11 @@ void moba_carve(void *scratch, int BH, int64_t len, int D, int block, int dtype,
 cudaError_t launch_moba(const MobaArgs &a, cudaStream_t s)
 {
     if (a.block < kMobaChunk || a.block % kMobaChunk != 0 || a.block % a.S != 0 || a.K < 2 || a.len < 1) return cudaErrorInvalidValue;
-    if ((a.len + a.block - 1) / a.block > kMobaMaxBlocks || a.B * a.H > 65535 || (a.len + kMobaMmaQueries - 1) / kMobaMmaQueries > 65535)
+    if ((a.len + a.block - 1) / a.block > kMobaMaxBlocks || a.B * a.H > 65535 || (a.len + 127) / 128 > 65535)
         return cudaErrorInvalidValue;
     if (a.dtype == RQ_BF16) {
-        if (a.D == 128) return moba_run_bf16<128>(a, s);
-        if (a.D == 64) return moba_run_bf16<64>(a, s);
+        const cudaError_t e = launch_moba_route_bf16(a, s);
+        return e != cudaSuccess ? e : launch_moba_attend_bf16(a, s);
     } else {
         if (a.D == 128) return moba_run_f32<128>(a, s);
         if (a.D == 64) return moba_run_f32<64>(a, s);

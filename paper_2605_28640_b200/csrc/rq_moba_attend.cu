@@ -1,0 +1,410 @@
+// MoBA attention for bf16 caches (Sec. 2.2, Eq. 4; App. A.1, MoBA paragraph): softmax attention of every prompt
+// position over the positions up to its own of the blocks it chose, both contractions on the tensor cores (tcgen05).
+#include <math_constants.h>
+
+#include "rq_async.cuh"
+#include "rq_device.cuh"
+#include "rq_internal.h"
+#include "rq_tmap.h"
+#include "rq_umma.cuh"
+
+namespace rq {
+
+namespace {
+
+constexpr unsigned FULL = 0xffffffffu;
+constexpr int kChunk = 64;                     // positions of a step
+constexpr int kTile = 128;                     // queries of an accumulator (its lanes)
+constexpr int kTiles = 2;                      // accumulators of a CTA: 256 consecutive queries share the keys and values
+constexpr int kStages = 4;                     // chunks of keys, and of values, in shared memory
+constexpr int kReadWarps = 4 * kTiles;         // warps that turn scores into weights: a thread per query
+constexpr int kThreads = (kReadWarps + 2) * 32;
+constexpr float kRaise = 8.0f;                 // powers of two a query's maximum may grow before its output is rescaled
+
+template <int D> struct AttGeom {
+    static constexpr int HALVES = D / 64;
+    static constexpr int Q_BYTES = HALVES * kTile * 128;           // the queries of one accumulator
+    static constexpr int C_BYTES = HALVES * kChunk * 128;          // the keys (or the values) of a chunk
+    static constexpr int OFF_K = kTiles * Q_BYTES;
+    static constexpr int OFF_V = OFF_K + kStages * C_BYTES;
+    static constexpr int OFF_LIST = OFF_V + kStages * C_BYTES;     // blocks to walk
+    static constexpr int SMEM_BYTES = OFF_LIST + kMobaMaxBlocks * 2 + 1024;   // + room to align the base to 1024 bytes
+};
+
+__device__ __forceinline__ uint64_t desc_sw128_mn(uint32_t saddr, uint32_t lbo_bytes)
+{
+    return (uint64_t)((saddr & 0x3FFFFu) >> 4) | ((uint64_t)(lbo_bytes >> 4) << 16) | ((uint64_t)(1024u >> 4) << 32) | (1ull << 46) |
+           (2ull << 61);
+}
+__device__ __forceinline__ float exp2_fast(float x)
+{
+    float y;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+
+// The walk over the chunks of the listed blocks: (entry of the list, chunk inside the block).
+struct Walk {
+    int bi = 0, r = 0;
+    __device__ __forceinline__ void next(int cpb)
+    {
+        if (++r == cpb) { r = 0; ++bi; }
+    }
+};
+
+// Grid (heads, tiles of 256 queries; the last queries of a head first: their work is the largest).  A CTA owns 256
+// consecutive queries as two accumulators of 128 lanes; everything per query (choice of blocks, causal cut, running
+// maximum, sum, weights) belongs to one thread.  The 64-position chunks of the blocks that any of the 256 queries chose
+// are walked once:
+//   S = Q K^T        128 x 64 per accumulator, fp32 in tensor memory, two score buffers per accumulator, so that the
+//                    product of the next chunk runs while the weights of this one are computed
+//   weights          2^(s - m) for the chosen blocks' positions up to the query's own, rounded to bf16, written over
+//                    the first half of their scores as the A operand of the second product; summed in fp32
+//   O += P V         accumulated in tensor memory over all chunks
+// m is the query's largest score so far, but it is raised (and the query's row of O multiplied down) only when a score
+// exceeds it by more than 8 powers of two: weights of up to 256 lose nothing in bf16 and fp32, and the output is divided
+// by their sum at the end, so that O is hardly ever touched between the products.
+// Warps 0..7 read scores, warp 8 starts the tensor-map copies, warp 9 the products; they meet through mbarriers only,
+// every wait bounded.  256 queries per CTA because keys and values come from L2 for every CTA.
+template <int D>
+__global__ void __launch_bounds__(kThreads, 1) moba_mma_kernel(const __grid_constant__ CUtensorMap tmap, int64_t page_cap, int S,
+                                                               int64_t len, const bf16 *q, int H, int block, int nb,
+                                                               const uint32_t *masks, float scale_log2, bf16 *o, int32_t *status)
+{
+    using G = AttGeom<D>;
+    constexpr int NST = kStages;
+    // tensor memory of accumulator s: columns s * 256: two score buffers of 64 columns (their first 32 hold the weights
+    // afterwards), then the output
+    constexpr uint32_t ACC = 256, OFF_O = 128;
+    extern __shared__ __align__(1024) unsigned char asm_raw[];
+    __shared__ __align__(8) uint64_t full_k[NST], full_v[NST], free_k[NST], free_v[NST];
+    __shared__ __align__(8) uint64_t s_ready[kTiles][2], p_ready[kTiles][2], pv_done[kTiles][2];
+    __shared__ uint32_t um[kTiles][kMobaMaxBlocks / 32];         // blocks chosen by any query of an accumulator
+    __shared__ uint32_t tbase;
+    __shared__ int n_list;
+    unsigned char *sm = asm_raw + ((1024u - (smem_addr(asm_raw) & 1023u)) & 1023u);
+    unsigned char *qs = sm, *kst = sm + G::OFF_K, *vst = sm + G::OFF_V;
+    uint16_t *list = reinterpret_cast<uint16_t *>(sm + G::OFF_LIST);   // block | 0x4000 (first accumulator) | 0x8000 (second)
+    const int words = (nb + 31) / 32;
+
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int bh = blockIdx.x, b = bh / H, h = bh % H;
+    const int64_t t0 = (int64_t)(gridDim.y - 1 - blockIdx.y) * (kTile * kTiles);
+    const int n_chunks_all = (int)((min(t0 + kTile * kTiles, len) + kChunk - 1) / kChunk);
+    const int cpb = block / kChunk;                              // chunks of a block
+    const int ppc = kChunk / S;                                  // pages of a chunk
+
+    if (tid == 0) {
+        for (int i = 0; i < NST; ++i) {
+            mbar_init(&full_k[i], 1); mbar_init(&full_v[i], 1);
+            mbar_init(&free_k[i], 1); mbar_init(&free_v[i], 1);
+        }
+        for (int s = 0; s < kTiles; ++s)
+            for (int i = 0; i < 2; ++i) {
+                mbar_init(&s_ready[s][i], 1);
+                mbar_init(&p_ready[s][i], kTile);
+                mbar_init(&pv_done[s][i], 1);
+            }
+        mbar_init_fence();
+    }
+    if (warp == kReadWarps) tmem_alloc(&tbase, 512);
+    for (int i = tid; i < kTiles * words; i += kThreads) um[i / words][i % words] = 0u;
+    // the queries (q is [B][T][H][D]) as K-major operands; rows past the prompt are zero
+    for (int i = tid; i < kTiles * kTile * (D / 8); i += kThreads) {
+        const int r = i / (D / 8), c = i % (D / 8);
+        uint4 v = make_uint4(0u, 0u, 0u, 0u);
+        if (t0 + r < len) v = *reinterpret_cast<const uint4 *>(q + (((int64_t)b * len + t0 + r) * H + h) * D + c * 8);
+        *reinterpret_cast<uint4 *>(qs + (r / kTile) * G::Q_BYTES + (c >> 3) * (kTile * 128) + umma_sw128_offset(r % kTile, c & 7)) = v;
+    }
+    __syncthreads();
+    if (warp < kReadWarps) {
+        const bool in = t0 + tid < len;
+        const uint32_t *row = masks + ((int64_t)bh * len + (in ? t0 + tid : 0)) * words;
+        for (int w = 0; w < words; ++w) {
+            const uint32_t m = __reduce_or_sync(FULL, in ? __ldg(row + w) : 0u);
+            if (lane == 0 && m) atomicOr(&um[warp >> 2][w], m);
+        }
+    }
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // the queries, written with ordinary stores, are read by the tensor core
+    __syncthreads();
+    if (warp == 0) {                                             // the list of blocks, ascending
+        int base = 0;
+        for (int w0 = 0; w0 < words; w0 += 32) {
+            const int w = w0 + lane;
+            const uint32_t m0 = w < words ? um[0][w] : 0u, m1 = w < words ? um[1][w] : 0u;
+            const int cnt = __popc(m0 | m1);
+            int inc = cnt;
+#pragma unroll
+            for (int off = 1; off < 32; off <<= 1) {
+                const int v = __shfl_up_sync(FULL, inc, off);
+                if (lane >= off) inc += v;
+            }
+            int pos = base + inc - cnt;
+            for (uint32_t bits = m0 | m1; bits; bits &= bits - 1u, ++pos) {
+                const int i = __ffs(bits) - 1;
+                list[pos] = (uint16_t)((w * 32 + i) | (((m0 >> i) & 1u) << 14) | (((m1 >> i) & 1u) << 15));
+            }
+            base += __shfl_sync(FULL, inc, 31);
+        }
+        if (lane == 0) n_list = base;
+    }
+    tcgen05_before_sync();
+    __syncthreads();
+    tcgen05_after_sync();
+    const uint32_t tb = tbase;
+    // steps of the walk: whole blocks, the last one (the last query's own) up to the CTA's last chunk
+    const int nl = n_list, n = (nl - 1) * cpb + min(cpb, n_chunks_all - (list[nl - 1] & 0x3fff) * cpb);
+    bool ok = true;
+
+    if (warp == kReadWarps) {
+        // ---- copies
+        if (lane == 0) {
+            Walk w;
+            int issued = 0;
+#pragma unroll 1
+            for (int i = 0; i < n; ++i, w.next(cpb)) {
+                const int st = i % NST;
+                if (i >= NST) {
+                    const uint32_t ph = (uint32_t)((i / NST - 1) & 1);
+                    ok = mbar_wait(&free_k[st], ph) && mbar_wait(&free_v[st], ph);
+                    if (!ok) break;
+                }
+                const int page = (int)((int64_t)bh * page_cap + (int64_t)((list[w.bi] & 0x3fff) * cpb + w.r) * ppc);
+                mbar_arrive_expect_tx(&full_k[st], G::C_BYTES);
+#pragma unroll
+                for (int hf = 0; hf < G::HALVES; ++hf)
+                    tma_load_4d(kst + (size_t)st * G::C_BYTES + hf * (kChunk * 128), &tmap, hf * 64, 0, 0, page, &full_k[st]);
+                mbar_arrive_expect_tx(&full_v[st], G::C_BYTES);
+#pragma unroll
+                for (int hf = 0; hf < G::HALVES; ++hf)
+                    tma_load_4d(vst + (size_t)st * G::C_BYTES + hf * (kChunk * 128), &tmap, hf * 64, 0, 1, page, &full_v[st]);
+                issued = i + 1;
+            }
+            // after a wait that ran out: no copy may still be on its way into this CTA's shared memory when it exits
+            if (!ok)
+                for (int k = max(0, issued - NST); k < issued; ++k) {
+                    mbar_wait(&full_k[k % NST], (uint32_t)((k / NST) & 1));
+                    mbar_wait(&full_v[k % NST], (uint32_t)((k / NST) & 1));
+                }
+        }
+    } else if (warp == kReadWarps + 1) {
+        // ---- products
+        if (lane == 0) {
+            constexpr uint32_t idesc_s = umma_idesc_bf16(kTile, kChunk);
+            constexpr uint32_t idesc_o = umma_idesc_bf16(kTile, D) | (1u << 16);       // the values are MN-major
+            const uint64_t qd = umma_desc_sw128(smem_addr(qs)), kd = umma_desc_sw128(smem_addr(kst));
+            const uint64_t vd = desc_sw128_mn(smem_addr(vst), kChunk * 128);
+            int us[kTiles] = {0, 0}, up[kTiles] = {0, 0};        // score products and output products started
+            Walk ws, wp;
+            auto scores = [&](int i) -> bool {
+                const int st = i % NST;
+                const uint32_t e = list[ws.bi];
+                ws.next(cpb);
+                if (!mbar_wait(&full_k[st], (uint32_t)((i / NST) & 1))) return false;
+                tcgen05_after_sync();
+#pragma unroll
+                for (int s = 0; s < kTiles; ++s) {
+                    if (!((e >> (14 + s)) & 1u)) continue;
+                    const int u = us[s]++;
+                    if (u >= 2 && !mbar_wait(&pv_done[s][u & 1], (uint32_t)(((u >> 1) - 1) & 1))) return false;   // the buffer's weights were used
+#pragma unroll
+                    for (int k = 0; k < D / 16; ++k)
+                        umma_bf16(tb + s * ACC + (uint32_t)(u & 1) * kChunk,
+                                  qd + (uint64_t)((s * G::Q_BYTES + (k >> 2) * (kTile * 128) + (k & 3) * 32) >> 4),
+                                  kd + (uint64_t)((st * G::C_BYTES + (k >> 2) * (kChunk * 128) + (k & 3) * 32) >> 4), idesc_s, k > 0);
+                    umma_commit(&s_ready[s][u & 1]);
+                }
+                umma_commit(&free_k[st]);
+                return true;
+            };
+            auto output = [&](int i) -> bool {
+                const int st = i % NST;
+                const uint32_t e = list[wp.bi];
+                wp.next(cpb);
+                if (!mbar_wait(&full_v[st], (uint32_t)((i / NST) & 1))) return false;
+#pragma unroll
+                for (int s = 0; s < kTiles; ++s) {
+                    if (!((e >> (14 + s)) & 1u)) continue;
+                    const int u = up[s]++;
+                    if (!mbar_wait(&p_ready[s][u & 1], (uint32_t)((u >> 1) & 1))) return false;
+                    tcgen05_after_sync();
+#pragma unroll
+                    for (int k = 0; k < kChunk / 16; ++k)
+                        umma_bf16_ta(tb + s * ACC + OFF_O, tb + s * ACC + (uint32_t)(u & 1) * kChunk + k * 8,
+                                     vd + (uint64_t)((st * G::C_BYTES + k * 2048) >> 4), idesc_o, (u > 0 || k > 0) ? 1u : 0u);
+                    umma_commit(&pv_done[s][u & 1]);
+                }
+                umma_commit(&free_v[st]);
+                return true;
+            };
+            ok = scores(0);
+#pragma unroll 1
+            for (int i = 0; i < n && ok; ++i) {
+                if (i + 1 < n) ok = scores(i + 1);
+                ok = ok && output(i);
+            }
+        }
+    } else {
+        // ---- weights: a thread per query
+        const int s = warp >> 2, lq = (warp & 3) * 32 + lane;
+        const int64_t tq = t0 + s * kTile + lq;
+        const bool in = tq < len;
+        const uint32_t tl = tb + s * ACC + ((uint32_t)((warp & 3) * 32) << 16);
+        const uint32_t *row = masks + ((int64_t)bh * len + (in ? tq : 0)) * words;
+        uint32_t w_cur = 0u, w_next = 0u;                        // the query's choice of the 32 blocks around the walk, and of the next 32
+        int w_at = -1;
+        float m = -CUDART_INF_F;                                 // what the weights are relative to (scaled, log2)
+        float2 l2 = make_float2(0.0f, 0.0f);                     // sums of the weights (even and odd positions)
+        const float2 sc2 = make_float2(scale_log2, scale_log2);
+        int u = 0;
+        Walk wk;
+#pragma unroll 1
+        for (int i = 0; i < n; ++i, wk.next(cpb)) {
+            const uint32_t e = list[wk.bi];
+            if (!((e >> (14 + s)) & 1u)) continue;
+            const int j = e & 0x3fff;
+            if ((j >> 5) != w_at) {
+                const int w = j >> 5;
+                w_cur = w_at >= 0 && w == w_at + 1 ? w_next : in ? __ldg(row + w) : 0u;
+                w_next = in && w + 1 < words ? __ldg(row + w + 1) : 0u;
+                w_at = w;
+            }
+            const int c = j * cpb + wk.r;
+            const int64_t p0 = (int64_t)c * kChunk;
+            // positions this query attends among the chunk's: none if it did not choose the block, else those up to its own
+            int nv = 0;
+            if (in && ((w_cur >> (j & 31)) & 1u)) nv = (int)max((int64_t)0, min((int64_t)kChunk, tq - p0 + 1));
+            ok = mbar_wait(&s_ready[s][u & 1], (uint32_t)((u >> 1) & 1));
+            if (!__all_sync(FULL, ok)) break;
+            tcgen05_after_sync();
+            const uint32_t ts = tl + (uint32_t)(u & 1) * kChunk;
+            if (__any_sync(FULL, nv > 0)) {
+                float v[kChunk];
+                tmem_ld64(ts, v);
+                const bool cut = __any_sync(FULL, nv > 0 && nv < kChunk);
+                if (cut) {
+#pragma unroll
+                    for (int k = 0; k < kChunk; ++k) v[k] = k < nv ? v[k] : -CUDART_INF_F;
+                }
+                float tm[4] = {v[0], v[1], v[2], v[3]};
+#pragma unroll
+                for (int k = 4; k < kChunk; ++k) tm[k & 3] = fmaxf(tm[k & 3], v[k]);
+                const float top = fmaxf(fmaxf(tm[0], tm[1]), fmaxf(tm[2], tm[3])) * scale_log2;
+                const bool raise = nv > 0 && top > m + kRaise;
+                if (__any_sync(FULL, raise)) {
+                    const bool touch = raise && m > -CUDART_INF_F;         // (otherwise the query's row of O is still zero)
+                    const float f = touch ? exp2_fast(m - top) : 1.0f;
+                    if (raise) m = top;
+                    if (__any_sync(FULL, touch)) {
+                        l2.x *= f;
+                        l2.y *= f;
+                        ok = mbar_wait(&pv_done[s][(u - 1) & 1], (uint32_t)(((u - 1) >> 1) & 1));   // nothing is being added to O
+                        if (!__all_sync(FULL, ok)) break;
+                        tcgen05_after_sync();
+#pragma unroll 1
+                        for (int cb = 0; cb < D; cb += 16) {
+                            uint32_t x[16];
+                            tmem_ld16(tl + OFF_O + cb, x);
+#pragma unroll
+                            for (int k = 0; k < 16; ++k) x[k] = __float_as_uint(__uint_as_float(x[k]) * f);
+                            tmem_st16(tl + OFF_O + cb, x);
+                        }
+                    }
+                }
+                const float nm = nv > 0 ? -m : -3.0e38f;         // a block the query did not choose: 2^-3e38 = 0
+                const float2 nm2 = make_float2(nm, nm), one2 = make_float2(1.0f, 1.0f);
+#pragma unroll
+                for (int hf = 0; hf < 2; ++hf) {
+                    uint32_t w[16];
+#pragma unroll
+                    for (int k = 0; k < 16; ++k) {
+                        const float2 x = fma2(make_float2(v[hf * 32 + 2 * k], v[hf * 32 + 2 * k + 1]), sc2, nm2);
+                        const float2 p = make_float2(exp2_fast(x.x), exp2_fast(x.y));
+                        l2 = fma2(p, one2, l2);
+                        w[k] = pack_bf16(p.x, p.y);
+                    }
+                    tmem_st16(ts + hf * 16, w);
+                }
+            } else {                                             // none of the warp's queries chose the block
+                const uint32_t z[16] = {0u, 0u, 0u, 0u, 0u, 0u, 0u, 0u, 0u, 0u, 0u, 0u, 0u, 0u, 0u, 0u};
+                tmem_st16(ts, z);
+                tmem_st16(ts + 16, z);
+            }
+            if (p0 + kChunk > len) {
+                // the prompt ends inside this chunk: the value rows past its end hold whatever the cache's memory held; a
+                // weight of zero would not stop a NaN there, so those rows are cleared once they have landed
+                ok = mbar_wait(&full_v[i % NST], (uint32_t)((i / NST) & 1));
+                if (!__all_sync(FULL, ok)) break;
+                const int r = lq & (kChunk - 1), hf = lq >> 6;
+                if (hf < G::HALVES && p0 + r >= len) {
+                    uint4 *vrow = reinterpret_cast<uint4 *>(vst + (size_t)(i % NST) * G::C_BYTES + hf * (kChunk * 128) + (r >> 3) * 1024 +
+                                                            (r & 7) * 128);
+#pragma unroll
+                    for (int k = 0; k < 8; ++k) vrow[k] = make_uint4(0u, 0u, 0u, 0u);
+                }
+                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // ordinary stores, read by the tensor core
+            }
+            tmem_st_wait();                                      // the weights are in tensor memory
+            tcgen05_before_sync();
+            mbar_arrive(&p_ready[s][u & 1]);
+            ++u;
+        }
+        // the output once the last product is complete, divided by the sum of the query's weights
+        if (__all_sync(FULL, ok) && u > 0) {
+            ok = mbar_wait(&pv_done[s][(u - 1) & 1], (uint32_t)(((u - 1) >> 1) & 1));
+            if (__all_sync(FULL, ok)) {
+                tcgen05_after_sync();
+                const float l = l2.x + l2.y, inv = l > 0.0f ? 1.0f / l : 0.0f;
+#pragma unroll 1
+                for (int cb = 0; cb < D; cb += 32) {
+                    float v[32];
+                    tmem_ld32(tl + OFF_O + cb, v);
+                    if (in) {
+                        bf16 *orow = o + (((int64_t)b * len + tq) * H + h) * D + cb;
+#pragma unroll
+                        for (int k = 0; k < 32; k += 8)
+                            *reinterpret_cast<uint4 *>(orow + k) =
+                                make_uint4(pack_bf16(v[k] * inv, v[k + 1] * inv), pack_bf16(v[k + 2] * inv, v[k + 3] * inv),
+                                           pack_bf16(v[k + 4] * inv, v[k + 5] * inv), pack_bf16(v[k + 6] * inv, v[k + 7] * inv));
+                    }
+                }
+            }
+        }
+    }
+    if (__any_sync(FULL, !ok) && lane == 0) atomicCAS(status, RQ_OK, RQ_ERR_TIMEOUT);
+    tcgen05_before_sync();
+    __syncthreads();
+    if (warp == kReadWarps) tmem_dealloc(tbase, 512);
+}
+
+template <int D> cudaError_t attend_run(const MobaArgs &a, cudaStream_t s)
+{
+    using G = AttGeom<D>;
+    const int BH = a.B * a.H, nb = (int)((a.len + a.block - 1) / a.block);
+    static bool ready[64];
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
+    if (!ready[dev]) {
+        e = cudaFuncSetAttribute(moba_mma_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, G::SMEM_BYTES);
+        if (e != cudaSuccess) return e;
+        ready[dev] = true;
+    }
+    alignas(64) CUtensorMap tmap;
+    e = cache_tensor_map(&tmap, a.kv, D, a.S, (int64_t)BH * a.page_cap, kChunk);
+    if (e != cudaSuccess) return e;
+    const unsigned tiles = (unsigned)((a.len + kTile * kTiles - 1) / (kTile * kTiles));
+    moba_mma_kernel<D><<<dim3((unsigned)BH, tiles), kThreads, G::SMEM_BYTES, s>>>(
+        tmap, a.page_cap, a.S, a.len, (const bf16 *)a.q, a.H, a.block, nb, a.masks, a.scale * 1.4426950408889634f, (bf16 *)a.o, a.status);
+    return cudaGetLastError();
+}
+
+}  // namespace
+
+cudaError_t launch_moba_attend_bf16(const MobaArgs &a, cudaStream_t s)
+{
+    return a.D == 128 ? attend_run<128>(a, s) : a.D == 64 ? attend_run<64>(a, s) : cudaErrorInvalidValue;
+}
+
+}  // namespace rq
