@@ -151,14 +151,14 @@ __global__ void __launch_bounds__(kThreads, 1) moba_mma_kernel(const __grid_cons
     tcgen05_before_sync();
     __syncthreads();
     tcgen05_after_sync();
-    const uint32_t tb = tbase;
+    const uint32_t tb = __shfl_sync(FULL, tbase, 0);             // (the shuffle tells the compiler that it is uniform)
     // steps of the walk: whole blocks, the last one (the last query's own) up to the CTA's last chunk
     const int nl = n_list, n = (nl - 1) * cpb + min(cpb, n_chunks_all - (list[nl - 1] & 0x3fff) * cpb);
     bool ok = true;
 
     if (warp == kReadWarps) {
-        // ---- copies
-        if (lane == 0) {
+        // ---- copies (the whole warp, like the products below: see rq_umma.cuh)
+        {
             Walk w;
             int issued = 0;
 #pragma unroll 1
@@ -167,14 +167,15 @@ __global__ void __launch_bounds__(kThreads, 1) moba_mma_kernel(const __grid_cons
                 if (i >= NST) {
                     const uint32_t ph = (uint32_t)((i / NST - 1) & 1);
                     ok = mbar_wait(&free_k[st], ph) && mbar_wait(&free_v[st], ph);
+                    ok = __all_sync(FULL, ok);
                     if (!ok) break;
                 }
-                const int page = (int)((int64_t)bh * page_cap + (int64_t)((list[w.bi] & 0x3fff) * cpb + w.r) * ppc);
-                mbar_arrive_expect_tx(&full_k[st], G::C_BYTES);
+                const int page = (int)((int64_t)bh * page_cap + (int64_t)(__shfl_sync(FULL, list[w.bi] & 0x3fff, 0) * cpb + w.r) * ppc);
+                mbar_expect_warp(&full_k[st], G::C_BYTES);
 #pragma unroll
                 for (int hf = 0; hf < G::HALVES; ++hf)
                     tma_load_4d(kst + (size_t)st * G::C_BYTES + hf * (kChunk * 128), &tmap, hf * 64, 0, 0, page, &full_k[st]);
-                mbar_arrive_expect_tx(&full_v[st], G::C_BYTES);
+                mbar_expect_warp(&full_v[st], G::C_BYTES);
 #pragma unroll
                 for (int hf = 0; hf < G::HALVES; ++hf)
                     tma_load_4d(vst + (size_t)st * G::C_BYTES + hf * (kChunk * 128), &tmap, hf * 64, 0, 1, page, &full_v[st]);
@@ -189,7 +190,7 @@ __global__ void __launch_bounds__(kThreads, 1) moba_mma_kernel(const __grid_cons
         }
     } else if (warp == kReadWarps + 1) {
         // ---- products
-        if (lane == 0) {
+        {
             constexpr uint32_t idesc_s = umma_idesc_bf16(kTile, kChunk);
             constexpr uint32_t idesc_o = umma_idesc_bf16(kTile, D) | (1u << 16);       // the values are MN-major
             const uint64_t qd = umma_desc_sw128(smem_addr(qs)), kd = umma_desc_sw128(smem_addr(kst));
@@ -198,15 +199,16 @@ __global__ void __launch_bounds__(kThreads, 1) moba_mma_kernel(const __grid_cons
             Walk ws, wp;
             auto scores = [&](int i) -> bool {
                 const int st = i % NST;
-                const uint32_t e = list[ws.bi];
+                const uint32_t e = __shfl_sync(FULL, (uint32_t)list[ws.bi], 0);
                 ws.next(cpb);
-                if (!mbar_wait(&full_k[st], (uint32_t)((i / NST) & 1))) return false;
+                if (!__all_sync(FULL, mbar_wait(&full_k[st], (uint32_t)((i / NST) & 1)))) return false;
                 tcgen05_after_sync();
 #pragma unroll
                 for (int s = 0; s < kTiles; ++s) {
                     if (!((e >> (14 + s)) & 1u)) continue;
                     const int u = us[s]++;
-                    if (u >= 2 && !mbar_wait(&pv_done[s][u & 1], (uint32_t)(((u >> 1) - 1) & 1))) return false;   // the buffer's weights were used
+                    if (u >= 2 && !__all_sync(FULL, mbar_wait(&pv_done[s][u & 1], (uint32_t)(((u >> 1) - 1) & 1))))
+                        return false;                            // (the product that uses the buffer's weights)
 #pragma unroll
                     for (int k = 0; k < D / 16; ++k)
                         umma_bf16(tb + s * ACC + (uint32_t)(u & 1) * kChunk,
@@ -219,14 +221,14 @@ __global__ void __launch_bounds__(kThreads, 1) moba_mma_kernel(const __grid_cons
             };
             auto output = [&](int i) -> bool {
                 const int st = i % NST;
-                const uint32_t e = list[wp.bi];
+                const uint32_t e = __shfl_sync(FULL, (uint32_t)list[wp.bi], 0);
                 wp.next(cpb);
-                if (!mbar_wait(&full_v[st], (uint32_t)((i / NST) & 1))) return false;
+                if (!__all_sync(FULL, mbar_wait(&full_v[st], (uint32_t)((i / NST) & 1)))) return false;
 #pragma unroll
                 for (int s = 0; s < kTiles; ++s) {
                     if (!((e >> (14 + s)) & 1u)) continue;
                     const int u = up[s]++;
-                    if (!mbar_wait(&p_ready[s][u & 1], (uint32_t)((u >> 1) & 1))) return false;
+                    if (!__all_sync(FULL, mbar_wait(&p_ready[s][u & 1], (uint32_t)((u >> 1) & 1)))) return false;
                     tcgen05_after_sync();
 #pragma unroll
                     for (int k = 0; k < kChunk / 16; ++k)

@@ -180,43 +180,45 @@ __global__ void __launch_bounds__(kRouteThreads) moba_route_mma_kernel(const bf1
         tcgen05_before_sync();
         __syncthreads();
         tcgen05_after_sync();
-        const uint32_t tb = tbase, tl = tb + ((uint32_t)((warp & 3) * 32) << 16);
+        const uint32_t tb = __shfl_sync(FULL, tbase, 0), tl = tb + ((uint32_t)((warp & 3) * 32) << 16);
         const unsigned char *src = planes + (int64_t)bh * groups_all * G::GROUP_BYTES;
-        int issued = 0, used = 0;                                              // thread 0: copies started, copies multiplied
+        int issued = 0, used = 0;                                              // warp 0: copies started, copies multiplied
         uint32_t panel_phase = 0u;
 
-        // the scores of panel p into tensor memory; thread 0 starts copies and products
+        // the scores of panel p into tensor memory; the first warp starts copies and products
         auto panel = [&](int p) {
-            if (tid == 0 && ok) {
+            if (warp == 0 && ok) {                                             // (the whole warp, see rq_umma.cuh)
                 const int g0 = p * kPanelGroups, gn = min(kPanelGroups, groups - g0);
                 auto issue = [&](int g) {
                     const int st = issued % stages;
-                    mbar_arrive_expect_tx(&full[st], G::GROUP_BYTES);
-                    bulk_g2s(bs + (size_t)st * G::GROUP_BYTES, src + (int64_t)g * G::GROUP_BYTES, G::GROUP_BYTES, &full[st]);
+                    if (lane == 0) {
+                        mbar_arrive_expect_tx(&full[st], G::GROUP_BYTES);
+                        bulk_g2s(bs + (size_t)st * G::GROUP_BYTES, src + (int64_t)g * G::GROUP_BYTES, G::GROUP_BYTES, &full[st]);
+                    }
+                    __syncwarp();
                     ++issued;
                 };
                 constexpr uint32_t idesc = umma_idesc_bf16(NQ, kRouteGroup);
-                const uint32_t qa = smem_addr(qs);
+                const uint64_t qd = umma_desc_sw128(smem_addr(qs)), bd = umma_desc_sw128(smem_addr(bs));
                 tcgen05_after_sync();
                 for (int g = 0; g < gn && g < stages; ++g) issue(g0 + g);
 #pragma unroll 1
                 for (int g = 0; g < gn; ++g) {
                     const int st = used % stages;
                     const uint32_t phase = (uint32_t)((used / stages) & 1);
-                    ok = mbar_wait(&full[st], phase);
+                    ok = __all_sync(FULL, mbar_wait(&full[st], phase));
                     if (!ok) break;
                     ++used;
-                    const uint32_t ba = smem_addr(bs + (size_t)st * G::GROUP_BYTES);
 #pragma unroll
                     for (int pl = 2; pl >= 0; --pl)                            // the smallest terms first
 #pragma unroll
                         for (int k = 0; k < D / 16; ++k)
-                            umma_bf16(tb + (uint32_t)g * kRouteGroup, umma_desc_sw128(qa + (k >> 2) * (NQ * 128) + (k & 3) * 32),
-                                      umma_desc_sw128(ba + pl * G::PLANE_BYTES + (k >> 2) * (kRouteGroup * 128) + (k & 3) * 32), idesc,
+                            umma_bf16(tb + (uint32_t)g * kRouteGroup, qd + (uint64_t)(((k >> 2) * (NQ * 128) + (k & 3) * 32) >> 4),
+                                      bd + (uint64_t)((st * G::GROUP_BYTES + pl * G::PLANE_BYTES + (k >> 2) * (kRouteGroup * 128) + (k & 3) * 32) >> 4), idesc,
                                       !(pl == 2 && k == 0));
                     umma_commit(&done[st]);
                     if (g + stages < gn) {
-                        ok = mbar_wait(&done[st], phase);
+                        ok = __all_sync(FULL, mbar_wait(&done[st], phase));
                         if (!ok) break;
                         issue(g0 + g + stages);
                     }

@@ -226,7 +226,7 @@ __global__ void __launch_bounds__(kMmaThreads) snap_mma_kernel(const __grid_cons
     const int t0 = blockIdx.x * tiles_per_cta, n = min(tiles_per_cta, ntiles - t0);
     const int64_t first_q = len - W;                           // position of query 0
     const int ppt = kMmaKeys / S;                              // pages per tile
-    int n_issued = 0, n_landed = 0;                            // thread 0: tiles whose copies were started / seen complete
+    int n_issued = 0, n_landed = 0;                            // the producing warp: tiles whose copies were started / seen complete
 
     if (tid == 0) {
         mbar_init(&bar[0], 1);
@@ -250,12 +250,12 @@ __global__ void __launch_bounds__(kMmaThreads) snap_mma_kernel(const __grid_cons
     }
     // the keys of tile t (relative to t0) into its stage: position j lives in page j / S, slot j % S of the
     // head's cache; pages past the head's last one hold somebody else's rows or nothing, and every key at
-    // or beyond `len` is masked where the scores are used.  One thread.
+    // or beyond `len` is masked where the scores are used.  One warp.
     auto issue = [&](int i) {
         const int stage = i % NST;
         unsigned char *dst = ks + (size_t)stage * G::TILE_BYTES;
         const int page = (int)((int64_t)bh * page_cap + (int64_t)(t0 + i) * ppt);
-        mbar_arrive_expect_tx(&full[stage], G::TILE_BYTES);
+        mbar_expect_warp(&full[stage], G::TILE_BYTES);
 #pragma unroll
         for (int hh = 0; hh < G::HALVES; ++hh) tma_load_4d(dst + hh * G::HALF_BYTES, &tmap, hh * 64, 0, 0, page, &full[stage]);
         n_issued = i + 1;
@@ -270,15 +270,15 @@ __global__ void __launch_bounds__(kMmaThreads) snap_mma_kernel(const __grid_cons
     tcgen05_before_sync();
     __syncthreads();
     tcgen05_after_sync();
-    const uint32_t tb = tbase;
+    const uint32_t tb = __shfl_sync(0xffffffffu, tbase, 0);     // (the shuffle tells the compiler that it is uniform)
 
     const int row = tid & (kSnapRows - 1), half = (tid >> 6) & 1;   // pass 1: this thread's query and half of the tile's keys
     float m = -CUDART_INF_F, l = 0.0f;                         // pass 1: running statistics
     bool ok = true;
     if (warp == kMmaWarps) {
-        // ---- the producing warp: one thread starts the copies and the products; nobody else waits for it
-        // except through the barriers
-        if (lane == 0) {
+        // ---- the producing warp starts the copies and the products (all its lanes run this, see rq_umma.cuh);
+        // nobody else waits for it except through the barriers
+        {
             for (int t = NST; t < kMmaAhead && t < n; ++t) {       // the tiles between the first copies and the first prefetch
                 const int page = (int)((int64_t)bh * page_cap + (int64_t)(t0 + t) * ppt);
 #pragma unroll
@@ -286,28 +286,27 @@ __global__ void __launch_bounds__(kMmaThreads) snap_mma_kernel(const __grid_cons
             }
             for (int s = 0; s < NST && s < n; ++s) issue(s);
             constexpr uint32_t idesc = PASS == 1 ? umma_idesc_bf16(128, kMmaKeys) : umma_idesc_bf16(kMmaKeys, kSnapRows);
-            const uint32_t qa = smem_addr(qs);
+            const uint64_t qd = umma_desc_sw128(smem_addr(qs)), kd = umma_desc_sw128(smem_addr(ks));
 #pragma unroll 1
             for (int i = 0; i < n && ok; ++i) {
                 // accumulator i & 1 has been read (tile i - 2), the tile's keys have landed
-                if (i >= 2) ok = mbar_wait(&acc_free[i & 1], (uint32_t)(((i >> 1) - 1) & 1));
-                ok = ok && mbar_wait(&full[i % NST], (uint32_t)((i / NST) & 1));
+                if (i >= 2) ok = __all_sync(0xffffffffu, mbar_wait(&acc_free[i & 1], (uint32_t)(((i >> 1) - 1) & 1)));
+                ok = ok && __all_sync(0xffffffffu, mbar_wait(&full[i % NST], (uint32_t)((i / NST) & 1)));
                 if (!ok) break;
                 n_landed = i + 1;
                 tcgen05_after_sync();
-                const uint32_t ka = smem_addr(ks + (size_t)(i % NST) * G::TILE_BYTES);
                 const uint32_t acc = tb + (uint32_t)(i & 1) * ACC;
 #pragma unroll
                 for (int k = 0; k < D / 16; ++k) {
                     const uint32_t off = (uint32_t)(k >> 2) * G::HALF_BYTES + (uint32_t)(k & 3) * 32u;
-                    const uint64_t dq = umma_desc_sw128(qa + off), dk = umma_desc_sw128(ka + off);
+                    const uint64_t dq = qd + (uint64_t)(off >> 4), dk = kd + (uint64_t)(((i % NST) * G::TILE_BYTES + off) >> 4);
                     if (PASS == 1) umma_bf16(acc, dq, dk, idesc, k > 0);
                     else umma_bf16(acc, dk, dq, idesc, k > 0);
                 }
                 umma_commit(&bar[i & 1]);
                 // the stage of tile i - 1 is free once its product has completed; it takes tile i - 1 + NST
                 if (i >= 1 && i - 1 + NST < n) {
-                    ok = mbar_wait(&bar[(i - 1) & 1], (uint32_t)(((i - 1) >> 1) & 1));
+                    ok = __all_sync(0xffffffffu, mbar_wait(&bar[(i - 1) & 1], (uint32_t)(((i - 1) >> 1) & 1)));
                     if (ok) issue(i - 1 + NST);
                 }
             }
