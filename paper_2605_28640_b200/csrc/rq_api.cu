@@ -603,16 +603,18 @@ int rq_snapkv_compact(const rq_cache *src, const int32_t *idx, int32_t keep, rq_
         return RQ_ERR_INVALID_ARG;
     if (keep > b.capacity_tokens) return RQ_ERR_CAPACITY;
     cudaStream_t s = (cudaStream_t)stream;
-    rc = rq_cache_reset(dst, stream);                    // empties dst, clears its bookkeeping
-    if (rc != RQ_OK) return rc;
-    const int BH = a.batch * a.heads;
-    if (launch_snap_compact(src->kv, src->page_capacity, dst->kv, dst->meta, dst->page_capacity, a.page_size, a.head_dim,
-                            a.dtype, idx, keep, absmax_of(dst), BH, s) != cudaSuccess)
-        return RQ_ERR_CUDA;
-    // the recurrence goes on from where the prompt ended
-    if (cudaMemcpyAsync(dst->state, src->state, (size_t)BH * 2 * a.head_dim * sizeof(float), cudaMemcpyDeviceToDevice, s) !=
-        cudaSuccess)
-        return RQ_ERR_CUDA;
+    // dst starts over: its bookkeeping is cleared here, its recurrence state comes from src in the kernel
+    const WorkspaceLayout w = workspace_layout(b);
+    if (cudaMemsetAsync((char *)dst->workspace + w.status, 0, w.scores - w.status, s) != cudaSuccess) return RQ_ERR_CUDA;
+    dst->len = 0;
+    SnapCompactArgs ca;
+    ca.skv = src->kv; ca.s_page_cap = src->page_capacity;
+    ca.dkv = dst->kv; ca.dmeta = dst->meta; ca.d_page_cap = dst->page_capacity;
+    ca.S = a.page_size; ca.D = a.head_dim; ca.dtype = a.dtype; ca.BH = a.batch * a.heads; ca.keep = keep;
+    ca.idx = idx;
+    ca.sstate = (const float *)src->state; ca.dstate = (float *)dst->state;
+    ca.absmax = absmax_of(dst);
+    if (launch_snap_compact(ca, s) != cudaSuccess) return RQ_ERR_CUDA;
     dst->len = keep;
     return RQ_OK;
 }

@@ -157,8 +157,18 @@ size_t snap_scratch_bytes(int BH, int64_t len);
 void snap_carve(void *scratch, int BH, int64_t len, float **imp, float2 **stats, float2 **rowstat);
 cudaError_t launch_snap_scores(const SnapArgs &a, cudaStream_t s);
 cudaError_t launch_snap_select(const float *imp, int BH, int64_t len, int window, int keep, int32_t *idx, cudaStream_t s);
-cudaError_t launch_snap_compact(const void *skv, int64_t s_page_cap, void *dkv, void *dmeta, int64_t d_page_cap, int S, int D,
-                                int dtype, const int32_t *idx, int keep, float *absmax, int BH, cudaStream_t s);
+struct SnapCompactArgs {
+    const void *skv;    // the source cache
+    int64_t s_page_cap;
+    void *dkv, *dmeta;  // the new cache
+    int64_t d_page_cap;
+    int S, D, dtype, BH, keep;
+    const int32_t *idx; // [BH][keep]
+    const float *sstate;
+    float *dstate;      // the recurrence state is carried over
+    float *absmax;      // [2][BH] of the new cache, zero before the launch (NULL: not tracked)
+};
+cudaError_t launch_snap_compact(const SnapCompactArgs &a, cudaStream_t s);
 
 // ---- MoBA-style block-sparse prefill attention (rq_moba.cu) ----
 struct MobaArgs {

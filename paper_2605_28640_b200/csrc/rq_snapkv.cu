@@ -535,60 +535,138 @@ __global__ void __launch_bounds__(1024) snap_select_kernel(const float *imp, int
 }
 
 // ---------------------------------------------------------------- compaction into the new cache
-// One CTA of 256 threads per (head, page of the new cache).  The page's retained rows move in 16-byte
-// pieces, keys and values alike (a thread per piece, a row's pieces on neighbouring threads); the keys
-// also pass through shared memory, from which a thread per channel then takes the page's bounds.
-constexpr int kCompactThreads = 256;
-constexpr int kCompactSmem = 64 * 128 * 4;                 // the keys of one page at most: 64 slots x 128 channels x 4 bytes
+// Grid (runs of 64 slots of the new cache, heads), four warps of 16 slots each.  A warp reads its 16 retained rows, keys
+// and values, in 16-byte pieces, LPR lanes to a row, all loads in flight before the first store; the page's bounds are
+// taken from the keys in registers (a page of 64 slots: the four warps' bounds meet in shared memory).  The CTA of a
+// head's first slots also carries the recurrence state over.
+// Bound: single rows of 256 bytes (D = 128, bf16) scattered over the source, i.e. the DRAM accesses in flight.  A CTA
+// per page with two loads per thread between barriers kept 57 KB in flight per SM; here up to 190 KB.  32 heads,
+// 8192 of 131000 entries each (268 MB moved): 143 -> 57 us; 256 heads, 1024 of 4096: 70 -> 42 us.
+constexpr int kCompactWarps = 4;
 
-template <typename T>
-__global__ void __launch_bounds__(kCompactThreads) snap_compact_kernel(const T *skv, int64_t s_page_cap, T *dkv, T *dmeta,
-                                                                       int64_t d_page_cap, int S, int D, const int32_t *idx,
-                                                                       int keep, float *absmax, int BH)
+__device__ __forceinline__ uint32_t min_word(bf16, uint32_t a, uint32_t b)
 {
-    __shared__ __align__(16) unsigned char krows[kCompactSmem];
-    __shared__ int32_t src_pos[64];
-    const int bh = blockIdx.y, page = blockIdx.x, tid = threadIdx.x;
-    const int rb = D * (int)sizeof(T), ppr = rb / 16;        // bytes and 16-byte pieces of a row
-    const int rows = min(S, keep - page * S);                // retained rows of this page (at least one)
-    if (tid < S) src_pos[tid] = tid < rows ? idx[(int64_t)bh * keep + page * S + tid] : -1;
-    __syncthreads();
-    unsigned char *dpage = reinterpret_cast<unsigned char *>(dkv + (((int64_t)bh * d_page_cap + page) * 2) * S * D);
-    const unsigned char *shead = reinterpret_cast<const unsigned char *>(skv + (int64_t)bh * s_page_cap * 2 * S * D);
-    for (int i = tid; i < S * ppr; i += kCompactThreads) {
-        const int r = i / ppr, c = i % ppr;
-        uint4 kq = make_uint4(0u, 0u, 0u, 0u), vq = kq;      // unused slots of the last page are defined (zero)
-        if (r < rows) {
-            const int64_t pos = src_pos[r];
-            const unsigned char *src = shead + ((pos / S) * 2 * S + pos % S) * (int64_t)rb + c * 16;
-            kq = *reinterpret_cast<const uint4 *>(src);
-            vq = *reinterpret_cast<const uint4 *>(src + (int64_t)S * rb);
-        }
-        *reinterpret_cast<uint4 *>(dpage + (int64_t)r * rb + c * 16) = kq;
-        *reinterpret_cast<uint4 *>(dpage + (int64_t)(S + r) * rb + c * 16) = vq;
-        *reinterpret_cast<uint4 *>(krows + r * rb + c * 16) = kq;
-    }
-    __syncthreads();
+    const __nv_bfloat162 m = __hmin2(*reinterpret_cast<__nv_bfloat162 *>(&a), *reinterpret_cast<__nv_bfloat162 *>(&b));
+    return *reinterpret_cast<const uint32_t *>(&m);
+}
+__device__ __forceinline__ uint32_t max_word(bf16, uint32_t a, uint32_t b)
+{
+    const __nv_bfloat162 m = __hmax2(*reinterpret_cast<__nv_bfloat162 *>(&a), *reinterpret_cast<__nv_bfloat162 *>(&b));
+    return *reinterpret_cast<const uint32_t *>(&m);
+}
+__device__ __forceinline__ uint32_t min_word(float, uint32_t a, uint32_t b)
+{
+    return __float_as_uint(fminf(__uint_as_float(a), __uint_as_float(b)));
+}
+__device__ __forceinline__ uint32_t max_word(float, uint32_t a, uint32_t b)
+{
+    return __float_as_uint(fmaxf(__uint_as_float(a), __uint_as_float(b)));
+}
+// largest absolute value in a word
+__device__ __forceinline__ float abs_word(bf16, uint32_t w) { return fmaxf(fabsf(bf16lo(w)), fabsf(bf16hi(w))); }
+__device__ __forceinline__ float abs_word(float, uint32_t w) { return fabsf(__uint_as_float(w)); }
+
+template <typename T, int D, int S>
+__global__ void __launch_bounds__(kCompactWarps * 32) snap_compact_kernel(const T *skv, int64_t s_page_cap, T *dkv, T *dmeta,
+                                                                          int64_t d_page_cap, const int32_t *idx, int keep,
+                                                                          const float *sstate, float *dstate, float *absmax, int BH)
+{
+    constexpr int RB = D * (int)sizeof(T), LPR = RB / 16, RPL = 32 / LPR;   // bytes and lanes of a row, rows of a warp-wide read
+    constexpr int NR = 16 / RPL;                             // reads of 16 rows
+    constexpr int NB = NR > 8 ? 8 : NR;                      // of which this many are in flight at a time, keys and values each
+    constexpr unsigned FULL = 0xffffffffu;
+    __shared__ __align__(16) uint4 smn[kCompactWarps][LPR], smx[kCompactWarps][LPR];
+    const int bh = blockIdx.y, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int slot0 = blockIdx.x * 64 + warp * 16;           // first slot (position in the new cache) of this warp
+    const int rsub = lane / LPR, piece = lane % LPR;
+    if (blockIdx.x == 0)
+        for (int i = tid; i < 2 * D; i += kCompactWarps * 32) dstate[(int64_t)bh * 2 * D + i] = sstate[(int64_t)bh * 2 * D + i];
+    const int rows = min(16, keep - slot0);                  // retained rows of this warp (none: <= 0)
+    const int64_t page = slot0 / S;
+    const bool here = page * S < keep;                       // the page exists (its unused slots are written as zero)
     float am = 0.0f;
-    if (tid < D) {
-        const T *kr = reinterpret_cast<const T *>(krows);
-        float mn = CUDART_INF_F, mx = -CUDART_INF_F;
-        for (int r = 0; r < rows; ++r) {
-            const float kf = load1<T>(kr + r * D + tid);
-            mn = fminf(mn, kf);
-            mx = fmaxf(mx, kf);
-        }
-        T *mrow = dmeta + (((int64_t)bh * d_page_cap + page) * 2) * D;
-        store1<T>(mrow + tid, mn);
-        store1<T>(mrow + D + tid, mx);
-        am = fmaxf(-mn, mx);
-    }
-    if (absmax && tid < D) {                                 // D is a multiple of 32: whole warps
+    uint32_t mn[4], mx[4];
 #pragma unroll
-        for (int off = 16; off > 0; off >>= 1) am = fmaxf(am, __shfl_xor_sync(0xffffffffu, am, off));
-        if ((tid & 31) == 0) {
-            atomicMax(reinterpret_cast<unsigned *>(absmax) + bh, __float_as_uint(am));
-            atomicMax(reinterpret_cast<unsigned *>(absmax) + BH + bh, __float_as_uint(am));
+    for (int i = 0; i < 4; ++i) {
+        mn[i] = sizeof(T) == 2 ? 0x7f807f80u : 0x7f800000u;  // +inf, -inf
+        mx[i] = sizeof(T) == 2 ? 0xff80ff80u : 0xff800000u;
+    }
+    if (here) {
+        const unsigned char *shead = reinterpret_cast<const unsigned char *>(skv + (int64_t)bh * s_page_cap * 2 * S * D);
+        unsigned char *dst = reinterpret_cast<unsigned char *>(dkv + ((int64_t)bh * d_page_cap + page) * 2 * S * D) +
+                             (int64_t)(slot0 % S) * RB + piece * 16;
+        const int pos_lane = lane < rows ? idx[(int64_t)bh * keep + slot0 + lane] : -1;
+#pragma unroll
+        for (int n0 = 0; n0 < NR; n0 += NB) {
+            uint4 kq[NB], vq[NB];
+#pragma unroll
+            for (int n = 0; n < NB; ++n) {
+                const int r = (n0 + n) * RPL + rsub, pos = __shfl_sync(FULL, pos_lane, r);
+                kq[n] = vq[n] = make_uint4(0u, 0u, 0u, 0u);
+                if (pos >= 0) {
+                    const unsigned char *src = shead + ((int64_t)(pos / S) * 2 * S + pos % S) * RB + piece * 16;
+                    kq[n] = __ldcs(reinterpret_cast<const uint4 *>(src));
+                    vq[n] = __ldcs(reinterpret_cast<const uint4 *>(src + (int64_t)S * RB));
+                }
+            }
+#pragma unroll
+            for (int n = 0; n < NB; ++n) {
+                const int r = (n0 + n) * RPL + rsub;
+                *reinterpret_cast<uint4 *>(dst + (int64_t)r * RB) = kq[n];
+                *reinterpret_cast<uint4 *>(dst + (int64_t)(S + r) * RB) = vq[n];
+                if (r < rows) {
+                    const uint32_t w[4] = {kq[n].x, kq[n].y, kq[n].z, kq[n].w};
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        mn[i] = min_word(T(), mn[i], w[i]);
+                        mx[i] = max_word(T(), mx[i], w[i]);
+                    }
+                }
+            }
+        }
+#pragma unroll
+        for (int off = LPR; off < 32; off <<= 1)             // the rows of the other lanes
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                mn[i] = min_word(T(), mn[i], __shfl_xor_sync(FULL, mn[i], off));
+                mx[i] = max_word(T(), mx[i], __shfl_xor_sync(FULL, mx[i], off));
+            }
+        if (rows > 0)
+#pragma unroll
+            for (int i = 0; i < 4; ++i) am = fmaxf(am, fmaxf(abs_word(T(), mn[i]), abs_word(T(), mx[i])));
+    }
+    T *mrow = dmeta + ((int64_t)bh * d_page_cap + page) * 2 * D;
+    if (S == 16) {
+        if (here && lane < LPR) {
+            *reinterpret_cast<uint4 *>(mrow + lane * (16 / (int)sizeof(T))) = make_uint4(mn[0], mn[1], mn[2], mn[3]);
+            *reinterpret_cast<uint4 *>(mrow + D + lane * (16 / (int)sizeof(T))) = make_uint4(mx[0], mx[1], mx[2], mx[3]);
+        }
+    } else {
+        if (lane < LPR) {
+            smn[warp][lane] = make_uint4(mn[0], mn[1], mn[2], mn[3]);
+            smx[warp][lane] = make_uint4(mx[0], mx[1], mx[2], mx[3]);
+        }
+        __syncthreads();
+        if (here && warp == 0 && lane < LPR) {
+#pragma unroll
+            for (int w = 1; w < kCompactWarps; ++w) {
+                const uint4 a = smn[w][lane], b = smx[w][lane];
+                const uint32_t aw[4] = {a.x, a.y, a.z, a.w}, bw[4] = {b.x, b.y, b.z, b.w};
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    mn[i] = min_word(T(), mn[i], aw[i]);
+                    mx[i] = max_word(T(), mx[i], bw[i]);
+                }
+            }
+            *reinterpret_cast<uint4 *>(mrow + lane * (16 / (int)sizeof(T))) = make_uint4(mn[0], mn[1], mn[2], mn[3]);
+            *reinterpret_cast<uint4 *>(mrow + D + lane * (16 / (int)sizeof(T))) = make_uint4(mx[0], mx[1], mx[2], mx[3]);
+        }
+    }
+    if (absmax) {                                            // the head's largest |key|, both copies: non-negative floats order like their bits
+        const unsigned m = __reduce_max_sync(FULL, __float_as_uint(am));
+        if (lane == 0 && m != 0u) {
+            atomicMax(reinterpret_cast<unsigned *>(absmax) + bh, m);
+            atomicMax(reinterpret_cast<unsigned *>(absmax) + BH + bh, m);
         }
     }
 }
@@ -714,16 +792,28 @@ cudaError_t launch_snap_select(const float *imp, int BH, int64_t len, int window
     return cudaGetLastError();
 }
 
-cudaError_t launch_snap_compact(const void *skv, int64_t s_page_cap, void *dkv, void *dmeta, int64_t d_page_cap, int S, int D,
-                                int dtype, const int32_t *idx, int keep, float *absmax, int BH, cudaStream_t s)
+template <typename T, int D>
+static void compact_shape(const SnapCompactArgs &a, cudaStream_t s)
 {
-    const dim3 grid((unsigned)((keep + S - 1) / S), (unsigned)BH);
-    if (dtype == RQ_BF16)
-        snap_compact_kernel<bf16><<<grid, kCompactThreads, 0, s>>>((const bf16 *)skv, s_page_cap, (bf16 *)dkv, (bf16 *)dmeta, d_page_cap, S, D, idx,
-                                                     keep, absmax, BH);
+    const dim3 grid((unsigned)((a.keep + 63) / 64), (unsigned)a.BH);
+    if (a.S == 16)
+        snap_compact_kernel<T, D, 16><<<grid, kCompactWarps * 32, 0, s>>>((const T *)a.skv, a.s_page_cap, (T *)a.dkv, (T *)a.dmeta, a.d_page_cap,
+                                                                         a.idx, a.keep, a.sstate, a.dstate, a.absmax, a.BH);
     else
-        snap_compact_kernel<float><<<grid, kCompactThreads, 0, s>>>((const float *)skv, s_page_cap, (float *)dkv, (float *)dmeta, d_page_cap, S, D,
-                                                      idx, keep, absmax, BH);
+        snap_compact_kernel<T, D, 64><<<grid, kCompactWarps * 32, 0, s>>>((const T *)a.skv, a.s_page_cap, (T *)a.dkv, (T *)a.dmeta, a.d_page_cap,
+                                                                         a.idx, a.keep, a.sstate, a.dstate, a.absmax, a.BH);
+}
+
+cudaError_t launch_snap_compact(const SnapCompactArgs &a, cudaStream_t s)
+{
+    if ((a.D != 64 && a.D != 128) || (a.S != 16 && a.S != 64)) return cudaErrorInvalidValue;
+    if (a.dtype == RQ_BF16) {
+        if (a.D == 128) compact_shape<bf16, 128>(a, s);
+        else compact_shape<bf16, 64>(a, s);
+    } else {
+        if (a.D == 128) compact_shape<float, 128>(a, s);
+        else compact_shape<float, 64>(a, s);
+    }
     return cudaGetLastError();
 }
 
