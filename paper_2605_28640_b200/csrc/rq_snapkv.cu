@@ -24,11 +24,11 @@
 //   snap_tile_kernel<1 / 2>   fp32 caches: the same two passes as plain fp32 FMA code (64 x 128
 //                             score tiles in registers, 8 rows x 4 keys per thread)
 //   snap_select_kernel        per head: the keep - W most important positions before the window
-//                             (most-significant-digit radix select on the order-preserving image of the
-//                             importance, equal importance to the lower position) plus the window,
-//                             written in ascending order
-//   snap_compact_kernel       per (head, page of the new cache): gathers the retained rows, rebuilds
-//                             the page's min/max bounds, tracks the head's largest |key|
+//                             (buckets on the order-preserving image of the importance, equal importance
+//                             to the lower position) plus the window, written in ascending order
+//   snap_compact_kernel       per (head, 64 slots of the new cache): gathers the retained rows, rebuilds
+//                             the pages' min/max bounds, tracks the head's largest |key|
+#include <cooperative_groups.h>
 #include <math.h>
 #include <math_constants.h>
 
@@ -412,126 +412,183 @@ __global__ void __launch_bounds__(128) snap_rows_kernel(const float2 *stats, flo
 }
 
 // ---------------------------------------------------------------- token-level selection
-// One CTA of 1024 threads per head.  Candidates: positions 0 .. C-1 (C = len - w, w = window
-// positions kept outright); `want` of them are taken: those with the largest importance, equal
-// importance to the lower position.  Radix select over the order-preserving keys, 11 bits per pass,
-// reading the importances from global memory (L2) each pass; then every warp walks its own
-// contiguous range twice (count, write), so the list comes out ascending.
-__global__ void __launch_bounds__(1024) snap_select_kernel(const float *imp, int64_t len, int w, int keep, int32_t *idx)
+// A cluster of CL CTAs per head.  Candidates: positions 0 .. C-1 (C = len - w, w = window positions kept outright);
+// `want` of them are taken: those with the largest importance, equal importance to the lower position.  A CTA owns a
+// contiguous range of the candidates, a warp a contiguous part of it, a lane every 32nd position, whose
+// order-preserving keys it keeps in registers (EPT per thread; EPT = 0: read again in every pass).  The key of the last
+// position taken is found with 2048 equal-width buckets between the head's smallest and largest key, then again inside
+// the bucket that holds it, at most three times in all; every CTA counts its own keys and adds up the buckets of all
+// CTAs through distributed shared memory.  Then ballots and scans over warps and CTAs give every taken position its
+// place in the ascending list.
+// Bound: latency (a chain of about ten block- or cluster-wide steps).  One CTA per head, digits of 11 bits from the
+// top and the importances read from L2 in every pass: 86 us for 32 heads x 131000 positions, 17 us for 256 x 4096; so: 29
+// and 11 us.
+constexpr int kSelMaxEpt = 32;
+
+template <int EPT, int NT>
+__global__ void __launch_bounds__(NT, 1024 / NT) snap_select_kernel(const float *imp, int64_t len, int w, int keep,
+                                                                                   int per_warp, int32_t *idx)
 {
+    namespace cg = cooperative_groups;
     constexpr unsigned FULL = 0xffffffffu;
-    __shared__ uint32_t hist[kSnapBins];
-    __shared__ uint32_t red[32], red2[32];
-    __shared__ uint32_t s_digit, s_krem, s_cnt;
+    constexpr int NW = NT / 32, BPT = kSnapBins / NT;            // a thread adds up BPT buckets
+    __shared__ __align__(16) uint32_t hist[2][kSnapBins];
+    __shared__ uint32_t red[NW], red2[NW], pub[2];
+    __shared__ uint32_t s_bin, s_krem, s_cnt;
+    cg::cluster_group cl = cg::this_cluster();
+    const int CL = (int)cl.num_blocks(), cr = (int)cl.block_rank();
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int bh = blockIdx.x;
+    const int bh = blockIdx.x / CL;
     const float *x = imp + (int64_t)bh * len;
     int32_t *out = idx + (int64_t)bh * keep;
-    const int C = (int)(len - w);
-    const int want = keep - w;
-    if (want >= C) {                                 // everything is kept
-        for (int j = tid; j < keep; j += 1024) out[j] = j < len ? j : -1;
-        return;
+    const int C = (int)(len - w), want = keep - w;
+    if (want >= C || want <= 0) {                    // everything is kept, or nothing but the window
+        if (cr == 0)
+            for (int j = tid; j < keep; j += NT) out[j] = want <= 0 ? C + j : j < len ? j : -1;
+        return;                                      // (the same for the whole cluster)
     }
-    uint32_t tau = 0xffffffffu;                      // want == 0: nothing but the window
-    int r_eq = 0;
-    if (want > 0) {
-        uint32_t prefix = 0u;
-        int k = want;
-        bool whole = false;
+    const int lo_j = min((int64_t)C, ((int64_t)cr * NW + warp) * per_warp), hi_j = min(C, lo_j + per_warp);
+    uint32_t key[EPT > 0 ? EPT : 1];
+    // body(element number, key) for every key of this thread, absent ones as 0 (below every key of a number)
+    auto for_keys = [&](auto body) {
+        if constexpr (EPT > 0) {
+#pragma unroll
+            for (int i = 0; i < EPT; ++i) body(i, key[i]);
+        } else {
 #pragma unroll 1
-        for (int hi = 31; hi >= 0 && !whole; hi -= 11) {
-            const int lo = hi >= 10 ? hi - 10 : 0;   // this pass decides bits hi .. lo
-            const uint32_t dmask = (1u << (hi - lo + 1)) - 1u;
-            const uint32_t himask = hi == 31 ? 0u : ~0u << (hi + 1);
-            for (int i = tid; i < kSnapBins; i += 1024) hist[i] = 0u;
-            __syncthreads();
-            // eight independent loads per thread are issued before the first is used
-            for (int j0 = tid; j0 < C; j0 += 8 * 1024) {
+            for (int j0 = lo_j; j0 < hi_j; j0 += 8 * 32) {
                 float f[8];
 #pragma unroll
-                for (int u = 0; u < 8; ++u) f[u] = j0 + u * 1024 < C ? __ldcg(x + j0 + u * 1024) : 0.0f;
+                for (int u = 0; u < 8; ++u) f[u] = j0 + u * 32 + lane < hi_j ? __ldcg(x + j0 + u * 32 + lane) : 0.0f;
 #pragma unroll
-                for (int u = 0; u < 8; ++u) {
-                    const uint32_t kx = order_key(f[u]);
-                    if (j0 + u * 1024 < C && (kx & himask) == (prefix & himask)) atomicAdd(&hist[(kx >> lo) & dmask], 1u);
+                for (int u = 0; u < 8; ++u) body((j0 - lo_j) / 32 + u, j0 + u * 32 + lane < hi_j ? order_key(f[u]) : 0u);
+            }
+        }
+    };
+    if constexpr (EPT > 0) {
+        float f[EPT];
+#pragma unroll
+        for (int i = 0; i < EPT; ++i) f[i] = lo_j + i * 32 + lane < hi_j ? __ldcg(x + lo_j + i * 32 + lane) : 0.0f;
+#pragma unroll
+        for (int i = 0; i < EPT; ++i) key[i] = lo_j + i * 32 + lane < hi_j ? order_key(f[i]) : 0u;
+    }
+    // smallest and largest key of the head
+    uint32_t kmin = 0xffffffffu, kmax = 0u;
+    for_keys([&](int, uint32_t k) {
+        kmin = min(kmin, k ? k : 0xffffffffu);
+        kmax = max(kmax, k);
+    });
+    kmin = __reduce_min_sync(FULL, kmin);
+    kmax = __reduce_max_sync(FULL, kmax);
+    if (lane == 0) { red[warp] = kmin; red2[warp] = kmax; }
+#pragma unroll
+    for (int i = 0; i < BPT; ++i) hist[0][tid + i * NT] = 0u;
+    __syncthreads();
+    if (warp == 0) {
+        const uint32_t a = __reduce_min_sync(FULL, lane < NW ? red[lane] : 0xffffffffu), b = __reduce_max_sync(FULL, lane < NW ? red2[lane] : 0u);
+        if (lane == 0) { pub[0] = a; pub[1] = b; }
+    }
+    cl.sync();
+    for (int r = 0; r < CL; ++r) {
+        const uint32_t *p = cl.map_shared_rank(pub, r);
+        kmin = min(kmin, p[0]);
+        kmax = max(kmax, p[1]);
+    }
+    uint32_t tau = 0u, rem = (uint32_t)want;         // keys above tau are taken, and of those equal to it the first r_eq
+    int r_eq = 0;
+#pragma unroll 1
+    for (int it = 0;; ++it) {
+        uint32_t *hs = hist[it & 1];
+        const int sh = max(0, 21 - __clz((int)(kmax - kmin)));           // (kmax - kmin) >> sh < 2048
+        for_keys([&](int, uint32_t k) {
+            if (k >= kmin && k <= kmax) atomicAdd(&hs[(k - kmin) >> sh], 1u);
+        });
+        cl.sync();                                   // (and nobody reads the other buckets any more)
+        uint32_t c[BPT], sum = 0u;                   // the head's buckets BPT tid .. BPT tid + BPT - 1
+#pragma unroll
+        for (int i = 0; i < BPT; ++i) c[i] = 0u;
+        for (int r = 0; r < CL; ++r) {
+            const uint2 *v = reinterpret_cast<const uint2 *>(cl.map_shared_rank(hs, r) + BPT * tid);
+#pragma unroll
+            for (int i = 0; i < BPT; i += 2) {
+                const uint2 y = v[i / 2];
+                c[i] += y.x;
+                c[i + 1] += y.y;
+            }
+        }
+#pragma unroll
+        for (int i = 0; i < BPT; ++i) hist[(it & 1) ^ 1][tid + i * NT] = 0u;
+        // walk the buckets from the top until `rem` keys are covered
+#pragma unroll
+        for (int i = 0; i < BPT; ++i) sum += c[i];
+        uint32_t suf = sum;
+#pragma unroll
+        for (int off = 1; off < 32; off <<= 1) {
+            const uint32_t t = __shfl_down_sync(FULL, suf, off);
+            if (lane + off < 32) suf += t;
+        }
+        if (lane == 0) red[warp] = suf;
+        __syncthreads();
+        uint32_t above = suf - sum;                  // keys in higher buckets
+#pragma unroll
+        for (int i = 0; i < NW; ++i) above += i > warp ? red[i] : 0u;
+        if (above < rem && above + sum >= rem) {
+            bool found = false;
+#pragma unroll
+            for (int i = BPT - 1; i >= 0; --i) {
+                if (!found && above + c[i] >= rem) {
+                    found = true;
+                    s_bin = (uint32_t)(BPT * tid + i);
+                    s_krem = rem - above;
+                    s_cnt = c[i];
                 }
+                above += c[i];
             }
-            __syncthreads();
-            // walk the bins from the top until k keys are covered: thread t owns bins 2t, 2t+1
-            const uint32_t c0 = hist[2 * tid], c1 = hist[2 * tid + 1];
-            uint32_t suf = c0 + c1;
-#pragma unroll
-            for (int off = 1; off < 32; off <<= 1) {
-                const uint32_t t = __shfl_down_sync(FULL, suf, off);
-                if (lane + off < 32) suf += t;
-            }
-            if (lane == 0) red[warp] = suf;
-            __syncthreads();
-            const uint32_t wtot = red[lane];
-            uint32_t wsuf = wtot;
-#pragma unroll
-            for (int off = 1; off < 32; off <<= 1) {
-                const uint32_t t = __shfl_down_sync(FULL, wsuf, off);
-                if (lane + off < 32) wsuf += t;
-            }
-            const uint32_t above = __shfl_sync(FULL, wsuf - wtot, warp);
-            const uint32_t incl1 = above + suf - c0, excl1 = incl1 - c1, incl0 = incl1 + c0, kr = (uint32_t)k;
-            if (incl1 >= kr && excl1 < kr) { s_digit = 2u * tid + 1u; s_krem = kr - excl1; s_cnt = c1; }
-            if (incl0 >= kr && incl1 < kr) { s_digit = 2u * tid; s_krem = kr - incl1; s_cnt = c0; }
-            __syncthreads();
-            prefix |= s_digit << lo;
-            k = (int)s_krem;
-            whole = s_cnt == s_krem;                 // the whole bin is wanted: its lowest possible key is a threshold
-            __syncthreads();
         }
-        tau = prefix;
-        r_eq = whole ? 0x7fffffff : k;               // keys equal to tau that are taken, lowest positions first
+        __syncthreads();
+        const uint32_t bin = s_bin, lo = kmin + (bin << sh);
+        rem = s_krem;
+        if (s_cnt == rem) { tau = lo - 1u; break; }                      // the whole bucket
+        if (sh == 0) { tau = lo; r_eq = (int)rem; break; }               // equal keys: the lowest positions
+        kmax = lo + min(kmax - lo, (1u << sh) - 1u);
+        kmin = lo;
     }
-    // every warp owns a contiguous range of the candidates: count, scan over the warps, write
-    const int per = (C + 31) / 32, lo_j = warp * per, hi_j = min(C, lo_j + per);
-    uint32_t wgt = 0, weq = 0;
-    for (int j0 = lo_j; j0 < hi_j; j0 += 8 * 32) {
-        float f[8];
-#pragma unroll
-        for (int u = 0; u < 8; ++u) f[u] = j0 + u * 32 + lane < hi_j ? __ldcg(x + j0 + u * 32 + lane) : 0.0f;
-#pragma unroll
-        for (int u = 0; u < 8; ++u) {
-            const bool in = j0 + u * 32 + lane < hi_j;
-            const uint32_t kx = order_key(f[u]);
-            wgt += __popc(__ballot_sync(FULL, in && kx > tau));
-            weq += __popc(__ballot_sync(FULL, in && kx == tau));
-        }
-    }
+    // places in the list: count, scan over the warps and the CTAs, write
+    uint32_t wgt = 0u, weq = 0u;
+    for_keys([&](int, uint32_t k) {
+        wgt += __popc(__ballot_sync(FULL, k > tau));
+        weq += __popc(__ballot_sync(FULL, k == tau && k));
+    });
+    __syncthreads();                                 // (red is read above)
     if (lane == 0) { red[warp] = wgt; red2[warp] = weq; }
     __syncthreads();
-    uint32_t g_inc = red[lane], e_inc = red2[lane];
-#pragma unroll
-    for (int off = 1; off < 32; off <<= 1) {
-        const uint32_t tg = __shfl_up_sync(FULL, g_inc, off), te = __shfl_up_sync(FULL, e_inc, off);
-        if (lane >= off) { g_inc += tg; e_inc += te; }
+    if (warp == 0) {
+        const uint32_t a = __reduce_add_sync(FULL, lane < NW ? red[lane] : 0u), b = __reduce_add_sync(FULL, lane < NW ? red2[lane] : 0u);
+        if (lane == 0) { pub[0] = a; pub[1] = b; }
     }
-    int gt_run = (int)(__shfl_sync(FULL, g_inc, warp) - wgt), eq_run = (int)(__shfl_sync(FULL, e_inc, warp) - weq);
+    cl.sync();
+    int gt_run = 0, eq_run = 0;
+    for (int r = 0; r < cr; ++r) {
+        const uint32_t *p = cl.map_shared_rank(pub, r);
+        gt_run += (int)p[0];
+        eq_run += (int)p[1];
+    }
+    cl.sync();                                       // no CTA's shared memory is read by another one any more
+#pragma unroll
+    for (int i = 0; i < NW; ++i)
+        if (i < warp) { gt_run += (int)red[i]; eq_run += (int)red2[i]; }
     const uint32_t lt = (1u << lane) - 1u;
-    for (int j0 = lo_j; j0 < hi_j; j0 += 8 * 32) {
-        float f[8];
-#pragma unroll
-        for (int u = 0; u < 8; ++u) f[u] = j0 + u * 32 + lane < hi_j ? __ldcg(x + j0 + u * 32 + lane) : 0.0f;
-#pragma unroll
-        for (int u = 0; u < 8; ++u) {
-            const int j = j0 + u * 32 + lane;
-            const bool in = j < hi_j;
-            const uint32_t kx = order_key(f[u]);
-            const bool is_gt = in && kx > tau, is_eq = in && kx == tau;
-            const uint32_t bg = __ballot_sync(FULL, is_gt), be = __ballot_sync(FULL, is_eq);
-            const int gb = gt_run + __popc(bg & lt), eb = eq_run + __popc(be & lt);
-            const int rank = is_gt ? gb + min(eb, r_eq) : (is_eq && eb < r_eq) ? gb + eb : -1;
-            if (rank >= 0 && rank < want) out[rank] = j;
-            gt_run += __popc(bg);
-            eq_run += __popc(be);
-        }
-    }
-    for (int i = tid; i < w; i += 1024) out[want + i] = C + i;       // the window, above every candidate
+    for_keys([&](int i, uint32_t k) {
+        const bool is_gt = k > tau, is_eq = k == tau && k;
+        const uint32_t bg = __ballot_sync(FULL, is_gt), be = __ballot_sync(FULL, is_eq);
+        const int gb = gt_run + __popc(bg & lt), eb = eq_run + __popc(be & lt);
+        const int rank = is_gt ? gb + min(eb, r_eq) : (is_eq && eb < r_eq) ? gb + eb : -1;
+        if (rank >= 0 && rank < want) out[rank] = lo_j + i * 32 + lane;
+        gt_run += __popc(bg);
+        eq_run += __popc(be);
+    });
+    if (cr == 0)
+        for (int i = tid; i < w; i += NT) out[want + i] = C + i;   // the window, above every candidate
 }
 
 // ---------------------------------------------------------------- compaction into the new cache
@@ -784,12 +841,42 @@ cudaError_t launch_snap_scores(const SnapArgs &a, cudaStream_t s)
     return cudaErrorInvalidValue;
 }
 
+template <int EPT, int NT>
+static cudaError_t select_run(const float *imp, int BH, int64_t len, int w, int keep, int cl, int per_warp, int32_t *idx, cudaStream_t s)
+{
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute at = {};
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = (unsigned)cl;
+    at.val.clusterDim.y = at.val.clusterDim.z = 1;
+    cfg.gridDim = dim3((unsigned)(BH * cl));
+    cfg.blockDim = dim3(NT);
+    cfg.stream = s;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, snap_select_kernel<EPT, NT>, imp, len, w, keep, per_warp, idx);
+}
+
 cudaError_t launch_snap_select(const float *imp, int BH, int64_t len, int window, int keep, int32_t *idx, cudaStream_t s)
 {
     int w = window < keep ? window : keep;
     if ((int64_t)w > len) w = (int)len;
-    snap_select_kernel<<<(unsigned)BH, 1024, 0, s>>>(imp, len, w, keep, idx);
-    return cudaGetLastError();
+    const int64_t C = len - w;
+    // Up to 64K positions: CTAs of 512 threads with at most 16 keys each, two to an SM; beyond, CTAs of 1024 threads with
+    // 32 keys: half as many CTAs then add up each other's buckets (131000 positions of 32 heads: 38 -> 29 us), but the
+    // barriers of the wider CTAs cost 8 us where one CTA is enough for a head (4096 positions).
+    const bool wide = C > 8 * 512 * 16;
+    const int64_t nt = wide ? 1024 : 512, room = wide ? sm_count() : 2 * (int64_t)sm_count();
+    int64_t cl = 1;                                  // CTAs per head: enough to hold its keys in registers (up to eight), then
+    while (cl < 8 && C > cl * nt * (wide ? kSelMaxEpt : 16)) cl *= 2;   // more while all find room on the chip at once
+    while (cl < 8 && 2 * cl * BH <= room && C >= 4 * cl * nt) cl *= 2;
+    const int ept = (int)((C + cl * nt - 1) / (cl * nt));
+    if (wide)
+        return ept <= kSelMaxEpt ? select_run<kSelMaxEpt, 1024>(imp, BH, len, w, keep, (int)cl, ept * 32, idx, s)
+                                 : select_run<0, 1024>(imp, BH, len, w, keep, (int)cl, ept * 32, idx, s);
+    if (ept <= 4) return select_run<4, 512>(imp, BH, len, w, keep, (int)cl, ept * 32, idx, s);
+    if (ept <= 8) return select_run<8, 512>(imp, BH, len, w, keep, (int)cl, ept * 32, idx, s);
+    return select_run<16, 512>(imp, BH, len, w, keep, (int)cl, ept * 32, idx, s);
 }
 
 template <typename T, int D>
