@@ -108,7 +108,8 @@ typedef struct rq_cache {
      *              status reads RQ_ERR_TIMEOUT; call rq_cache_reset before the cache is used again.
      * reserved[2]: how rq_decode_step runs: 0 = the library chooses, 1 = always as separate
      *              kernels, 2 / 4 / 8 = as one launch with that many groups of heads whenever the
-     *              shape allows it.  The results are the same.
+     *              shape allows it, 16 = as one launch of a thread-block cluster per head (at most
+     *              2048 pages).  The results are the same.
      * reserved[3]: must be 0. */
     int64_t reserved[4];
 } rq_cache;
@@ -299,12 +300,14 @@ RQ_API int64_t rq_cache_len(const rq_cache *cache);
 
 /* Kernel launches the next rq_decode_step on this cache will enqueue for this budget when
  * sel_idx_out is NULL [no counterpart in the paper: bookkeeping for benchmarks]: ONE when the whole
- * step runs as one launch (chosen by the library for 64 to 128 (batch, head) pairs of 4096 to
+ * step runs as one launch (chosen by the library for short contexts: fewer than 1024 pages per head
+ * with up to a few MB to read per head, or up to 2048 pages when there are more (batch, head) pairs
+ * than SMs; and for 64 to 128 (batch, head) pairs of 4096 to
  * 12284 pages each that split into 4, 8 or 2 equal groups which keep the GPU's resident CTAs
  * busy, budget below the number of pages; cache.reserved[2] asks for it on other shapes);
- * otherwise three (update + scoring, selection, attention), or two when the context is short
- * enough (at most 256 pages per head, at least 16 heads) for one CTA per head to do the first
- * two kernels' work in one launch.  A non-NULL sel_idx_out can add a launch that sorts the list.
+ * otherwise three (update + scoring, selection, attention), or two when they are asked for on a
+ * context short enough (at most 256 pages per head, at least 16 heads) for one CTA per head to do
+ * the first two kernels' work in one launch.  A non-NULL sel_idx_out can add a launch that sorts the list.
  * The first call on a device looks up launch parameters (occupancy).  -1 for an invalid cache. */
 RQ_API int rq_decode_step_launches(const rq_cache *cache, int32_t budget_pages);
 

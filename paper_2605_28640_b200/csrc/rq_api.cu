@@ -91,7 +91,7 @@ int sm_count()
 // per-head counters the one-launch step uses, the step clearing the other one.)  [1] poll limit of
 // device-side copy waits (0: the default, < 0: none at all; a testing aid), [2] choice of the decode
 // path (0: automatic, 1: always the separate kernels, 2, 4, 8: the one-launch step with that many
-// waves whenever the shape allows it)
+// waves whenever the shape allows it, 16: one launch of a cluster per head)
 static float *absmax_of(const rq_cache *c)
 {
     if ((int64_t)c->cfg.batch * c->cfg.heads > kStepMaxHeads) return nullptr;
@@ -222,6 +222,16 @@ static int step_waves(const rq_cache *c, const DecodeArgs &a, int budget, int *g
     return team <= slots ? waves : 0;
 }
 
+// CTAs per head of the cluster form of the next decode step, 0 if the step runs otherwise
+static int step_cluster(const rq_cache *c, int64_t pages, int budget)
+{
+    const int64_t choice = c->reserved[2];
+    if (choice != 0 && choice != 16) return 0;
+    const int BH = c->cfg.batch * c->cfg.heads, cl = cluster_step_size(BH, pages, sm_count());
+    const int64_t row = 2 * c->cfg.head_dim * (int64_t)elem_size(c->cfg.dtype), kept = budget < pages ? budget : pages;
+    return choice == 16 || cluster_step_wins(BH, pages, (pages + kept * c->cfg.page_size) * row, sm_count()) ? cl : 0;
+}
+
 static int decode_step_impl(rq_cache *cache, const void *q, const void *k_t, const void *v_t,
                             const void *g_t, int32_t budget_pages, float scale, void *o,
                             int32_t *sel_idx_out, cudaStream_t s, cudaEvent_t *ev)
@@ -243,8 +253,19 @@ static int decode_step_impl(rq_cache *cache, const void *q, const void *k_t, con
     int st;
     int grid = 0;
     DecodeArgs a = decode_args(cache, new_len);
-    const int waves = step_waves(cache, a, budget_pages, &grid);
-    if (waves > 0) {
+    const int cl = step_cluster(cache, P, budget_pages);
+    const int waves = cl > 0 ? 0 : step_waves(cache, a, budget_pages, &grid);
+    if (cl > 0) {
+        if (!(scale > 0.0f)) scale = 1.0f / sqrtf((float)a.D);
+        int32_t *other = a.absmax ? (int32_t *)((char *)cache->workspace + w.step_ctr) + (size_t)((a.epoch & 1) ^ 1) * a.B * a.H * kStepCtrInts
+                                  : nullptr;
+        st = launch_cluster_step(a, q, k_t, v_t, g_t, scores, budget_pages, scale, o, sel_idx_out, other, cl, s) == cudaSuccess
+                 ? RQ_OK : RQ_ERR_CUDA;
+        mark(ev, 1, s);
+        mark(ev, 2, s);
+        mark(ev, 3, s);
+        if (st == RQ_OK) cache->reserved[0] += 1;
+    } else if (waves > 0) {
         // one launch; the list lands in the workspace in no particular order and is sorted for the caller
         const StepBuffers b = step_buffers(cache, w);
         if (!(scale > 0.0f)) scale = 1.0f / sqrtf((float)a.D);
@@ -673,6 +694,7 @@ int rq_decode_step_launches(const rq_cache *cache, int32_t budget_pages)
     const int64_t P = (cache->len + 1 + c.page_size - 1) / c.page_size;     // after the step's append
     int grid = 0;
     const DecodeArgs a = decode_args(cache, cache->len + 1);
+    if (budget_pages >= 1 && step_cluster(cache, P, budget_pages) > 0) return 1;
     if (budget_pages >= 1 && step_waves(cache, a, budget_pages, &grid) > 0) return 1;
     return P <= kSmallStepPages && c.batch * c.heads >= kSmallStepMinHeads ? 2 : 3;
 }

@@ -1,0 +1,467 @@
+// A whole decode step (Eq. 1, Eq. 3, Eq. 4) of a short context as ONE launch, a thread-block cluster per (batch, head).
+//
+// With up to 2048 pages per head a step is latency, not memory traffic: three dependent launches cost more than the
+// bytes they move.  Here the CTAs of a cluster do everything for their head and meet twice, through distributed shared
+// memory:
+//   1. the first CTA appends the token (update_head); all CTAs score the pages, a warp-wide read per record or two
+//      straight from global memory, and write every score to all CTAs of the cluster;
+//   2. after a cluster barrier every CTA selects the head's pages for itself (the same ones) and takes its share of
+//      their tiles, a tile of up to 16 rows per warp at a time, keys and values of a tile in flight together, folded
+//      into the warp's online softmax from registers;
+//   3. the warps' partial results meet in the CTA, the CTAs' in the first CTA, which writes the output row.
+// No tickets, no copies to wait for, nothing in the workspace but the newest page's score.
+// Bound: the chain of about five memory or barrier latencies.  Figures at cluster_step_wins below.
+#include <cooperative_groups.h>
+#include <math_constants.h>
+
+#include "rq_async.cuh"
+#include "rq_device.cuh"
+#include "rq_internal.h"
+#include "rq_stream.cuh"
+
+namespace rq {
+
+namespace {
+
+namespace cg = cooperative_groups;
+
+constexpr unsigned FULL = 0xffffffffu;
+constexpr int NT = 256, NW = NT / 32;          // threads, warps of a CTA
+constexpr int kMaxCl = 8;                      // CTAs of a cluster at most
+constexpr int kRows = kClusterPages / NT;      // pages of a thread in the selection
+constexpr int kRankPages = 96;                 // heads of up to this many pages: every page is ranked against every other
+constexpr int kBins = 256;                     // buckets of the threshold search beyond
+
+template <typename T, int D> struct TileGeom {
+    static constexpr int CH = VecOf<T>::N, LPR = D / CH, RPI = 32 / LPR;       // elements of a vector, lanes of a row, rows of a read
+    static constexpr int TR = 8 * RPI < 16 ? 8 * RPI : 16, NI = TR / RPI;      // rows and reads of a tile
+    static constexpr int HALVINGS = LPR / NI;                                  // lanes that end up with a row's score
+    static constexpr int SH = HALVINGS == 4 ? 2 : HALVINGS == 2 ? 1 : 0;
+    static_assert((NI << SH) == LPR, "a row's score must end up in at least one lane");
+};
+
+// One tile, keys and values in registers, folded into the warp's online softmax (the arithmetic of attend_tile).
+template <typename T, int D>
+__device__ __forceinline__ void fold_tile(AttendState<T> &st, const uint4 (&kr)[TileGeom<T, D>::NI],
+                                          const uint4 (&vr)[TileGeom<T, D>::NI], int valid, int lane)
+{
+    using G = TileGeom<T, D>;
+    constexpr int CH = G::CH, LPR = G::LPR, RPI = G::RPI, NI = G::NI;
+    const int rsub = lane / LPR, cgp = lane % LPR;
+    float s[NI];
+#pragma unroll
+    for (int n = 0; n < NI; ++n) {
+        float kf[CH];
+        unpack16<T>(kr[n], kf);
+        float2 d2 = make_float2(0.0f, 0.0f);
+#pragma unroll
+        for (int c = 0; c < CH; c += 2) d2 = fma2(make_float2(st.qf[c], st.qf[c + 1]), make_float2(kf[c], kf[c + 1]), d2);
+        s[n] = d2.x + d2.y;
+    }
+    int nv = NI;
+#pragma unroll
+    for (int off = LPR / 2; off > 0; off >>= 1) {
+        if (nv > 1) {
+            const int half = nv / 2;
+            const bool hi = (lane & off) != 0;
+#pragma unroll
+            for (int i = 0; i < NI / 2; ++i) {
+                if (i < half) {
+                    const float send = hi ? s[i] : s[i + half];
+                    const float keep = hi ? s[i + half] : s[i];
+                    s[i] = keep + __shfl_xor_sync(FULL, send, off);
+                }
+            }
+            nv = half;
+        } else {
+            s[0] += __shfl_xor_sync(FULL, s[0], off);
+        }
+    }
+    const int row = ((cgp >> G::SH) & (NI - 1)) * RPI + rsub;
+    const float sc = row < valid ? s[0] : -CUDART_INF_F;
+    float m_new = fmaxf(st.m, sc);
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) m_new = fmaxf(m_new, __shfl_xor_sync(FULL, m_new, off));
+    const float alpha = exp2f(st.m - m_new);         // 0 on the first tile (m = -inf)
+    const float p_row = exp2f(sc - m_new);           // 0 for a masked row
+    st.m = m_new;
+    st.l = fmaf(st.l, alpha, p_row);
+#pragma unroll
+    for (int c = 0; c < CH; c += 2) {
+        const float2 a2 = mul2(make_float2(st.acc[c], st.acc[c + 1]), make_float2(alpha, alpha));
+        st.acc[c] = a2.x;
+        st.acc[c + 1] = a2.y;
+    }
+#pragma unroll
+    for (int n = 0; n < NI; ++n) {
+        const float p = __shfl_sync(FULL, p_row, rsub * LPR + (n << G::SH));
+        float vf[CH];
+        unpack16<T>(vr[n], vf);
+#pragma unroll
+        for (int c = 0; c < CH; c += 2) {
+            const float2 a2 = fma2(make_float2(p, p), make_float2(vf[c], vf[c + 1]), make_float2(st.acc[c], st.acc[c + 1]));
+            st.acc[c] = a2.x;
+            st.acc[c + 1] = a2.y;
+        }
+    }
+}
+
+struct ClusterShared {
+    alignas(16) uint32_t key[kClusterPages];   // order-preserving images of the page scores; 0: forced, or no page
+    uint32_t ckey[kClusterPages];              // pages of the threshold's bucket
+    uint16_t cidx[kClusterPages];
+    uint16_t list[kClusterPages];              // the selected pages, ascending
+    alignas(16) uint32_t hist[2][kBins];
+    uint32_t mask[kClusterPages / 32];         // the selected pages as bits
+    uint32_t red[NW], red2[NW], ncand;
+    float upd[32];
+};
+
+// The `want` best of the pages with a key, equal keys to the lower page, as bits of sh.mask beside the forced ones
+// (pages below ns, and from P - nl on).  One CTA.
+__device__ __forceinline__ void select_pages(ClusterShared &sh, int P, int ns, int nl, int want, int tid)
+{
+    const int lane = tid & 31, warp = tid >> 5;
+    if (P <= kRankPages) {
+        // a page's rank is the number of pages that beat it
+        const uint32_t k = tid < P ? sh.key[tid] : 0u;
+        int rank = 0;
+        for (int j = 0; j < P; j += 4) {
+            const uint4 o = *reinterpret_cast<const uint4 *>(sh.key + j);
+            rank += (o.x > k || (o.x == k && j < tid)) + (o.y > k || (o.y == k && j + 1 < tid)) + (o.z > k || (o.z == k && j + 2 < tid)) +
+                    (o.w > k || (o.w == k && j + 3 < tid));
+        }
+        const bool take = tid < P && (tid < ns || tid >= P - nl || (k != 0u && rank < want));
+        const uint32_t bits = __ballot_sync(FULL, take);
+        if (lane == 0) sh.mask[warp] = bits;                            // (NW words, zero beyond the last page)
+        __syncthreads();
+        return;
+    }
+    uint32_t key[kRows];
+    uint32_t kmin = 0xffffffffu, kmax = 0u;
+#pragma unroll
+    for (int r = 0; r < kRows; ++r) {
+        key[r] = r * NT + tid < P ? sh.key[r * NT + tid] : 0u;
+        kmin = min(kmin, key[r] ? key[r] : 0xffffffffu);
+        kmax = max(kmax, key[r]);
+    }
+    kmin = __reduce_min_sync(FULL, kmin);
+    kmax = __reduce_max_sync(FULL, kmax);
+    if (lane == 0) { sh.red[warp] = kmin; sh.red2[warp] = kmax; }
+    sh.hist[0][tid] = 0u;
+    if (tid == 0) sh.ncand = 0u;
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < NW; ++i) {
+        kmin = min(kmin, sh.red[i]);
+        kmax = max(kmax, sh.red2[i]);
+    }
+    // the bucket that holds the last page taken, in ever finer buckets between its smallest and largest key
+    uint32_t rem = (uint32_t)want, cnt = 0u;
+    if (want > 0) {
+#pragma unroll 1
+        for (int it = 0;; ++it) {
+            uint32_t *hs = sh.hist[it & 1];
+            const int shift = max(0, 24 - __clz((int)(kmax - kmin)));    // (kmax - kmin) >> shift < 256
+#pragma unroll
+            for (int r = 0; r < kRows; ++r)
+                if (key[r] && key[r] >= kmin && key[r] <= kmax) atomicAdd(&hs[(key[r] - kmin) >> shift], 1u);
+            __syncthreads();
+            sh.hist[(it & 1) ^ 1][tid] = 0u;
+            // every warp: lane l adds up buckets 8 l .. 8 l + 7 and the sums of the lanes above
+            const uint4 a = *reinterpret_cast<const uint4 *>(hs + 8 * lane), b = *reinterpret_cast<const uint4 *>(hs + 8 * lane + 4);
+            const uint32_t c[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+            uint32_t suf = a.x + a.y + a.z + a.w + b.x + b.y + b.z + b.w;
+            const uint32_t own = suf;
+#pragma unroll
+            for (int off = 1; off < 32; off <<= 1) {
+                const uint32_t t = __shfl_down_sync(FULL, suf, off);
+                if (lane + off < 32) suf += t;
+            }
+            uint32_t above = suf - own, bin = 0u, krem = 0u, kcnt = 0u;
+            const bool mine = above < rem && suf >= rem;
+            bool found = false;
+#pragma unroll
+            for (int i = 7; i >= 0; --i) {
+                if (!found && above + c[i] >= rem) { found = true; bin = 8u * lane + i; krem = rem - above; kcnt = c[i]; }
+                above += c[i];
+            }
+            const int src = __ffs(__ballot_sync(FULL, mine)) - 1;        // (the counts add up to at least `rem`)
+            bin = __shfl_sync(FULL, bin, src);
+            rem = __shfl_sync(FULL, krem, src);
+            cnt = __shfl_sync(FULL, kcnt, src);
+            const uint32_t lo = kmin + (bin << shift);
+            kmax = lo + min(kmax - lo, (1u << shift) - 1u);
+            kmin = lo;
+            if (cnt == rem || cnt <= 32u || shift == 0) break;
+            __syncthreads();                                             // (the other buckets are zero)
+        }
+    } else {
+        kmin = kmax = 0xffffffffu;                                       // nothing beside the forced pages
+    }
+    const bool rank_them = rem > 0u && cnt != rem;
+#pragma unroll
+    for (int r = 0; r < kRows; ++r) {
+        const int p = r * NT + tid;
+        const bool in = key[r] && key[r] >= kmin && key[r] <= kmax && want > 0;
+        const bool take = p < P && (p < ns || p >= P - nl || (key[r] > kmax) || (in && !rank_them));
+        const uint32_t bits = __ballot_sync(FULL, take);
+        if (lane == 0 && r * NT + warp * 32 < P) sh.mask[r * NW + warp] = bits;
+        if (in && rank_them) {
+            const uint32_t at = atomicAdd(&sh.ncand, 1u);
+            sh.ckey[at] = key[r];
+            sh.cidx[at] = (uint16_t)p;
+        }
+    }
+    __syncthreads();
+    if (rank_them) {
+        const int n = (int)sh.ncand;
+        for (int i = tid; i < n; i += NT) {
+            const uint32_t k = sh.ckey[i];
+            const int p = sh.cidx[i];
+            uint32_t rank = 0u;
+            for (int j = 0; j < n; ++j) rank += sh.ckey[j] > k || (sh.ckey[j] == k && (int)sh.cidx[j] < p);
+            if (rank < rem) atomicOr(&sh.mask[p >> 5], 1u << (p & 31));
+        }
+        __syncthreads();
+    }
+}
+
+// Grid (heads x cluster size).  K: pages to keep (at most P); ns, nl: forced first and newest pages inside K.
+template <typename T, int D, int S>
+__global__ void __launch_bounds__(NT, 2) cluster_step_kernel(DecodeArgs a, const T *q, const T *k_t, const T *v_t, const void *g_t,
+                                                             float *scores, int K, int ns, int nl, float scale_log2, T *o,
+                                                             int32_t *sel_out, int budget, int32_t *ctr_other)
+{
+    using SG = ScoreGeom<T, D>;
+    using G = TileGeom<T, D>;
+    constexpr int CH = G::CH, LPR = G::LPR, NI = G::NI, TR = G::TR, TPP = S / TR;
+    static_assert(S % TR == 0, "a page is a whole number of tiles");
+    __shared__ ClusterShared sh;
+    __shared__ __align__(16) float wpart[NW][D + 4], cpart[kMaxCl][D + 4];     // m, l, -, -, acc of the warps, of the CTAs
+    cg::cluster_group cl = cg::this_cluster();
+    const int CL = (int)cl.num_blocks(), cr = (int)cl.block_rank();
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int bh = blockIdx.x / CL;
+    const int P = (int)((a.len + S - 1) / S);
+    const int gw = cr * NW + warp, GW = CL * NW;                         // this warp inside the cluster
+    const bool dense = K >= P;                                           // every page is kept: no scores
+    if (tid < 4 && P + tid < kClusterPages) sh.key[P + tid] = 0u;        // (the ranking reads four keys at a time)
+    cl.barrier_arrive();                                                 // all CTAs have started: their shared memory may be written
+    grid_dependency_wait();                                              // earlier kernels may still write what is read here
+    grid_launch_dependents();
+
+    // ---- 1. append and scores.  The first records are on their way while the first CTA appends the token
+    const unsigned char *meta = static_cast<const unsigned char *>(a.meta) + (int64_t)bh * a.page_cap * SG::REC_BYTES;
+    constexpr int U = 4;                                                 // records of a lane group in flight
+    const int sub = lane / SG::LPP, c = lane % SG::LPP;
+    uint4 raw[U][SG::VPL];
+    auto load_records = [&](int r0) {
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int rec = r0 + u * GW * SG::PPW + sub;
+#pragma unroll
+            for (int v = 0; v < SG::VPL; ++v)
+                raw[u][v] = !dense && rec < P - 1 ? __ldcg(reinterpret_cast<const uint4 *>(meta + (int64_t)rec * SG::REC_BYTES) + c + v * SG::LPP)
+                                                  : make_uint4(0u, 0u, 0u, 0u);
+        }
+    };
+    load_records(gw * SG::PPW);
+    float qs[SG::VPL][SG::CH];
+    score_load_q<T, D>(q, bh, lane, qs);
+    AttendState<T> st;
+    attend_begin_head<T, D>(st, q, bh, scale_log2, lane);
+    float newest = 0.0f;
+    if (cr == 0) {
+        newest = update_head<T, D>(a, bh, q, k_t, v_t, g_t, scores, sh.upd);
+        if (ctr_other && tid < kStepCtrInts) ctr_other[bh * kStepCtrInts + tid] = 0;   // the other one-launch form's counters of the next step
+    }
+    cl.barrier_wait();
+    if (!dense) {
+        // (the loop bound is the same for every lane of a warp: the shuffles below need all of them)
+        for (int rb = gw * SG::PPW; rb < P - 1; rb += U * GW * SG::PPW) {
+            float s[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                float2 s2 = make_float2(0.0f, 0.0f);                     // even and odd channels summed apart, then together
+#pragma unroll
+                for (int v = 0; v < SG::VPL; ++v) {
+                    float m[SG::CH];
+                    unpack16<T>(raw[u][v], m);
+#pragma unroll
+                    for (int i = 0; i < SG::CH; i += 2) s2 = fma2(make_float2(qs[v][i], qs[v][i + 1]), make_float2(m[i], m[i + 1]), s2);
+                }
+                s[u] = s2.x + s2.y;
+            }
+            const int rn = rb;
+            if (rb + U * GW * SG::PPW < P - 1) load_records(rb + U * GW * SG::PPW);
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+#pragma unroll
+                for (int off = SG::LPP / 2; off > 0; off >>= 1) s[u] += __shfl_xor_sync(FULL, s[u], off);
+                const int rec = rn + u * GW * SG::PPW + sub;
+                if (c < CL && rec < P - 1) cl.map_shared_rank(sh.key, c)[rec] = rec < ns || rec >= P - nl ? 0u : order_key(s[u]);
+            }
+        }
+        if (cr == 0 && tid == 0)
+            for (int r = 0; r < CL; ++r) cl.map_shared_rank(sh.key, r)[P - 1] = nl > 0 || P - 1 < ns ? 0u : order_key(newest);
+    }
+    cl.sync();                                                           // all scores are in, the token is in the cache
+
+    // ---- 2. the head's pages, ascending
+    if (dense) {
+        for (int p = tid; p < P; p += NT) sh.list[p] = (uint16_t)p;
+    } else {
+        select_pages(sh, P, ns, nl, K - ns - nl, tid);
+        const int words = (P + 31) / 32;
+        const uint32_t w0 = lane < words ? sh.mask[lane] : 0u, w1 = lane + 32 < words ? sh.mask[lane + 32] : 0u;
+        int i0 = __popc(w0), i1 = __popc(w1);
+#pragma unroll
+        for (int off = 1; off < 32; off <<= 1) {
+            const int t0 = __shfl_up_sync(FULL, i0, off), t1 = __shfl_up_sync(FULL, i1, off);
+            if (lane >= off) { i0 += t0; i1 += t1; }
+        }
+        i1 += __shfl_sync(FULL, i0, 31);
+        i0 -= __popc(w0);
+        i1 -= __popc(w1);
+        for (int w = warp; w < words; w += NW) {
+            const uint32_t bits = __shfl_sync(FULL, w < 32 ? w0 : w1, w & 31);
+            const int at = __shfl_sync(FULL, w < 32 ? i0 : i1, w & 31);
+            if ((bits >> lane) & 1u) sh.list[at + __popc(bits & ((1u << lane) - 1u))] = (uint16_t)(w * 32 + lane);
+        }
+    }
+    __syncthreads();
+    if (sel_out && cr == 0)
+        for (int i = tid; i < budget; i += NT) sel_out[(int64_t)bh * budget + i] = i < K ? (int)sh.list[i] : -1;
+
+    // ---- 3. attention: tiles gw, gw + GW, ... of the list
+    const T *kv = static_cast<const T *>(a.kv) + (int64_t)bh * a.page_cap * 2 * S * D;
+    const int n_tiles = min(K, P) * TPP, rsub = lane / LPR;
+    for (int t = gw; t < n_tiles; t += GW) {
+        const int page = sh.list[t / TPP], row0 = (t % TPP) * TR;
+        const int valid = (int)min((int64_t)TR, a.len - (int64_t)page * S - row0);
+        const T *kp = kv + ((int64_t)page * 2 * S + row0) * D + lane * CH;
+        uint4 kr[NI], vr[NI];
+#pragma unroll
+        for (int n = 0; n < NI; ++n) {
+            const bool in = n * G::RPI + rsub < valid;
+            kr[n] = in ? __ldcg(reinterpret_cast<const uint4 *>(kp + n * 32 * CH)) : make_uint4(0u, 0u, 0u, 0u);
+        }
+#pragma unroll
+        for (int n = 0; n < NI; ++n) {
+            const bool in = n * G::RPI + rsub < valid;
+            vr[n] = in ? __ldcg(reinterpret_cast<const uint4 *>(kp + (int64_t)S * D + n * 32 * CH)) : make_uint4(0u, 0u, 0u, 0u);
+        }
+        if (valid > 0) fold_tile<T, D>(st, kr, vr, valid, lane);
+    }
+    // the row groups of a warp (all share m), the warps of the CTA, the CTAs of the cluster
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) st.l += __shfl_xor_sync(FULL, st.l, off);
+    st.l *= 1.0f / (float)(1 << G::SH);
+#pragma unroll
+    for (int off = LPR; off < 32; off <<= 1)
+#pragma unroll
+        for (int i = 0; i < CH; ++i) st.acc[i] += __shfl_xor_sync(FULL, st.acc[i], off);
+    if (lane < LPR)
+#pragma unroll
+        for (int i = 0; i < CH; ++i) wpart[warp][4 + lane * CH + i] = st.acc[i];
+    if (lane == 0) { wpart[warp][0] = st.m; wpart[warp][1] = st.l; }
+    __syncthreads();
+    // thread d: channel d of n partial results
+    auto merge = [&](const float (*part)[D + 4], int n, float &M, float &L) {
+        M = -CUDART_INF_F;
+        for (int i = 0; i < n; ++i) M = fmaxf(M, part[i][0]);
+        float A = 0.0f;
+        L = 0.0f;
+        for (int i = 0; i < n; ++i) {
+            const float f = part[i][0] == -CUDART_INF_F ? 0.0f : exp2f(part[i][0] - M);
+            L = fmaf(part[i][1], f, L);
+            A = fmaf(part[i][4 + tid], f, A);
+        }
+        return A;
+    };
+    if (tid < D) {
+        float M, L;
+        const float A = merge(wpart, NW, M, L);
+        float *dst = cl.map_shared_rank(&cpart[0][0], 0) + cr * (D + 4);
+        dst[4 + tid] = A;
+        if (tid == 0) { dst[0] = M; dst[1] = L; }
+    }
+    cl.sync();
+    if (cr == 0 && tid < D) {
+        float M, L;
+        const float A = merge(cpart, CL, M, L);
+        store1<T>(o + (int64_t)bh * D + tid, A / L);
+    }
+}
+
+template <typename T, int D, int S>
+cudaError_t run(const DecodeArgs &a, const void *q, const void *k_t, const void *v_t, const void *g_t, float *scores, int budget,
+                float scale, void *o, int32_t *sel_out, int32_t *ctr_other, int cl, cudaStream_t s)
+{
+    const int P = (int)((a.len + S - 1) / S), K = budget < P ? budget : P;
+    int ns = a.n_sink < K ? a.n_sink : K;
+    int nl = a.n_local < K - ns ? a.n_local : K - ns;
+    if (nl > P - ns) nl = P - ns;
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute at[2] = {};
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = (unsigned)cl;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.gridDim = dim3((unsigned)(a.B * a.H * cl));
+    cfg.blockDim = dim3(NT);
+    cfg.stream = s;
+    cfg.attrs = at;
+    cfg.numAttrs = 2;
+    return cudaLaunchKernelEx(&cfg, cluster_step_kernel<T, D, S>, a, (const T *)q, (const T *)k_t, (const T *)v_t, g_t, scores, K, ns, nl,
+                              scale * 1.4426950408889634f, (T *)o, sel_out, budget, ctr_other);
+}
+
+}  // namespace
+
+// CTAs of a cluster: as many as all find room for at once (two to an SM, less what the shape of the GPU's processing
+// clusters leaves out)
+int cluster_step_size(int BH, int64_t pages, int sms)
+{
+    if (pages > kClusterPages) return 0;
+    int cl = kMaxCl;
+    while (cl > 1 && (int64_t)BH * cl > 2 * (int64_t)sms - sms / 4) cl /= 2;
+    return cl;
+}
+
+// Below 1024 pages one launch wins on every shape as long as the CTAs have little to read each (device time, 32 heads x 128,
+// separate launches / cluster, us: 4090 tokens in pages of 64, 16 kept 16.9 / 10.2; 1000 tokens 16.1 / 8.5; 8000 tokens, 125
+// of 500 pages 23.1 / 15.7; 4 heads, 1000 tokens 19.0 / 6.8; 256 heads, 8000 tokens, 31 of 500 47.6 / 33.4), and up to 2048
+// where the heads alone fill the chip (256 heads, 32000 tokens, 125 kept 107 / 102, 500 kept 224 / 215; 64 to 128 heads of
+// 2000 pages: 0.95 to 1.03).  Few heads with much to read leave most of the chip idle, and the separate kernels, which spread
+// a head over all of it, win: 4 heads, 2000 pages of 64 tokens, 500 kept (2 MB per CTA) 39 / 55.
+bool cluster_step_wins(int BH, int64_t pages, int64_t head_bytes, int sms)
+{
+    const int cl = cluster_step_size(BH, pages, sms);
+    if (cl == 0) return false;
+    if (BH >= sms) return true;
+    return pages < 1024 && head_bytes / cl <= (512 << 10);
+}
+
+cudaError_t launch_cluster_step(const DecodeArgs &a, const void *q, const void *k_t, const void *v_t, const void *g_t, float *scores,
+                                int budget, float scale, void *o, int32_t *sel_out, int32_t *ctr_other, int cl, cudaStream_t s)
+{
+#define RQ_CLUSTER(T, D, S) return run<T, D, S>(a, q, k_t, v_t, g_t, scores, budget, scale, o, sel_out, ctr_other, cl, s)
+    if (a.dtype == RQ_BF16) {
+        if (a.D == 128 && a.S == 16) RQ_CLUSTER(bf16, 128, 16);
+        if (a.D == 128 && a.S == 64) RQ_CLUSTER(bf16, 128, 64);
+        if (a.D == 64 && a.S == 16) RQ_CLUSTER(bf16, 64, 16);
+        if (a.D == 64 && a.S == 64) RQ_CLUSTER(bf16, 64, 64);
+    } else {
+        if (a.D == 128 && a.S == 16) RQ_CLUSTER(float, 128, 16);
+        if (a.D == 128 && a.S == 64) RQ_CLUSTER(float, 128, 64);
+        if (a.D == 64 && a.S == 16) RQ_CLUSTER(float, 64, 16);
+        if (a.D == 64 && a.S == 64) RQ_CLUSTER(float, 64, 64);
+    }
+#undef RQ_CLUSTER
+    return cudaErrorInvalidValue;
+}
+
+}  // namespace rq
