@@ -651,8 +651,7 @@ int rq_moba_scratch_bytes(const rq_cache *cache, int32_t block, int32_t budget_b
     const int rc = check_cache(cache);
     if (rc != RQ_OK) return rc;
     if (!bytes || !moba_shape_ok(cache, block, budget_blocks)) return RQ_ERR_INVALID_ARG;
-    *bytes = moba_scratch_bytes(cache->cfg.batch * cache->cfg.heads, cache->len, cache->cfg.head_dim, block, budget_blocks,
-                                cache->cfg.dtype);
+    *bytes = moba_scratch_bytes(cache->cfg.batch * cache->cfg.heads, cache->len, cache->cfg.head_dim, block, budget_blocks);
     return RQ_OK;
 }
 
@@ -671,14 +670,10 @@ int rq_moba_prefill(rq_cache *cache, const void *q, int32_t block, int32_t budge
     a.q = q; a.block = block; a.K = budget_blocks; a.o = o;
     a.scale = scale > 0.0f ? scale : 1.0f / sqrtf((float)c.head_dim);
     const int BH = c.batch * c.heads;
-    moba_carve(scratch, BH, cache->len, c.head_dim, block, c.dtype, a);
-    a.blocks_out = blocks_out;
+    moba_carve(scratch, blocks_out, a);
     a.status = (int32_t *)((char *)cache->workspace + workspace_layout(c).status);
     if (launch_moba(a, s) != cudaSuccess) return RQ_ERR_CUDA;
     const size_t nb = (size_t)((cache->len + block - 1) / block);
-    if (blocks_out && a.sel && cudaMemcpyAsync(blocks_out, a.sel, (size_t)BH * cache->len * budget_blocks * sizeof(int32_t),
-                                      cudaMemcpyDeviceToDevice, s) != cudaSuccess)
-        return RQ_ERR_CUDA;
     if (means_out && cudaMemcpyAsync(means_out, a.means, (size_t)BH * nb * c.head_dim * sizeof(float), cudaMemcpyDeviceToDevice,
                                      s) != cudaSuccess)
         return RQ_ERR_CUDA;

@@ -186,19 +186,19 @@ struct MobaArgs {
     int block, K;       // block size in positions; blocks per query (first and own block included)
     float scale;
     float *means;       // [BH][blocks][D] block representatives
-    int32_t *sel;       // fp32 caches: [BH][len][K] chosen blocks of every query, ascending, -1 beyond
-    unsigned char *planes;  // bf16 caches: the representatives as three bf16 terms, as the tensor core reads them
-    uint32_t *masks;    // bf16 caches: [BH][len][words] chosen blocks of every query as bits
-    int32_t *blocks_out;    // NULL, or the caller's [BH][len][K]
+    // Chosen blocks of every query: as bits [BH][len][words], 32 blocks to a word (bf16 caches, where that takes no more
+    // room than the lists), and as lists [BH][len][K], ascending, -1 beyond.  One of the two may be NULL for bf16 caches
+    uint32_t *masks;
+    int32_t *list;
     void *o;            // [B][len][H][D]
     int32_t *status;    // the cache's device status word
 };
 constexpr int kMobaMaxBlocks = 2048;           // blocks of a prompt at most
-size_t moba_scratch_bytes(int BH, int64_t len, int D, int block, int K, int dtype);
-void moba_carve(void *scratch, int BH, int64_t len, int D, int block, int dtype, MobaArgs &a);
+size_t moba_scratch_bytes(int BH, int64_t len, int D, int block, int K);
+// means, masks and list of `a` (its shape filled in) from the scratch and, if not NULL, the caller's lists
+void moba_carve(void *scratch, int32_t *blocks_out, MobaArgs &a);
 cudaError_t launch_moba(const MobaArgs &a, cudaStream_t s);
 // bf16 caches: representatives and routing (rq_moba_route.cu)
-size_t moba_plane_bytes(int BH, int nb, int D);
 cudaError_t launch_moba_route_bf16(const MobaArgs &a, cudaStream_t s);
 // bf16 caches: the attention (rq_moba_attend.cu)
 cudaError_t launch_moba_attend_bf16(const MobaArgs &a, cudaStream_t s);

@@ -434,38 +434,30 @@ cudaError_t moba_run_f32(const MobaArgs &a, cudaStream_t s)
                                                                           a.means, nb);
     const dim3 rgrid((unsigned)((a.len + kMobaRouteWarps * rq - 1) / (kMobaRouteWarps * rq)), (unsigned)BH);
     if (staged)
-        moba_route_kernel<float, D, true><<<rgrid, kMobaRouteWarps * 32, rs, s>>>((const float *)a.q, a.means, a.len, a.H, a.block, nb, a.K, a.sel);
+        moba_route_kernel<float, D, true><<<rgrid, kMobaRouteWarps * 32, rs, s>>>((const float *)a.q, a.means, a.len, a.H, a.block, nb, a.K, a.list);
     else
-        moba_route_kernel<float, D, false><<<rgrid, kMobaRouteWarps * 32, rs, s>>>((const float *)a.q, a.means, a.len, a.H, a.block, nb, a.K, a.sel);
+        moba_route_kernel<float, D, false><<<rgrid, kMobaRouteWarps * 32, rs, s>>>((const float *)a.q, a.means, a.len, a.H, a.block, nb, a.K, a.list);
     moba_attend_kernel<float, D><<<dim3((unsigned)((a.len + kMobaQueries - 1) / kMobaQueries), (unsigned)BH), kMobaQueries * 32, as, s>>>(
-        (const float *)a.kv, a.page_cap, a.S, a.len, (const float *)a.q, a.H, a.block, nb, a.K, a.sel, a.scale * 1.4426950408889634f,
+        (const float *)a.kv, a.page_cap, a.S, a.len, (const float *)a.q, a.H, a.block, nb, a.K, a.list, a.scale * 1.4426950408889634f,
         (float *)a.o);
     return cudaGetLastError();
 }
 
 }  // namespace
 
-size_t moba_scratch_bytes(int BH, int64_t len, int D, int block, int K, int dtype)
-{
-    const size_t nb = (size_t)((len + block - 1) / block), means = round256((size_t)BH * nb * D * sizeof(float));
-    if (dtype != RQ_BF16) return means + round256((size_t)BH * (size_t)len * K * sizeof(int32_t));
-    return means + round256(moba_plane_bytes(BH, (int)nb, D)) + round256((size_t)BH * (size_t)len * ((nb + 31) / 32) * sizeof(uint32_t));
-}
-
-void moba_carve(void *scratch, int BH, int64_t len, int D, int block, int dtype, MobaArgs &a)
+size_t moba_scratch_bytes(int BH, int64_t len, int D, int block, int K)
 {
     const size_t nb = (size_t)((len + block - 1) / block);
+    return round256((size_t)BH * nb * D * sizeof(float)) + round256((size_t)BH * (size_t)len * K * sizeof(int32_t));
+}
+
+void moba_carve(void *scratch, int32_t *blocks_out, MobaArgs &a)
+{
+    const size_t nb = (size_t)((a.len + a.block - 1) / a.block);
     a.means = (float *)scratch;
-    a.sel = nullptr;
-    a.planes = nullptr;
-    a.masks = nullptr;
-    char *p = (char *)scratch + round256((size_t)BH * nb * D * sizeof(float));
-    if (dtype != RQ_BF16) {
-        a.sel = (int32_t *)p;
-    } else {
-        a.planes = (unsigned char *)p;
-        a.masks = (uint32_t *)(p + round256(moba_plane_bytes(BH, (int)nb, D)));
-    }
+    void *rest = (char *)scratch + round256((size_t)a.B * a.H * nb * a.D * sizeof(float));     // room for the lists
+    a.masks = a.dtype == RQ_BF16 && (nb + 31) / 32 <= (size_t)a.K ? (uint32_t *)rest : nullptr;
+    a.list = blocks_out ? blocks_out : a.masks ? nullptr : (int32_t *)rest;
 }
 
 cudaError_t launch_moba(const MobaArgs &a, cudaStream_t s)

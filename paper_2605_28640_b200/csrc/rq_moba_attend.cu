@@ -69,7 +69,7 @@ struct Walk {
 template <int D>
 __global__ void __launch_bounds__(kThreads, 1) moba_mma_kernel(const __grid_constant__ CUtensorMap tmap, int64_t page_cap, int S,
                                                                int64_t len, const bf16 *q, int H, int block, int nb,
-                                                               const uint32_t *masks, float scale_log2, bf16 *o, int32_t *status)
+                                                               const uint32_t *masks, const int32_t *lists, int K, float scale_log2, bf16 *o, int32_t *status)
 {
     using G = AttGeom<D>;
     constexpr int NST = kStages;
@@ -119,10 +119,18 @@ __global__ void __launch_bounds__(kThreads, 1) moba_mma_kernel(const __grid_cons
     __syncthreads();
     if (warp < kReadWarps) {
         const bool in = t0 + tid < len;
-        const uint32_t *row = masks + ((int64_t)bh * len + (in ? t0 + tid : 0)) * words;
-        for (int w = 0; w < words; ++w) {
-            const uint32_t m = __reduce_or_sync(FULL, in ? __ldg(row + w) : 0u);
-            if (lane == 0 && m) atomicOr(&um[warp >> 2][w], m);
+        if (masks) {
+            const uint32_t *row = masks + ((int64_t)bh * len + (in ? t0 + tid : 0)) * words;
+            for (int w = 0; w < words; ++w) {
+                const uint32_t m = __reduce_or_sync(FULL, in ? __ldg(row + w) : 0u);
+                if (lane == 0 && m) atomicOr(&um[warp >> 2][w], m);
+            }
+        } else if (in) {
+            const int32_t *mine = lists + ((int64_t)bh * len + t0 + tid) * K;
+            for (int i = 0; i < K; ++i) {
+                const int j = __ldg(mine + i);
+                if (j >= 0) atomicOr(&um[warp >> 2][j >> 5], 1u << (j & 31));
+            }
         }
     }
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // the queries, written with ordinary stores, are read by the tensor core
@@ -255,6 +263,8 @@ __global__ void __launch_bounds__(kThreads, 1) moba_mma_kernel(const __grid_cons
         const uint32_t *row = masks + ((int64_t)bh * len + (in ? tq : 0)) * words;
         uint32_t w_cur = 0u, w_next = 0u;                        // the query's choice of the 32 blocks around the walk, and of the next 32
         int w_at = -1;
+        const int32_t *mine = lists + ((int64_t)bh * len + (in ? tq : 0)) * K;
+        int at = 0;                                              // without masks: the query's first list entry that is not behind the walk
         float m = -CUDART_INF_F;                                 // what the weights are relative to (scaled, log2)
         float2 l2 = make_float2(0.0f, 0.0f);                     // sums of the weights (even and odd positions)
         const float2 sc2 = make_float2(scale_log2, scale_log2);
@@ -265,17 +275,24 @@ __global__ void __launch_bounds__(kThreads, 1) moba_mma_kernel(const __grid_cons
             const uint32_t e = list[wk.bi];
             if (!((e >> (14 + s)) & 1u)) continue;
             const int j = e & 0x3fff;
-            if ((j >> 5) != w_at) {
-                const int w = j >> 5;
-                w_cur = w_at >= 0 && w == w_at + 1 ? w_next : in ? __ldg(row + w) : 0u;
-                w_next = in && w + 1 < words ? __ldg(row + w + 1) : 0u;
-                w_at = w;
+            bool chosen;
+            if (masks) {
+                if ((j >> 5) != w_at) {
+                    const int w = j >> 5;
+                    w_cur = w_at >= 0 && w == w_at + 1 ? w_next : in ? __ldg(row + w) : 0u;
+                    w_next = in && w + 1 < words ? __ldg(row + w + 1) : 0u;
+                    w_at = w;
+                }
+                chosen = (w_cur >> (j & 31)) & 1u;
+            } else {
+                while (in && at < K && (uint32_t)__ldg(mine + at) < (uint32_t)j) ++at;     // (-1: beyond every block)
+                chosen = in && at < K && __ldg(mine + at) == j;
             }
             const int c = j * cpb + wk.r;
             const int64_t p0 = (int64_t)c * kChunk;
             // positions this query attends among the chunk's: none if it did not choose the block, else those up to its own
             int nv = 0;
-            if (in && ((w_cur >> (j & 31)) & 1u)) nv = (int)max((int64_t)0, min((int64_t)kChunk, tq - p0 + 1));
+            if (in && chosen) nv = (int)max((int64_t)0, min((int64_t)kChunk, tq - p0 + 1));
             ok = mbar_wait(&s_ready[s][u & 1], (uint32_t)((u >> 1) & 1));
             if (!__all_sync(FULL, ok)) break;
             tcgen05_after_sync();
@@ -398,7 +415,7 @@ template <int D> cudaError_t attend_run(const MobaArgs &a, cudaStream_t s)
     if (e != cudaSuccess) return e;
     const unsigned tiles = (unsigned)((a.len + kTile * kTiles - 1) / (kTile * kTiles));
     moba_mma_kernel<D><<<dim3((unsigned)BH, tiles), kThreads, G::SMEM_BYTES, s>>>(
-        tmap, a.page_cap, a.S, a.len, (const bf16 *)a.q, a.H, a.block, nb, a.masks, a.scale * 1.4426950408889634f, (bf16 *)a.o, a.status);
+        tmap, a.page_cap, a.S, a.len, (const bf16 *)a.q, a.H, a.block, nb, a.masks, a.list, a.K, a.scale * 1.4426950408889634f, (bf16 *)a.o, a.status);
     return cudaGetLastError();
 }
 

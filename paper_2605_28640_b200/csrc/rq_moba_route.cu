@@ -2,12 +2,11 @@
 // representatives, the scores of every query against the representatives of the blocks before it, and the
 // budget's best blocks of every query as a bit mask.
 //
-//   moba_means_bf16_kernel   per (head, block): the mean of the block's stored keys in fp32, and the same numbers
-//                            cut into three bf16 terms (hi + mid + lo: 24 significand bits, nothing of the fp32
-//                            mean is lost) laid out as the tensor core reads them
-//   moba_route_mma_kernel    per (head, 128 consecutive queries): scores = Q (hi + mid + lo)^T in tensor memory,
-//                            then per query the threshold of the budget by value buckets, the mask and, if asked
-//                            for, the ascending list
+//   moba_means_bf16_kernel   per (head, block): the mean of the block's stored keys, fp32
+//   moba_route_mma_kernel    per (head, 128 consecutive queries): the representatives cut into three bf16 terms (hi + mid
+//                            + lo: 24 significand bits, nothing of the fp32 mean is lost), scores = Q (hi + mid + lo)^T in
+//                            tensor memory, then per query the threshold of the budget by value buckets, the mask and,
+//                            if asked for, the ascending list
 #include <limits.h>
 #include <math_constants.h>
 
@@ -23,7 +22,7 @@ namespace {
 constexpr unsigned FULL = 0xffffffffu;
 constexpr int kRouteQueries = 128;             // queries of a CTA: the lanes of the accumulator
 constexpr int kRouteThreads = 512;             // four threads per query, each a quarter of the score words
-constexpr int kRouteGroup = 64;                // blocks of one product (N), and of one copy of representatives
+constexpr int kRouteGroup = 64;                // blocks of one product (N)
 constexpr int kPanelGroups = 8;                // groups whose scores fit in tensor memory at once (512 columns)
 constexpr int kRouteBins = 64;                 // value buckets of the threshold search
 constexpr int kRouteCap = 16;                  // blocks of the threshold's bucket that are ranked directly
@@ -31,9 +30,8 @@ constexpr int kRouteCap = 16;                  // blocks of the threshold's buck
 // ---------------------------------------------------------------- block representatives
 // Grid (ceil(blocks / R), heads), R = 256 / (D / 2) blocks per CTA, a thread per two channels of a block.  The sum
 // runs over the block's valid positions in order.
-// planes: [head][group of 64 blocks][hi, mid, lo][half of 64 channels][64 rows x 128 bytes, 128-byte swizzle]
 __global__ void __launch_bounds__(256) moba_means_bf16_kernel(const bf16 *kv, int64_t page_cap, int S, int D, int64_t len, int block,
-                                                             float *means, unsigned char *planes, int nb)
+                                                             float *means, int nb)
 {
     const int per = D / 2, r = threadIdx.x / per, c = 2 * (threadIdx.x % per);
     const int j = blockIdx.x * (256 / per) + r, bh = blockIdx.y;
@@ -58,17 +56,6 @@ __global__ void __launch_bounds__(256) moba_means_bf16_kernel(const bf16 *kv, in
     }
     const float n = (float)(hi - lo), m0 = s0 / n, m1 = s1 / n;
     *reinterpret_cast<float2 *>(means + ((int64_t)bh * nb + j) * D + c) = make_float2(m0, m1);
-    const int groups = (nb + kRouteGroup - 1) / kRouteGroup, plane_bytes = kRouteGroup * D * 2;
-    unsigned char *dst = planes + ((int64_t)bh * groups + j / kRouteGroup) * 3 * plane_bytes + (c >> 6) * (kRouteGroup * 128) +
-                         umma_sw128_offset(j % kRouteGroup, (c & 63) >> 3) + (c & 7) * 2;
-    float a = m0, b = m1;
-#pragma unroll
-    for (int t = 0; t < 3; ++t) {                       // the remainders are exact: each term takes the next 8 bits
-        const uint32_t w = pack_bf16(a, b);
-        *reinterpret_cast<uint32_t *>(dst + t * plane_bytes) = w;
-        a -= bf16lo(w);
-        b -= bf16hi(w);
-    }
 }
 
 // ---------------------------------------------------------------- routing
@@ -79,16 +66,15 @@ template <int D> struct RouteGeom {
     static constexpr int GROUP_BYTES = 3 * PLANE_BYTES;
     static constexpr int WORK_BYTES = kRouteBins * kRouteQueries * 4 + kRouteCap * kRouteQueries * 6;   // buckets, ranked blocks
     static constexpr int SMALL_BYTES = (12 + 6) * kRouteQueries * 4;
-    // `stages` copies of representatives; a prompt of one panel is done with queries and representatives when the
-    // buckets are needed, so these share the space
-    static __host__ __device__ int front_bytes(int stages, bool one_panel)
+    // a prompt of one panel is done with queries and representatives when the buckets are needed, so these share the space
+    static __host__ __device__ int front_bytes(bool one_panel)
     {
-        const int qb = Q_BYTES + stages * GROUP_BYTES;
+        const int qb = Q_BYTES + GROUP_BYTES;
         return one_panel ? (qb > WORK_BYTES ? qb : WORK_BYTES) : qb + WORK_BYTES;
     }
-    static int smem_bytes(int stages, bool one_panel, int words)
+    static int smem_bytes(bool one_panel, int words)
     {
-        return 1024 + front_bytes(stages, one_panel) + 2 * words * kRouteQueries * 4 + SMALL_BYTES;
+        return 1024 + front_bytes(one_panel) + 2 * words * kRouteQueries * 4 + SMALL_BYTES;
     }
 };
 
@@ -119,23 +105,23 @@ __device__ __forceinline__ uint32_t score_bin(float v, float lo, float inv)
 // each, 28.9 -> 1.35 ms (before: fp32 FMA scores, a lane per block, then a bit-wise vote search up to 128 blocks and one
 // round per taken block beyond).
 template <int D>
-__global__ void __launch_bounds__(kRouteThreads) moba_route_mma_kernel(const bf16 *q, const unsigned char *planes, int64_t len, int H,
+__global__ void __launch_bounds__(kRouteThreads, 2) moba_route_mma_kernel(const bf16 *q, const float *means, int64_t len, int H,
                                                                       int block, int nb, int K, int words, uint32_t *masks,
-                                                                      int32_t *list, int stages, int32_t *status)
+                                                                      int32_t *list, int32_t *status)
 {
     using G = RouteGeom<D>;
     constexpr int NQ = kRouteQueries, NB = kRouteBins, CAP = kRouteCap;
     extern __shared__ __align__(1024) unsigned char rsm_raw[];
-    __shared__ __align__(8) uint64_t full[2], done[2], panel_done;
+    __shared__ __align__(8) uint64_t done;                                    // a product is complete
     __shared__ uint32_t tbase;
     unsigned char *sm = rsm_raw + ((1024u - (smem_addr(rsm_raw) & 1023u)) & 1023u);
     const int groups_all = (nb + kRouteGroup - 1) / kRouteGroup;
     const bool one_panel_launch = groups_all <= kPanelGroups;
     unsigned char *qs = sm, *bs = sm + G::Q_BYTES;
-    uint32_t *hist = reinterpret_cast<uint32_t *>(one_panel_launch ? sm : sm + G::Q_BYTES + stages * G::GROUP_BYTES);   // [NB][NQ]
+    uint32_t *hist = reinterpret_cast<uint32_t *>(one_panel_launch ? sm : sm + G::Q_BYTES + G::GROUP_BYTES);   // [NB][NQ]
     uint32_t *ckey = hist + NB * NQ;                                           // [CAP][NQ]
     uint16_t *cidx = reinterpret_cast<uint16_t *>(ckey + CAP * NQ);            // [CAP][NQ]
-    uint32_t *mk = reinterpret_cast<uint32_t *>(sm + G::front_bytes(stages, one_panel_launch));   // [words][NQ] chosen blocks
+    uint32_t *mk = reinterpret_cast<uint32_t *>(sm + G::front_bytes(one_panel_launch));   // [words][NQ] chosen blocks
     uint32_t *tie = mk + words * NQ;                                           // [words][NQ] equal scores at the threshold
     uint32_t *part_a = tie + words * NQ, *part_b = part_a + 4 * NQ, *part_c = part_b + 4 * NQ;    // [4][NQ] each
     int32_t *s_tb = reinterpret_cast<int32_t *>(part_c + 4 * NQ), *s_need = s_tb + NQ, *s_cnt = s_need + NQ;
@@ -164,8 +150,7 @@ __global__ void __launch_bounds__(kRouteThreads) moba_route_mma_kernel(const bf1
     bool ok = true;
     if (any) {
         if (tid == 0) {
-            for (int s = 0; s < 2; ++s) { mbar_init(&full[s], 1); mbar_init(&done[s], 1); }
-            mbar_init(&panel_done, 1);
+            mbar_init(&done, 1);
             mbar_init_fence();
         }
         if (warp == 0) tmem_alloc(&tbase, tcols);
@@ -181,53 +166,58 @@ __global__ void __launch_bounds__(kRouteThreads) moba_route_mma_kernel(const bf1
         __syncthreads();
         tcgen05_after_sync();
         const uint32_t tb = __shfl_sync(FULL, tbase, 0), tl = tb + ((uint32_t)((warp & 3) * 32) << 16);
-        const unsigned char *src = planes + (int64_t)bh * groups_all * G::GROUP_BYTES;
-        int issued = 0, used = 0;                                              // warp 0: copies started, copies multiplied
-        uint32_t panel_phase = 0u;
+        int used = 0;                                                          // products started
 
-        // the scores of panel p into tensor memory; the first warp starts copies and products
+        // the scores of panel p into tensor memory, 64 blocks at a time: all threads cut representatives into terms, the
+        // first warp starts the products (the whole warp, see rq_umma.cuh)
+        constexpr int PER = kRouteGroup * D / 4 / kRouteThreads;               // float4 of a thread
         auto panel = [&](int p) {
-            if (warp == 0 && ok) {                                             // (the whole warp, see rq_umma.cuh)
-                const int g0 = p * kPanelGroups, gn = min(kPanelGroups, groups - g0);
-                auto issue = [&](int g) {
-                    const int st = issued % stages;
-                    if (lane == 0) {
-                        mbar_arrive_expect_tx(&full[st], G::GROUP_BYTES);
-                        bulk_g2s(bs + (size_t)st * G::GROUP_BYTES, src + (int64_t)g * G::GROUP_BYTES, G::GROUP_BYTES, &full[st]);
-                    }
-                    __syncwarp();
-                    ++issued;
-                };
-                constexpr uint32_t idesc = umma_idesc_bf16(NQ, kRouteGroup);
-                const uint64_t qd = umma_desc_sw128(smem_addr(qs)), bd = umma_desc_sw128(smem_addr(bs));
-                tcgen05_after_sync();
-                for (int g = 0; g < gn && g < stages; ++g) issue(g0 + g);
+            const int g0 = p * kPanelGroups, gn = min(kPanelGroups, groups - g0);
+            float4 f[PER];
+            auto load = [&](int g) {
+#pragma unroll
+                for (int i = 0; i < PER; ++i) {
+                    const int e = tid + i * kRouteThreads, j = g * kRouteGroup + e / (D / 4);
+                    f[i] = j < nb ? __ldg(reinterpret_cast<const float4 *>(means + ((int64_t)bh * nb + j) * D) + e % (D / 4))
+                                  : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+                }
+            };
+            load(g0);
 #pragma unroll 1
-                for (int g = 0; g < gn; ++g) {
-                    const int st = used % stages;
-                    const uint32_t phase = (uint32_t)((used / stages) & 1);
-                    ok = __all_sync(FULL, mbar_wait(&full[st], phase));
-                    if (!ok) break;
-                    ++used;
+            for (int g = 0; g < gn; ++g) {
+                if (used > 0) ok = ok && mbar_wait(&done, (uint32_t)((used - 1) & 1));     // the product before has read its terms
+#pragma unroll
+                for (int i = 0; i < PER; ++i) {
+                    const int e = tid + i * kRouteThreads, r = e / (D / 4), c = 4 * (e % (D / 4));
+                    unsigned char *dst = bs + (c >> 6) * (kRouteGroup * 128) + umma_sw128_offset(r, (c & 63) >> 3) + (c & 7) * 2;
+                    float4 x = f[i];
+#pragma unroll
+                    for (int t = 0; t < 3; ++t) {                              // the remainders are exact: each term takes the next 8 bits
+                        const uint2 w = make_uint2(pack_bf16(x.x, x.y), pack_bf16(x.z, x.w));
+                        *reinterpret_cast<uint2 *>(dst + t * G::PLANE_BYTES) = w;
+                        x.x -= bf16lo(w.x); x.y -= bf16hi(w.x); x.z -= bf16lo(w.y); x.w -= bf16hi(w.y);
+                    }
+                }
+                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // ordinary stores, read by the tensor core
+                if (g + 1 < gn) load(g0 + g + 1);
+                ok = __syncthreads_and(ok);
+                if (!ok) break;
+                if (warp == 0) {
+                    constexpr uint32_t idesc = umma_idesc_bf16(NQ, kRouteGroup);
+                    const uint64_t qd = umma_desc_sw128(smem_addr(qs)), bd = umma_desc_sw128(smem_addr(bs));
+                    tcgen05_after_sync();
 #pragma unroll
                     for (int pl = 2; pl >= 0; --pl)                            // the smallest terms first
 #pragma unroll
                         for (int k = 0; k < D / 16; ++k)
                             umma_bf16(tb + (uint32_t)g * kRouteGroup, qd + (uint64_t)(((k >> 2) * (NQ * 128) + (k & 3) * 32) >> 4),
-                                      bd + (uint64_t)((st * G::GROUP_BYTES + pl * G::PLANE_BYTES + (k >> 2) * (kRouteGroup * 128) + (k & 3) * 32) >> 4), idesc,
+                                      bd + (uint64_t)((pl * G::PLANE_BYTES + (k >> 2) * (kRouteGroup * 128) + (k & 3) * 32) >> 4), idesc,
                                       !(pl == 2 && k == 0));
-                    umma_commit(&done[st]);
-                    if (g + stages < gn) {
-                        ok = __all_sync(FULL, mbar_wait(&done[st], phase));
-                        if (!ok) break;
-                        issue(g0 + g + stages);
-                    }
+                    umma_commit(&done);
                 }
-                umma_commit(&panel_done);
+                ++used;
             }
-            __syncwarp();
-            if (!mbar_wait(&panel_done, panel_phase)) ok = false;
-            panel_phase ^= 1u;
+            ok = ok && mbar_wait(&done, (uint32_t)((used - 1) & 1));
             ok = __syncthreads_and(ok);
             tcgen05_after_sync();
         };
@@ -428,8 +418,6 @@ __global__ void __launch_bounds__(kRouteThreads) moba_route_mma_kernel(const bf1
                 }
             }
         }
-        if (tid == 0)                                                          // after a wait that ran out: no copy may still be on its way
-            for (int k = used; k < issued; ++k) mbar_wait(&full[k % stages], (uint32_t)((k / stages) & 1));
         tcgen05_before_sync();
         __syncthreads();
         if (warp == 0) tmem_dealloc(tbase, tcols);
@@ -445,7 +433,7 @@ __global__ void __launch_bounds__(kRouteThreads) moba_route_mma_kernel(const bf1
         uint32_t m;
         if (K >= o + 1) m = hi >= 32 ? 0xffffffffu : hi <= 0 ? 0u : (1u << hi) - 1u;
         else m = mk[w * NQ + r] | (w == 0 ? 1u : 0u) | (w == (o >> 5) ? 1u << (o & 31) : 0u);
-        masks[((int64_t)bh * len + t0) * words + i] = m;
+        if (masks) masks[((int64_t)bh * len + t0) * words + i] = m;
         if (list) mk[w * NQ + r] = m;
     }
     if (!list) return;
@@ -478,35 +466,27 @@ template <int D> cudaError_t route_run(const MobaArgs &a, cudaStream_t s)
     const int BH = a.B * a.H, nb = (int)((a.len + a.block - 1) / a.block), words = (nb + 31) / 32;
     const int groups = (nb + kRouteGroup - 1) / kRouteGroup;
     const bool one_panel = groups <= kPanelGroups;
-    // more than 256 blocks: tensor memory leaves room for one CTA per SM, which then takes the shared memory of a second
-    // stage; up to 256, a second CTA is worth more than a second stage
-    const int stages = one_panel && groups * kRouteGroup > 256 ? 2 : 1;
     static bool ready[64];
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
     if (!ready[dev]) {
-        const int one = G::smem_bytes(2, true, kPanelGroups * kRouteGroup / 32), more = G::smem_bytes(1, false, kMobaMaxBlocks / 32);
+        const int one = G::smem_bytes(true, kPanelGroups * kRouteGroup / 32), more = G::smem_bytes(false, kMobaMaxBlocks / 32);
         e = cudaFuncSetAttribute(moba_route_mma_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, one > more ? one : more);
         if (e != cudaSuccess) return e;
         ready[dev] = true;
     }
     const int per = 256 / (D / 2);
     moba_means_bf16_kernel<<<dim3((unsigned)((nb + per - 1) / per), (unsigned)BH), 256, 0, s>>>(
-        (const bf16 *)a.kv, a.page_cap, a.S, D, a.len, a.block, a.means, a.planes, nb);
+        (const bf16 *)a.kv, a.page_cap, a.S, D, a.len, a.block, a.means, nb);
     moba_route_mma_kernel<D><<<dim3((unsigned)BH, (unsigned)((a.len + kRouteQueries - 1) / kRouteQueries)), kRouteThreads,
-                               G::smem_bytes(stages, one_panel, words), s>>>((const bf16 *)a.q, a.planes, a.len, a.H, a.block, nb, a.K,
-                                                                            words, a.masks, a.blocks_out, stages, a.status);
+                               G::smem_bytes(one_panel, words), s>>>((const bf16 *)a.q, a.means, a.len, a.H, a.block, nb, a.K,
+                                                                            words, a.masks, a.list, a.status);
     return cudaGetLastError();
 }
 
 }  // namespace
-
-size_t moba_plane_bytes(int BH, int nb, int D)
-{
-    return (size_t)BH * ((nb + kRouteGroup - 1) / kRouteGroup) * 3 * kRouteGroup * D * 2;
-}
 
 cudaError_t launch_moba_route_bf16(const MobaArgs &a, cudaStream_t s)
 {

@@ -15,13 +15,15 @@ DEV = "cuda"
 
 
 def route(levels, T, D, block, K):
-    """levels: the value of channel 0 of every block's keys; queries have 1 in channel 0 and nothing else."""
+    """levels: the value of channel 0 of every block's keys; queries have 1 in channel 0 and nothing else.  Also that the
+    attention is the same whether the caller asks for the lists or not (bit masks then, where they fit)."""
     nb = -(-T // block)
     cache = rq.Cache(1, 1, D, 16, T, torch.bfloat16)
     k = torch.zeros(1, T, 1, D, dtype=torch.bfloat16, device=DEV)
     k[0, :, 0, 0] = torch.tensor(np.repeat(levels, block)[:T], dtype=torch.bfloat16, device=DEV)
     z = torch.zeros_like(k)
-    rq.rq_build_cache(cache.handle, k, z, z)                      # zero gates: the cache holds the keys themselves
+    v = torch.randn(1, T, 1, D, device=DEV, dtype=torch.bfloat16)
+    rq.rq_build_cache(cache.handle, k, v, z)                      # zero gates: the cache holds the keys themselves
     q = torch.zeros(1, T, 1, D, dtype=torch.bfloat16, device=DEV)
     q[..., 0] = 1.0
     o = torch.empty_like(q)
@@ -30,6 +32,9 @@ def route(levels, T, D, block, K):
     rq.rq_moba_prefill(cache.handle, q, block, K, 0.0, o, blocks, None, scratch)
     torch.cuda.synchronize()
     assert rq.rq_device_status(cache.handle) == rq.RQ_OK
+    o2 = torch.empty_like(q)
+    rq.rq_moba_prefill(cache.handle, q, block, K, 0.0, o2, None, None, scratch)
+    assert torch.equal(o, o2)
     return blocks[0, 0].cpu().numpy(), nb
 
 
