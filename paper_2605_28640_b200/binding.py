@@ -91,15 +91,23 @@ def _check(status, where):
 
 
 def _ptr(t):
-    """Device (or host) address of a torch tensor, or None."""
-    return None if t is None else C.c_void_p(t.data_ptr())
+    """Device (or host) address of a torch tensor, or None (plain values: the argument types above convert them)."""
+    return None if t is None else t.data_ptr()
+
+
+_torch = None
 
 
 def _stream(stream):
-    import torch
-    if stream is None:
-        stream = torch.cuda.current_stream()
-    return C.c_void_p(stream.cuda_stream)
+    """The stream's handle; of None, torch's current stream.  The handle is asked for directly: building the stream
+    object around it takes 3 us, more than the rest of a call's marshalling."""
+    if stream is not None:
+        return stream.cuda_stream
+    global _torch
+    if _torch is None:
+        import torch
+        _torch = torch
+    return _torch._C._cuda_getCurrentRawStream(_torch.cuda.current_device())
 
 
 # ---------------------------------------------------------------- ABI-named calls
@@ -128,8 +136,10 @@ def rq_build_cache(cache: rq_cache, k, v, g, stream=None):
 
 
 def rq_decode_step(cache: rq_cache, q, k_t, v_t, g_t, budget_pages, scale, o, sel_idx_out=None, stream=None):
-    _check(lib().rq_decode_step(C.byref(cache), _ptr(q), _ptr(k_t), _ptr(v_t), _ptr(g_t), budget_pages,
-                                scale, _ptr(o), _ptr(sel_idx_out), _stream(stream)), "rq_decode_step")
+    status = (_lib or lib()).rq_decode_step(cache, q.data_ptr(), k_t.data_ptr(), v_t.data_ptr(), g_t.data_ptr(), budget_pages, scale,
+                                            o.data_ptr(), _ptr(sel_idx_out), _stream(stream))
+    if status != RQ_OK:
+        raise RqError(status, "rq_decode_step")
 
 
 def rq_decode_step_host(cache: rq_cache, q, k_t, v_t, g_t, budget_pages, scale, o, sel_idx_out=None,
