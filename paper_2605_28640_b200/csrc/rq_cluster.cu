@@ -41,9 +41,10 @@ template <typename T, int D> struct TileGeom {
 };
 
 // One tile, keys and values in registers, folded into the warp's online softmax (the arithmetic of attend_tile).
-template <typename T, int D>
+// keys_read() is called when the keys are not needed any more.
+template <typename T, int D, typename F>
 __device__ __forceinline__ void fold_tile(AttendState<T> &st, const uint4 (&kr)[TileGeom<T, D>::NI],
-                                          const uint4 (&vr)[TileGeom<T, D>::NI], int valid, int lane)
+                                          const uint4 (&vr)[TileGeom<T, D>::NI], int valid, int lane, F keys_read)
 {
     using G = TileGeom<T, D>;
     constexpr int CH = G::CH, LPR = G::LPR, RPI = G::RPI, NI = G::NI;
@@ -58,6 +59,7 @@ __device__ __forceinline__ void fold_tile(AttendState<T> &st, const uint4 (&kr)[
         for (int c = 0; c < CH; c += 2) d2 = fma2(make_float2(st.qf[c], st.qf[c + 1]), make_float2(kf[c], kf[c + 1]), d2);
         s[n] = d2.x + d2.y;
     }
+    keys_read();
     int nv = NI;
 #pragma unroll
     for (int off = LPR / 2; off > 0; off >>= 1) {
@@ -253,7 +255,7 @@ __global__ void __launch_bounds__(NT, 2) cluster_step_kernel(DecodeArgs a, const
 
     // ---- 1. append and scores.  The first records are on their way while the first CTA appends the token
     const unsigned char *meta = static_cast<const unsigned char *>(a.meta) + (int64_t)bh * a.page_cap * SG::REC_BYTES;
-    constexpr int U = 4;                                                 // records of a lane group in flight
+    constexpr int U = 4;                                                 // records of a lane group in flight (8: 0.6 us more where there are few)
     const int sub = lane / SG::LPP, c = lane % SG::LPP;
     uint4 raw[U][SG::VPL];
     auto load_records = [&](int r0) {
@@ -337,22 +339,36 @@ __global__ void __launch_bounds__(NT, 2) cluster_step_kernel(DecodeArgs a, const
     // ---- 3. attention: tiles gw, gw + GW, ... of the list
     const T *kv = static_cast<const T *>(a.kv) + (int64_t)bh * a.page_cap * 2 * S * D;
     const int n_tiles = min(K, P) * TPP, rsub = lane / LPR;
-    for (int t = gw; t < n_tiles; t += GW) {
+    int valid = 0;
+    const T *kp = kv;
+    uint4 kr[NI], vr[NI];
+    auto find = [&](int t) {                                             // rows of tile t that hold tokens, and where they are
         const int page = sh.list[t / TPP], row0 = (t % TPP) * TR;
-        const int valid = (int)min((int64_t)TR, a.len - (int64_t)page * S - row0);
-        const T *kp = kv + ((int64_t)page * 2 * S + row0) * D + lane * CH;
-        uint4 kr[NI], vr[NI];
+        valid = (int)max((int64_t)0, min((int64_t)TR, a.len - (int64_t)page * S - row0));
+        kp = kv + ((int64_t)page * 2 * S + row0) * D + lane * CH;
+    };
+    auto load = [&](uint4 (&x)[NI], const T *p) {
 #pragma unroll
-        for (int n = 0; n < NI; ++n) {
-            const bool in = n * G::RPI + rsub < valid;
-            kr[n] = in ? __ldcg(reinterpret_cast<const uint4 *>(kp + n * 32 * CH)) : make_uint4(0u, 0u, 0u, 0u);
-        }
-#pragma unroll
-        for (int n = 0; n < NI; ++n) {
-            const bool in = n * G::RPI + rsub < valid;
-            vr[n] = in ? __ldcg(reinterpret_cast<const uint4 *>(kp + (int64_t)S * D + n * 32 * CH)) : make_uint4(0u, 0u, 0u, 0u);
-        }
-        if (valid > 0) fold_tile<T, D>(st, kr, vr, valid, lane);
+        for (int n = 0; n < NI; ++n)
+            x[n] = n * G::RPI + rsub < valid ? __ldcg(reinterpret_cast<const uint4 *>(p + n * 32 * CH)) : make_uint4(0u, 0u, 0u, 0u);
+    };
+    if (gw < n_tiles) {
+        find(gw);
+        load(kr, kp);
+        load(vr, kp + (int64_t)S * D);
+    }
+    for (int t = gw; t < n_tiles; t += GW) {                             // the next tile's loads start as soon as the registers are free
+        const int now = valid;
+        const bool more = t + GW < n_tiles;
+        auto keys_read = [&]() {
+            if (more) {
+                find(t + GW);
+                load(kr, kp);
+            }
+        };
+        if (now > 0) fold_tile<T, D>(st, kr, vr, now, lane, keys_read);
+        else keys_read();
+        if (more) load(vr, kp + (int64_t)S * D);
     }
     // the row groups of a warp (all share m), the warps of the CTA, the CTAs of the cluster
 #pragma unroll
