@@ -424,6 +424,7 @@ int rq_build_cache(rq_cache *cache, const void *k, const void *v, const void *g,
     a.len0 = cache->len; a.T = T; a.page_cap = cache->page_capacity;
     a.absmax = absmax_of(cache);
     a.chunk_scratch = (float *)((char *)cache->workspace + w.scan);
+    a.status = (int32_t *)((char *)cache->workspace + w.status);
     if (launch_scan(a, (cudaStream_t)stream) != cudaSuccess) return RQ_ERR_CUDA;
     cache->len += T;
     return RQ_OK;

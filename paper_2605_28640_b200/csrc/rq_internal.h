@@ -66,6 +66,7 @@ struct ScanArgs {
     int64_t len0, T, page_cap;
     float *absmax;      // [2][BH] largest |stored key| per head, both copies brought up to date (NULL: not tracked)
     float *chunk_scratch;   // kScanScratchBytes of device memory for the time-chunked form (NULL: one chunk always)
+    int32_t *status;    // the cache's device status word
 };
 constexpr size_t kScanScratchBytes = (size_t)2 << 20;
 cudaError_t launch_scan(const ScanArgs &a, cudaStream_t s);

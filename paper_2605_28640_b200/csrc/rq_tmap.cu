@@ -39,4 +39,23 @@ cudaError_t cache_tensor_map(CUtensorMap *out, const void *kv, int D, int S, int
     return cudaSuccess;
 }
 
+cudaError_t prompt_tensor_map(CUtensorMap *out, const void *x, int es, int D, int H, int64_t T, int B, int64_t sh, int64_t st, int64_t sb,
+                              int channels, int positions)
+{
+    const TensorMapEncodeTiled encode = tensor_map_encoder();
+    if (!encode) return cudaErrorNotSupported;
+    // (a dimension of one element has no stride of its own)
+    const int64_t bytes[3] = {(H > 1 ? sh : D) * es, st * es, (B > 1 ? sb : D) * es};
+    for (int i = 0; i < 3; ++i)
+        if (bytes[i] <= 0 || bytes[i] % 16 != 0 || bytes[i] >= ((int64_t)1 << 40)) return cudaErrorInvalidValue;
+    const cuuint64_t dims[4] = {(cuuint64_t)D, (cuuint64_t)H, (cuuint64_t)T, (cuuint64_t)B};
+    const cuuint64_t strides[3] = {(cuuint64_t)bytes[0], (cuuint64_t)bytes[1], (cuuint64_t)bytes[2]};
+    const cuuint32_t box[4] = {(cuuint32_t)channels, 1, (cuuint32_t)positions, 1}, steps[4] = {1, 1, 1, 1};
+    if (encode(out, es == 2 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, const_cast<void *>(x), dims, strides,
+               box, steps, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
+               CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+        return cudaErrorInvalidValue;
+    return cudaSuccess;
+}
+
 }  // namespace rq
