@@ -21,7 +21,7 @@
 // by 16 lanes (warp w takes channels 2w and 2w+1), which, with the state entering the tile,
 // gives the state entering every warp and the state entering the next tile; after a second
 // barrier every thread applies the recurrence token by token (pass 2), rounds to the storage
-// type and stores its rows straight to the cache, 64 bytes of a row per half-warp.  Page
+// type and its rows go out to the cache, 64 or 128 bytes of a row per half-warp.  Page
 // bounds are taken before rounding (rounding is monotone: the rounded minimum is the minimum
 // of the rounded).
 //
@@ -32,7 +32,11 @@
 //
 // The order of all floating-point operations is fixed: the same bits on every run.
 //
-// SCAN_FIGURES
+// Bound: the phases of a tile between its two barriers, with DRAM close behind (131072 tokens of 32 heads x 128, bf16: 5.5
+// GB in 0.96 to 1.07 ms, 5.2 to 5.7 TB/s; the copies alone run at 5.8 TB/s).  Before (copies started and rows stored in
+// 16-byte pieces by all threads, one CTA per unit, three barriers, the inputs read twice for few heads) / now, us: 32 heads,
+// 131072 tokens 1120 / 957; 8 heads, 50003 tokens, fp32 gates 195 / 121; 8 heads, 8000 tokens 76 / 33; 4 heads, 8000 tokens
+// 75 / 31; fp32, 12 heads, 20000 tokens 176 / 120; fp32, 32 heads, 8000 tokens, pages of 16 120 / 126.
 #include "rq_async.cuh"
 #include "rq_device.cuh"
 #include "rq_internal.h"
@@ -56,8 +60,8 @@ constexpr int kMapStride = 3 * CG + 2;          // floats between two warps' map
                                                 // the same channel of 16 consecutive maps hit 16 different banks
 constexpr int kInStride = 2 * CG + 2;           // likewise for the states entering the warps
 constexpr int LPC = NW;                         // lanes that scan the warp maps of one channel
-constexpr int kMaxCluster = 8;
-static_assert(CG == 32 && NW == 16 && RT == 8 && TT == 256, "the layouts below");
+constexpr int kMaxCluster = 4;
+static_assert(CG == 32 && NW == 16 && RT == 8, "the layouts below");
 
 // two neighbouring elements as floats
 __device__ __forceinline__ float2 unpack2(uint32_t w) { return make_float2(bf16lo(w), bf16hi(w)); }
@@ -115,7 +119,7 @@ __device__ __forceinline__ void send_float(uint32_t dst, float x, uint32_t bar)
 }
 
 struct ScanMaps {
-    CUtensorMap k, v, g;
+    CUtensorMap k, v, g, cache;
 };
 struct ScanPlan {
     int64_t tile0;          // first tile (of 256 cache positions) that the call touches
@@ -137,6 +141,9 @@ __global__ void __launch_bounds__(NT) scan_kernel(ScanArgs a, const __grid_const
     constexpr int NST = scan_stages<T, G>();
     constexpr int STAGE = scan_stage_bytes<T, G>();
     constexpr int OFF_V = TT * CG * (int)sizeof(T), OFF_G = 2 * OFF_V;
+    // 2-byte storage: a warp's rows go back into their stage and out with tensor-map stores (32 heads x 128, 131072 tokens:
+    // 973 -> 956 us); 4-byte storage: straight from registers (12 heads, 20000 tokens: 120 us, through the stage 138)
+    constexpr bool BY_STAGE = sizeof(T) == 2;
     constexpr int WPP = S / (2 * RT);                                          // warps that share a page
     constexpr unsigned FULLMASK = 0xffffffffu;
     static_assert(D % CG == 0, "a head is a whole number of channel groups");
@@ -178,6 +185,7 @@ __global__ void __launch_bounds__(NT) scan_kernel(ScanArgs a, const __grid_const
         const int64_t t = (tile0 + i) * TT;
         return plan.tma && t >= a.len0 && t + TT <= end;
     };
+    const uint64_t once = l2_evict_first_policy();
     // start the copies of this CTA's j-th tile.  The whole first warp.
     auto issue = [&](int j) {
         const int i = cr + j * CL, st = j % NST;
@@ -185,9 +193,17 @@ __global__ void __launch_bounds__(NT) scan_kernel(ScanArgs a, const __grid_const
             unsigned char *dst = dsm + (size_t)st * STAGE;
             const int tok = (int)((tile0 + i) * TT - a.len0);
             mbar_expect_warp(&full[st], STAGE);
-            tma_load_4d(dst, &tm.k, c0, h, tok, b, &full[st]);
-            tma_load_4d(dst + OFF_V, &tm.v, c0, h, tok, b, &full[st]);
-            tma_load_4d(dst + OFF_G, &tm.g, c0, h, tok, b, &full[st]);
+            // (rows of 128 bytes are whole lines that nobody else reads; of 64 bytes, half a line whose other half another CTA
+            // reads at about the same time)
+            if (sizeof(T) == 4) {
+                tma_load_4d_hint(dst, &tm.k, c0, h, tok, b, &full[st], once);
+                tma_load_4d_hint(dst + OFF_V, &tm.v, c0, h, tok, b, &full[st], once);
+            } else {
+                tma_load_4d(dst, &tm.k, c0, h, tok, b, &full[st]);
+                tma_load_4d(dst + OFF_V, &tm.v, c0, h, tok, b, &full[st]);
+            }
+            if (sizeof(G) == 4) tma_load_4d_hint(dst + OFF_G, &tm.g, c0, h, tok, b, &full[st], once);
+            else tma_load_4d(dst + OFF_G, &tm.g, c0, h, tok, b, &full[st]);
         } else if (lane == 0) {
             mbar_arrive(&full[st]);
         }
@@ -312,8 +328,10 @@ __global__ void __launch_bounds__(NT) scan_kernel(ScanArgs a, const __grid_const
             *reinterpret_cast<float2 *>(wm + CG) = fma2(A2, LBk, Bk2);
             *reinterpret_cast<float2 *>(wm + 2 * CG) = fma2(A2, LBv, Bv2);
         }
-        __syncthreads();                                         // the maps are there, and the stage has been read
-        if (warp == 0 && j + NST < mine) issue(j + NST);
+        if (BY_STAGE) tma_store_wait_read();                     // the warp's rows of the tile before have left their stage
+        __syncthreads();                                         // the maps are there
+        // the stage of the tile before (of this tile, if nothing goes back into it) is free
+        if (warp == 0 && (!BY_STAGE || j >= 1) && j - BY_STAGE + NST < mine) issue(j - BY_STAGE + NST);
         if (WPP > 1 && MODE == 0 && j > 0) wide_bounds(j - 1);
 
         // ---- scan of the 16 warp maps of channels 2 warp and 2 warp + 1 (one per half-warp) by 16 lanes
@@ -379,14 +397,30 @@ __global__ void __launch_bounds__(NT) scan_kernel(ScanArgs a, const __grid_const
             if (MAP || (row0 + r >= lo && row0 + r < hi)) {
                 sk2 = fma2(g2[r], sk2, k2[r]);
                 sv2 = fma2(g2[r], sv2, v2[r]);
-                store2_cs(dst + r * D, sk2);
-                store2_cs(dst + (S + r) * D, sv2);
+                if constexpr (MAP && BY_STAGE) {
+                    T *kt = reinterpret_cast<T *>(dsm + (size_t)(j % NST) * STAGE) + (row0 + r) * CG + ch2;
+                    store2(kt, sk2.x, sk2.y);
+                    store2(kt + TT * CG, sv2.x, sv2.y);
+                } else {
+                    store2_cs(dst + r * D, sk2);
+                    store2_cs(dst + (S + r) * D, sv2);
+                }
                 mn0 = fminf(mn0, sk2.x); mx0 = fmaxf(mx0, sk2.x);
                 mn1 = fminf(mn1, sk2.y); mx1 = fmaxf(mx1, sk2.y);
             } else if (row0 + r >= hi && row0 + r < fill_hi) {   // unused slots of the last page
                 store2_cs(dst + r * D, make_float2(0.0f, 0.0f));
                 store2_cs(dst + (S + r) * D, make_float2(0.0f, 0.0f));
             }
+        }
+        if constexpr (MAP && BY_STAGE) {
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+            __syncwarp();
+            const T *kt = reinterpret_cast<const T *>(dsm + (size_t)(j % NST) * STAGE) + warp * 2 * RT * CG;
+            const int64_t wpos = tile_start + 2 * warp * RT;
+            const int page = (int)(bh * a.page_cap + wpos / S), slot = (int)(wpos % S);
+            tma_store_4d(kt, &tm.cache, c0, slot, 0, page);
+            tma_store_4d(kt + TT * CG, &tm.cache, c0, slot, 1, page);
+            tma_store_commit();
         }
         if (mn0 <= mx0) amax = fmaxf(amax, fmaxf(fmaxf(-mn0, mx0), fmaxf(-mn1, mx1)));   // this run held new tokens
         // the warp's two runs together (16 positions)
@@ -408,6 +442,7 @@ __global__ void __launch_bounds__(NT) scan_kernel(ScanArgs a, const __grid_const
         if (by_map(cr + j * CL)) tile(BoolTag<true>(), j);
         else tile(BoolTag<false>(), j);
     }
+    if (BY_STAGE) tma_store_wait_read();
     __syncthreads();
     if (MODE == 1) {
         if (tid < CG) {                          // the chunk's map
@@ -498,16 +533,22 @@ cudaError_t run(const ScanArgs &a, cudaStream_t s)
     p.tma = a.T >= TT && a.T < ((int64_t)1 << 31) &&
             prompt_tensor_map(&tm.k, a.k, sizeof(T), D, a.H, a.T, a.B, a.sh, a.st, a.sb, CG, TT) == cudaSuccess &&
             prompt_tensor_map(&tm.v, a.v, sizeof(T), D, a.H, a.T, a.B, a.sh, a.st, a.sb, CG, TT) == cudaSuccess &&
-            prompt_tensor_map(&tm.g, a.g, sizeof(G), D, a.H, a.T, a.B, a.sh, a.st, a.sb, CG, TT) == cudaSuccess;
-    // As many CTAs per unit as leave every SM at most one, with at least four tiles each.  Where not even clusters of eight
-    // fill half of the chip: time chunks, as many as give every SM a CTA, of at least 16 tiles and within the scratch.
+            prompt_tensor_map(&tm.g, a.g, sizeof(G), D, a.H, a.T, a.B, a.sh, a.st, a.sb, CG, TT) == cudaSuccess &&
+            page_tensor_map(&tm.cache, a.kv, sizeof(T), D, S, (int64_t)a.B * a.H * a.page_cap, CG, 2 * RT) == cudaSuccess;
+    // Time chunks: as many as give every SM a CTA, of at least 16 tiles and within the scratch.  They read the inputs
+    // twice, so they only pay where they are at least seven (4 heads x 128, 131072 tokens: 223 us; a cluster of four, bound
+    // by its hops of about 0.55 us, 290).  Otherwise as many CTAs per unit as leave every SM at most one, with at least four
+    // tiles each (8 heads, 131072 tokens: 469 -> 283 us; 16 heads: 913 -> 543; clusters of eight find too little room: 386 for
+    // the 4 heads).
     const int sms = sm_count();
     int cl = 1, chunks = 1;
-    if (a.chunk_scratch && units * kMaxCluster * 2 <= sms && p.ntiles >= 32) {
+    if (a.chunk_scratch && 2 * units <= sms) {
         chunks = sms / p.units;
         if (chunks > p.ntiles / 16) chunks = p.ntiles / 16;
         while (chunks > 1 && (size_t)p.units * chunks * 5 * CG * sizeof(float) > kScanScratchBytes) --chunks;
-    } else {
+    }
+    if (chunks < 7) {
+        chunks = 1;
         while (cl < kMaxCluster && 2 * cl * units <= sms && p.ntiles >= 8 * cl) cl *= 2;
     }
     p.chunk_tiles = (p.ntiles + chunks - 1) / chunks;

@@ -39,6 +39,21 @@ cudaError_t cache_tensor_map(CUtensorMap *out, const void *kv, int D, int S, int
     return cudaSuccess;
 }
 
+cudaError_t page_tensor_map(CUtensorMap *out, void *kv, int es, int D, int S, int64_t pages_total, int channels, int slots)
+{
+    if (pages_total < 1 || pages_total >= ((int64_t)1 << 31)) return cudaErrorInvalidValue;   // box coordinates are 32-bit
+    const TensorMapEncodeTiled encode = tensor_map_encoder();
+    if (!encode) return cudaErrorNotSupported;
+    const cuuint64_t dims[4] = {(cuuint64_t)D, (cuuint64_t)S, 2, (cuuint64_t)pages_total};
+    const cuuint64_t strides[3] = {(cuuint64_t)D * es, (cuuint64_t)S * D * es, (cuuint64_t)2 * S * D * es};
+    const cuuint32_t box[4] = {(cuuint32_t)channels, (cuuint32_t)slots, 1, 1}, steps[4] = {1, 1, 1, 1};
+    if (encode(out, es == 2 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, kv, dims, strides, box, steps,
+               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_NONE,
+               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+        return cudaErrorInvalidValue;
+    return cudaSuccess;
+}
+
 cudaError_t prompt_tensor_map(CUtensorMap *out, const void *x, int es, int D, int H, int64_t T, int B, int64_t sh, int64_t st, int64_t sb,
                               int channels, int positions)
 {

@@ -57,6 +57,39 @@ __device__ __forceinline__ void tma_load_4d(void *dst_smem, const void *tmap, in
         "l"(tmap), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(smem_addr(bar))
         : "memory");
 }
+// The same copy with an L2 cache policy for the lines it reads.
+__device__ __forceinline__ void tma_load_4d_hint(void *dst_smem, const void *tmap, int c0, int c1, int c2, int c3, uint64_t *bar, uint64_t policy)
+{
+    asm volatile(
+        "{\n\t.reg .pred e;\n\t"
+        "elect.sync _|e, 0xffffffff;\n\t"
+        "@e cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1, {%2, %3, %4, %5}], [%6], %7;\n\t}" ::"r"(
+            smem_addr(dst_smem)),
+        "l"(tmap), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(smem_addr(bar)), "l"(policy)
+        : "memory");
+}
+// The way back: a box of shared memory into the tensor, as (part of) the elected lane's current bulk group.  The shared
+// memory was written with ordinary stores: a proxy fence comes between.  One whole warp.
+__device__ __forceinline__ void tma_store_4d(const void *src_smem, const void *tmap, int c0, int c1, int c2, int c3)
+{
+    asm volatile(
+        "{\n\t.reg .pred e;\n\t"
+        "elect.sync _|e, 0xffffffff;\n\t"
+        "@e cp.async.bulk.tensor.4d.global.shared::cta.tile.bulk_group [%0, {%1, %2, %3, %4}], [%5];\n\t}" ::"l"(tmap), "r"(c0), "r"(c1),
+        "r"(c2), "r"(c3), "r"(smem_addr(src_smem))
+        : "memory");
+}
+__device__ __forceinline__ void tma_store_commit()
+{
+    asm volatile(
+        "{\n\t.reg .pred e;\n\t"
+        "elect.sync _|e, 0xffffffff;\n\t"
+        "@e cp.async.bulk.commit_group;\n\t}" ::
+            : "memory");
+}
+// the elected lane's stores have read their shared memory (a lane without stores does not wait)
+__device__ __forceinline__ void tma_store_wait_read() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
+
 // one arrival that also announces `bytes` of copy traffic to wait for, by the elected lane of a whole warp
 __device__ __forceinline__ void mbar_expect_warp(uint64_t *bar, uint32_t bytes)
 {

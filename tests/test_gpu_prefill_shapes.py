@@ -1,0 +1,80 @@
+"""Prefill where its forms meet: lengths around a tile (256 positions), the first and last tile ragged, tiles taken in turn
+by clusters of two and four CTAs, input layouts that a tensor map describes ([B][T][H][D], [B][H][T][D], heads of a wider
+row) and one that it does not (a gate shared by all heads: a stride of zero), all element types, a call that starts inside a
+page.  The reference is the recurrence in fp64, step by step; the cache is compared with the rounded reference.
+
+Bounds: an fp32 recurrence with gates up to 0.999 carries at most about 1000 roundings of 2^-24, i.e. 6e-5 of the largest
+state; a stored bf16 value next to a rounding boundary is one step of 2^-8 off, and nearly none are."""
+import pytest
+import torch
+
+import paper_2605_28640_b200 as rq
+
+pytestmark = pytest.mark.gpu
+DEV = "cuda"
+BF, F32 = torch.bfloat16, torch.float32
+
+
+def laid_out(layout, x):
+    """The same numbers as x [B][T][H][D] (contiguous) with other strides; "shared": the first head's for all heads."""
+    B, T, H, D = x.shape
+    if layout == "bhtd":
+        return x.transpose(1, 2).contiguous().transpose(1, 2)
+    if layout == "wide":                                         # heads inside a row of twice the width
+        w = torch.zeros(B, T, 2 * H, D, device=DEV, dtype=x.dtype)
+        w[:, :, :H] = x
+        return w[:, :, :H]
+    if layout == "shared":                                       # a stride of zero
+        return x[:, :, :1].contiguous().expand(B, T, H, D)
+    return x
+
+
+def recurrence(k, v, g, T0=0):
+    out = []
+    for x in (k, v):
+        s = torch.zeros(x.shape[0], x.shape[2], x.shape[3], dtype=torch.float64, device=DEV)
+        rows = torch.empty(x.shape, dtype=torch.float64, device=DEV)
+        for t in range(x.shape[1]):
+            gt = g[:, t].double()
+            s = gt * s + (1 - gt) * x[:, t].double()
+            rows[:, t] = s
+        out.append(rows)
+    return out
+
+
+@pytest.mark.parametrize("layout", ["bthd", "bhtd", "wide", "shared"])
+@pytest.mark.parametrize("B,H,D,S,T,cuts,dtype,gdtype", [
+    (1, 2, 64, 16, 255, [], BF, BF), (1, 2, 128, 16, 256, [], BF, BF), (2, 1, 64, 64, 257, [], F32, F32),
+    (1, 3, 128, 16, 1300, [7, 300], BF, F32),                    # starts inside pages and tiles
+    (1, 2, 128, 64, 2100, [100], BF, BF),                        # cluster of two or four: eight tiles and a bit
+    (1, 8, 128, 16, 4200, [], BF, BF), (1, 4, 64, 16, 4300, [129], F32, BF), (1, 20, 128, 16, 2600, [], BF, BF),
+    (2, 40, 64, 64, 600, [64], F32, F32)])
+def test_states_cache_and_bounds(B, H, D, S, T, cuts, dtype, gdtype, layout):
+    gen = torch.Generator(device=DEV)
+    gen.manual_seed(T + H)
+    k, v, g = (torch.randn(B, T, H, D, generator=gen, device=DEV) for _ in range(3))
+    k, v, g = (laid_out(layout, x) for x in (k.to(dtype), v.to(dtype), torch.sigmoid(4.12 + 0.5 * g).to(gdtype)))
+    c = rq.Cache(B, H, D, S, T + 70, dtype, gdtype)
+    c.kv.fill_(0xFF)
+    c.meta.fill_(0xFF)
+    edges = [0, *cuts, T]
+    for a, b in zip(edges[:-1], edges[1:]):
+        rq.rq_build_cache(c.handle, k[:, a:b], v[:, a:b], g[:, a:b])
+    torch.cuda.synchronize()
+    assert rq.rq_device_status(c.handle) == rq.RQ_OK and len(c) == T
+    P = -(-T // S)
+    for i, want in enumerate(recurrence(k, v, g)):
+        top = want.abs().max()
+        assert (c.state_view()[:, :, i].double() - want[:, -1]).abs().max() <= 6e-5 * top
+        got = c.kv_view()[:, :, :P, i].reshape(B, H, P * S, D)
+        assert (got[:, :, T:] == 0).all()
+        got, want = got[:, :, :T], want.transpose(1, 2)
+        off = (got.double() - want.to(dtype).double()).abs()
+        if dtype == BF:
+            assert (off <= 2 ** -7 * want.abs() + 6e-5 * top).all() and (off > 0).float().mean() <= 2e-3
+        else:
+            assert off.max() <= 6e-5 * top
+    keys = c.kv_view()[:, :, :P, 0]
+    for p in range(P):
+        rows = keys[:, :, p, :min(S, T - p * S)]
+        assert torch.equal(c.meta_view()[:, :, p, 0], rows.amin(2)) and torch.equal(c.meta_view()[:, :, p, 1], rows.amax(2))
