@@ -67,10 +67,12 @@ struct Walk {
 // Warps 0..7 read scores, warp 8 starts the tensor-map copies, warps 9 and 10 the score products of an accumulator each,
 // warp 11 the output products; they meet through mbarriers only, every wait bounded.  One warp for all products was the
 // limit: 24 products, six commits and as many waits a chunk (32 heads x 128, 30011 positions: 7.61 -> 6.13 ms; 4096: 234 -> 206 us).  256 queries per CTA because keys and values come
-// from L2 for every CTA.
+// from L2 for every CTA.  A CTA's queries come by tensor map, and it may start before the routing kernel has ended: at 4096
+// positions a CTA lives 50 us only, and the 20 us before its first product were a third of that (206 -> 186 us).
 template <int D>
-__global__ void __launch_bounds__(kThreads, 1) moba_mma_kernel(const __grid_constant__ CUtensorMap tmap, int64_t page_cap, int S,
-                                                               int64_t len, const bf16 *q, int H, int block, int nb,
+__global__ void __launch_bounds__(kThreads, 1) moba_mma_kernel(const __grid_constant__ CUtensorMap tmap,
+                                                               const __grid_constant__ CUtensorMap qmap, int64_t page_cap, int S,
+                                                               int64_t len, int H, int block, int nb,
                                                                const uint32_t *masks, const int32_t *lists, int K, float scale_log2, bf16 *o, int32_t *status)
 {
     using G = AttGeom<D>;
@@ -79,7 +81,7 @@ __global__ void __launch_bounds__(kThreads, 1) moba_mma_kernel(const __grid_cons
     // afterwards), then the output
     constexpr uint32_t ACC = 256, OFF_O = 128;
     extern __shared__ __align__(1024) unsigned char asm_raw[];
-    __shared__ __align__(8) uint64_t full_k[NST], full_v[NST], free_k[NST], free_v[NST];
+    __shared__ __align__(8) uint64_t full_k[NST], full_v[NST], free_k[NST], free_v[NST], full_q;
     __shared__ __align__(8) uint64_t s_ready[kTiles][2], p_ready[kTiles][2], pv_done[kTiles][2];
     __shared__ uint32_t um[kTiles][kMobaMaxBlocks / 32];         // blocks chosen by any query of an accumulator
     __shared__ uint32_t tbase;
@@ -101,6 +103,7 @@ __global__ void __launch_bounds__(kThreads, 1) moba_mma_kernel(const __grid_cons
             mbar_init(&full_k[i], 1); mbar_init(&full_v[i], 1);
             mbar_init(&free_k[i], kTiles); mbar_init(&free_v[i], 1);
         }
+        mbar_init(&full_q, 1);
         for (int s = 0; s < kTiles; ++s)
             for (int i = 0; i < 2; ++i) {
                 mbar_init(&s_ready[s][i], 1);
@@ -111,31 +114,38 @@ __global__ void __launch_bounds__(kThreads, 1) moba_mma_kernel(const __grid_cons
     }
     if (warp == kReadWarps) tmem_alloc(&tbase, 512);
     for (int i = tid; i < kTiles * words; i += kThreads) um[i / words][i % words] = 0u;
-    // the queries (q is [B][T][H][D]) as K-major operands; rows past the prompt are zero
-    for (int i = tid; i < kTiles * kTile * (D / 8); i += kThreads) {
-        const int r = i / (D / 8), c = i % (D / 8);
-        uint4 v = make_uint4(0u, 0u, 0u, 0u);
-        if (t0 + r < len) v = *reinterpret_cast<const uint4 *>(q + (((int64_t)b * len + t0 + r) * H + h) * D + c * 8);
-        *reinterpret_cast<uint4 *>(qs + (r / kTile) * G::Q_BYTES + (c >> 3) * (kTile * 128) + umma_sw128_offset(r % kTile, c & 7)) = v;
-    }
     __syncthreads();
+    if (warp == kReadWarps) {                                    // the queries; rows past the prompt come as zeros
+        mbar_expect_warp(&full_q, kTiles * G::Q_BYTES);
+#pragma unroll
+        for (int s = 0; s < kTiles; ++s)
+#pragma unroll
+            for (int hf = 0; hf < G::HALVES; ++hf)
+                tma_load_4d(qs + s * G::Q_BYTES + hf * (kTile * 128), &qmap, hf * 64, h, (int)t0 + s * kTile, b, &full_q);
+    }
+    grid_dependency_wait();                                      // the choices of blocks come from the kernel before
     if (warp < kReadWarps) {
         const bool in = t0 + tid < len;
         if (masks) {
             const uint32_t *row = masks + ((int64_t)bh * len + (in ? t0 + tid : 0)) * words;
-            for (int w = 0; w < words; ++w) {
-                const uint32_t m = __reduce_or_sync(FULL, in ? __ldg(row + w) : 0u);
-                if (lane == 0 && m) atomicOr(&um[warp >> 2][w], m);
+            for (int w0 = 0; w0 < words; w0 += 8) {              // eight loads in flight
+                uint32_t m[8];
+#pragma unroll
+                for (int u = 0; u < 8; ++u) m[u] = in && w0 + u < words ? __ldcg(row + w0 + u) : 0u;
+#pragma unroll
+                for (int u = 0; u < 8; ++u) {
+                    m[u] = __reduce_or_sync(FULL, m[u]);
+                    if (lane == 0 && m[u]) atomicOr(&um[warp >> 2][w0 + u], m[u]);
+                }
             }
         } else if (in) {
             const int32_t *mine = lists + ((int64_t)bh * len + t0 + tid) * K;
             for (int i = 0; i < K; ++i) {
-                const int j = __ldg(mine + i);
+                const int j = __ldcg(mine + i);
                 if (j >= 0) atomicOr(&um[warp >> 2][j >> 5], 1u << (j & 31));
             }
         }
     }
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // the queries, written with ordinary stores, are read by the tensor core
     __syncthreads();
     if (warp == 0) {                                             // the list of blocks, ascending
         int base = 0;
@@ -191,7 +201,8 @@ __global__ void __launch_bounds__(kThreads, 1) moba_mma_kernel(const __grid_cons
                     tma_load_4d(vst + (size_t)st * G::C_BYTES + hf * (kChunk * 128), &tmap, hf * 64, 0, 1, page, &full_v[st]);
                 issued = i + 1;
             }
-            // after a wait that ran out: no copy may still be on its way into this CTA's shared memory when it exits
+            // no copy may still be on its way into this CTA's shared memory when it exits, after a wait that ran out either
+            ok = mbar_wait(&full_q, 0u) && ok;
             if (!ok)
                 for (int k = max(0, issued - NST); k < issued; ++k) {
                     mbar_wait(&full_k[k % NST], (uint32_t)((k / NST) & 1));
@@ -206,8 +217,9 @@ __global__ void __launch_bounds__(kThreads, 1) moba_mma_kernel(const __grid_cons
         const uint32_t ts = tb + s * ACC;
         int u = 0;                                               // products started
         Walk w;
+        ok = __all_sync(FULL, mbar_wait(&full_q, 0u));
 #pragma unroll 1
-        for (int i = 0; i < n; ++i, w.next(cpb)) {
+        for (int i = 0; i < n && ok; ++i, w.next(cpb)) {
             const int st = i % NST;
             // (waited for even if not used: the stage's release counts one arrival of each of the two warps per filling)
             ok = __all_sync(FULL, mbar_wait(&full_k[st], (uint32_t)((i / NST) & 1)));
@@ -275,14 +287,14 @@ __global__ void __launch_bounds__(kThreads, 1) moba_mma_kernel(const __grid_cons
             if (masks) {
                 if ((j >> 5) != w_at) {
                     const int w = j >> 5;
-                    w_cur = w_at >= 0 && w == w_at + 1 ? w_next : in ? __ldg(row + w) : 0u;
-                    w_next = in && w + 1 < words ? __ldg(row + w + 1) : 0u;
+                    w_cur = w_at >= 0 && w == w_at + 1 ? w_next : in ? __ldcg(row + w) : 0u;
+                    w_next = in && w + 1 < words ? __ldcg(row + w + 1) : 0u;
                     w_at = w;
                 }
                 chosen = (w_cur >> (j & 31)) & 1u;
             } else {
-                while (in && at < K && (uint32_t)__ldg(mine + at) < (uint32_t)j) ++at;     // (-1: beyond every block)
-                chosen = in && at < K && __ldg(mine + at) == j;
+                while (in && at < K && (uint32_t)__ldcg(mine + at) < (uint32_t)j) ++at;    // (-1: beyond every block)
+                chosen = in && at < K && __ldcg(mine + at) == j;
             }
             const int c = j * cpb + wk.r;
             const int64_t p0 = (int64_t)c * kChunk;
@@ -406,13 +418,24 @@ template <int D> cudaError_t attend_run(const MobaArgs &a, cudaStream_t s)
         if (e != cudaSuccess) return e;
         ready[dev] = true;
     }
-    alignas(64) CUtensorMap tmap;
+    alignas(64) CUtensorMap tmap, qmap;
     e = cache_tensor_map(&tmap, a.kv, D, a.S, (int64_t)BH * a.page_cap, kChunk);
     if (e != cudaSuccess) return e;
+    e = query_tensor_map(&qmap, a.q, D, a.H, a.len, a.B, kTile);
+    if (e != cudaSuccess) return e;
     const unsigned tiles = (unsigned)((a.len + kTile * kTiles - 1) / (kTile * kTiles));
-    moba_mma_kernel<D><<<dim3((unsigned)BH, tiles), kThreads, G::SMEM_BYTES, s>>>(
-        tmap, a.page_cap, a.S, a.len, (const bf16 *)a.q, a.H, a.block, nb, a.masks, a.list, a.K, a.scale * 1.4426950408889634f, (bf16 *)a.o, a.status);
-    return cudaGetLastError();
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute at = {};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cfg.gridDim = dim3((unsigned)BH, tiles);
+    cfg.blockDim = dim3(kThreads);
+    cfg.dynamicSmemBytes = G::SMEM_BYTES;
+    cfg.stream = s;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, moba_mma_kernel<D>, tmap, qmap, a.page_cap, a.S, a.len, a.H, a.block, nb, (const uint32_t *)a.masks,
+                              (const int32_t *)a.list, a.K, a.scale * 1.4426950408889634f, (bf16 *)a.o, a.status);
 }
 
 }  // namespace

@@ -13,6 +13,7 @@
 #include "rq_async.cuh"
 #include "rq_device.cuh"
 #include "rq_internal.h"
+#include "rq_tmap.h"
 #include "rq_umma.cuh"
 
 namespace rq {
@@ -35,6 +36,7 @@ __global__ void __launch_bounds__(256) moba_means_bf16_kernel(const bf16 *kv, in
 {
     const int per = D / 2, r = threadIdx.x / per, c = 2 * (threadIdx.x % per);
     const int j = blockIdx.x * (256 / per) + r, bh = blockIdx.y;
+    grid_launch_dependents();
     if (j >= nb) return;
     const int64_t lo = (int64_t)j * block, hi = min(lo + block, len);
     float s0 = 0.0f, s1 = 0.0f;
@@ -101,18 +103,18 @@ __device__ __forceinline__ uint32_t score_bin(float v, float lo, float inv)
 // A threshold bucket of more than 16 blocks is cut further by buckets on the scores' integer images until at most 16
 // are left or all left are equal (equal scores: the lowest blocks).  More than 512 blocks are taken in panels of 512,
 // whose scores are computed again for each pass (the tensor cores have nothing else to do here).
-// Measured, 32 heads x 128 channels: 4096 queries, 16 of 64 blocks each, 158 -> 58 us; 30011 queries, 30 of 469 blocks
-// each, 28.9 -> 1.35 ms (before: fp32 FMA scores, a lane per block, then a bit-wise vote search up to 128 blocks and one
+// Measured, 32 heads x 128 channels: 4096 queries, 16 of 64 blocks each, 158 -> 52 us; 30011 queries, 30 of 469 blocks
+// each, 28.9 -> 1.1 ms (queries by tensor map and four product steps per election: 58 -> 52 us of the former; before: fp32 FMA scores, a lane per block, then a bit-wise vote search up to 128 blocks and one
 // round per taken block beyond).
 template <int D>
-__global__ void __launch_bounds__(kRouteThreads, 2) moba_route_mma_kernel(const bf16 *q, const float *means, int64_t len, int H,
+__global__ void __launch_bounds__(kRouteThreads, 2) moba_route_mma_kernel(const __grid_constant__ CUtensorMap qmap, const float *means, int64_t len, int H,
                                                                       int block, int nb, int K, int words, uint32_t *masks,
                                                                       int32_t *list, int32_t *status)
 {
     using G = RouteGeom<D>;
     constexpr int NQ = kRouteQueries, NB = kRouteBins, CAP = kRouteCap;
     extern __shared__ __align__(1024) unsigned char rsm_raw[];
-    __shared__ __align__(8) uint64_t done;                                    // a product is complete
+    __shared__ __align__(8) uint64_t full_q, done;                                    // a product is complete
     __shared__ uint32_t tbase;
     unsigned char *sm = rsm_raw + ((1024u - (smem_addr(rsm_raw) & 1023u)) & 1023u);
     const int groups_all = (nb + kRouteGroup - 1) / kRouteGroup;
@@ -151,20 +153,19 @@ __global__ void __launch_bounds__(kRouteThreads, 2) moba_route_mma_kernel(const 
     if (any) {
         if (tid == 0) {
             mbar_init(&done, 1);
+            mbar_init(&full_q, 1);
             mbar_init_fence();
         }
         if (warp == 0) tmem_alloc(&tbase, tcols);
-        // the queries (q is [B][T][H][D]) as the K-major operand; rows past the prompt are zero
-        for (int i = tid; i < NQ * (D / 8); i += kRouteThreads) {
-            const int r = i / (D / 8), c = i % (D / 8);
-            uint4 v = make_uint4(0u, 0u, 0u, 0u);
-            if (t0 + r < len) v = *reinterpret_cast<const uint4 *>(q + (((int64_t)b * len + t0 + r) * H + h) * D + c * 8);
-            *reinterpret_cast<uint4 *>(qs + (c >> 3) * (NQ * 128) + umma_sw128_offset(r, c & 7)) = v;
-        }
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");           // ordinary stores, read by the tensor core
         tcgen05_before_sync();
         __syncthreads();
         tcgen05_after_sync();
+        if (warp == 0) {                                                       // the queries; rows past the prompt come as zeros
+            mbar_expect_warp(&full_q, G::Q_BYTES);
+#pragma unroll
+            for (int hf = 0; hf < G::HALVES; ++hf) tma_load_4d(qs + hf * (NQ * 128), &qmap, hf * 64, h, (int)t0, b, &full_q);
+        }
+        grid_dependency_wait();                                                // the representatives come from the kernel before
         const uint32_t tb = __shfl_sync(FULL, tbase, 0), tl = tb + ((uint32_t)((warp & 3) * 32) << 16);
         int used = 0;                                                          // products started
 
@@ -178,7 +179,7 @@ __global__ void __launch_bounds__(kRouteThreads, 2) moba_route_mma_kernel(const 
 #pragma unroll
                 for (int i = 0; i < PER; ++i) {
                     const int e = tid + i * kRouteThreads, j = g * kRouteGroup + e / (D / 4);
-                    f[i] = j < nb ? __ldg(reinterpret_cast<const float4 *>(means + ((int64_t)bh * nb + j) * D) + e % (D / 4))
+                    f[i] = j < nb ? __ldcg(reinterpret_cast<const float4 *>(means + ((int64_t)bh * nb + j) * D) + e % (D / 4))
                                   : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
                 }
             };
@@ -205,14 +206,14 @@ __global__ void __launch_bounds__(kRouteThreads, 2) moba_route_mma_kernel(const 
                 if (warp == 0) {
                     constexpr uint32_t idesc = umma_idesc_bf16(NQ, kRouteGroup);
                     const uint64_t qd = umma_desc_sw128(smem_addr(qs)), bd = umma_desc_sw128(smem_addr(bs));
+                    if (used == 0) ok = __all_sync(FULL, mbar_wait(&full_q, 0u) || mbar_wait(&full_q, 0u));
                     tcgen05_after_sync();
 #pragma unroll
                     for (int pl = 2; pl >= 0; --pl)                            // the smallest terms first
 #pragma unroll
-                        for (int k = 0; k < D / 16; ++k)
-                            umma_bf16(tb + (uint32_t)g * kRouteGroup, qd + (uint64_t)(((k >> 2) * (NQ * 128) + (k & 3) * 32) >> 4),
-                                      bd + (uint64_t)((pl * G::PLANE_BYTES + (k >> 2) * (kRouteGroup * 128) + (k & 3) * 32) >> 4), idesc,
-                                      !(pl == 2 && k == 0));
+                        for (int hf = 0; hf < G::HALVES; ++hf)
+                            umma_bf16_x4<2, 2>(tb + (uint32_t)g * kRouteGroup, qd + (uint64_t)((hf * (NQ * 128)) >> 4),
+                                               bd + (uint64_t)((pl * G::PLANE_BYTES + hf * (kRouteGroup * 128)) >> 4), idesc, !(pl == 2 && hf == 0));
                     umma_commit(&done);
                 }
                 ++used;
@@ -423,6 +424,8 @@ __global__ void __launch_bounds__(kRouteThreads, 2) moba_route_mma_kernel(const 
         if (warp == 0) tmem_dealloc(tbase, tcols);
     }
     if (!ok && tid == 0) atomicCAS(status, RQ_OK, RQ_ERR_TIMEOUT);
+    grid_dependency_wait();
+    grid_launch_dependents();
     __syncthreads();
     // the masks go out, with the first block and the query's own
     for (int i = tid; i < NQ * words; i += kRouteThreads) {
@@ -480,10 +483,23 @@ template <int D> cudaError_t route_run(const MobaArgs &a, cudaStream_t s)
     const int per = 256 / (D / 2);
     moba_means_bf16_kernel<<<dim3((unsigned)((nb + per - 1) / per), (unsigned)BH), 256, 0, s>>>(
         (const bf16 *)a.kv, a.page_cap, a.S, D, a.len, a.block, a.means, nb);
-    moba_route_mma_kernel<D><<<dim3((unsigned)BH, (unsigned)((a.len + kRouteQueries - 1) / kRouteQueries)), kRouteThreads,
-                               G::smem_bytes(one_panel, words), s>>>((const bf16 *)a.q, a.means, a.len, a.H, a.block, nb, a.K,
-                                                                            words, a.masks, a.list, a.status);
-    return cudaGetLastError();
+    e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    alignas(64) CUtensorMap qmap;
+    e = query_tensor_map(&qmap, a.q, D, a.H, a.len, a.B, kRouteQueries);
+    if (e != cudaSuccess) return e;
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute at = {};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cfg.gridDim = dim3((unsigned)BH, (unsigned)((a.len + kRouteQueries - 1) / kRouteQueries));
+    cfg.blockDim = dim3(kRouteThreads);
+    cfg.dynamicSmemBytes = (size_t)G::smem_bytes(one_panel, words);
+    cfg.stream = s;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, moba_route_mma_kernel<D>, qmap, (const float *)a.means, a.len, a.H, a.block, nb, a.K, words, a.masks,
+                              a.list, a.status);
 }
 
 }  // namespace

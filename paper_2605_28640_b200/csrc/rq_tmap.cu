@@ -39,6 +39,20 @@ cudaError_t cache_tensor_map(CUtensorMap *out, const void *kv, int D, int S, int
     return cudaSuccess;
 }
 
+cudaError_t query_tensor_map(CUtensorMap *out, const void *q, int D, int H, int64_t T, int B, int positions)
+{
+    const TensorMapEncodeTiled encode = tensor_map_encoder();
+    if (!encode) return cudaErrorNotSupported;
+    const cuuint64_t dims[4] = {(cuuint64_t)D, (cuuint64_t)H, (cuuint64_t)T, (cuuint64_t)B};
+    const cuuint64_t strides[3] = {(cuuint64_t)D * 2, (cuuint64_t)H * D * 2, (cuuint64_t)T * H * D * 2};
+    const cuuint32_t box[4] = {64, 1, (cuuint32_t)positions, 1}, steps[4] = {1, 1, 1, 1};
+    if (encode(out, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void *>(q), dims, strides, box, steps,
+               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+        return cudaErrorInvalidValue;
+    return cudaSuccess;
+}
+
 cudaError_t page_tensor_map(CUtensorMap *out, void *kv, int es, int D, int S, int64_t pages_total, int channels, int slots)
 {
     if (pages_total < 1 || pages_total >= ((int64_t)1 << 31)) return cudaErrorInvalidValue;   // box coordinates are 32-bit
