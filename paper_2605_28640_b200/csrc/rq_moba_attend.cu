@@ -68,12 +68,14 @@ struct Walk {
 // warp 11 the output products; they meet through mbarriers only, every wait bounded.  One warp for all products was the
 // limit: 24 products, six commits and as many waits a chunk (32 heads x 128, 30011 positions: 7.61 -> 6.13 ms; 4096: 234 -> 206 us).  256 queries per CTA because keys and values come
 // from L2 for every CTA.  A CTA's queries come by tensor map, and it may start before the routing kernel has ended: at 4096
-// positions a CTA lives 50 us only, and the 20 us before its first product were a third of that (206 -> 186 us).
+// positions a CTA lives 50 us only, and the 20 us before its first product were a third of that (206 -> 186 us; the
+// list by a lane per block and the outputs through shared memory 186 -> 181 us).
 template <int D>
 __global__ void __launch_bounds__(kThreads, 1) moba_mma_kernel(const __grid_constant__ CUtensorMap tmap,
-                                                               const __grid_constant__ CUtensorMap qmap, int64_t page_cap, int S,
+                                                               const __grid_constant__ CUtensorMap qmap,
+                                                               const __grid_constant__ CUtensorMap omap, int64_t page_cap, int S,
                                                                int64_t len, int H, int block, int nb,
-                                                               const uint32_t *masks, const int32_t *lists, int K, float scale_log2, bf16 *o, int32_t *status)
+                                                               const uint32_t *masks, const int32_t *lists, int K, float scale_log2, int32_t *status)
 {
     using G = AttGeom<D>;
     constexpr int NST = kStages;
@@ -149,22 +151,13 @@ __global__ void __launch_bounds__(kThreads, 1) moba_mma_kernel(const __grid_cons
     __syncthreads();
     if (warp == 0) {                                             // the list of blocks, ascending
         int base = 0;
-        for (int w0 = 0; w0 < words; w0 += 32) {
-            const int w = w0 + lane;
-            const uint32_t m0 = w < words ? um[0][w] : 0u, m1 = w < words ? um[1][w] : 0u;
-            const int cnt = __popc(m0 | m1);
-            int inc = cnt;
-#pragma unroll
-            for (int off = 1; off < 32; off <<= 1) {
-                const int v = __shfl_up_sync(FULL, inc, off);
-                if (lane >= off) inc += v;
-            }
-            int pos = base + inc - cnt;
-            for (uint32_t bits = m0 | m1; bits; bits &= bits - 1u, ++pos) {
-                const int i = __ffs(bits) - 1;
-                list[pos] = (uint16_t)((w * 32 + i) | (((m0 >> i) & 1u) << 14) | (((m1 >> i) & 1u) << 15));
-            }
-            base += __shfl_sync(FULL, inc, 31);
+#pragma unroll 4
+        for (int w = 0; w < words; ++w) {                        // a lane per block
+            const uint32_t m0 = um[0][w], m1 = um[1][w], m = m0 | m1;
+            if ((m >> lane) & 1u)
+                list[base + __popc(m & ((1u << lane) - 1u))] =
+                    (uint16_t)((w * 32 + lane) | (((m0 >> lane) & 1u) << 14) | (((m1 >> lane) & 1u) << 15));
+            base += __popc(m);
         }
         if (lane == 0) n_list = base;
     }
@@ -382,18 +375,27 @@ __global__ void __launch_bounds__(kThreads, 1) moba_mma_kernel(const __grid_cons
             if (__all_sync(FULL, ok)) {
                 tcgen05_after_sync();
                 const float l = l2.x + l2.y, inv = l > 0.0f ? 1.0f / l : 0.0f;
+                // (the accumulator's queries are not read any more: its rows go out through their room, a store per warp and
+                // 64 channels; rows past the prompt are cut off by the map)
+                unsigned char *os = qs + s * G::Q_BYTES + (warp & 3) * 32 * 128;
 #pragma unroll 1
                 for (int cb = 0; cb < D; cb += 32) {
                     float v[32];
                     tmem_ld32(tl + OFF_O + cb, v);
-                    if (in) {
-                        bf16 *orow = o + (((int64_t)b * len + tq) * H + h) * D + cb;
 #pragma unroll
-                        for (int k = 0; k < 32; k += 8)
-                            *reinterpret_cast<uint4 *>(orow + k) =
-                                make_uint4(pack_bf16(v[k] * inv, v[k + 1] * inv), pack_bf16(v[k + 2] * inv, v[k + 3] * inv),
-                                           pack_bf16(v[k + 4] * inv, v[k + 5] * inv), pack_bf16(v[k + 6] * inv, v[k + 7] * inv));
-                    }
+                    for (int k = 0; k < 32; k += 8)
+                        *reinterpret_cast<uint4 *>(os + (cb >> 6) * (kTile * 128) + umma_sw128_offset(lane, ((cb & 63) + k) >> 3)) =
+                            make_uint4(pack_bf16(v[k] * inv, v[k + 1] * inv), pack_bf16(v[k + 2] * inv, v[k + 3] * inv),
+                                       pack_bf16(v[k + 4] * inv, v[k + 5] * inv), pack_bf16(v[k + 6] * inv, v[k + 7] * inv));
+                }
+                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                __syncwarp();
+                if (tq - lane < len) {
+#pragma unroll
+                    for (int hf = 0; hf < G::HALVES; ++hf)
+                        tma_store_4d(os + hf * (kTile * 128), &omap, hf * 64, h, (int)(tq - lane), b);
+                    tma_store_commit();
+                    tma_store_wait_read();
                 }
             }
         }
@@ -418,10 +420,12 @@ template <int D> cudaError_t attend_run(const MobaArgs &a, cudaStream_t s)
         if (e != cudaSuccess) return e;
         ready[dev] = true;
     }
-    alignas(64) CUtensorMap tmap, qmap;
+    alignas(64) CUtensorMap tmap, qmap, omap;
     e = cache_tensor_map(&tmap, a.kv, D, a.S, (int64_t)BH * a.page_cap, kChunk);
     if (e != cudaSuccess) return e;
     e = query_tensor_map(&qmap, a.q, D, a.H, a.len, a.B, kTile);
+    if (e != cudaSuccess) return e;
+    e = query_tensor_map(&omap, a.o, D, a.H, a.len, a.B, 32);
     if (e != cudaSuccess) return e;
     const unsigned tiles = (unsigned)((a.len + kTile * kTiles - 1) / (kTile * kTiles));
     cudaLaunchConfig_t cfg = {};
@@ -434,8 +438,8 @@ template <int D> cudaError_t attend_run(const MobaArgs &a, cudaStream_t s)
     cfg.stream = s;
     cfg.attrs = &at;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, moba_mma_kernel<D>, tmap, qmap, a.page_cap, a.S, a.len, a.H, a.block, nb, (const uint32_t *)a.masks,
-                              (const int32_t *)a.list, a.K, a.scale * 1.4426950408889634f, (bf16 *)a.o, a.status);
+    return cudaLaunchKernelEx(&cfg, moba_mma_kernel<D>, tmap, qmap, omap, a.page_cap, a.S, a.len, a.H, a.block, nb, (const uint32_t *)a.masks,
+                              (const int32_t *)a.list, a.K, a.scale * 1.4426950408889634f, a.status);
 }
 
 }  // namespace

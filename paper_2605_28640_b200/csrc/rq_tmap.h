@@ -19,8 +19,9 @@ cudaError_t cache_tensor_map(CUtensorMap *out, const void *kv, int D, int S, int
 cudaError_t prompt_tensor_map(CUtensorMap *out, const void *x, int es, int D, int H, int64_t T, int B, int64_t sh, int64_t st, int64_t sb,
                               int channels, int positions);
 
-// [B][T][H][D] bf16 queries as a rank-4 tensor (channel, head, position, batch item); box = 64 channels x one head x
-// `positions` positions, 128-byte swizzle (the layout the tensor core reads); positions beyond T read as zero.
+// [B][T][H][D] bf16 queries (or outputs) as a rank-4 tensor (channel, head, position, batch item); box = 64 channels x one head x
+// `positions` positions, 128-byte swizzle (the layout the tensor core reads); positions beyond T read as
+// zero and are not stored.
 cudaError_t query_tensor_map(CUtensorMap *out, const void *q, int D, int H, int64_t T, int B, int positions);
 
 // The paged cache with elements of `es` bytes as a rank-4 tensor (channel, slot, key / value, page); box = `channels` channels
