@@ -32,6 +32,8 @@
 #include <math.h>
 #include <math_constants.h>
 
+#include <utility>
+
 #include "rq_async.cuh"
 #include "rq_device.cuh"
 #include "rq_internal.h"
@@ -41,6 +43,8 @@
 namespace rq {
 
 namespace {
+
+namespace cg = cooperative_groups;
 
 constexpr int kSnapRows = 64;                  // queries of the window (fewer: the rest is masked)
 constexpr int kSnapKeys = 128;                 // keys per tile
@@ -385,6 +389,243 @@ __global__ void __launch_bounds__(kMmaThreads) snap_mma_kernel(const __grid_cons
     if (warp == 0) tmem_dealloc(tbase, TCOLS);
 }
 
+// ---------------------------------------------------------------- short prompts: the keys read once
+// A cluster of up to kOnceCluster CTAs per head, each with up to RT tiles of 128 keys.  The scores of the head, 64 columns
+// of fp32 per tile, stay in the cluster's tensor memory between the passes, so that the keys come from HBM once:
+//   tiles    D[key][query] = K Q^T as they land; running maximum of every query over the thread's keys
+//   maximum  of a query over the lanes, the warps and (distributed shared memory) the CTAs of the cluster
+//   weights  2^(s - max) written over the scores, their sums over lanes, warps and CTAs in the same way
+//   sums     of a key's weights, each times 1 / (sum of its query): the importance
+// Warps 0..7 read the accumulators (a lane per key, a warp per half of the queries), warp 8 copies and multiplies.  The
+// maximum is the head's before a weight is taken, as in the two-pass kernels: equal keys get equal importance wherever they
+// lie.
+constexpr int kOnceWarps = 8;
+constexpr int kOnceThreads = (kOnceWarps + 1) * 32;
+constexpr int kOnceCluster = 8;
+
+template <int D>
+struct SnapOnceGeom {
+    static constexpr int HALVES = D / 64;
+    static constexpr int QH_BYTES = kSnapRows * 128;           // 64 channels of the window's queries
+    static constexpr int KH_BYTES = kMmaKeys * 128;            // 64 channels of a tile
+    static constexpr int OFF_K = HALVES * QH_BYTES;
+    static constexpr int TILE_BYTES = HALVES * KH_BYTES;
+    static constexpr int SMEM_BYTES = OFF_K + 2 * TILE_BYTES + 1024;
+};
+
+// Lane l's result: OP over the 32 lanes of their v[l].
+template <bool MAX> __device__ __forceinline__ float lanes_reduce(float (&v)[32], int lane)
+{
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) {
+        const bool up = lane & off;
+#pragma unroll
+        for (int i = 0; i < off; ++i) {
+            const float got = __shfl_xor_sync(0xffffffffu, up ? v[i] : v[i + off], off), mine = up ? v[i + off] : v[i];
+            v[i] = MAX ? fmaxf(mine, got) : mine + got;
+        }
+    }
+    return v[0];
+}
+
+template <int D, int RT>
+__global__ void __launch_bounds__(kOnceThreads, RT <= 4 ? 2 : 1) snap_once_kernel(const __grid_constant__ CUtensorMap tmap,
+                                                                                int64_t page_cap, int S, int64_t len, const bf16 *qw,
+                                                                                int W, int H, float scale_log2, float *imp, int ntiles,
+                                                                                int tiles_per_cta, int32_t *status)
+{
+    using G = SnapOnceGeom<D>;
+    constexpr uint32_t TCOLS = RT * kSnapRows;
+    extern __shared__ __align__(1024) unsigned char osm_raw[];
+    __shared__ __align__(8) uint64_t bar[RT], full[2];         // a tile's product is complete; a stage's keys have landed
+    __shared__ uint32_t tbase;
+    __shared__ float red[4][kSnapRows];                        // per quarter of the keys and query
+    __shared__ float xch[2][kOnceCluster][kSnapRows];          // what every CTA of the cluster found: maxima, sums
+    __shared__ __align__(16) float ref[kSnapRows];             // per query: the maximum, then 1 / sum
+    __shared__ float part[RT][kMmaKeys];                       // importance of a key from the upper half of the queries
+    cg::cluster_group cl = cg::this_cluster();
+    cg::cluster_group::arrival_token started = cl.barrier_arrive();
+    unsigned char *dsm = osm_raw + ((1024u - (smem_addr(osm_raw) & 1023u)) & 1023u);
+    unsigned char *qs = dsm, *ks = dsm + G::OFF_K;
+
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int bh = blockIdx.y, b = bh / H, h = bh % H, rank = blockIdx.x, ranks = gridDim.x;
+    const int t0 = rank * tiles_per_cta, n = max(0, min(tiles_per_cta, ntiles - t0));
+    const int64_t first_q = len - W;
+    const int ppt = kMmaKeys / S;
+    if (tid == 0) {
+        for (int i = 0; i < RT; ++i) mbar_init(&bar[i], 1);
+        mbar_init(&full[0], 1);
+        mbar_init(&full[1], 1);
+        mbar_init_fence();
+    }
+    if (warp == kOnceWarps) tmem_alloc(&tbase, TCOLS);
+    for (int i = tid; i < kSnapRows * (D / 8); i += kOnceThreads) {   // the window's queries (qw is [B][W][H][D])
+        const int r = i / (D / 8), c = i % (D / 8);
+        uint4 v = make_uint4(0u, 0u, 0u, 0u);
+        if (r < W) v = *reinterpret_cast<const uint4 *>(qw + (((int64_t)b * W + r) * H + h) * D + c * 8);
+        *reinterpret_cast<uint4 *>(qs + (c >> 3) * G::QH_BYTES + umma_sw128_offset(r, c & 7)) = v;
+    }
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // the queries, written with ordinary stores, are read by the tensor core
+    tcgen05_before_sync();
+    __syncthreads();
+    tcgen05_after_sync();
+    const uint32_t tb = __shfl_sync(0xffffffffu, tbase, 0);
+
+    bool ok = true;
+    const int half = (warp >> 2) & 1, quad = warp & 3, row = quad * 32 + lane;   // readers: half of the queries, key of a tile
+    const bool reader = warp < kOnceWarps;
+    const uint32_t tl = tb + (uint32_t)half * 32u + ((uint32_t)(quad * 32) << 16);
+    float v[32], a[32];
+    // query half * 32 + c of the window sees this thread's key of tile i if c >= the result (32: none does)
+    auto first_seen = [&](int i) -> int {
+        const int64_t q_lo = (int64_t)(t0 + i) * kMmaKeys + row - first_q;
+        return (int)min((int64_t)32, max((int64_t)0, q_lo - half * 32));
+    };
+    const int c_end = min(32, max(0, W - half * 32));          // queries of this half
+    auto cut = [&](int i) { return W < kSnapRows || (int64_t)(t0 + i + 1) * kMmaKeys - 1 > first_q; };   // some key is not seen by all 64
+    if (!reader) {
+        // ---- copies and products (the whole warp, see rq_umma.cuh)
+        auto page_of = [&](int i) { return (int)((int64_t)bh * page_cap + (int64_t)(t0 + i) * ppt); };
+        auto issue = [&](int i) {
+            mbar_expect_warp(&full[i & 1], G::TILE_BYTES);
+#pragma unroll
+            for (int hf = 0; hf < G::HALVES; ++hf)
+                tma_load_4d(ks + (i & 1) * G::TILE_BYTES + hf * G::KH_BYTES, &tmap, hf * 64, 0, 0, page_of(i), &full[i & 1]);
+        };
+        for (int i = 0; i < n && i < 2; ++i) issue(i);
+        for (int i = 2; i < n; ++i)                            // the rest is asked into L2: its copies are short when their turn comes
+#pragma unroll
+            for (int hf = 0; hf < G::HALVES; ++hf) tma_prefetch_4d(&tmap, hf * 64, 0, 0, page_of(i));
+        constexpr uint32_t idesc = umma_idesc_bf16(kMmaKeys, kSnapRows);
+        const uint64_t qd = umma_desc_sw128(smem_addr(qs)), kd = umma_desc_sw128(smem_addr(ks));
+        int issued = min(n, 2), landed = 0;
+#pragma unroll 1
+        for (int i = 0; i < n; ++i) {
+            ok = __all_sync(0xffffffffu, mbar_wait(&full[i & 1], (uint32_t)((i >> 1) & 1)));
+            if (!ok) break;
+            landed = i + 1;
+            tcgen05_after_sync();
+#pragma unroll
+            for (int hf = 0; hf < G::HALVES; ++hf)
+                umma_bf16_x4<2, 2>(tb + (uint32_t)i * kSnapRows, kd + (uint64_t)(((i & 1) * G::TILE_BYTES + hf * G::KH_BYTES) >> 4),
+                                   qd + (uint64_t)((hf * G::QH_BYTES) >> 4), idesc, hf > 0);
+            umma_commit(&bar[i]);
+            if (i + 2 < n) {
+                ok = __all_sync(0xffffffffu, mbar_wait(&bar[i], 0u));    // the product has read the stage
+                if (!ok) break;
+                issue(i + 2);
+                issued = i + 3;
+            }
+        }
+        // after a wait that ran out: no copy may still be on its way into this CTA's shared memory when it exits
+        for (int i = landed; i < issued; ++i) mbar_wait(&full[i & 1], (uint32_t)((i >> 1) & 1));
+    } else {
+#pragma unroll
+        for (int c = 0; c < 32; ++c) a[c] = -CUDART_INF_F;
+#pragma unroll 1
+        for (int i = 0; i < n; ++i) {
+            ok = __all_sync(0xffffffffu, mbar_wait(&bar[i], 0u));
+            if (!ok) break;
+            tcgen05_after_sync();
+            tmem_ld32(tl + (uint32_t)i * kSnapRows, v);
+            if (cut(i)) {
+                const int c_lo = first_seen(i);
+#pragma unroll
+                for (int c = 0; c < 32; ++c) a[c] = c >= c_lo && c < c_end ? fmaxf(a[c], v[c] * scale_log2) : a[c];
+            } else {
+#pragma unroll
+                for (int c = 0; c < 32; ++c) a[c] = fmaxf(a[c], v[c] * scale_log2);
+            }
+        }
+        red[quad][half * 32 + lane] = lanes_reduce<true>(a, lane);
+    }
+    // one number per query from every CTA: red over the quarters, out to all, in again
+    auto exchange = [&](int which, auto op) -> float {
+        __syncthreads();
+        const int q = tid & (kSnapRows - 1);
+        const float mine = op(op(red[0][q], red[1][q]), op(red[2][q], red[3][q]));
+        if (reader)
+            for (int r = tid / kSnapRows; r < ranks; r += kOnceWarps * 32 / kSnapRows) *cl.map_shared_rank(&xch[which][rank][q], r) = mine;
+        cl.sync();
+        float x = xch[which][0][q];
+        for (int r = 1; r < ranks; ++r) x = op(x, xch[which][r][q]);
+        return x;
+    };
+    cl.barrier_wait(std::move(started));                       // every CTA of the cluster runs: its shared memory may be written
+    const float top = exchange(0, [](float x, float y) { return fmaxf(x, y); });
+    if (tid < kSnapRows) ref[tid] = top > -CUDART_INF_F ? top : 0.0f;
+    __syncthreads();
+    if (reader) {
+#pragma unroll
+        for (int c = 0; c < 32; ++c) a[c] = 0.0f;
+        if (ok) {
+#pragma unroll 1
+            for (int i = 0; i < n; ++i) {
+                tmem_ld32(tl + (uint32_t)i * kSnapRows, v);
+#pragma unroll
+                for (int c = 0; c < 32; c += 4) {
+                    const float4 m = *reinterpret_cast<const float4 *>(&ref[half * 32 + c]);
+                    v[c] = exp2_fast(fmaf(v[c], scale_log2, -m.x));
+                    v[c + 1] = exp2_fast(fmaf(v[c + 1], scale_log2, -m.y));
+                    v[c + 2] = exp2_fast(fmaf(v[c + 2], scale_log2, -m.z));
+                    v[c + 3] = exp2_fast(fmaf(v[c + 3], scale_log2, -m.w));
+                }
+                if (cut(i)) {
+                    const int c_lo = first_seen(i);
+#pragma unroll
+                    for (int c = 0; c < 32; ++c) v[c] = c >= c_lo && c < c_end ? v[c] : 0.0f;
+                }
+#pragma unroll
+                for (int hf = 0; hf < 2; ++hf) {
+                    uint32_t w[16];
+#pragma unroll
+                    for (int c = 0; c < 16; ++c) {
+                        a[hf * 16 + c] += v[hf * 16 + c];
+                        w[c] = __float_as_uint(v[hf * 16 + c]);
+                    }
+                    tmem_st16(tl + (uint32_t)i * kSnapRows + hf * 16, w);
+                }
+            }
+            tmem_st_wait();
+        }
+        red[quad][half * 32 + lane] = lanes_reduce<false>(a, lane);
+    }
+    const float sum = exchange(1, [](float x, float y) { return x + y; });
+    if (tid < kSnapRows) ref[tid] = tid < W && sum > 0.0f ? 1.0f / sum : 0.0f;
+    __syncthreads();
+    float acc[RT];
+    if (reader && ok) {
+#pragma unroll
+        for (int i = 0; i < RT; ++i) {
+            if (i >= n) break;
+            tmem_ld32(tl + (uint32_t)i * kSnapRows, v);
+            float s = 0.0f;
+#pragma unroll
+            for (int c = 0; c < 32; c += 4) {
+                const float4 f = *reinterpret_cast<const float4 *>(&ref[half * 32 + c]);
+                s = fmaf(v[c], f.x, s);
+                s = fmaf(v[c + 1], f.y, s);
+                s = fmaf(v[c + 2], f.z, s);
+                s = fmaf(v[c + 3], f.w, s);
+            }
+            acc[i] = s;
+            if (half) part[i][row] = s;
+        }
+    }
+    if (__any_sync(0xffffffffu, !ok) && lane == 0) atomicCAS(status, RQ_OK, RQ_ERR_TIMEOUT);
+    tcgen05_before_sync();
+    __syncthreads();
+    if (reader && ok && !half) {
+#pragma unroll
+        for (int i = 0; i < RT; ++i) {
+            const int64_t j = (int64_t)(t0 + i) * kMmaKeys + row;
+            if (i < n && j < len) imp[(int64_t)bh * len + j] = acc[i] + part[i][row];
+        }
+    }
+    if (warp == kOnceWarps) tmem_dealloc(tbase, TCOLS);
+}
+
 // Final statistics of a row: merge of its tiles' (max, sum exp).  One warp per (head, row).
 __global__ void __launch_bounds__(128) snap_rows_kernel(const float2 *stats, float2 *rowstat, int ntiles, int n_rows_total)
 {
@@ -429,7 +670,6 @@ template <int EPT, int NT>
 __global__ void __launch_bounds__(NT, 1024 / NT) snap_select_kernel(const float *imp, int64_t len, int w, int keep,
                                                                                    int per_warp, int32_t *idx)
 {
-    namespace cg = cooperative_groups;
     constexpr unsigned FULL = 0xffffffffu;
     constexpr int NW = NT / 32, BPT = kSnapBins / NT;            // a thread adds up BPT buckets
     __shared__ __align__(16) uint32_t hist[2][kSnapBins];
@@ -757,6 +997,41 @@ cudaError_t snap_scores_t(const SnapArgs &a, cudaStream_t s)
     return cudaGetLastError();
 }
 
+// The same for prompts whose scores fit in the tensor memory of a cluster: tiles per CTA and CTAs per head.
+template <int D, int RT>
+cudaError_t snap_scores_once(const SnapArgs &a, const CUtensorMap &tmap, int ntiles, cudaStream_t s)
+{
+    using G = SnapOnceGeom<D>;
+    static bool ready[64];
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
+    if (!ready[dev]) {
+        e = cudaFuncSetAttribute(snap_once_kernel<D, RT>, cudaFuncAttributeMaxDynamicSharedMemorySize, G::SMEM_BYTES);
+        if (e != cudaSuccess) return e;
+        ready[dev] = true;
+    }
+    const int BH = a.B * a.H, slots = (RT <= 4 ? 2 : 1) * sm_count();
+    // as few CTAs per head as hold its tiles, more while the chip has room for them at once
+    int cl = (ntiles + RT - 1) / RT;
+    while (cl < kOnceCluster && cl < ntiles && BH * (cl + 1) <= slots) ++cl;
+    const int tpc = (ntiles + cl - 1) / cl;
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute at = {};
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = (unsigned)cl;
+    at.val.clusterDim.y = at.val.clusterDim.z = 1;
+    cfg.gridDim = dim3((unsigned)cl, (unsigned)BH);
+    cfg.blockDim = dim3(kOnceThreads);
+    cfg.dynamicSmemBytes = G::SMEM_BYTES;
+    cfg.stream = s;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, snap_once_kernel<D, RT>, tmap, a.page_cap, a.S, a.len, (const bf16 *)a.qw, a.W, a.H,
+                              a.scale * 1.4426950408889634f, a.imp, ntiles, tpc, a.status);
+}
+
 template <int D>
 cudaError_t snap_scores_mma(const SnapArgs &a, cudaStream_t s)
 {
@@ -779,6 +1054,8 @@ cudaError_t snap_scores_mma(const SnapArgs &a, cudaStream_t s)
     e = cache_tensor_map(&tmap, a.kv, D, a.S, (int64_t)BH * a.page_cap, kMmaKeys);
     if (e != cudaSuccess) return e;
     const int ntiles = (int)((a.len + kMmaKeys - 1) / kMmaKeys);
+    if (ntiles <= 4 * kOnceCluster) return snap_scores_once<D, 4>(a, tmap, ntiles, s);
+    if (ntiles <= 8 * kOnceCluster) return snap_scores_once<D, 8>(a, tmap, ntiles, s);
     // tiles per CTA: two CTAs share an SM, so the launch runs in rounds of 2 * SMs CTAs; the choice with the fewest
     // rounds * (tiles of a CTA + what a CTA costs before its first tile, about two tiles' time) ends soonest
     const int64_t slots = 2 * (int64_t)sm_count();
