@@ -7,10 +7,12 @@
 //   importance[j] = sum_i softmax_j(scale * q_i . k~_j),  query i at position T - W + i sees j <= T - W + i
 //
 // Kernels.  The importance is a dense contraction (W x D x T per head) followed by a softmax over T
-// and a sum over the window.  The 64 x T scores of a head are never stored: the keys are read twice,
+// and a sum over the window.  The 64 x T scores of a long head are not stored: its keys are read twice,
 // once for the row statistics (maximum and sum of exponentials of every query) and once for the
 // weights.
-//   snap_mma_kernel<PASS 1>   bf16 caches.  Per (head, run of 128-key tiles): the scores of a tile on the
+//   snap_once_kernel          bf16 caches, up to 8192 positions: the scores do fit in the tensor memory of a cluster of CTAs
+//                             and the keys are read once
+//   snap_mma_kernel<PASS 1>   longer bf16 caches.  Per (head, run of 128-key tiles): the scores of a tile on the
 //                             tensor cores (tcgen05.mma, operands in shared memory, fp32 accumulator
 //                             in tensor memory): D[query][key] with the window's queries as the M
 //                             side (both halves of the 128 rows hold the same 64 queries, so that all
@@ -248,10 +250,6 @@ __global__ void __launch_bounds__(kMmaThreads) snap_mma_kernel(const __grid_cons
         if (qr < W) v = *reinterpret_cast<const uint4 *>(qw + (((int64_t)b * W + qr) * H + h) * D + c * 8);
         *reinterpret_cast<uint4 *>(qs + (c >> 3) * G::HALF_BYTES + umma_sw128_offset(r, c & 7)) = v;
     }
-    if (PASS == 2 && tid < kSnapRows) {
-        const float2 f = tid < W ? rowstat[(int64_t)bh * kSnapRows + tid] : make_float2(0.0f, 1.0f);
-        qst[tid] = make_float2(f.x, 1.0f / f.y);
-    }
     // the keys of tile t (relative to t0) into its stage: position j lives in page j / S, slot j % S of the
     // head's cache; pages past the head's last one hold somebody else's rows or nothing, and every key at
     // or beyond `len` is masked where the scores are used.  One warp.
@@ -278,6 +276,7 @@ __global__ void __launch_bounds__(kMmaThreads) snap_mma_kernel(const __grid_cons
 
     const int row = tid & (kSnapRows - 1), half = (tid >> 6) & 1;   // pass 1: this thread's query and half of the tile's keys
     float m = -CUDART_INF_F, l = 0.0f;                         // pass 1: running statistics
+    grid_launch_dependents();
     bool ok = true;
     if (warp == kMmaWarps) {
         // ---- the producing warp starts the copies and the products (all its lanes run this, see rq_umma.cuh);
@@ -318,6 +317,14 @@ __global__ void __launch_bounds__(kMmaThreads) snap_mma_kernel(const __grid_cons
             for (int k = n_landed; k < n_issued; ++k) mbar_wait(&full[k % NST], (uint32_t)((k / NST) & 1));
         }
     } else {
+    if (PASS == 2) {
+        grid_dependency_wait();                                // the statistics come from the kernel before, the keys do not
+        if (tid < kSnapRows) {
+            const float2 f = tid < W ? __ldcg(rowstat + (int64_t)bh * kSnapRows + tid) : make_float2(0.0f, 1.0f);
+            qst[tid] = make_float2(f.x, 1.0f / f.y);
+        }
+        asm volatile("bar.sync 1, %0;" ::"n"(kMmaWarps * 32) : "memory");
+    }
 #pragma unroll 1
     for (int i = 0; i < n; ++i) {
         ok = mbar_wait(&bar[i & 1], (uint32_t)((i >> 1) & 1));
@@ -398,7 +405,8 @@ __global__ void __launch_bounds__(kMmaThreads) snap_mma_kernel(const __grid_cons
 //   sums     of a key's weights, each times 1 / (sum of its query): the importance
 // Warps 0..7 read the accumulators (a lane per key, a warp per half of the queries), warp 8 copies and multiplies.  The
 // maximum is the head's before a weight is taken, as in the two-pass kernels: equal keys get equal importance wherever they
-// lie.
+// lie.  Bound by the chain of a CTA (copies, two exchanges over the cluster, three walks over the scores: 11 us for 512
+// keys), which two CTAs per SM overlap.  256 heads x 4096 keys x 128 channels: 124 (two passes and the merge) -> 95 us.
 constexpr int kOnceWarps = 8;
 constexpr int kOnceThreads = (kOnceWarps + 1) * 32;
 constexpr int kOnceCluster = 8;
@@ -430,14 +438,15 @@ template <bool MAX> __device__ __forceinline__ float lanes_reduce(float (&v)[32]
 
 template <int D, int RT>
 __global__ void __launch_bounds__(kOnceThreads, RT <= 4 ? 2 : 1) snap_once_kernel(const __grid_constant__ CUtensorMap tmap,
-                                                                                int64_t page_cap, int S, int64_t len, const bf16 *qw,
-                                                                                int W, int H, float scale_log2, float *imp, int ntiles,
+                                                                                const __grid_constant__ CUtensorMap qmap,
+                                                                                int64_t page_cap, int S, int64_t len, int W, int H,
+                                                                                float scale_log2, float *imp, int ntiles,
                                                                                 int tiles_per_cta, int32_t *status)
 {
     using G = SnapOnceGeom<D>;
     constexpr uint32_t TCOLS = RT * kSnapRows;
     extern __shared__ __align__(1024) unsigned char osm_raw[];
-    __shared__ __align__(8) uint64_t bar[RT], full[2];         // a tile's product is complete; a stage's keys have landed
+    __shared__ __align__(8) uint64_t bar[RT], full[2], full_q; // a tile's product is complete; a stage's keys, the queries have landed
     __shared__ uint32_t tbase;
     __shared__ float red[4][kSnapRows];                        // per quarter of the keys and query
     __shared__ float xch[2][kOnceCluster][kSnapRows];          // what every CTA of the cluster found: maxima, sums
@@ -453,20 +462,31 @@ __global__ void __launch_bounds__(kOnceThreads, RT <= 4 ? 2 : 1) snap_once_kerne
     const int t0 = rank * tiles_per_cta, n = max(0, min(tiles_per_cta, ntiles - t0));
     const int64_t first_q = len - W;
     const int ppt = kMmaKeys / S;
-    if (tid == 0) {
-        for (int i = 0; i < RT; ++i) mbar_init(&bar[i], 1);
-        mbar_init(&full[0], 1);
-        mbar_init(&full[1], 1);
-        mbar_init_fence();
+    auto page_of = [&](int i) { return (int)((int64_t)bh * page_cap + (int64_t)(t0 + i) * ppt); };
+    auto issue = [&](int i) {
+        mbar_expect_warp(&full[i & 1], G::TILE_BYTES);
+#pragma unroll
+        for (int hf = 0; hf < G::HALVES; ++hf)
+            tma_load_4d(ks + (i & 1) * G::TILE_BYTES + hf * G::KH_BYTES, &tmap, hf * 64, 0, 0, page_of(i), &full[i & 1]);
+    };
+    if (warp == kOnceWarps) {                                  // copies start before anything else
+        if (lane == 0) {
+            for (int i = 0; i < RT; ++i) mbar_init(&bar[i], 1);
+            mbar_init(&full[0], 1);
+            mbar_init(&full[1], 1);
+            mbar_init(&full_q, 1);
+            mbar_init_fence();
+        }
+        __syncwarp();
+        mbar_expect_warp(&full_q, G::HALVES * G::QH_BYTES);    // the window's queries; rows beyond the window come as zeros
+#pragma unroll
+        for (int hf = 0; hf < G::HALVES; ++hf) tma_load_4d(qs + hf * G::QH_BYTES, &qmap, hf * 64, h, 0, b, &full_q);
+        for (int i = 0; i < n && i < 2; ++i) issue(i);
+        for (int i = 2; i < n; ++i)                            // the rest is asked into L2: its copies are short when their turn comes
+#pragma unroll
+            for (int hf = 0; hf < G::HALVES; ++hf) tma_prefetch_4d(&tmap, hf * 64, 0, 0, page_of(i));
     }
-    if (warp == kOnceWarps) tmem_alloc(&tbase, TCOLS);
-    for (int i = tid; i < kSnapRows * (D / 8); i += kOnceThreads) {   // the window's queries (qw is [B][W][H][D])
-        const int r = i / (D / 8), c = i % (D / 8);
-        uint4 v = make_uint4(0u, 0u, 0u, 0u);
-        if (r < W) v = *reinterpret_cast<const uint4 *>(qw + (((int64_t)b * W + r) * H + h) * D + c * 8);
-        *reinterpret_cast<uint4 *>(qs + (c >> 3) * G::QH_BYTES + umma_sw128_offset(r, c & 7)) = v;
-    }
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // the queries, written with ordinary stores, are read by the tensor core
+    if (warp == 0) tmem_alloc(&tbase, TCOLS);
     tcgen05_before_sync();
     __syncthreads();
     tcgen05_after_sync();
@@ -486,22 +506,12 @@ __global__ void __launch_bounds__(kOnceThreads, RT <= 4 ? 2 : 1) snap_once_kerne
     auto cut = [&](int i) { return W < kSnapRows || (int64_t)(t0 + i + 1) * kMmaKeys - 1 > first_q; };   // some key is not seen by all 64
     if (!reader) {
         // ---- copies and products (the whole warp, see rq_umma.cuh)
-        auto page_of = [&](int i) { return (int)((int64_t)bh * page_cap + (int64_t)(t0 + i) * ppt); };
-        auto issue = [&](int i) {
-            mbar_expect_warp(&full[i & 1], G::TILE_BYTES);
-#pragma unroll
-            for (int hf = 0; hf < G::HALVES; ++hf)
-                tma_load_4d(ks + (i & 1) * G::TILE_BYTES + hf * G::KH_BYTES, &tmap, hf * 64, 0, 0, page_of(i), &full[i & 1]);
-        };
-        for (int i = 0; i < n && i < 2; ++i) issue(i);
-        for (int i = 2; i < n; ++i)                            // the rest is asked into L2: its copies are short when their turn comes
-#pragma unroll
-            for (int hf = 0; hf < G::HALVES; ++hf) tma_prefetch_4d(&tmap, hf * 64, 0, 0, page_of(i));
         constexpr uint32_t idesc = umma_idesc_bf16(kMmaKeys, kSnapRows);
         const uint64_t qd = umma_desc_sw128(smem_addr(qs)), kd = umma_desc_sw128(smem_addr(ks));
         int issued = min(n, 2), landed = 0;
+        ok = __all_sync(0xffffffffu, mbar_wait(&full_q, 0u) || mbar_wait(&full_q, 0u));
 #pragma unroll 1
-        for (int i = 0; i < n; ++i) {
+        for (int i = 0; i < n && ok; ++i) {
             ok = __all_sync(0xffffffffu, mbar_wait(&full[i & 1], (uint32_t)((i >> 1) & 1)));
             if (!ok) break;
             landed = i + 1;
@@ -614,6 +624,7 @@ __global__ void __launch_bounds__(kOnceThreads, RT <= 4 ? 2 : 1) snap_once_kerne
         }
     }
     if (__any_sync(0xffffffffu, !ok) && lane == 0) atomicCAS(status, RQ_OK, RQ_ERR_TIMEOUT);
+    grid_launch_dependents();
     tcgen05_before_sync();
     __syncthreads();
     if (reader && ok && !half) {
@@ -623,18 +634,20 @@ __global__ void __launch_bounds__(kOnceThreads, RT <= 4 ? 2 : 1) snap_once_kerne
             if (i < n && j < len) imp[(int64_t)bh * len + j] = acc[i] + part[i][row];
         }
     }
-    if (warp == kOnceWarps) tmem_dealloc(tbase, TCOLS);
+    if (warp == 0) tmem_dealloc(tbase, TCOLS);
 }
 
 // Final statistics of a row: merge of its tiles' (max, sum exp).  One warp per (head, row).
 __global__ void __launch_bounds__(128) snap_rows_kernel(const float2 *stats, float2 *rowstat, int ntiles, int n_rows_total)
 {
     const int w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+    grid_launch_dependents();
     if (w >= n_rows_total) return;
+    grid_dependency_wait();
     const int bh = w / kSnapRows, row = w % kSnapRows;
     float m = -CUDART_INF_F, l = 0.0f;
     for (int t = lane; t < ntiles; t += 32) {
-        const float2 f = stats[((int64_t)bh * ntiles + t) * kSnapRows + row];
+        const float2 f = __ldcg(stats + ((int64_t)bh * ntiles + t) * kSnapRows + row);
         if (f.x > -CUDART_INF_F) {
             const float mn = fmaxf(m, f.x);
             l = l * exp2f(m - mn) + f.y * exp2f(f.x - mn);     // exp2f(-inf) = 0 on the first merge
@@ -682,6 +695,7 @@ __global__ void __launch_bounds__(NT, 1024 / NT) snap_select_kernel(const float 
     const float *x = imp + (int64_t)bh * len;
     int32_t *out = idx + (int64_t)bh * keep;
     const int C = (int)(len - w), want = keep - w;
+    grid_dependency_wait();                          // the importances come from the kernel before
     if (want >= C || want <= 0) {                    // everything is kept, or nothing but the window
         if (cr == 0)
             for (int j = tid; j < keep; j += NT) out[j] = want <= 0 ? C + j : j < len ? j : -1;
@@ -1017,6 +1031,9 @@ cudaError_t snap_scores_once(const SnapArgs &a, const CUtensorMap &tmap, int nti
     int cl = (ntiles + RT - 1) / RT;
     while (cl < kOnceCluster && cl < ntiles && BH * (cl + 1) <= slots) ++cl;
     const int tpc = (ntiles + cl - 1) / cl;
+    alignas(64) CUtensorMap qmap;
+    e = query_tensor_map(&qmap, a.qw, D, a.H, a.W, a.B, kSnapRows);
+    if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute at = {};
     at.id = cudaLaunchAttributeClusterDimension;
@@ -1028,8 +1045,8 @@ cudaError_t snap_scores_once(const SnapArgs &a, const CUtensorMap &tmap, int nti
     cfg.stream = s;
     cfg.attrs = &at;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, snap_once_kernel<D, RT>, tmap, a.page_cap, a.S, a.len, (const bf16 *)a.qw, a.W, a.H,
-                              a.scale * 1.4426950408889634f, a.imp, ntiles, tpc, a.status);
+    return cudaLaunchKernelEx(&cfg, snap_once_kernel<D, RT>, tmap, qmap, a.page_cap, a.S, a.len, a.W, a.H, a.scale * 1.4426950408889634f, a.imp,
+                              ntiles, tpc, a.status);
 }
 
 template <int D>
@@ -1074,11 +1091,26 @@ cudaError_t snap_scores_mma(const SnapArgs &a, cudaStream_t s)
     const float sl2 = a.scale * 1.4426950408889634f;
     snap_mma_kernel<D, 1><<<grid, kMmaThreads, G::SMEM_BYTES, s>>>(tmap, a.page_cap, a.S, a.len, (const bf16 *)a.qw, a.W, a.H, sl2,
                                                                  a.stats, nullptr, nullptr, ntiles, tpc, a.status);
+    e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    // the next two may start before the one ahead of them has ended: the second pass's first keys are on their way by then
     const int rows = BH * kSnapRows;
-    snap_rows_kernel<<<(rows * 32 + 127) / 128, 128, 0, s>>>(a.stats, a.rowstat, runs, rows);
-    snap_mma_kernel<D, 2><<<grid, kMmaThreads, G::SMEM_BYTES, s>>>(tmap, a.page_cap, a.S, a.len, (const bf16 *)a.qw, a.W, a.H, sl2,
-                                                                 nullptr, a.rowstat, a.imp, ntiles, tpc, a.status);
-    return cudaGetLastError();
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute at = {};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cfg.gridDim = dim3((unsigned)((rows * 32 + 127) / 128));
+    cfg.blockDim = dim3(128);
+    cfg.stream = s;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    e = cudaLaunchKernelEx(&cfg, snap_rows_kernel, (const float2 *)a.stats, a.rowstat, runs, rows);
+    if (e != cudaSuccess) return e;
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(kMmaThreads);
+    cfg.dynamicSmemBytes = G::SMEM_BYTES;
+    return cudaLaunchKernelEx(&cfg, snap_mma_kernel<D, 2>, tmap, a.page_cap, a.S, a.len, (const bf16 *)a.qw, a.W, a.H, sl2, (float2 *)nullptr,
+                              (const float2 *)a.rowstat, a.imp, ntiles, tpc, a.status);
 }
 
 size_t round256(size_t x) { return (x + 255) & ~(size_t)255; }
@@ -1122,15 +1154,17 @@ template <int EPT, int NT>
 static cudaError_t select_run(const float *imp, int BH, int64_t len, int w, int keep, int cl, int per_warp, int32_t *idx, cudaStream_t s)
 {
     cudaLaunchConfig_t cfg = {};
-    cudaLaunchAttribute at = {};
-    at.id = cudaLaunchAttributeClusterDimension;
-    at.val.clusterDim.x = (unsigned)cl;
-    at.val.clusterDim.y = at.val.clusterDim.z = 1;
+    cudaLaunchAttribute at[2] = {};
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = (unsigned)cl;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.gridDim = dim3((unsigned)(BH * cl));
     cfg.blockDim = dim3(NT);
     cfg.stream = s;
-    cfg.attrs = &at;
-    cfg.numAttrs = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 2;
     return cudaLaunchKernelEx(&cfg, snap_select_kernel<EPT, NT>, imp, len, w, keep, per_warp, idx);
 }
 
