@@ -103,8 +103,9 @@ __device__ __forceinline__ uint32_t score_bin(float v, float lo, float inv)
 // A threshold bucket of more than 16 blocks is cut further by buckets on the scores' integer images until at most 16
 // are left or all left are equal (equal scores: the lowest blocks).  More than 512 blocks are taken in panels of 512,
 // whose scores are computed again for each pass (the tensor cores have nothing else to do here).
-// Measured, 32 heads x 128 channels: 4096 queries, 16 of 64 blocks each, 158 -> 52 us; 30011 queries, 30 of 469 blocks
-// each, 28.9 -> 1.1 ms (queries by tensor map and four product steps per election: 58 -> 52 us of the former; before: fp32 FMA scores, a lane per block, then a bit-wise vote search up to 128 blocks and one
+// Measured, 32 heads x 128 channels: 4096 queries, 16 of 64 blocks each, 158 -> 47 us; 30011 queries, 30 of 469 blocks
+// each, 28.9 -> 1.0 ms (queries by tensor map and four product steps per election: 58 -> 52 us of the former, candidates noted by one atomic per
+// word instead of one each: 52 -> 47 us; before: fp32 FMA scores, a lane per block, then a bit-wise vote search up to 128 blocks and one
 // round per taken block beyond).
 template <int D>
 __global__ void __launch_bounds__(kRouteThreads, 2) moba_route_mma_kernel(const __grid_constant__ CUtensorMap qmap, const float *means, int64_t len, int H,
@@ -367,8 +368,31 @@ __global__ void __launch_bounds__(kRouteThreads, 2) moba_route_mma_kernel(const 
         if (ok) {
             const int tbin = s_tb[ql], need = s_need[ql];
             const uint32_t klo = s_klo[ql], khi = s_khi[ql];
+            const bool refined = klo != 0u || khi != 0xffffffffu || tied;
             for_scores(false, [&](int w, float (&v)[32], uint32_t cand) {
                 uint32_t bits = 0u, eq = 0u;
+                if (!__any_sync(FULL, refined)) {
+                    // one atomic per thread and word: one per candidate, each waited for while most lanes had none, took
+                    // half of a CTA's time
+#pragma unroll
+                    for (int c = 0; c < 32; ++c) {
+                        const int bin = (int)score_bin(v[c], mn, inv);
+                        if (bin > tbin) bits |= 1u << c;
+                        if (bin == tbin) eq |= 1u << c;
+                    }
+                    mk[w * NQ + ql] = bits & cand;
+                    eq = need > 0 ? eq & cand : 0u;
+                    if (!__any_sync(FULL, eq != 0u)) return;
+                    uint32_t at = eq ? atomicAdd(&s_n[ql], (uint32_t)__popc(eq)) : (uint32_t)CAP;
+#pragma unroll
+                    for (int c = 0; c < 32; ++c)
+                        if (((eq >> c) & 1u) && at < (uint32_t)CAP) {
+                            ckey[at * NQ + ql] = score_key(v[c]);
+                            cidx[at * NQ + ql] = (uint16_t)(32 * w + c);
+                            ++at;
+                        }
+                    return;
+                }
 #pragma unroll
                 for (int c = 0; c < 32; ++c) {
                     const int bin = (int)score_bin(v[c], mn, inv);
