@@ -216,6 +216,8 @@ __global__ void __launch_bounds__(NT) scan_kernel(ScanArgs a, const __grid_const
         mbar_init(&carried[1], 1);
         mbar_init_fence();
     }
+    grid_dependency_wait();                      // earlier kernels may still write what is read here, or read what is written
+    grid_launch_dependents();
     __syncthreads();
     if (warp == 0) {
         for (int j = 0; j < NST && j < mine; ++j) issue(j);
@@ -488,16 +490,18 @@ template <typename T, typename G, int D, int S, int MODE>
 cudaError_t start(const ScanArgs &a, const ScanMaps &tm, const ScanPlan &p, int cl, float *maps, const float *entry, int smem, cudaStream_t s)
 {
     cudaLaunchConfig_t cfg = {};
-    cudaLaunchAttribute at = {};
-    at.id = cudaLaunchAttributeClusterDimension;
-    at.val.clusterDim.x = (unsigned)cl;
-    at.val.clusterDim.y = at.val.clusterDim.z = 1;
+    cudaLaunchAttribute at[2] = {};
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = (unsigned)cl;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.gridDim = dim3((unsigned)(p.units * p.chunks * cl));
     cfg.blockDim = dim3(NT);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
-    cfg.attrs = &at;
-    cfg.numAttrs = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 2;
     return cudaLaunchKernelEx(&cfg, scan_kernel<T, G, D, S, MODE>, a, tm, p, maps, entry);
 }
 

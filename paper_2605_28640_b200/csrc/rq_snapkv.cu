@@ -887,6 +887,8 @@ __global__ void __launch_bounds__(kCompactWarps * 32) snap_compact_kernel(const 
     constexpr int NB = NR > 8 ? 8 : NR;                      // of which this many are in flight at a time, keys and values each
     constexpr unsigned FULL = 0xffffffffu;
     __shared__ __align__(16) uint4 smn[kCompactWarps][LPR], smx[kCompactWarps][LPR];
+    grid_dependency_wait();                                  // the list and the cleared bookkeeping come from the kernels before
+    grid_launch_dependents();
     const int bh = blockIdx.y, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int slot0 = blockIdx.x * 64 + warp * 16;           // first slot (position in the new cache) of this warp
     const int rsub = lane / LPR, piece = lane % LPR;
@@ -1191,28 +1193,29 @@ cudaError_t launch_snap_select(const float *imp, int BH, int64_t len, int window
 }
 
 template <typename T, int D>
-static void compact_shape(const SnapCompactArgs &a, cudaStream_t s)
+static cudaError_t compact_shape(const SnapCompactArgs &a, cudaStream_t s)
 {
     const dim3 grid((unsigned)((a.keep + 63) / 64), (unsigned)a.BH);
-    if (a.S == 16)
-        snap_compact_kernel<T, D, 16><<<grid, kCompactWarps * 32, 0, s>>>((const T *)a.skv, a.s_page_cap, (T *)a.dkv, (T *)a.dmeta, a.d_page_cap,
-                                                                         a.idx, a.keep, a.sstate, a.dstate, a.absmax, a.BH);
-    else
-        snap_compact_kernel<T, D, 64><<<grid, kCompactWarps * 32, 0, s>>>((const T *)a.skv, a.s_page_cap, (T *)a.dkv, (T *)a.dmeta, a.d_page_cap,
-                                                                         a.idx, a.keep, a.sstate, a.dstate, a.absmax, a.BH);
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute at = {};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(kCompactWarps * 32);
+    cfg.stream = s;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, a.S == 16 ? snap_compact_kernel<T, D, 16> : snap_compact_kernel<T, D, 64>, (const T *)a.skv, a.s_page_cap,
+                              (T *)a.dkv, (T *)a.dmeta, a.d_page_cap, a.idx, a.keep, a.sstate, a.dstate, a.absmax, a.BH);
 }
 
 cudaError_t launch_snap_compact(const SnapCompactArgs &a, cudaStream_t s)
 {
     if ((a.D != 64 && a.D != 128) || (a.S != 16 && a.S != 64)) return cudaErrorInvalidValue;
     if (a.dtype == RQ_BF16) {
-        if (a.D == 128) compact_shape<bf16, 128>(a, s);
-        else compact_shape<bf16, 64>(a, s);
-    } else {
-        if (a.D == 128) compact_shape<float, 128>(a, s);
-        else compact_shape<float, 64>(a, s);
+        return a.D == 128 ? compact_shape<bf16, 128>(a, s) : compact_shape<bf16, 64>(a, s);
     }
-    return cudaGetLastError();
+    return a.D == 128 ? compact_shape<float, 128>(a, s) : compact_shape<float, 64>(a, s);
 }
 
 }  // namespace rq
