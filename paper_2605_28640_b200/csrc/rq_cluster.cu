@@ -125,17 +125,21 @@ __device__ __forceinline__ void select_pages(ClusterShared &sh, int P, int ns, i
 {
     const int lane = tid & 31, warp = tid >> 5;
     if (P <= kRankPages) {
-        // a page's rank is the number of pages that beat it
-        const uint32_t k = tid < P ? sh.key[tid] : 0u;
-        int rank = 0;
-        for (int j = 0; j < P; j += 4) {
-            const uint4 o = *reinterpret_cast<const uint4 *>(sh.key + j);
-            rank += (o.x > k || (o.x == k && j < tid)) + (o.y > k || (o.y == k && j + 1 < tid)) + (o.z > k || (o.z == k && j + 2 < tid)) +
-                    (o.w > k || (o.w == k && j + 3 < tid));
+        // a page's rank is the number of pages that beat it.  A warp takes every NW-th page; its lanes hold the keys of all
+        constexpr int W = kRankPages / 32, R = kRankPages / NW;
+        uint32_t k[W], bits[W] = {};
+#pragma unroll
+        for (int w = 0; w < W; ++w) k[w] = w * 32 + lane < P ? sh.key[w * 32 + lane] : 0u;
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            const int p = r * NW + warp;                                 // (page p's key is in word r * NW / 32)
+            const uint32_t own = __shfl_sync(FULL, k[r * NW / 32], p & 31);
+            int rank = 0;
+#pragma unroll
+            for (int w = 0; w < W; ++w) rank += __popc(__ballot_sync(FULL, k[w] > own || (k[w] == own && w * 32 + lane < p)));
+            if (p < P && (p < ns || p >= P - nl || (own != 0u && rank < want))) bits[r * NW / 32] |= 1u << (p & 31);
         }
-        const bool take = tid < P && (tid < ns || tid >= P - nl || (k != 0u && rank < want));
-        const uint32_t bits = __ballot_sync(FULL, take);
-        if (lane == 0) sh.mask[warp] = bits;                            // (NW words, zero beyond the last page)
+        if (lane < W && (lane == 0 ? bits[0] : lane == 1 ? bits[1] : bits[2])) atomicOr(&sh.mask[lane], lane == 0 ? bits[0] : lane == 1 ? bits[1] : bits[2]);
         __syncthreads();
         return;
     }
@@ -248,7 +252,7 @@ __global__ void __launch_bounds__(NT, 2) cluster_step_kernel(DecodeArgs a, const
     const int P = (int)((a.len + S - 1) / S);
     const int gw = cr * NW + warp, GW = CL * NW;                         // this warp inside the cluster
     const bool dense = K >= P;                                           // every page is kept: no scores
-    if (tid < 4 && P + tid < kClusterPages) sh.key[P + tid] = 0u;        // (the ranking reads four keys at a time)
+    if (tid < kClusterPages / 32) sh.mask[tid] = 0u;
     cl.barrier_arrive();                                                 // all CTAs have started: their shared memory may be written
     grid_dependency_wait();                                              // earlier kernels may still write what is read here
     grid_launch_dependents();
@@ -258,17 +262,20 @@ __global__ void __launch_bounds__(NT, 2) cluster_step_kernel(DecodeArgs a, const
     constexpr int U = 4;                                                 // records of a lane group in flight (8: 0.6 us more where there are few)
     const int sub = lane / SG::LPP, c = lane % SG::LPP;
     uint4 raw[U][SG::VPL];
+    // the first CTA, busy with the token, takes no records where the others can load theirs at once (about 1 us to the scores)
+    const int skip = CL > 1 && P - 1 <= U * (CL - 1) * NW * SG::PPW ? 1 : 0;
+    const int first_rec = skip && cr == 0 ? P : (gw - skip * NW) * SG::PPW, step_rec = (GW - skip * NW) * SG::PPW;
     auto load_records = [&](int r0) {
 #pragma unroll
         for (int u = 0; u < U; ++u) {
-            const int rec = r0 + u * GW * SG::PPW + sub;
+            const int rec = r0 + u * step_rec + sub;
 #pragma unroll
             for (int v = 0; v < SG::VPL; ++v)
                 raw[u][v] = !dense && rec < P - 1 ? __ldcg(reinterpret_cast<const uint4 *>(meta + (int64_t)rec * SG::REC_BYTES) + c + v * SG::LPP)
                                                   : make_uint4(0u, 0u, 0u, 0u);
         }
     };
-    load_records(gw * SG::PPW);
+    load_records(first_rec);
     float qs[SG::VPL][SG::CH];
     score_load_q<T, D>(q, bh, lane, qs);
     AttendState<T> st;
@@ -281,7 +288,7 @@ __global__ void __launch_bounds__(NT, 2) cluster_step_kernel(DecodeArgs a, const
     cl.barrier_wait();
     if (!dense) {
         // (the loop bound is the same for every lane of a warp: the shuffles below need all of them)
-        for (int rb = gw * SG::PPW; rb < P - 1; rb += U * GW * SG::PPW) {
+        for (int rb = first_rec; rb < P - 1; rb += U * step_rec) {
             float s[U];
 #pragma unroll
             for (int u = 0; u < U; ++u) {
@@ -296,12 +303,12 @@ __global__ void __launch_bounds__(NT, 2) cluster_step_kernel(DecodeArgs a, const
                 s[u] = s2.x + s2.y;
             }
             const int rn = rb;
-            if (rb + U * GW * SG::PPW < P - 1) load_records(rb + U * GW * SG::PPW);
+            if (rb + U * step_rec < P - 1) load_records(rb + U * step_rec);
 #pragma unroll
             for (int u = 0; u < U; ++u) {
 #pragma unroll
                 for (int off = SG::LPP / 2; off > 0; off >>= 1) s[u] += __shfl_xor_sync(FULL, s[u], off);
-                const int rec = rn + u * GW * SG::PPW + sub;
+                const int rec = rn + u * step_rec + sub;
                 if (c < CL && rec < P - 1) cl.map_shared_rank(sh.key, c)[rec] = rec < ns || rec >= P - nl ? 0u : order_key(s[u]);
             }
         }

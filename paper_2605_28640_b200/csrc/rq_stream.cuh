@@ -331,13 +331,21 @@ __device__ __forceinline__ float update_head(const DecodeArgs &a, int h, const T
     const int64_t page = pos / S;
     const int slot = (int)(pos % S);
     float term = 0.0f, amax = 0.0f;
+    const int cur = a.epoch & 1;
+    const float largest = d == 0 && a.absmax ? a.absmax[cur * a.B * a.H + h] : 0.0f;
     if (d < D) {
+        // every load before the first store: behind a store that might overlap them they would wait for another round trip
+        // each (2.1 us from the first load to the score instead of 1.1)
         float *st = a.state + (int64_t)h * 2 * D;
+        T *m = static_cast<T *>(a.meta) + (((int64_t)h * a.page_cap + page) * 2) * D;
         const float g = a.gate_dtype == RQ_BF16 ? load1<bf16>(static_cast<const bf16 *>(g_t) + (int64_t)h * D + d)
                                                 : load1<float>(static_cast<const float *>(g_t) + (int64_t)h * D + d);
+        const float s_k = st[d], s_v = st[D + d], x_k = load1<T>(k_t + (int64_t)h * D + d), x_v = load1<T>(v_t + (int64_t)h * D + d);
+        const float qd = load1<T>(q + (int64_t)h * D + d);
+        const float mn_old = slot ? load1<T>(m + d) : 0.0f, mx_old = slot ? load1<T>(m + D + d) : 0.0f;
         const float om = 1.0f - g;
-        const float sk = fmaf(g, st[d], om * load1<T>(k_t + (int64_t)h * D + d));
-        const float sv = fmaf(g, st[D + d], om * load1<T>(v_t + (int64_t)h * D + d));
+        const float sk = fmaf(g, s_k, om * x_k);
+        const float sv = fmaf(g, s_v, om * x_v);
         st[d] = sk;
         st[D + d] = sv;
         T *pg = static_cast<T *>(a.kv) + (((int64_t)h * a.page_cap + page) * 2) * S * D;
@@ -345,7 +353,6 @@ __device__ __forceinline__ float update_head(const DecodeArgs &a, int h, const T
         store1<T>(pg + (int64_t)(S + slot) * D + d, sv);
         const float r = round_storage<T>(sk);
         amax = fabsf(r);
-        T *m = static_cast<T *>(a.meta) + (((int64_t)h * a.page_cap + page) * 2) * D;
         float mn = r, mx = r;
         if (slot == 0) {
             // a fresh page: clear its unused slots so that later reads are defined
@@ -354,12 +361,11 @@ __device__ __forceinline__ float update_head(const DecodeArgs &a, int h, const T
                 store1<T>(pg + (int64_t)(S + s2) * D + d, 0.0f);
             }
         } else {
-            mn = fminf(load1<T>(m + d), r);
-            mx = fmaxf(load1<T>(m + D + d), r);
+            mn = fminf(mn_old, r);
+            mx = fmaxf(mx_old, r);
         }
         store1<T>(m + d, mn);
         store1<T>(m + D + d, mx);
-        const float qd = load1<T>(q + (int64_t)h * D + d);
         term = fmaxf(qd * mn, qd * mx);
     }
     // score of the newest page: sum of the D terms; largest |stored key| of the new row
@@ -375,11 +381,7 @@ __device__ __forceinline__ float update_head(const DecodeArgs &a, int h, const T
         float m = 0.0f;
         for (int w = 0; w < (D + 31) / 32; ++w) { s += red[w]; m = fmaxf(m, red[8 + w]); }
         scores[(int64_t)h * a.page_cap + page] = s;
-        if (a.absmax) {
-            const int BH = a.B * a.H, cur = a.epoch & 1;
-            const float nv = fmaxf(a.absmax[cur * BH + h], m);
-            a.absmax[(cur ^ 1) * BH + h] = nv;
-        }
+        if (a.absmax) a.absmax[(cur ^ 1) * a.B * a.H + h] = fmaxf(largest, m);
     }
     __syncthreads();
     return s;
