@@ -301,7 +301,6 @@ static int decode_step_impl(rq_cache *cache, const void *q, const void *k_t, con
 __global__ void stage_in_kernel(const uint4 *q, const uint4 *k, const uint4 *v, const uint4 *g, uint4 *dq,
                                 uint4 *dk, uint4 *dv, uint4 *dg, int nv, int ng)
 {
-    grid_launch_dependents();
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i < nv) { dq[i] = q[i]; return; }
     i -= nv;

@@ -323,20 +323,28 @@ __global__ void __launch_bounds__(NT, 2) cluster_step_kernel(DecodeArgs a, const
     } else {
         select_pages(sh, P, ns, nl, K - ns - nl, tid);
         const int words = (P + 31) / 32;
-        const uint32_t w0 = lane < words ? sh.mask[lane] : 0u, w1 = lane + 32 < words ? sh.mask[lane + 32] : 0u;
-        int i0 = __popc(w0), i1 = __popc(w1);
+        if (words <= NW) {                                               // a warp per word, every lane adds up the words before
+            int at = 0;
 #pragma unroll
-        for (int off = 1; off < 32; off <<= 1) {
-            const int t0 = __shfl_up_sync(FULL, i0, off), t1 = __shfl_up_sync(FULL, i1, off);
-            if (lane >= off) { i0 += t0; i1 += t1; }
-        }
-        i1 += __shfl_sync(FULL, i0, 31);
-        i0 -= __popc(w0);
-        i1 -= __popc(w1);
-        for (int w = warp; w < words; w += NW) {
-            const uint32_t bits = __shfl_sync(FULL, w < 32 ? w0 : w1, w & 31);
-            const int at = __shfl_sync(FULL, w < 32 ? i0 : i1, w & 31);
-            if ((bits >> lane) & 1u) sh.list[at + __popc(bits & ((1u << lane) - 1u))] = (uint16_t)(w * 32 + lane);
+            for (int w = 0; w < NW; ++w) at += w < warp ? __popc(sh.mask[w]) : 0;
+            const uint32_t bits = sh.mask[warp];
+            if ((bits >> lane) & 1u) sh.list[at + __popc(bits & ((1u << lane) - 1u))] = (uint16_t)(warp * 32 + lane);
+        } else {
+            const uint32_t w0 = lane < words ? sh.mask[lane] : 0u, w1 = lane + 32 < words ? sh.mask[lane + 32] : 0u;
+            int i0 = __popc(w0), i1 = __popc(w1);
+#pragma unroll
+            for (int off = 1; off < 32; off <<= 1) {
+                const int t0 = __shfl_up_sync(FULL, i0, off), t1 = __shfl_up_sync(FULL, i1, off);
+                if (lane >= off) { i0 += t0; i1 += t1; }
+            }
+            i1 += __shfl_sync(FULL, i0, 31);
+            i0 -= __popc(w0);
+            i1 -= __popc(w1);
+            for (int w = warp; w < words; w += NW) {
+                const uint32_t bits = __shfl_sync(FULL, w < 32 ? w0 : w1, w & 31);
+                const int at = __shfl_sync(FULL, w < 32 ? i0 : i1, w & 31);
+                if ((bits >> lane) & 1u) sh.list[at + __popc(bits & ((1u << lane) - 1u))] = (uint16_t)(w * 32 + lane);
+            }
         }
     }
     __syncthreads();
