@@ -133,11 +133,13 @@ __device__ __forceinline__ void select_pages(ClusterShared &sh, int P, int ns, i
 #pragma unroll
         for (int r = 0; r < R; ++r) {
             const int p = r * NW + warp;                                 // (page p's key is in word r * NW / 32)
+            if (p >= P) break;
             const uint32_t own = __shfl_sync(FULL, k[r * NW / 32], p & 31);
             int rank = 0;
 #pragma unroll
-            for (int w = 0; w < W; ++w) rank += __popc(__ballot_sync(FULL, k[w] > own || (k[w] == own && w * 32 + lane < p)));
-            if (p < P && (p < ns || p >= P - nl || (own != 0u && rank < want))) bits[r * NW / 32] |= 1u << (p & 31);
+            for (int w = 0; w < W; ++w)
+                if (w * 32 < P) rank += __popc(__ballot_sync(FULL, k[w] > own || (k[w] == own && w * 32 + lane < p)));
+            if ((p < ns || p >= P - nl || (own != 0u && rank < want))) bits[r * NW / 32] |= 1u << (p & 31);
         }
         if (lane < W && (lane == 0 ? bits[0] : lane == 1 ? bits[1] : bits[2])) atomicOr(&sh.mask[lane], lane == 0 ? bits[0] : lane == 1 ? bits[1] : bits[2]);
         __syncthreads();
@@ -276,15 +278,15 @@ __global__ void __launch_bounds__(NT, 2) cluster_step_kernel(DecodeArgs a, const
         }
     };
     load_records(first_rec);
+    float newest = 0.0f;
+    if (cr == 0) {                                                       // (before the queries are waited for: one round trip for both)
+        newest = update_head<T, D>(a, bh, q, k_t, v_t, g_t, scores, sh.upd);
+        if (ctr_other && tid < kStepCtrInts) ctr_other[bh * kStepCtrInts + tid] = 0;   // the other one-launch form's counters of the next step
+    }
     float qs[SG::VPL][SG::CH];
     score_load_q<T, D>(q, bh, lane, qs);
     AttendState<T> st;
     attend_begin_head<T, D>(st, q, bh, scale_log2, lane);
-    float newest = 0.0f;
-    if (cr == 0) {
-        newest = update_head<T, D>(a, bh, q, k_t, v_t, g_t, scores, sh.upd);
-        if (ctr_other && tid < kStepCtrInts) ctr_other[bh * kStepCtrInts + tid] = 0;   // the other one-launch form's counters of the next step
-    }
     cl.barrier_wait();
     if (!dense) {
         // (the loop bound is the same for every lane of a warp: the shuffles below need all of them)
@@ -312,8 +314,10 @@ __global__ void __launch_bounds__(NT, 2) cluster_step_kernel(DecodeArgs a, const
                 if (c < CL && rec < P - 1) cl.map_shared_rank(sh.key, c)[rec] = rec < ns || rec >= P - nl ? 0u : order_key(s[u]);
             }
         }
-        if (cr == 0 && tid == 0)
-            for (int r = 0; r < CL; ++r) cl.map_shared_rank(sh.key, r)[P - 1] = nl > 0 || P - 1 < ns ? 0u : order_key(newest);
+        if (cr == 0 && warp == 0) {
+            newest = __shfl_sync(FULL, newest, 0);
+            if (lane < CL) cl.map_shared_rank(sh.key, lane)[P - 1] = nl > 0 || P - 1 < ns ? 0u : order_key(newest);
+        }
     }
     cl.sync();                                                           // all scores are in, the token is in the cache
 
