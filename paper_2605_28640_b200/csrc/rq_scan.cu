@@ -33,9 +33,9 @@
 // The order of all floating-point operations is fixed: the same bits on every run.
 //
 // Bound: the phases of a tile between its two barriers, with DRAM close behind (131072 tokens of 32 heads x 128, bf16: 5.5
-// GB in 0.96 to 1.07 ms, 5.2 to 5.7 TB/s; the copies alone run at 5.8 TB/s).  Before (copies started and rows stored in
+// GB in 0.90 to 0.99 ms, 5.6 to 6.1 TB/s; the copies alone run at 5.8 TB/s).  Before (copies started and rows stored in
 // 16-byte pieces by all threads, one CTA per unit, three barriers, the inputs read twice for few heads) / now, us: 32 heads,
-// 131072 tokens 1120 / 957; 8 heads, 50003 tokens, fp32 gates 195 / 121; 8 heads, 8000 tokens 76 / 33; 4 heads, 8000 tokens
+// 131072 tokens 1120 / 900; 4001 tokens 46 / 37; 8 heads, 50003 tokens, fp32 gates 195 / 110; 8 heads, 8000 tokens 76 / 33; 4 heads, 8000 tokens
 // 75 / 31; fp32, 12 heads, 20000 tokens 176 / 120; fp32, 32 heads, 8000 tokens, pages of 16 120 / 126.
 #include "rq_async.cuh"
 #include "rq_device.cuh"
@@ -129,6 +129,7 @@ struct ScanPlan {
 };
 
 // MODE 0: the scan proper.  MODE 1: the affine map of a time chunk only (no output), for the time-chunked form.
+// MODE 2: MODE 0 with one CTA per unit and the CTAs of a head as a cluster that keeps them within a tile of each other.
 // Time chunks (chunks > 1; so few units that not even clusters fill the chip, and a long prompt): CTA x works on unit
 // x % units and the chunk_tiles tiles of chunk x / units.  First every chunk but the last is reduced to its map s -> A s + B
 // (MODE 1), a small kernel chains the maps into the state that enters every chunk, then every chunk runs the scan proper
@@ -159,7 +160,7 @@ __global__ void __launch_bounds__(NT) scan_kernel(ScanArgs a, const __grid_const
     __shared__ __align__(8) uint64_t full[NST], carried[2]; // a stage has landed; the state entering a tile has arrived
 
     cg::cluster_group cl = cg::this_cluster();
-    const int CL = (int)cl.num_blocks(), cr = (int)cl.block_rank();
+    const int CL = MODE == 2 ? 1 : (int)cl.num_blocks(), cr = MODE == 2 ? 0 : (int)cl.block_rank();
     const int unit = blockIdx.x / CL % plan.units, chunk = blockIdx.x / CL / plan.units, chunks = plan.chunks;
     const int64_t tile0 = plan.tile0 + (int64_t)chunk * plan.chunk_tiles;
     const int ntiles = min(plan.chunk_tiles, plan.ntiles - chunk * plan.chunk_tiles);
@@ -180,11 +181,9 @@ __global__ void __launch_bounds__(NT) scan_kernel(ScanArgs a, const __grid_const
     const G *gp = static_cast<const G *>(a.g) + in_base;
     const int row0 = (2 * warp + half) * RT;     // first row of this thread's run
 
-    // tile i of the unit (chunk): does it come through the tensor maps?
-    auto by_map = [&](int i) {
-        const int64_t t = (tile0 + i) * TT;
-        return plan.tma && t >= a.len0 && t + TT <= end;
-    };
+    // tile i of the unit (chunk): does it come through the tensor maps (rows past the prompt's end as zeros), and is it full?
+    auto by_map = [&](int i) { return plan.tma && (tile0 + i) * TT >= a.len0; };
+    auto full_tile = [&](int i) { return by_map(i) && (tile0 + i + 1) * TT <= end; };
     const uint64_t once = l2_evict_first_policy();
     // start the copies of this CTA's j-th tile.  The whole first warp.
     auto issue = [&](int j) {
@@ -276,7 +275,7 @@ __global__ void __launch_bounds__(NT) scan_kernel(ScanArgs a, const __grid_const
         }
     };
 
-    // this CTA's j-th tile; MAP: it has landed in its stage and every row of it is a new token
+    // this CTA's j-th tile; MAP: it lands in its stage and every row of it is a new token
     auto tile = [&](auto map_tag, int j) {
         constexpr bool MAP = decltype(map_tag)::value;
         const int i = cr + j * CL;
@@ -288,7 +287,7 @@ __global__ void __launch_bounds__(NT) scan_kernel(ScanArgs a, const __grid_const
 
         // ---- pass 1: this thread's run as a map from a zero state (identity outside the new range)
         float2 g2[RT], k2[RT], v2[RT];                           // g, (1-g) k, (1-g) v of the two channels
-        if constexpr (MAP) {
+        if (MAP || by_map(i)) {
             ok = ok && mbar_wait(&full[j % NST], (uint32_t)((j / NST) & 1));
             // (2-byte elements: the two halves of a warp, eight rows of 64 bytes apart, share banks: two reads instead of one)
             const unsigned char *st = dsm + (size_t)(j % NST) * STAGE;
@@ -299,6 +298,7 @@ __global__ void __launch_bounds__(NT) scan_kernel(ScanArgs a, const __grid_const
                 g2[r] = load2(gt + r * CG);
                 k2[r] = load2(kt + r * CG);
                 v2[r] = load2(vt + r * CG);
+                if (!MAP && row0 + r >= hi) g2[r] = make_float2(1.0f, 1.0f);     // (k and v are zero there)
             }
         } else {
 #pragma unroll
@@ -334,7 +334,7 @@ __global__ void __launch_bounds__(NT) scan_kernel(ScanArgs a, const __grid_const
         __syncthreads();                                         // the maps are there
         // the stage of the tile before (of this tile, if nothing goes back into it) is free
         if (warp == 0 && (!BY_STAGE || j >= 1) && j - BY_STAGE + NST < mine) issue(j - BY_STAGE + NST);
-        if (WPP > 1 && MODE == 0 && j > 0) wide_bounds(j - 1);
+        if (WPP > 1 && MODE != 1 && j > 0) wide_bounds(j - 1);
 
         // ---- scan of the 16 warp maps of channels 2 warp and 2 warp + 1 (one per half-warp) by 16 lanes
         {
@@ -360,7 +360,7 @@ __global__ void __launch_bounds__(NT) scan_kernel(ScanArgs a, const __grid_const
             const float ck = carry[j & 1][0][ci], cv = carry[j & 1][1][ci];
             if (m == LPC - 1) {                              // the state after the tile: to the next tile, or the end
                 const float nk = fmaf(sa, ck, sbk), nv = fmaf(sa, cv, sbv);
-                if (MODE == 0 && i == ntiles - 1 && chunk == chunks - 1) {
+                if (MODE != 1 && i == ntiles - 1 && chunk == chunks - 1) {
                     a.state[(int64_t)bh * 2 * D + c0 + ci] = nk;
                     a.state[(int64_t)bh * 2 * D + D + c0 + ci] = nv;
                 } else if (CL > 1) {
@@ -439,10 +439,21 @@ __global__ void __launch_bounds__(NT) scan_kernel(ScanArgs a, const __grid_const
         }
     };
 
+    // (full tiles in a loop of their own: 42.2 -> 41.0 us for 4001 tokens)
+    const int64_t full_from = plan.tma ? (a.len0 + TT - 1) / TT - tile0 : (int64_t)ntiles, full_to = plan.tma ? end / TT - tile0 : (int64_t)0;
+    int j = 0;
 #pragma unroll 1
-    for (int j = 0; j < mine; ++j) {
-        if (by_map(cr + j * CL)) tile(BoolTag<true>(), j);
-        else tile(BoolTag<false>(), j);
+    while (j < mine) {
+#pragma unroll 1
+        for (; j < mine && cr + j * CL >= full_from && cr + j * CL < full_to; ++j) {
+            if (MODE == 2) asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
+            tile(BoolTag<true>(), j);
+            if (MODE == 2) asm volatile("barrier.cluster.wait.aligned;" ::: "memory");
+        }
+        if (j < mine) {
+            tile(BoolTag<false>(), j);
+            ++j;
+        }
     }
     if (BY_STAGE) tma_store_wait_read();
     __syncthreads();
@@ -492,7 +503,7 @@ cudaError_t start(const ScanArgs &a, const ScanMaps &tm, const ScanPlan &p, int 
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute at[2] = {};
     at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = (unsigned)cl;
+    at[0].val.clusterDim.x = (unsigned)(MODE == 2 ? D / CG : cl);
     at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
     at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at[1].val.programmaticStreamSerializationAllowed = 1;
@@ -526,6 +537,8 @@ cudaError_t run(const ScanArgs &a, cudaStream_t s)
         if (e != cudaSuccess) return e;
         e = cudaFuncSetAttribute(scan_kernel<T, G, D, S, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, DSM);
         if (e != cudaSuccess) return e;
+        e = cudaFuncSetAttribute(scan_kernel<T, G, D, S, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, DSM);
+        if (e != cudaSuccess) return e;
         ready[dev] = true;
     }
     ScanPlan p;
@@ -555,6 +568,10 @@ cudaError_t run(const ScanArgs &a, cudaStream_t s)
         chunks = 1;
         while (cl < kMaxCluster && 2 * cl * units <= sms && p.ntiles >= 8 * cl) cl *= 2;
     }
+    // Long prompts of nearly as many units as SMs are bound by DRAM, and it likes a head's units, neighbours in every row,
+    // together: 32 heads, 131072 tokens 923 -> 900 us.  Short ones lose by the barriers (4001 tokens 41.0 -> 42.1), and so
+    // would more units than the clusters find room for at once.
+    const bool abreast = cl == 1 && chunks == 1 && p.ntiles >= 64 && 9 * units <= 8 * sms;
     p.chunk_tiles = (p.ntiles + chunks - 1) / chunks;
     p.chunks = (p.ntiles + p.chunk_tiles - 1) / p.chunk_tiles;
     float *maps = a.chunk_scratch, *entry = a.chunk_scratch ? a.chunk_scratch + (size_t)units * p.chunks * 3 * CG : nullptr;
@@ -563,7 +580,7 @@ cudaError_t run(const ScanArgs &a, cudaStream_t s)
         if (e != cudaSuccess) return e;
         scan_chain_kernel<<<(unsigned)units, 2 * CG, 0, s>>>(a.state, D, D / CG, p.chunks, maps, entry);
     }
-    e = start<T, G, D, S, 0>(a, tm, p, cl, maps, entry, DSM, s);
+    e = abreast ? start<T, G, D, S, 2>(a, tm, p, 1, maps, entry, DSM, s) : start<T, G, D, S, 0>(a, tm, p, cl, maps, entry, DSM, s);
     return e != cudaSuccess ? e : cudaGetLastError();
 }
 

@@ -78,3 +78,24 @@ def test_states_cache_and_bounds(B, H, D, S, T, cuts, dtype, gdtype, layout):
     for p in range(P):
         rows = keys[:, :, p, :min(S, T - p * S)]
         assert torch.equal(c.meta_view()[:, :, p, 0], rows.amin(2)) and torch.equal(c.meta_view()[:, :, p, 1], rows.amax(2))
+
+
+@pytest.mark.parametrize("H,D,S,T,dtype,gdtype", [(20, 128, 16, 16384, BF, BF), (32, 128, 64, 16500, BF, F32), (40, 64, 16, 16385, F32, BF),
+                                                  (65, 64, 64, 16639, BF, BF)])
+def test_units_abreast(H, D, S, T, dtype, gdtype):
+    """The form that keeps a head's units abreast (64 tiles and more, nearly as many units as SMs) against two calls of fewer
+    tiles each, cut between tiles: the order of the operations is the same, and so are the bits."""
+    gen = torch.Generator(device=DEV)
+    gen.manual_seed(T + H)
+    k, v, g = (torch.randn(1, T, H, D, generator=gen, device=DEV) for _ in range(3))
+    k, v, g = k.to(dtype), v.to(dtype), torch.sigmoid(4.12 + 0.5 * g).to(gdtype)
+    caches = []
+    for edges in ([0, T], [0, 8192, T]):
+        c = rq.Cache(1, H, D, S, T, dtype, gdtype)
+        for a, b in zip(edges[:-1], edges[1:]):
+            rq.rq_build_cache(c.handle, k[:, a:b], v[:, a:b], g[:, a:b])
+        torch.cuda.synchronize()
+        assert rq.rq_device_status(c.handle) == rq.RQ_OK
+        caches.append(c)
+    a, b = caches
+    assert torch.equal(a.state, b.state) and torch.equal(a.kv, b.kv) and torch.equal(a.meta, b.meta)
