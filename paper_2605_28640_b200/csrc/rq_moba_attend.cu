@@ -66,10 +66,14 @@ struct Walk {
 // by their sum at the end, so that O is hardly ever touched between the products.
 // Warps 0..7 read scores, warp 8 starts the tensor-map copies, warps 9 and 10 the score products of an accumulator each,
 // warp 11 the output products; they meet through mbarriers only, every wait bounded.  One warp for all products was the
-// limit: 24 products, six commits and as many waits a chunk (32 heads x 128, 30011 positions: 7.61 -> 6.13 ms; 4096: 234 -> 206 us).  256 queries per CTA because keys and values come
-// from L2 for every CTA.  A CTA's queries come by tensor map, and it may start before the routing kernel has ended: at 4096
-// positions a CTA lives 50 us only, and the 20 us before its first product were a third of that (206 -> 186 us; the
-// list by a lane per block and the outputs through shared memory 186 -> 181 us).
+// limit: 24 products, six commits and as many waits a chunk.  256 queries per CTA because keys and values come from L2 for
+// every CTA.  A CTA's queries come by tensor map, and it may start before the routing kernel has ended: at 4096 positions
+// a CTA lives 50 us only, and the 20 us before its first product were a third of that.
+// Measured, 32 heads x 128 channels, 30011 positions (30 of 469 blocks) / 4096 (16 of 64): a warp per kind of product 7.61 ->
+// 6.13 ms / 234 -> 206 us; queries by tensor map, early start 206 -> 186 us; list by a lane per block, outputs through shared
+// memory 186 -> 181 us.  Bound: the readers' chain per chunk (about 1900 cycles, of which ex2 alone takes 1024, against 1280
+// for the products).  Slower were a quarter of the exponentials by polynomial, 16 reading warps, and pairs of chunks as one
+// product of 128 columns.
 template <int D>
 __global__ void __launch_bounds__(kThreads, 1) moba_mma_kernel(const __grid_constant__ CUtensorMap tmap,
                                                                const __grid_constant__ CUtensorMap qmap,

@@ -104,9 +104,9 @@ __device__ __forceinline__ uint32_t score_bin(float v, float lo, float inv)
 // are left or all left are equal (equal scores: the lowest blocks).  More than 512 blocks are taken in panels of 512,
 // whose scores are computed again for each pass (the tensor cores have nothing else to do here).
 // Measured, 32 heads x 128 channels: 4096 queries, 16 of 64 blocks each, 158 -> 47 us; 30011 queries, 30 of 469 blocks
-// each, 28.9 -> 1.0 ms (queries by tensor map and four product steps per election: 58 -> 52 us of the former, candidates noted by one atomic per
-// word instead of one each: 52 -> 47 us; before: fp32 FMA scores, a lane per block, then a bit-wise vote search up to 128 blocks and one
-// round per taken block beyond).
+// each, 28.9 -> 1.0 ms.  (Before: fp32 FMA scores, a lane per block, then a bit-wise vote search up to 128 blocks and one
+// round per taken block beyond.  Of the former: queries by tensor map and four product steps per election 58 -> 52 us,
+// candidates noted by one atomic per word instead of one each 52 -> 47 us.)
 template <int D>
 __global__ void __launch_bounds__(kRouteThreads, 2) moba_route_mma_kernel(const __grid_constant__ CUtensorMap qmap, const float *means, int64_t len, int H,
                                                                       int block, int nb, int K, int words, uint32_t *masks,

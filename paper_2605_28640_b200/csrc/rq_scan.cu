@@ -35,7 +35,7 @@
 // Bound: the phases of a tile between its two barriers, with DRAM close behind (131072 tokens of 32 heads x 128, bf16: 5.5
 // GB in 0.90 to 0.99 ms, 5.6 to 6.1 TB/s; the copies alone run at 5.8 TB/s).  Before (copies started and rows stored in
 // 16-byte pieces by all threads, one CTA per unit, three barriers, the inputs read twice for few heads) / now, us: 32 heads,
-// 131072 tokens 1120 / 900; 4001 tokens 46 / 37; 8 heads, 50003 tokens, fp32 gates 195 / 110; 8 heads, 8000 tokens 76 / 33; 4 heads, 8000 tokens
+// 131072 tokens 1120 / 900; 4001 tokens and the clearing before them 50 / 40; 8 heads, 50003 tokens, fp32 gates 195 / 110; 8 heads, 8000 tokens 76 / 33; 4 heads, 8000 tokens
 // 75 / 31; fp32, 12 heads, 20000 tokens 176 / 120; fp32, 32 heads, 8000 tokens, pages of 16 120 / 126.
 #include "rq_async.cuh"
 #include "rq_device.cuh"

@@ -209,8 +209,9 @@ __device__ __forceinline__ float exp2_fast(float x)
 // x the slots of a page x keys only x the pages of 128 positions, 128-byte swizzle: one copy brings one
 // 64-channel half of a tile's keys into shared memory in the layout the tensor core reads.
 template <int D, int PASS>
-__global__ void __launch_bounds__(kMmaThreads) snap_mma_kernel(const __grid_constant__ CUtensorMap tmap, int64_t page_cap, int S,
-                                                               int64_t len, const bf16 *qw, int W, int H, float scale_log2,
+__global__ void __launch_bounds__(kMmaThreads) snap_mma_kernel(const __grid_constant__ CUtensorMap tmap,
+                                                               const __grid_constant__ CUtensorMap qmap, int64_t page_cap, int S,
+                                                               int64_t len, int W, int H, float scale_log2,
                                                                float2 *stats, const float2 *rowstat, float *imp,
                                                                int ntiles, int tiles_per_cta, int32_t *status)
 {
@@ -220,7 +221,7 @@ __global__ void __launch_bounds__(kMmaThreads) snap_mma_kernel(const __grid_cons
     constexpr uint32_t TCOLS = 2 * ACC;                        // two accumulators: one is filled while the other is read
     extern __shared__ __align__(1024) unsigned char dsm_raw[];
     __shared__ __align__(8) uint64_t bar[2];                   // an accumulator's product is complete
-    __shared__ __align__(8) uint64_t full[NST];                // a stage's keys have landed
+    __shared__ __align__(8) uint64_t full[NST], full_q;        // a stage's keys, the queries have landed
     __shared__ __align__(8) uint64_t acc_free[2];              // an accumulator has been read by all four warps
     __shared__ uint32_t tbase;
     __shared__ float2 qst[kSnapRows];                          // pass 1: merge of the two halves; pass 2: (max, 1 / sum) per query
@@ -234,22 +235,7 @@ __global__ void __launch_bounds__(kMmaThreads) snap_mma_kernel(const __grid_cons
     const int ppt = kMmaKeys / S;                              // pages per tile
     int n_issued = 0, n_landed = 0;                            // the producing warp: tiles whose copies were started / seen complete
 
-    if (tid == 0) {
-        mbar_init(&bar[0], 1);
-        mbar_init(&bar[1], 1);
-        for (int s = 0; s < NST; ++s) mbar_init(&full[s], 1);
-        mbar_init(&acc_free[0], kMmaWarps * 32);
-        mbar_init(&acc_free[1], kMmaWarps * 32);
-        mbar_init_fence();
-    }
     if (warp == 0) tmem_alloc(&tbase, TCOLS);
-    // the window's queries of this head (qw is [B][W][H][D]) in rows r and r + 64; rows beyond the window are zero
-    for (int i = tid; i < 128 * (D / 8); i += kMmaThreads) {
-        const int r = i / (D / 8), c = i % (D / 8), qr = r & (kSnapRows - 1);
-        uint4 v = make_uint4(0u, 0u, 0u, 0u);
-        if (qr < W) v = *reinterpret_cast<const uint4 *>(qw + (((int64_t)b * W + qr) * H + h) * D + c * 8);
-        *reinterpret_cast<uint4 *>(qs + (c >> 3) * G::HALF_BYTES + umma_sw128_offset(r, c & 7)) = v;
-    }
     // the keys of tile t (relative to t0) into its stage: position j lives in page j / S, slot j % S of the
     // head's cache; pages past the head's last one hold somebody else's rows or nothing, and every key at
     // or beyond `len` is masked where the scores are used.  One warp.
@@ -268,7 +254,31 @@ __global__ void __launch_bounds__(kMmaThreads) snap_mma_kernel(const __grid_cons
             for (int hh = 0; hh < G::HALVES; ++hh) tma_prefetch_4d(&tmap, hh * 64, 0, 0, page + kMmaAhead * ppt);
         }
     };
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // the queries, written with ordinary stores, are read by the tensor core
+    if (warp == kMmaWarps) {                                   // copies start before anything else
+        if (lane == 0) {
+            mbar_init(&bar[0], 1);
+            mbar_init(&bar[1], 1);
+            for (int s = 0; s < NST; ++s) mbar_init(&full[s], 1);
+            mbar_init(&full_q, 1);
+            mbar_init(&acc_free[0], kMmaWarps * 32);
+            mbar_init(&acc_free[1], kMmaWarps * 32);
+            mbar_init_fence();
+        }
+        __syncwarp();
+        // the window's queries of this head in rows r and, for the first pass, r + 64; rows beyond the window come as zeros
+        mbar_expect_warp(&full_q, G::Q_BYTES / (PASS == 1 ? 1 : 2));
+#pragma unroll
+        for (int hh = 0; hh < G::HALVES; ++hh) {
+            tma_load_4d(qs + hh * G::HALF_BYTES, &qmap, hh * 64, h, 0, b, &full_q);
+            if (PASS == 1) tma_load_4d(qs + hh * G::HALF_BYTES + G::HALF_BYTES / 2, &qmap, hh * 64, h, 0, b, &full_q);
+        }
+        for (int s = 0; s < NST && s < n; ++s) issue(s);
+        for (int t = NST; t < kMmaAhead && t < n; ++t) {       // the tiles between the first copies and the first prefetch
+            const int page = (int)((int64_t)bh * page_cap + (int64_t)(t0 + t) * ppt);
+#pragma unroll
+            for (int hh = 0; hh < G::HALVES; ++hh) tma_prefetch_4d(&tmap, hh * 64, 0, 0, page);
+        }
+    }
     tcgen05_before_sync();
     __syncthreads();
     tcgen05_after_sync();
@@ -282,12 +292,7 @@ __global__ void __launch_bounds__(kMmaThreads) snap_mma_kernel(const __grid_cons
         // ---- the producing warp starts the copies and the products (all its lanes run this, see rq_umma.cuh);
         // nobody else waits for it except through the barriers
         {
-            for (int t = NST; t < kMmaAhead && t < n; ++t) {       // the tiles between the first copies and the first prefetch
-                const int page = (int)((int64_t)bh * page_cap + (int64_t)(t0 + t) * ppt);
-#pragma unroll
-                for (int hh = 0; hh < G::HALVES; ++hh) tma_prefetch_4d(&tmap, hh * 64, 0, 0, page);
-            }
-            for (int s = 0; s < NST && s < n; ++s) issue(s);
+            ok = __all_sync(0xffffffffu, mbar_wait(&full_q, 0u) || mbar_wait(&full_q, 0u));
             constexpr uint32_t idesc = PASS == 1 ? umma_idesc_bf16(128, kMmaKeys) : umma_idesc_bf16(kMmaKeys, kSnapRows);
             const uint64_t qd = umma_desc_sw128(smem_addr(qs)), kd = umma_desc_sw128(smem_addr(ks));
 #pragma unroll 1
@@ -300,11 +305,10 @@ __global__ void __launch_bounds__(kMmaThreads) snap_mma_kernel(const __grid_cons
                 tcgen05_after_sync();
                 const uint32_t acc = tb + (uint32_t)(i & 1) * ACC;
 #pragma unroll
-                for (int k = 0; k < D / 16; ++k) {
-                    const uint32_t off = (uint32_t)(k >> 2) * G::HALF_BYTES + (uint32_t)(k & 3) * 32u;
-                    const uint64_t dq = qd + (uint64_t)(off >> 4), dk = kd + (uint64_t)(((i % NST) * G::TILE_BYTES + off) >> 4);
-                    if (PASS == 1) umma_bf16(acc, dq, dk, idesc, k > 0);
-                    else umma_bf16(acc, dk, dq, idesc, k > 0);
+                for (int hh = 0; hh < G::HALVES; ++hh) {
+                    const uint64_t dq = qd + (uint64_t)((hh * G::HALF_BYTES) >> 4), dk = kd + (uint64_t)(((i % NST) * G::TILE_BYTES + hh * G::HALF_BYTES) >> 4);
+                    if (PASS == 1) umma_bf16_x4<2, 2>(acc, dq, dk, idesc, hh > 0);
+                    else umma_bf16_x4<2, 2>(acc, dk, dq, idesc, hh > 0);
                 }
                 umma_commit(&bar[i & 1]);
                 // the stage of tile i - 1 is free once its product has completed; it takes tile i - 1 + NST
@@ -1015,7 +1019,7 @@ cudaError_t snap_scores_t(const SnapArgs &a, cudaStream_t s)
 
 // The same for prompts whose scores fit in the tensor memory of a cluster: tiles per CTA and CTAs per head.
 template <int D, int RT>
-cudaError_t snap_scores_once(const SnapArgs &a, const CUtensorMap &tmap, int ntiles, cudaStream_t s)
+cudaError_t snap_scores_once(const SnapArgs &a, const CUtensorMap &tmap, const CUtensorMap &qmap, int ntiles, cudaStream_t s)
 {
     using G = SnapOnceGeom<D>;
     static bool ready[64];
@@ -1033,9 +1037,6 @@ cudaError_t snap_scores_once(const SnapArgs &a, const CUtensorMap &tmap, int nti
     int cl = (ntiles + RT - 1) / RT;
     while (cl < kOnceCluster && cl < ntiles && BH * (cl + 1) <= slots) ++cl;
     const int tpc = (ntiles + cl - 1) / cl;
-    alignas(64) CUtensorMap qmap;
-    e = query_tensor_map(&qmap, a.qw, D, a.H, a.W, a.B, kSnapRows);
-    if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute at = {};
     at.id = cudaLaunchAttributeClusterDimension;
@@ -1069,12 +1070,14 @@ cudaError_t snap_scores_mma(const SnapArgs &a, cudaStream_t s)
     }
     const int BH = a.B * a.H;
     if (kMmaKeys % a.S != 0) return cudaErrorInvalidValue;
-    alignas(64) CUtensorMap tmap;
+    alignas(64) CUtensorMap tmap, qmap;
     e = cache_tensor_map(&tmap, a.kv, D, a.S, (int64_t)BH * a.page_cap, kMmaKeys);
     if (e != cudaSuccess) return e;
+    e = query_tensor_map(&qmap, a.qw, D, a.H, a.W, a.B, kSnapRows);
+    if (e != cudaSuccess) return e;
     const int ntiles = (int)((a.len + kMmaKeys - 1) / kMmaKeys);
-    if (ntiles <= 4 * kOnceCluster) return snap_scores_once<D, 4>(a, tmap, ntiles, s);
-    if (ntiles <= 8 * kOnceCluster) return snap_scores_once<D, 8>(a, tmap, ntiles, s);
+    if (ntiles <= 4 * kOnceCluster) return snap_scores_once<D, 4>(a, tmap, qmap, ntiles, s);
+    if (ntiles <= 8 * kOnceCluster) return snap_scores_once<D, 8>(a, tmap, qmap, ntiles, s);
     // tiles per CTA: two CTAs share an SM, so the launch runs in rounds of 2 * SMs CTAs; the choice with the fewest
     // rounds * (tiles of a CTA + what a CTA costs before its first tile, about two tiles' time) ends soonest
     const int64_t slots = 2 * (int64_t)sm_count();
@@ -1091,7 +1094,7 @@ cudaError_t snap_scores_mma(const SnapArgs &a, cudaStream_t s)
     const int runs = (ntiles + tpc - 1) / tpc;
     const dim3 grid((unsigned)runs, (unsigned)BH);
     const float sl2 = a.scale * 1.4426950408889634f;
-    snap_mma_kernel<D, 1><<<grid, kMmaThreads, G::SMEM_BYTES, s>>>(tmap, a.page_cap, a.S, a.len, (const bf16 *)a.qw, a.W, a.H, sl2,
+    snap_mma_kernel<D, 1><<<grid, kMmaThreads, G::SMEM_BYTES, s>>>(tmap, qmap, a.page_cap, a.S, a.len, a.W, a.H, sl2,
                                                                  a.stats, nullptr, nullptr, ntiles, tpc, a.status);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
@@ -1111,7 +1114,7 @@ cudaError_t snap_scores_mma(const SnapArgs &a, cudaStream_t s)
     cfg.gridDim = grid;
     cfg.blockDim = dim3(kMmaThreads);
     cfg.dynamicSmemBytes = G::SMEM_BYTES;
-    return cudaLaunchKernelEx(&cfg, snap_mma_kernel<D, 2>, tmap, a.page_cap, a.S, a.len, (const bf16 *)a.qw, a.W, a.H, sl2, (float2 *)nullptr,
+    return cudaLaunchKernelEx(&cfg, snap_mma_kernel<D, 2>, tmap, qmap, a.page_cap, a.S, a.len, a.W, a.H, sl2, (float2 *)nullptr,
                               (const float2 *)a.rowstat, a.imp, ntiles, tpc, a.status);
 }
 

@@ -136,29 +136,6 @@ __device__ __forceinline__ void tmem_dealloc(uint32_t taddr, uint32_t cols)
 // runs, the operands have to be moved to the warp's uniform registers for each instruction, which costs more cycles than
 // the product itself takes.
 
-// one product step; accumulate = 0 overwrites D
-__device__ __forceinline__ void umma_bf16(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc, uint32_t accumulate)
-{
-    asm volatile(
-        "{\n\t.reg .pred p, e;\n\t"
-        "elect.sync _|e, 0xffffffff;\n\t"
-        "setp.ne.b32 p, %4, 0;\n\t"
-        "@e tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
-        ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
-        : "memory");
-}
-// the same with the A operand in tensor memory: lane = row, a 32-bit column holds two consecutive bf16 of the
-// row's K extent (the lower index in the low half), so a K step of 16 elements is 8 columns
-__device__ __forceinline__ void umma_bf16_ta(uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc, uint32_t idesc, uint32_t accumulate)
-{
-    asm volatile(
-        "{\n\t.reg .pred p, e;\n\t"
-        "elect.sync _|e, 0xffffffff;\n\t"
-        "setp.ne.b32 p, %4, 0;\n\t"
-        "@e tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}"
-        ::"r"(d_tmem), "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(accumulate)
-        : "memory");
-}
 // Four consecutive K steps of a product (64 elements), the descriptors of A and B `A_STEP` and `B_STEP` further on from step
 // to step (descriptor units of 16 bytes; for an A operand in tensor memory, columns); the first step overwrites D if
 // accumulate = 0.  One election and a handful of additions instead of four times as much: a warp starts an instruction
@@ -181,6 +158,8 @@ __device__ __forceinline__ void umma_bf16_x4(uint32_t d_tmem, uint64_t a_desc, u
         "n"(2 * B_STEP), "n"(3 * B_STEP)
         : "memory");
 }
+// The same with the A operand in tensor memory: lane = row, a 32-bit column holds two consecutive bf16 of the row's K extent
+// (the lower index in the low half), so a K step of 16 elements is 8 columns.
 template <int A_STEP, int B_STEP>
 __device__ __forceinline__ void umma_bf16_ta_x4(uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc, uint32_t idesc, uint32_t accumulate)
 {
