@@ -103,11 +103,13 @@ __device__ __forceinline__ uint32_t score_bin(float v, float lo, float inv)
 // A threshold bucket of more than 16 blocks is cut further by buckets on the scores' integer images until at most 16
 // are left or all left are equal (equal scores: the lowest blocks).  More than 512 blocks are taken in panels of 512,
 // whose scores are computed again for each pass (the tensor cores have nothing else to do here).
-// Measured, 32 heads x 128 channels: 4096 queries, 16 of 64 blocks each, 158 -> 47 us; 30011 queries, 30 of 469 blocks
+// Measured, 32 heads x 128 channels: 4096 queries, 16 of 64 blocks each, 158 -> 42 us; 30011 queries, 30 of 469 blocks
 // each, 28.9 -> 1.0 ms.  (Before: fp32 FMA scores, a lane per block, then a bit-wise vote search up to 128 blocks and one
 // round per taken block beyond.  Of the former: queries by tensor map and four product steps per election 58 -> 52 us,
-// candidates noted by one atomic per word instead of one each 52 -> 47 us.)
-template <int D>
+// candidates noted by one atomic per word instead of one each 52 -> 47 us, half words for up to 64 blocks 47 -> 42 us.)
+// HALF: prompts of at most 64 blocks, whose two words of scores are taken by half words, so that all four threads of a query
+// have some.
+template <int D, bool HALF>
 __global__ void __launch_bounds__(kRouteThreads, 2) moba_route_mma_kernel(const __grid_constant__ CUtensorMap qmap, const float *means, int64_t len, int H,
                                                                       int block, int nb, int K, int words, uint32_t *masks,
                                                                       int32_t *list, int32_t *status)
@@ -223,11 +225,24 @@ __global__ void __launch_bounds__(kRouteThreads, 2) moba_route_mma_kernel(const 
             ok = __syncthreads_and(ok);
             tcgen05_after_sync();
         };
-        // body(word, scores, candidates among them as bits) for this thread's words of every panel
+        // body(word, its first column taken, scores, candidates among them as bits) for this thread's words of every panel
         auto for_scores = [&](bool first, auto body) {
             for (int p = 0; p < panels && ok; ++p) {
                 if (first || panels > 1) panel(p);
                 if (!ok) break;
+                if constexpr (HALF) {
+                    if ((part >> 1) < words_cta) {
+                        uint32_t x[16];
+                        float v[16];
+                        tmem_ld16(tl + (uint32_t)part * 16u, x);
+#pragma unroll
+                        for (int c = 0; c < 16; ++c) v[c] = __uint_as_float(x[c]);
+                        const int hi = c_hi - 16 * part;
+                        uint32_t cand = hi >= 16 ? 0xffffu : hi <= 0 ? 0u : (1u << hi) - 1u;
+                        if (part == 0) cand &= ~1u;
+                        body(part >> 1, (part & 1) * 16, v, cand);
+                    }
+                } else
 #pragma unroll 1
                 for (int wl = part; wl < 2 * kPanelGroups; wl += 4) {
                     const int w = p * 2 * kPanelGroups + wl;
@@ -238,7 +253,7 @@ __global__ void __launch_bounds__(kRouteThreads, 2) moba_route_mma_kernel(const 
                     const int hi = c_hi - 32 * w;
                     uint32_t cand = hi >= 32 ? 0xffffffffu : hi <= 0 ? 0u : (1u << hi) - 1u;
                     if (w == 0) cand &= ~1u;
-                    body(w, v, cand);
+                    body(w, 0, v, cand);
                 }
                 tcgen05_before_sync();
                 if (panels > 1) __syncthreads();                               // the scores may be overwritten
@@ -273,13 +288,14 @@ __global__ void __launch_bounds__(kRouteThreads, 2) moba_route_mma_kernel(const 
 
         // ---- 1. smallest and largest
         float mn = CUDART_INF_F, mx = -CUDART_INF_F;
-        for_scores(true, [&](int w, float (&v)[32], uint32_t cand) {
-            if (w > 0 && 32 * w + 32 <= own_first && own_first >= K) {         // every score is a candidate of every query
+        constexpr int N = HALF ? 16 : 32;                                      // scores taken at a time
+        for_scores(true, [&](int w, int c0, float (&v)[N], uint32_t cand) {
+            if (w + c0 > 0 && 32 * w + c0 + N <= own_first && own_first >= K) {         // every score is a candidate of every query
 #pragma unroll
-                for (int c = 0; c < 32; ++c) { mn = fminf(mn, v[c]); mx = fmaxf(mx, v[c]); }
+                for (int c = 0; c < N; ++c) { mn = fminf(mn, v[c]); mx = fmaxf(mx, v[c]); }
             } else {
 #pragma unroll
-                for (int c = 0; c < 32; ++c)
+                for (int c = 0; c < N; ++c)
                     if ((cand >> c) & 1u) { mn = fminf(mn, v[c]); mx = fmaxf(mx, v[c]); }
             }
         });
@@ -298,9 +314,9 @@ __global__ void __launch_bounds__(kRouteThreads, 2) moba_route_mma_kernel(const 
         const float inv = range > 0.0f ? fminf((float)(NB - 3) / range, 3.0e38f) : 0.0f;
 
         // ---- 2. buckets
-        for_scores(false, [&](int w, float (&v)[32], uint32_t cand) {
+        for_scores(false, [&](int, int, float (&v)[N], uint32_t cand) {
 #pragma unroll
-            for (int c = 0; c < 32; ++c)
+            for (int c = 0; c < N; ++c)
                 if ((cand >> c) & 1u) atomicAdd(&hist[score_bin(v[c], mn, inv) * NQ + ql], 1u);
         });
         if (ok) {
@@ -321,9 +337,9 @@ __global__ void __launch_bounds__(kRouteThreads, 2) moba_route_mma_kernel(const 
             if (over && klo == khi) { tied = true; over = false; }             // all equal: the lowest blocks are taken below
             if (!__syncthreads_or(over)) break;
             uint32_t kmin = 0xffffffffu, kmax = 0u;
-            for_scores(false, [&](int w, float (&v)[32], uint32_t cand) {
+            for_scores(false, [&](int, int, float (&v)[N], uint32_t cand) {
 #pragma unroll
-                for (int c = 0; c < 32; ++c) {
+                for (int c = 0; c < N; ++c) {
                     const uint32_t k = score_key(v[c]);
                     if (over && ((cand >> c) & 1u) && (int)score_bin(v[c], mn, inv) == tbin && k >= klo && k <= khi) {
                         kmin = min(kmin, k);
@@ -343,9 +359,9 @@ __global__ void __launch_bounds__(kRouteThreads, 2) moba_route_mma_kernel(const 
             }
             const uint32_t span = over ? kmax - kmin : 0u;
             const int sh = max(0, 26 - __clz((int)span));                      // (span >> sh) < 64
-            for_scores(false, [&](int w, float (&v)[32], uint32_t cand) {
+            for_scores(false, [&](int, int, float (&v)[N], uint32_t cand) {
 #pragma unroll
-                for (int c = 0; c < 32; ++c) {
+                for (int c = 0; c < N; ++c) {
                     const uint32_t k = score_key(v[c]);
                     if (over && ((cand >> c) & 1u) && (int)score_bin(v[c], mn, inv) == tbin && k >= kmin && k <= kmax)
                         atomicAdd(&hist[((k - kmin) >> sh) * NQ + ql], 1u);
@@ -369,32 +385,36 @@ __global__ void __launch_bounds__(kRouteThreads, 2) moba_route_mma_kernel(const 
             const int tbin = s_tb[ql], need = s_need[ql];
             const uint32_t klo = s_klo[ql], khi = s_khi[ql];
             const bool refined = klo != 0u || khi != 0xffffffffu || tied;
-            for_scores(false, [&](int w, float (&v)[32], uint32_t cand) {
+            auto put = [&](uint32_t *words_of, int w, int c0, uint32_t x) {
+                if constexpr (HALF) reinterpret_cast<uint16_t *>(words_of)[(w * NQ + ql) * 2 + (c0 >> 4)] = (uint16_t)x;
+                else words_of[w * NQ + ql] = x;
+            };
+            for_scores(false, [&](int w, int c0, float (&v)[N], uint32_t cand) {
                 uint32_t bits = 0u, eq = 0u;
                 if (!__any_sync(FULL, refined)) {
                     // one atomic per thread and word: one per candidate, each waited for while most lanes had none, took
                     // half of a CTA's time
 #pragma unroll
-                    for (int c = 0; c < 32; ++c) {
+                    for (int c = 0; c < N; ++c) {
                         const int bin = (int)score_bin(v[c], mn, inv);
                         if (bin > tbin) bits |= 1u << c;
                         if (bin == tbin) eq |= 1u << c;
                     }
-                    mk[w * NQ + ql] = bits & cand;
+                    put(mk, w, c0, bits & cand);
                     eq = need > 0 ? eq & cand : 0u;
                     if (!__any_sync(FULL, eq != 0u)) return;
                     uint32_t at = eq ? atomicAdd(&s_n[ql], (uint32_t)__popc(eq)) : (uint32_t)CAP;
 #pragma unroll
-                    for (int c = 0; c < 32; ++c)
+                    for (int c = 0; c < N; ++c)
                         if (((eq >> c) & 1u) && at < (uint32_t)CAP) {
                             ckey[at * NQ + ql] = score_key(v[c]);
-                            cidx[at * NQ + ql] = (uint16_t)(32 * w + c);
+                            cidx[at * NQ + ql] = (uint16_t)(32 * w + c0 + c);
                             ++at;
                         }
                     return;
                 }
 #pragma unroll
-                for (int c = 0; c < 32; ++c) {
+                for (int c = 0; c < N; ++c) {
                     const int bin = (int)score_bin(v[c], mn, inv);
                     if (bin > tbin) bits |= 1u << c;
                     if (bin == tbin && ((cand >> c) & 1u)) {
@@ -408,14 +428,14 @@ __global__ void __launch_bounds__(kRouteThreads, 2) moba_route_mma_kernel(const 
                                 const uint32_t at = atomicAdd(&s_n[ql], 1u);
                                 if (at < (uint32_t)CAP) {
                                     ckey[at * NQ + ql] = k;
-                                    cidx[at * NQ + ql] = (uint16_t)(32 * w + c);
+                                    cidx[at * NQ + ql] = (uint16_t)(32 * w + c0 + c);
                                 }
                             }
                         }
                     }
                 }
-                mk[w * NQ + ql] = bits & cand;
-                if (tied) tie[w * NQ + ql] = eq;
+                put(mk, w, c0, bits & cand);
+                if (tied) put(tie, w, c0, eq);
             });
             __syncthreads();
             if (active && need > 0) {
@@ -500,7 +520,9 @@ template <int D> cudaError_t route_run(const MobaArgs &a, cudaStream_t s)
     if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
     if (!ready[dev]) {
         const int one = G::smem_bytes(true, kPanelGroups * kRouteGroup / 32), more = G::smem_bytes(false, kMobaMaxBlocks / 32);
-        e = cudaFuncSetAttribute(moba_route_mma_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, one > more ? one : more);
+        e = cudaFuncSetAttribute(moba_route_mma_kernel<D, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, one > more ? one : more);
+        if (e != cudaSuccess) return e;
+        e = cudaFuncSetAttribute(moba_route_mma_kernel<D, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, G::smem_bytes(true, 2));
         if (e != cudaSuccess) return e;
         ready[dev] = true;
     }
@@ -522,7 +544,7 @@ template <int D> cudaError_t route_run(const MobaArgs &a, cudaStream_t s)
     cfg.stream = s;
     cfg.attrs = &at;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, moba_route_mma_kernel<D>, qmap, (const float *)a.means, a.len, a.H, a.block, nb, a.K, words, a.masks,
+    return cudaLaunchKernelEx(&cfg, words <= 2 ? moba_route_mma_kernel<D, true> : moba_route_mma_kernel<D, false>, qmap, (const float *)a.means, a.len, a.H, a.block, nb, a.K, words, a.masks,
                               a.list, a.status);
 }
 

@@ -49,7 +49,7 @@ def expected(levels, own, K):
 
 
 @pytest.mark.parametrize("D", [64, 128])
-@pytest.mark.parametrize("T,K", [(64 * 64, 16), (64 * 65 + 1, 9), (64 * 257, 40), (64 * 512, 100), (64 * 513 + 7, 33), (64 * 130, 2)])
+@pytest.mark.parametrize("T,K", [(64 * 64, 16), (64 * 17, 4), (64 * 33 + 5, 6), (64 * 48 + 1, 47), (64 * 65 + 1, 9), (64 * 257, 40), (64 * 512, 100), (64 * 513 + 7, 33), (64 * 130, 2)])
 @pytest.mark.parametrize("kind", ["distinct", "runs", "equal", "clustered"])
 def test_lists_at_the_edges(kind, T, K, D):
     block = 64
