@@ -513,18 +513,18 @@ template <int D> cudaError_t route_run(const MobaArgs &a, cudaStream_t s)
     const int BH = a.B * a.H, nb = (int)((a.len + a.block - 1) / a.block), words = (nb + 31) / 32;
     const int groups = (nb + kRouteGroup - 1) / kRouteGroup;
     const bool one_panel = groups <= kPanelGroups;
-    static bool ready[64];
+    const bool half = words <= 2;
+    static bool ready[2][64];
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
-    if (!ready[dev]) {
+    const auto kernel = half ? moba_route_mma_kernel<D, true> : moba_route_mma_kernel<D, false>;
+    if (!ready[half][dev]) {
         const int one = G::smem_bytes(true, kPanelGroups * kRouteGroup / 32), more = G::smem_bytes(false, kMobaMaxBlocks / 32);
-        e = cudaFuncSetAttribute(moba_route_mma_kernel<D, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, one > more ? one : more);
+        e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, half ? G::smem_bytes(true, 2) : one > more ? one : more);
         if (e != cudaSuccess) return e;
-        e = cudaFuncSetAttribute(moba_route_mma_kernel<D, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, G::smem_bytes(true, 2));
-        if (e != cudaSuccess) return e;
-        ready[dev] = true;
+        ready[half][dev] = true;
     }
     const int per = 256 / (D / 2);
     moba_means_bf16_kernel<<<dim3((unsigned)((nb + per - 1) / per), (unsigned)BH), 256, 0, s>>>(
@@ -544,7 +544,7 @@ template <int D> cudaError_t route_run(const MobaArgs &a, cudaStream_t s)
     cfg.stream = s;
     cfg.attrs = &at;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, words <= 2 ? moba_route_mma_kernel<D, true> : moba_route_mma_kernel<D, false>, qmap, (const float *)a.means, a.len, a.H, a.block, nb, a.K, words, a.masks,
+    return cudaLaunchKernelEx(&cfg, kernel, qmap, (const float *)a.means, a.len, a.H, a.block, nb, a.K, words, a.masks,
                               a.list, a.status);
 }
 

@@ -500,6 +500,16 @@ __global__ void scan_chain_kernel(const float *state, int D, int gph, int chunks
 template <typename T, typename G, int D, int S, int MODE>
 cudaError_t start(const ScanArgs &a, const ScanMaps &tm, const ScanPlan &p, int cl, float *maps, const float *entry, int smem, cudaStream_t s)
 {
+    static bool ready[64];                                       // (set up form by form: the first use of a kernel loads it)
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
+    if (!ready[dev]) {
+        e = cudaFuncSetAttribute(scan_kernel<T, G, D, S, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        if (e != cudaSuccess) return e;
+        ready[dev] = true;
+    }
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute at[2] = {};
     at[0].id = cudaLaunchAttributeClusterDimension;
@@ -527,20 +537,7 @@ cudaError_t run(const ScanArgs &a, cudaStream_t s)
     const int64_t units = (int64_t)a.B * a.H * (D / CG);
     if (units >= (int64_t)1 << 28) return cudaErrorInvalidValue;
     constexpr int DSM = scan_stages<T, G>() * scan_stage_bytes<T, G>();
-    static bool ready[64];
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return e;
-    if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
-    if (!ready[dev]) {
-        e = cudaFuncSetAttribute(scan_kernel<T, G, D, S, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, DSM);
-        if (e != cudaSuccess) return e;
-        e = cudaFuncSetAttribute(scan_kernel<T, G, D, S, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, DSM);
-        if (e != cudaSuccess) return e;
-        e = cudaFuncSetAttribute(scan_kernel<T, G, D, S, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, DSM);
-        if (e != cudaSuccess) return e;
-        ready[dev] = true;
-    }
+    cudaError_t e;
     ScanPlan p;
     p.tile0 = t0;
     p.ntiles = (int)(t1 - t0);

@@ -1061,13 +1061,6 @@ cudaError_t snap_scores_mma(const SnapArgs &a, cudaStream_t s)
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
-    if (!ready[dev]) {
-        e = cudaFuncSetAttribute(snap_mma_kernel<D, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, G::SMEM_BYTES);
-        if (e != cudaSuccess) return e;
-        e = cudaFuncSetAttribute(snap_mma_kernel<D, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, G::SMEM_BYTES);
-        if (e != cudaSuccess) return e;
-        ready[dev] = true;
-    }
     const int BH = a.B * a.H;
     if (kMmaKeys % a.S != 0) return cudaErrorInvalidValue;
     alignas(64) CUtensorMap tmap, qmap;
@@ -1078,6 +1071,13 @@ cudaError_t snap_scores_mma(const SnapArgs &a, cudaStream_t s)
     const int ntiles = (int)((a.len + kMmaKeys - 1) / kMmaKeys);
     if (ntiles <= 4 * kOnceCluster) return snap_scores_once<D, 4>(a, tmap, qmap, ntiles, s);
     if (ntiles <= 8 * kOnceCluster) return snap_scores_once<D, 8>(a, tmap, qmap, ntiles, s);
+    if (!ready[dev]) {
+        e = cudaFuncSetAttribute(snap_mma_kernel<D, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, G::SMEM_BYTES);
+        if (e != cudaSuccess) return e;
+        e = cudaFuncSetAttribute(snap_mma_kernel<D, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, G::SMEM_BYTES);
+        if (e != cudaSuccess) return e;
+        ready[dev] = true;
+    }
     // tiles per CTA: two CTAs share an SM, so the launch runs in rounds of 2 * SMs CTAs; the choice with the fewest
     // rounds * (tiles of a CTA + what a CTA costs before its first tile, about two tiles' time) ends soonest
     const int64_t slots = 2 * (int64_t)sm_count();
