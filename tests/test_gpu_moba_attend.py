@@ -42,3 +42,25 @@ def test_dense_budget(growth, T, D):
     ref = torch.nn.functional.scaled_dot_product_attention(*(x.double().transpose(1, 2) for x in (q, k, v)), is_causal=True)
     err = (o.double().transpose(1, 2) - ref).abs().max().item()
     assert err <= 1.1 * 2 ** -8 * v.float().abs().max().item()
+
+
+@pytest.mark.parametrize("D,T,gain", [(64, 500, 3.0), (128, 700, 3.0), (128, 1300, 12.0)])
+def test_weights_add_up_to_one(D, T, gain):
+    """Where all values are the same, so is every output, whatever the weights: what divides the output is the sum of the
+    weights as they were multiplied.  The fp32 sums are good to 2^-20, an eighth of a thousandth of a bf16 step: nothing that
+    rounding to bf16 leaves visible (the values are bf16 themselves, in the middle of their rounding interval)."""
+    block, H = 64, 2
+    g = torch.Generator(device=DEV)
+    g.manual_seed(T + D)
+    k, q = (torch.randn(1, T, H, D, generator=g, device=DEV) for _ in range(2))
+    v = torch.randn(1, 1, H, D, generator=g, device=DEV).to(torch.bfloat16).expand(1, T, H, D).contiguous()
+    k, q = k.to(torch.bfloat16), (gain * q).to(torch.bfloat16)
+    cache = rq.Cache(1, H, D, 16, T, torch.bfloat16)
+    rq.rq_build_cache(cache.handle, k, v, torch.zeros_like(k))    # zero gates: the cache holds k and v themselves
+    o = torch.empty_like(q)
+    K = -(-T // block)
+    scratch = torch.empty(rq.rq_moba_scratch_bytes(cache.handle, block, K), dtype=torch.uint8, device=DEV)
+    rq.rq_moba_prefill(cache.handle, q, block, K, 0.0, o, None, None, scratch)
+    torch.cuda.synchronize()
+    assert rq.rq_device_status(cache.handle) == rq.RQ_OK
+    assert torch.equal(o, v)
