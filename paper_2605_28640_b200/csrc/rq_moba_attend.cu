@@ -43,6 +43,14 @@ __device__ __forceinline__ float exp2_fast(float x)
     return y;
 }
 
+// the larger one; NaN if one is NaN
+__device__ __forceinline__ float max_nan(float a, float b)
+{
+    float y;
+    asm("max.NaN.f32 %0, %1, %2;" : "=f"(y) : "f"(a), "f"(b));
+    return y;
+}
+
 // The walk over the chunks of the listed blocks: (entry of the list, chunk inside the block).
 struct Walk {
     int bi = 0, r = 0;
@@ -317,10 +325,13 @@ __global__ void __launch_bounds__(kThreads, 1) moba_mma_kernel(const __grid_cons
                 }
                 float tm[4] = {v[0], v[1], v[2], v[3]};
 #pragma unroll
-                for (int k = 4; k < kChunk; ++k) tm[k & 3] = fmaxf(tm[k & 3], v[k]);
-                const float top = fmaxf(fmaxf(tm[0], tm[1]), fmaxf(tm[2], tm[3])) * scale_log2;
+                for (int k = 4; k < kChunk; ++k) tm[k & 3] = max_nan(tm[k & 3], v[k]);
+                const float top = max_nan(max_nan(tm[0], tm[1]), max_nan(tm[2], tm[3])) * scale_log2;
                 const bool raise = nv > 0 && top > m + kRaise;
-                if (__any_sync(FULL, raise)) {
+                const bool stray = nv == 0 && !(top < CUDART_INF_F);       // infinite or NaN scores of a block the query did not choose
+                if (__any_sync(FULL, raise || stray)) {
+#pragma unroll
+                    for (int k = 0; k < kChunk; ++k) v[k] = stray ? -CUDART_INF_F : v[k];
                     const bool touch = raise && m > -CUDART_INF_F;         // (otherwise the query's row of O is still zero)
                     const float f = touch ? exp2_fast(m - top) : 1.0f;
                     if (raise) m = top;
@@ -340,7 +351,8 @@ __global__ void __launch_bounds__(kThreads, 1) moba_mma_kernel(const __grid_cons
                         }
                     }
                 }
-                const float nm = nv > 0 ? -m : -3.0e38f;         // a block the query did not choose: 2^-3e38 = 0
+                // a block the query did not choose: 2^-3e38 = 0; nor do scores of -inf weigh anything while there is no other
+                const float nm = nv > 0 ? fminf(-m, 3.0e38f) : -3.0e38f;
                 const float2 nm2 = make_float2(nm, nm), one2 = make_float2(1.0f, 1.0f);
 #pragma unroll
                 for (int hf = 0; hf < 2; ++hf) {
@@ -383,7 +395,7 @@ __global__ void __launch_bounds__(kThreads, 1) moba_mma_kernel(const __grid_cons
             ok = mbar_wait(&pv_done[s][(u - 1) & 1], (uint32_t)(((u - 1) >> 1) & 1));
             if (__all_sync(FULL, ok)) {
                 tcgen05_after_sync();
-                const float l = l2.x + l2.y, inv = l > 0.0f ? 1.0f / l : 0.0f;
+                const float inv = 1.0f / (l2.x + l2.y);          // (nothing but scores of -inf: NaN; rows past the prompt are not stored)
                 // (the accumulator's queries are not read any more: its rows go out through their room, a store per warp and
                 // 64 channels; rows past the prompt are cut off by the map)
                 unsigned char *os = qs + s * G::Q_BYTES + (warp & 3) * 32 * 128;

@@ -175,6 +175,7 @@ __global__ void __launch_bounds__(kRouteThreads, 2) moba_route_mma_kernel(const 
         // the scores of panel p into tensor memory, 64 blocks at a time: all threads cut representatives into terms, the
         // first warp starts the products (the whole warp, see rq_umma.cuh)
         constexpr int PER = kRouteGroup * D / 4 / kRouteThreads;               // float4 of a thread
+        auto rest = [](float x, float term) { return fabsf(term) == CUDART_INF_F ? 0.0f : x - term; };     // of an infinite mean: nothing
         auto panel = [&](int p) {
             const int g0 = p * kPanelGroups, gn = min(kPanelGroups, groups - g0);
             float4 f[PER];
@@ -199,7 +200,7 @@ __global__ void __launch_bounds__(kRouteThreads, 2) moba_route_mma_kernel(const 
                     for (int t = 0; t < 3; ++t) {                              // the remainders are exact: each term takes the next 8 bits
                         const uint2 w = make_uint2(pack_bf16(x.x, x.y), pack_bf16(x.z, x.w));
                         *reinterpret_cast<uint2 *>(dst + t * G::PLANE_BYTES) = w;
-                        x.x -= bf16lo(w.x); x.y -= bf16hi(w.x); x.z -= bf16lo(w.y); x.w -= bf16hi(w.y);
+                        x = make_float4(rest(x.x, bf16lo(w.x)), rest(x.y, bf16hi(w.x)), rest(x.z, bf16lo(w.y)), rest(x.w, bf16hi(w.y)));
                     }
                 }
                 asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // ordinary stores, read by the tensor core
