@@ -10,7 +10,7 @@
 // and a sum over the window.  The 64 x T scores of a long head are not stored: its keys are read twice,
 // once for the row statistics (maximum and sum of exponentials of every query) and once for the
 // weights.
-//   snap_once_kernel          bf16 caches, up to 8192 positions: the scores do fit in the tensor memory of a cluster of CTAs
+//   snap_once_kernel          bf16 caches, up to 4096 positions: the scores do fit in the tensor memory of a cluster of CTAs
 //                             and the keys are read once
 //   snap_mma_kernel<PASS 1>   longer bf16 caches.  Per (head, run of 128-key tiles): the scores of a tile on the
 //                             tensor cores (tcgen05.mma, operands in shared memory, fp32 accumulator
@@ -401,8 +401,8 @@ __global__ void __launch_bounds__(kMmaThreads) snap_mma_kernel(const __grid_cons
 }
 
 // ---------------------------------------------------------------- short prompts: the keys read once
-// A cluster of up to kOnceCluster CTAs per head, each with up to RT tiles of 128 keys.  The scores of the head, 64 columns
-// of fp32 per tile, stay in the cluster's tensor memory between the passes, so that the keys come from HBM once:
+// A cluster of up to kOnceCluster CTAs per head, each with up to kOnceTiles tiles of 128 keys.  The scores of the head, 64
+// columns of fp32 per tile, stay in the cluster's tensor memory between the passes, so that the keys come from HBM once:
 //   tiles    D[key][query] = K Q^T as they land; running maximum of every query over the thread's keys
 //   maximum  of a query over the lanes, the warps and (distributed shared memory) the CTAs of the cluster
 //   weights  2^(s - max) written over the scores, their sums over lanes, warps and CTAs in the same way
@@ -411,9 +411,18 @@ __global__ void __launch_bounds__(kMmaThreads) snap_mma_kernel(const __grid_cons
 // maximum is the head's before a weight is taken, as in the two-pass kernels: equal keys get equal importance wherever they
 // lie.  Bound by the chain of a CTA (copies, two exchanges over the cluster, three walks over the scores: 11 us for 512
 // keys), which two CTAs per SM overlap.  256 heads x 4096 keys x 128 channels: 124 (two passes and the merge) -> 95 us.
+// Eight tiles per CTA, for up to 8192 positions, fill tensor memory with one CTA per SM and were slower than two passes at
+// every number of heads (8192 positions, a call, us: 4 heads 24 / 20, 32 heads 55 / 40, 256 heads 266 / 229).
+// CTAs wait for one another with their tensor memory in hand, so a CTA must never stand in tcgen05.alloc behind another
+// cluster's: two clusters that each hold what the other needs would wait for ever.  Shared memory sees to it: a CTA takes
+// more than a third of an SM's, so that at most two share an SM, whatever their registers, and two times 256 columns are
+// there.  (Kernels without such waits, the other users of tensor memory here, give theirs back in time.)
 constexpr int kOnceWarps = 8;
 constexpr int kOnceThreads = (kOnceWarps + 1) * 32;
 constexpr int kOnceCluster = 8;
+constexpr int kOnceTiles = 4;
+constexpr int kTmemColumns = 512;              // of an SM
+constexpr int kSmBytes = 228 * 1024;           // shared memory of an SM, 1 KB of it reserved for every CTA
 
 template <int D>
 struct SnapOnceGeom {
@@ -422,7 +431,10 @@ struct SnapOnceGeom {
     static constexpr int KH_BYTES = kMmaKeys * 128;            // 64 channels of a tile
     static constexpr int OFF_K = HALVES * QH_BYTES;
     static constexpr int TILE_BYTES = HALVES * KH_BYTES;
-    static constexpr int SMEM_BYTES = OFF_K + 2 * TILE_BYTES + 1024;
+    static constexpr int NEEDED_BYTES = OFF_K + 2 * TILE_BYTES + 1024;
+    static constexpr int SMEM_BYTES = NEEDED_BYTES > 76 * 1024 ? NEEDED_BYTES : 76 * 1024;
+    static constexpr uint32_t TCOLS = kOnceTiles * kSnapRows;
+    static_assert((kTmemColumns / TCOLS + 1) * (SMEM_BYTES + 1024) > kSmBytes, "an SM must not take more CTAs than its tensor memory holds");
 };
 
 // Lane l's result: OP over the 32 lanes of their v[l].
@@ -440,15 +452,16 @@ template <bool MAX> __device__ __forceinline__ float lanes_reduce(float (&v)[32]
     return v[0];
 }
 
-template <int D, int RT>
-__global__ void __launch_bounds__(kOnceThreads, RT <= 4 ? 2 : 1) snap_once_kernel(const __grid_constant__ CUtensorMap tmap,
+template <int D>
+__global__ void __launch_bounds__(kOnceThreads, 2) snap_once_kernel(const __grid_constant__ CUtensorMap tmap,
                                                                                 const __grid_constant__ CUtensorMap qmap,
                                                                                 int64_t page_cap, int S, int64_t len, int W, int H,
                                                                                 float scale_log2, float *imp, int ntiles,
                                                                                 int tiles_per_cta, int32_t *status)
 {
     using G = SnapOnceGeom<D>;
-    constexpr uint32_t TCOLS = RT * kSnapRows;
+    constexpr int RT = kOnceTiles;
+    constexpr uint32_t TCOLS = G::TCOLS;
     extern __shared__ __align__(1024) unsigned char osm_raw[];
     __shared__ __align__(8) uint64_t bar[RT], full[2], full_q; // a tile's product is complete; a stage's keys, the queries have landed
     __shared__ uint32_t tbase;
@@ -1017,8 +1030,8 @@ cudaError_t snap_scores_t(const SnapArgs &a, cudaStream_t s)
     return cudaGetLastError();
 }
 
-// The same for prompts whose scores fit in the tensor memory of a cluster: tiles per CTA and CTAs per head.
-template <int D, int RT>
+// The same for prompts whose scores fit in the tensor memory of a cluster.
+template <int D>
 cudaError_t snap_scores_once(const SnapArgs &a, const CUtensorMap &tmap, const CUtensorMap &qmap, int ntiles, cudaStream_t s)
 {
     using G = SnapOnceGeom<D>;
@@ -1028,13 +1041,13 @@ cudaError_t snap_scores_once(const SnapArgs &a, const CUtensorMap &tmap, const C
     if (e != cudaSuccess) return e;
     if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
     if (!ready[dev]) {
-        e = cudaFuncSetAttribute(snap_once_kernel<D, RT>, cudaFuncAttributeMaxDynamicSharedMemorySize, G::SMEM_BYTES);
+        e = cudaFuncSetAttribute(snap_once_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, G::SMEM_BYTES);
         if (e != cudaSuccess) return e;
         ready[dev] = true;
     }
-    const int BH = a.B * a.H, slots = (RT <= 4 ? 2 : 1) * sm_count();
+    const int BH = a.B * a.H, slots = 2 * sm_count();
     // as few CTAs per head as hold its tiles, more while the chip has room for them at once
-    int cl = (ntiles + RT - 1) / RT;
+    int cl = (ntiles + kOnceTiles - 1) / kOnceTiles;
     while (cl < kOnceCluster && cl < ntiles && BH * (cl + 1) <= slots) ++cl;
     const int tpc = (ntiles + cl - 1) / cl;
     cudaLaunchConfig_t cfg = {};
@@ -1048,7 +1061,7 @@ cudaError_t snap_scores_once(const SnapArgs &a, const CUtensorMap &tmap, const C
     cfg.stream = s;
     cfg.attrs = &at;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, snap_once_kernel<D, RT>, tmap, qmap, a.page_cap, a.S, a.len, a.W, a.H, a.scale * 1.4426950408889634f, a.imp,
+    return cudaLaunchKernelEx(&cfg, snap_once_kernel<D>, tmap, qmap, a.page_cap, a.S, a.len, a.W, a.H, a.scale * 1.4426950408889634f, a.imp,
                               ntiles, tpc, a.status);
 }
 
@@ -1069,8 +1082,7 @@ cudaError_t snap_scores_mma(const SnapArgs &a, cudaStream_t s)
     e = query_tensor_map(&qmap, a.qw, D, a.H, a.W, a.B, kSnapRows);
     if (e != cudaSuccess) return e;
     const int ntiles = (int)((a.len + kMmaKeys - 1) / kMmaKeys);
-    if (ntiles <= 4 * kOnceCluster) return snap_scores_once<D, 4>(a, tmap, qmap, ntiles, s);
-    if (ntiles <= 8 * kOnceCluster) return snap_scores_once<D, 8>(a, tmap, qmap, ntiles, s);
+    if (ntiles <= kOnceTiles * kOnceCluster) return snap_scores_once<D>(a, tmap, qmap, ntiles, s);
     if (!ready[dev]) {
         e = cudaFuncSetAttribute(snap_mma_kernel<D, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, G::SMEM_BYTES);
         if (e != cudaSuccess) return e;

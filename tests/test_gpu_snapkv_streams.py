@@ -1,0 +1,33 @@
+"""Importance and selection of short prompts on several streams at once: CTAs that wait for the others of their cluster with
+tensor memory in hand must all find room, whoever else is on the chip.  The results are those of one call after the other."""
+import pytest
+import torch
+
+import paper_2605_28640_b200 as rq
+
+pytestmark = pytest.mark.gpu
+DEV = "cuda"
+
+
+def test_concurrent_reductions():
+    calls = []
+    for i, (D, H, T) in enumerate([(64, 40, 4096), (128, 24, 4000), (64, 33, 8192), (128, 40, 2500), (64, 64, 3333), (128, 8, 20000)]):
+        g = torch.Generator(device=DEV)
+        g.manual_seed(i)
+        cache = rq.Cache(1, H, D, 16, T, torch.bfloat16)
+        k = torch.randn(1, T, H, D, generator=g, device=DEV, dtype=torch.bfloat16)
+        rq.rq_build_cache(cache.handle, k, k, torch.zeros_like(k))
+        qw = torch.randn(1, 64, H, D, generator=g, device=DEV, dtype=torch.bfloat16)
+        scratch = torch.empty(rq.rq_snapkv_scratch_bytes(cache.handle), dtype=torch.uint8, device=DEV)
+        outs = [(torch.empty(1, H, 300, dtype=torch.int32, device=DEV), torch.empty(1, H, T, device=DEV)) for _ in range(2)]
+        calls.append((cache, qw, scratch, outs, torch.cuda.Stream()))
+    for cache, qw, scratch, outs, _ in calls:
+        rq.rq_snapkv_select(cache.handle, qw, 64, 300, 0.0, *outs[0], scratch)
+    torch.cuda.synchronize()
+    for _ in range(20):
+        for cache, qw, scratch, outs, stream in calls:
+            rq.rq_snapkv_select(cache.handle, qw, 64, 300, 0.0, *outs[1], scratch, stream=stream)
+    torch.cuda.synchronize()
+    for cache, _, _, outs, _ in calls:
+        assert rq.rq_device_status(cache.handle) == rq.RQ_OK
+        assert torch.equal(outs[0][0], outs[1][0]) and torch.equal(outs[0][1], outs[1][1])
