@@ -28,6 +28,7 @@
 //   snap_select_kernel        per head: the keep - W most important positions before the window
 //                             (buckets on the order-preserving image of the importance, equal importance
 //                             to the lower position) plus the window, written in ascending order
+//   snap_select_one_kernel    the same for many heads of a long prompt, one CTA per head
 //   snap_compact_kernel       per (head, 64 slots of the new cache): gathers the retained rows, rebuilds
 //                             the pages' min/max bounds, tracks the head's largest |key|
 #include <cooperative_groups.h>
@@ -683,18 +684,19 @@ __global__ void __launch_bounds__(128) snap_rows_kernel(const float2 *stats, flo
 }
 
 // ---------------------------------------------------------------- token-level selection
-// A cluster of CL CTAs per head.  Candidates: positions 0 .. C-1 (C = len - w, w = window positions kept outright);
-// `want` of them are taken: those with the largest importance, equal importance to the lower position.  A CTA owns a
+// Candidates: positions 0 .. C-1 (C = len - w, w = window positions kept outright); `want` of them are taken: those with the
+// largest importance, equal importance to the lower position.
+//
+// snap_select_kernel: a cluster of CL CTAs per head.  A CTA owns a
 // contiguous range of the candidates, a warp a contiguous part of it, a lane every 32nd position, whose
 // order-preserving keys it keeps in registers (EPT per thread; EPT = 0: read again in every pass).  The key of the last
 // position taken is found with 2048 equal-width buckets between the head's smallest and largest key, then again inside
 // the bucket that holds it, at most three times in all; every CTA counts its own keys and adds up the buckets of all
 // CTAs through distributed shared memory.  Then ballots and scans over warps and CTAs give every taken position its
 // place in the ascending list.
-// Bound: latency (a chain of about ten block- or cluster-wide steps).  One CTA per head, digits of 11 bits from the
-// top and the importances read from L2 in every pass: 86 us for 32 heads x 131000 positions, 17 us for 256 x 4096; so: 29
-// and 11 us.
+// Bound: latency (a chain of about ten block- or cluster-wide steps).  Figures at launch_snap_select below.
 constexpr int kSelMaxEpt = 32;
+constexpr int kSelOneThreads = 1024;
 
 template <int EPT, int NT>
 __global__ void __launch_bounds__(NT, 1024 / NT) snap_select_kernel(const float *imp, int64_t len, int w, int keep,
@@ -860,6 +862,127 @@ __global__ void __launch_bounds__(NT, 1024 / NT) snap_select_kernel(const float 
     });
     if (cr == 0)
         for (int i = tid; i < w; i += NT) out[want + i] = C + i;   // the window, above every candidate
+}
+
+// The same for many heads, each with one CTA of 1024 threads: radix select over the order-preserving keys, 11 bits from the
+// top per pass, the importances read from L2 in every pass; then every warp walks its own contiguous range twice (count,
+// write), so the list comes out ascending.  Two CTAs share an SM.
+__global__ void __launch_bounds__(kSelOneThreads, 2) snap_select_one_kernel(const float *imp, int64_t len, int w, int keep, int32_t *idx)
+{
+    constexpr unsigned FULL = 0xffffffffu;
+    __shared__ uint32_t hist[kSnapBins];
+    __shared__ uint32_t red[32], red2[32];
+    __shared__ uint32_t s_digit, s_krem, s_cnt;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int bh = blockIdx.x;
+    const float *x = imp + (int64_t)bh * len;
+    int32_t *out = idx + (int64_t)bh * keep;
+    const int C = (int)(len - w);
+    const int want = keep - w;
+    grid_dependency_wait();                          // the importances come from the kernel before
+    if (want >= C) {                                 // everything is kept
+        for (int j = tid; j < keep; j += kSelOneThreads) out[j] = j < len ? j : -1;
+        return;
+    }
+    uint32_t tau = 0xffffffffu;                      // want == 0: nothing but the window
+    int r_eq = 0;
+    if (want > 0) {
+        uint32_t prefix = 0u;
+        int k = want;
+        bool whole = false;
+#pragma unroll 1
+        for (int hi = 31; hi >= 0 && !whole; hi -= 11) {
+            const int lo = hi >= 10 ? hi - 10 : 0;   // this pass decides bits hi .. lo
+            const uint32_t dmask = (1u << (hi - lo + 1)) - 1u;
+            const uint32_t himask = hi == 31 ? 0u : ~0u << (hi + 1);
+            for (int i = tid; i < kSnapBins; i += kSelOneThreads) hist[i] = 0u;
+            __syncthreads();
+            // eight independent loads per thread are issued before the first is used
+            for (int j0 = tid; j0 < C; j0 += 8 * kSelOneThreads) {
+                float f[8];
+#pragma unroll
+                for (int u = 0; u < 8; ++u) f[u] = j0 + u * kSelOneThreads < C ? __ldcg(x + j0 + u * kSelOneThreads) : 0.0f;
+#pragma unroll
+                for (int u = 0; u < 8; ++u) {
+                    const uint32_t kx = order_key(f[u]);
+                    if (j0 + u * kSelOneThreads < C && (kx & himask) == (prefix & himask)) atomicAdd(&hist[(kx >> lo) & dmask], 1u);
+                }
+            }
+            __syncthreads();
+            // walk the bins from the top until k keys are covered: thread t owns bins 2t, 2t+1
+            const uint32_t c0 = hist[2 * tid], c1 = hist[2 * tid + 1];
+            uint32_t suf = c0 + c1;
+#pragma unroll
+            for (int off = 1; off < 32; off <<= 1) {
+                const uint32_t t = __shfl_down_sync(FULL, suf, off);
+                if (lane + off < 32) suf += t;
+            }
+            if (lane == 0) red[warp] = suf;
+            __syncthreads();
+            const uint32_t wtot = red[lane];
+            uint32_t wsuf = wtot;
+#pragma unroll
+            for (int off = 1; off < 32; off <<= 1) {
+                const uint32_t t = __shfl_down_sync(FULL, wsuf, off);
+                if (lane + off < 32) wsuf += t;
+            }
+            const uint32_t above = __shfl_sync(FULL, wsuf - wtot, warp);
+            const uint32_t incl1 = above + suf - c0, excl1 = incl1 - c1, incl0 = incl1 + c0, kr = (uint32_t)k;
+            if (incl1 >= kr && excl1 < kr) { s_digit = 2u * tid + 1u; s_krem = kr - excl1; s_cnt = c1; }
+            if (incl0 >= kr && incl1 < kr) { s_digit = 2u * tid; s_krem = kr - incl1; s_cnt = c0; }
+            __syncthreads();
+            prefix |= s_digit << lo;
+            k = (int)s_krem;
+            whole = s_cnt == s_krem;                 // the whole bin is wanted: its lowest possible key is a threshold
+            __syncthreads();
+        }
+        tau = prefix;
+        r_eq = whole ? 0x7fffffff : k;               // keys equal to tau that are taken, lowest positions first
+    }
+    // every warp owns a contiguous range of the candidates: count, scan over the warps, write
+    const int per = (C + 31) / 32, lo_j = warp * per, hi_j = min(C, lo_j + per);
+    uint32_t wgt = 0, weq = 0;
+    for (int j0 = lo_j; j0 < hi_j; j0 += 8 * 32) {
+        float f[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) f[u] = j0 + u * 32 + lane < hi_j ? __ldcg(x + j0 + u * 32 + lane) : 0.0f;
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            const bool in = j0 + u * 32 + lane < hi_j;
+            const uint32_t kx = order_key(f[u]);
+            wgt += __popc(__ballot_sync(FULL, in && kx > tau));
+            weq += __popc(__ballot_sync(FULL, in && kx == tau));
+        }
+    }
+    if (lane == 0) { red[warp] = wgt; red2[warp] = weq; }
+    __syncthreads();
+    uint32_t g_inc = red[lane], e_inc = red2[lane];
+#pragma unroll
+    for (int off = 1; off < 32; off <<= 1) {
+        const uint32_t tg = __shfl_up_sync(FULL, g_inc, off), te = __shfl_up_sync(FULL, e_inc, off);
+        if (lane >= off) { g_inc += tg; e_inc += te; }
+    }
+    int gt_run = (int)(__shfl_sync(FULL, g_inc, warp) - wgt), eq_run = (int)(__shfl_sync(FULL, e_inc, warp) - weq);
+    const uint32_t lt = (1u << lane) - 1u;
+    for (int j0 = lo_j; j0 < hi_j; j0 += 8 * 32) {
+        float f[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) f[u] = j0 + u * 32 + lane < hi_j ? __ldcg(x + j0 + u * 32 + lane) : 0.0f;
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            const int j = j0 + u * 32 + lane;
+            const bool in = j < hi_j;
+            const uint32_t kx = order_key(f[u]);
+            const bool is_gt = in && kx > tau, is_eq = in && kx == tau;
+            const uint32_t bg = __ballot_sync(FULL, is_gt), be = __ballot_sync(FULL, is_eq);
+            const int gb = gt_run + __popc(bg & lt), eb = eq_run + __popc(be & lt);
+            const int rank = is_gt ? gb + min(eb, r_eq) : (is_eq && eb < r_eq) ? gb + eb : -1;
+            if (rank >= 0 && rank < want) out[rank] = j;
+            gt_run += __popc(bg);
+            eq_run += __popc(be);
+        }
+    }
+    for (int i = tid; i < w; i += kSelOneThreads) out[want + i] = C + i;       // the window, above every candidate
 }
 
 // ---------------------------------------------------------------- compaction into the new cache
@@ -1190,14 +1313,37 @@ cudaError_t launch_snap_select(const float *imp, int BH, int64_t len, int window
     int w = window < keep ? window : keep;
     if ((int64_t)w > len) w = (int)len;
     const int64_t C = len - w;
-    // Up to 64K positions: CTAs of 512 threads with at most 16 keys each, two to an SM; beyond, CTAs of 1024 threads with
-    // 32 keys: half as many CTAs then add up each other's buckets (131000 positions of 32 heads: 38 -> 29 us), but the
-    // barriers of the wider CTAs cost 8 us where one CTA is enough for a head (4096 positions).
-    const bool wide = C > 8 * 512 * 16;
-    const int64_t nt = wide ? 1024 : 512, room = wide ? sm_count() : 2 * (int64_t)sm_count();
-    int64_t cl = 1;                                  // CTAs per head: enough to hold its keys in registers (up to eight), then
-    while (cl < 8 && C > cl * nt * (wide ? kSelMaxEpt : 16)) cl *= 2;   // more while all find room on the chip at once
-    while (cl < 8 && 2 * cl * BH <= room && C >= 4 * cl * nt) cl *= 2;
+    // Clusters are worth it while all their CTAs find room at once, and the larger they are the more of the chip their shape
+    // leaves out: sixteen clusters of eight already wait for one another.  Device time of the selection alone, us, clusters
+    // of 1 / 2 / 4 / 8 CTAs with the better number of threads, and one CTA per head by digits:
+    //   16 heads, 16384 positions    16 / 13 / 13 / 28, 17         131000   111 / 64 / 32 / 46, 88
+    //   32 heads, 16384              16 / 13 / 14 / 38, 17         131000    99 / 57 / 31 / 60, 89
+    //   64 heads, 16384              17 / 13 / 20 / 76, 17         131000   111 / 67 / 61 / 107, 90
+    //   128 heads, 8192   12 / 13 / 30 / -, 11;   16384   19 / 18 / 36 / 139, 18;   65536   64 / 55 / 72 / 161, 51
+    //   256 heads, 8192   15 / 24 / 57 / -, 20;   16384   33 / 32 / 67 / 262, 30;   65536  110 / 107 / 137 / 305, 97
+    //   8 heads, 65536              55 / 27 / 19 / 19, 47          131000   110 / 63 / 32 / 25, 88
+    const int64_t sms = sm_count(), room = sms - sms / 8;
+    const int64_t most = 16 * (int64_t)BH <= sms ? 8 : 4 * BH <= room ? 4 : 2 * BH <= room ? 2 : 1;
+    if (most == 1 && C > 512 * 16) {
+        cudaLaunchConfig_t cfg = {};
+        cudaLaunchAttribute at = {};
+        at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        at.val.programmaticStreamSerializationAllowed = 1;
+        cfg.gridDim = dim3((unsigned)BH);
+        cfg.blockDim = dim3(kSelOneThreads);
+        cfg.stream = s;
+        cfg.attrs = &at;
+        cfg.numAttrs = 1;
+        return cudaLaunchKernelEx(&cfg, snap_select_one_kernel, imp, len, w, keep, idx);
+    }
+    // 512 threads with up to 16 keys each, in as many CTAs as that takes (up to 4096 positions one does as well as two); beyond
+    // four of these, or where there is room for two only, 1024 threads with up to 32 keys
+    int64_t cl = C <= 4096 ? 1 : C <= 2 * 512 * 16 ? 2 : 4;
+    if (cl > most) cl = most;
+    const bool wide = C > cl * 512 * 16;
+    if (wide)
+        while (cl < most && C > cl * 512 * kSelMaxEpt) cl *= 2;
+    const int64_t nt = wide ? 1024 : 512;
     const int ept = (int)((C + cl * nt - 1) / (cl * nt));
     if (wide)
         return ept <= kSelMaxEpt ? select_run<kSelMaxEpt, 1024>(imp, BH, len, w, keep, (int)cl, ept * 32, idx, s)

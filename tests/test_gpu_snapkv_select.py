@@ -41,3 +41,12 @@ def test_index_for_index(BH, T, keeps, kinds):
             best = np.lexsort((np.arange(T - W), -x))[:keep - W]
             want = np.concatenate([np.sort(best), np.arange(T - W, T)])
             assert np.array_equal(idx[0, h].cpu().numpy(), want), f"head {h}, keep {keep}"
+
+
+@pytest.mark.parametrize("kinds", [3, 0])
+@pytest.mark.parametrize("BH,T,keeps", [(9, 66000, (4000,)), (10, 66000, (64, 66000 - 1)), (32, 16449, (900,)), (32, 33000, (2000,)),
+                                        (33, 8257, (900,)), (64, 16449, (1500,)), (64, 70000, (3000,)), (65, 8256, (700,)),
+                                        (65, 8257, (64, 65, 700, 8257))])
+def test_forms_by_heads(BH, T, keeps, kinds):
+    """At the edges of the rule that gives a head one CTA, a cluster of two, four or eight, or the one-CTA form by digits."""
+    test_index_for_index(BH, T, keeps, kinds)
