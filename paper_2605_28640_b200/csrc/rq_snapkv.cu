@@ -195,6 +195,8 @@ struct SnapMmaGeom {
     static constexpr int Q_BYTES = HALVES * HALF_BYTES;        // the window's queries, twice (128 rows)
     static constexpr int TILE_BYTES = HALVES * HALF_BYTES;     // 128 keys
     static constexpr int SMEM_BYTES = Q_BYTES + kMmaStages * TILE_BYTES + 1024;   // + room to align the base to 1024 bytes
+    // as much as leaves an SM no room for a third CTA
+    static constexpr int TWO_BYTES = SMEM_BYTES > 76 * 1024 ? SMEM_BYTES : 76 * 1024;
 };
 
 // 2^x for x <= 0 (and -inf): the hardware approximation, relative error about 2^-22
@@ -1207,9 +1209,9 @@ cudaError_t snap_scores_mma(const SnapArgs &a, cudaStream_t s)
     const int ntiles = (int)((a.len + kMmaKeys - 1) / kMmaKeys);
     if (ntiles <= kOnceTiles * kOnceCluster) return snap_scores_once<D>(a, tmap, qmap, ntiles, s);
     if (!ready[dev]) {
-        e = cudaFuncSetAttribute(snap_mma_kernel<D, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, G::SMEM_BYTES);
+        e = cudaFuncSetAttribute(snap_mma_kernel<D, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, G::TWO_BYTES);
         if (e != cudaSuccess) return e;
-        e = cudaFuncSetAttribute(snap_mma_kernel<D, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, G::SMEM_BYTES);
+        e = cudaFuncSetAttribute(snap_mma_kernel<D, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, G::TWO_BYTES);
         if (e != cudaSuccess) return e;
         ready[dev] = true;
     }
@@ -1229,7 +1231,10 @@ cudaError_t snap_scores_mma(const SnapArgs &a, cudaStream_t s)
     const int runs = (ntiles + tpc - 1) / tpc;
     const dim3 grid((unsigned)runs, (unsigned)BH);
     const float sl2 = a.scale * 1.4426950408889634f;
-    snap_mma_kernel<D, 1><<<grid, kMmaThreads, G::SMEM_BYTES, s>>>(tmap, qmap, a.page_cap, a.S, a.len, a.W, a.H, sl2,
+    // One round of CTAs: two on every SM.  Four of 64 channels would fit, and the second pass, which starts while the first one
+    // ends, would pile up on the SMs that are free first (32 heads x 64, 32768 positions: 121 -> 102 us a call).
+    const int smem = (int64_t)runs * BH <= slots ? G::TWO_BYTES : G::SMEM_BYTES;
+    snap_mma_kernel<D, 1><<<grid, kMmaThreads, smem, s>>>(tmap, qmap, a.page_cap, a.S, a.len, a.W, a.H, sl2,
                                                                  a.stats, nullptr, nullptr, ntiles, tpc, a.status);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
@@ -1248,7 +1253,7 @@ cudaError_t snap_scores_mma(const SnapArgs &a, cudaStream_t s)
     if (e != cudaSuccess) return e;
     cfg.gridDim = grid;
     cfg.blockDim = dim3(kMmaThreads);
-    cfg.dynamicSmemBytes = G::SMEM_BYTES;
+    cfg.dynamicSmemBytes = smem;
     return cudaLaunchKernelEx(&cfg, snap_mma_kernel<D, 2>, tmap, qmap, a.page_cap, a.S, a.len, a.W, a.H, sl2, (float2 *)nullptr,
                               (const float2 *)a.rowstat, a.imp, ntiles, tpc, a.status);
 }
