@@ -130,6 +130,7 @@ struct ScanPlan {
 
 // MODE 0: the scan proper.  MODE 1: the affine map of a time chunk only (no output), for the time-chunked form.
 // MODE 2: MODE 0 with one CTA per unit and the CTAs of a head as a cluster that keeps them within a tile of each other.
+// MODE 3: MODE 0 for a call inside one tile, with plain loads and without the ring, so that two CTAs share an SM.
 // Time chunks (chunks > 1; so few units that not even clusters fill the chip, and a long prompt): CTA x works on unit
 // x % units and the chunk_tiles tiles of chunk x / units.  First every chunk but the last is reduced to its map s -> A s + B
 // (MODE 1), a small kernel chains the maps into the state that enters every chunk, then every chunk runs the scan proper
@@ -137,7 +138,7 @@ struct ScanPlan {
 //   maps   [units][chunks][3][CG]   A, B of the keys, B of the values
 //   entry  [units][chunks][2][CG]   state entering a chunk (chunk 0: the cache's state)
 template <typename T, typename G, int D, int S, int MODE>
-__global__ void __launch_bounds__(NT) scan_kernel(ScanArgs a, const __grid_constant__ ScanMaps tm, ScanPlan plan, float *maps, const float *entry)
+__global__ void __launch_bounds__(NT, MODE == 3 ? 2 : 1) scan_kernel(ScanArgs a, const __grid_constant__ ScanMaps tm, ScanPlan plan, float *maps, const float *entry)
 {
     constexpr int NST = scan_stages<T, G>();
     constexpr int STAGE = scan_stage_bytes<T, G>();
@@ -160,7 +161,7 @@ __global__ void __launch_bounds__(NT) scan_kernel(ScanArgs a, const __grid_const
     __shared__ __align__(8) uint64_t full[NST], carried[2]; // a stage has landed; the state entering a tile has arrived
 
     cg::cluster_group cl = cg::this_cluster();
-    const int CL = MODE == 2 ? 1 : (int)cl.num_blocks(), cr = MODE == 2 ? 0 : (int)cl.block_rank();
+    const int CL = MODE >= 2 ? 1 : (int)cl.num_blocks(), cr = MODE >= 2 ? 0 : (int)cl.block_rank();
     const int unit = blockIdx.x / CL % plan.units, chunk = blockIdx.x / CL / plan.units, chunks = plan.chunks;
     const int64_t tile0 = plan.tile0 + (int64_t)chunk * plan.chunk_tiles;
     const int ntiles = min(plan.chunk_tiles, plan.ntiles - chunk * plan.chunk_tiles);
@@ -182,7 +183,7 @@ __global__ void __launch_bounds__(NT) scan_kernel(ScanArgs a, const __grid_const
     const int row0 = (2 * warp + half) * RT;     // first row of this thread's run
 
     // tile i of the unit (chunk): does it come through the tensor maps (rows past the prompt's end as zeros), and is it full?
-    auto by_map = [&](int i) { return plan.tma && (tile0 + i) * TT >= a.len0; };
+    auto by_map = [&](int i) { return MODE != 3 && plan.tma && (tile0 + i) * TT >= a.len0; };
     auto full_tile = [&](int i) { return by_map(i) && (tile0 + i + 1) * TT <= end; };
     const uint64_t once = l2_evict_first_policy();
     // start the copies of this CTA's j-th tile.  The whole first warp.
@@ -209,7 +210,7 @@ __global__ void __launch_bounds__(NT) scan_kernel(ScanArgs a, const __grid_const
         __syncwarp();
     };
     bool ok = true;
-    if (tid == 0) {
+    if (MODE != 3 && tid == 0) {
         for (int s = 0; s < NST; ++s) mbar_init(&full[s], 1);
         mbar_init(&carried[0], 1);
         mbar_init(&carried[1], 1);
@@ -217,8 +218,8 @@ __global__ void __launch_bounds__(NT) scan_kernel(ScanArgs a, const __grid_const
     }
     grid_dependency_wait();                      // earlier kernels may still write what is read here, or read what is written
     grid_launch_dependents();
-    __syncthreads();
-    if (warp == 0) {
+    if (MODE != 3) __syncthreads();
+    if (MODE != 3 && warp == 0) {
         for (int j = 0; j < NST && j < mine; ++j) issue(j);
         if (CL > 1 && lane == 0) {
             // the first tile's state is the cache's, every other one comes as 2 * CG floats from the CTA before
@@ -227,11 +228,15 @@ __global__ void __launch_bounds__(NT) scan_kernel(ScanArgs a, const __grid_const
             mbar_arrive_expect_tx(&carried[1], 2 * CG * sizeof(float));
         }
     }
+    float first_k = 0.0f, first_v = 0.0f;        // MODE 3: the state, on its way while the tile is
     if (tid < CG && cr == 0) {                   // the state the (chunk of the) sequence starts from
         if (MODE == 1) {
             carry[0][0][tid] = 0.0f;
             carry[0][1][tid] = 0.0f;
             carry_a[0][tid] = 1.0f;
+        } else if (MODE == 3) {
+            first_k = a.state[(int64_t)bh * 2 * D + c0 + tid];
+            first_v = a.state[(int64_t)bh * 2 * D + D + c0 + tid];
         } else if (chunk == 0) {
             carry[0][0][tid] = a.state[(int64_t)bh * 2 * D + c0 + tid];
             carry[0][1][tid] = a.state[(int64_t)bh * 2 * D + D + c0 + tid];
@@ -287,6 +292,10 @@ __global__ void __launch_bounds__(NT) scan_kernel(ScanArgs a, const __grid_const
 
         // ---- pass 1: this thread's run as a map from a zero state (identity outside the new range)
         float2 g2[RT], k2[RT], v2[RT];                           // g, (1-g) k, (1-g) v of the two channels
+        float2 A2 = make_float2(1.0f, 1.0f), Bk2 = make_float2(0.0f, 0.0f), Bv2 = make_float2(0.0f, 0.0f);
+        // (a warp without new rows leaves its part of a short prompt out; elsewhere the branches cost more than they save)
+        const bool idle = MODE == 3 && (2 * warp * RT >= hi || 2 * (warp + 1) * RT <= lo);
+        if (!idle) {
         if (MAP || by_map(i)) {
             ok = ok && mbar_wait(&full[j % NST], (uint32_t)((j / NST) & 1));
             // (2-byte elements: the two halves of a warp, eight rows of 64 bytes apart, share banks: two reads instead of one)
@@ -310,7 +319,6 @@ __global__ void __launch_bounds__(NT) scan_kernel(ScanArgs a, const __grid_const
                 v2[r] = in ? load2(vp + src) : make_float2(0.0f, 0.0f);
             }
         }
-        float2 A2 = make_float2(1.0f, 1.0f), Bk2 = make_float2(0.0f, 0.0f), Bv2 = make_float2(0.0f, 0.0f);
 #pragma unroll
         for (int r = 0; r < RT; ++r) {
             const float2 o2 = fma2(g2[r], make_float2(-1.0f, -1.0f), make_float2(1.0f, 1.0f));   // 1 - g
@@ -319,6 +327,11 @@ __global__ void __launch_bounds__(NT) scan_kernel(ScanArgs a, const __grid_const
             A2 = mul2(A2, g2[r]);
             Bk2 = fma2(g2[r], Bk2, k2[r]);
             Bv2 = fma2(g2[r], Bv2, v2[r]);
+        }
+        }
+        if (MODE == 3 && tid < CG) {
+            carry[0][0][tid] = first_k;
+            carry[0][1][tid] = first_v;
         }
         // the map of the warp's first run, for the second run; the second run's lanes publish the warp's map
         const float2 LA = make_float2(__shfl_sync(FULLMASK, A2.x, hl), __shfl_sync(FULLMASK, A2.y, hl));
@@ -333,7 +346,7 @@ __global__ void __launch_bounds__(NT) scan_kernel(ScanArgs a, const __grid_const
         if (BY_STAGE) tma_store_wait_read();                     // the warp's rows of the tile before have left their stage
         __syncthreads();                                         // the maps are there
         // the stage of the tile before (of this tile, if nothing goes back into it) is free
-        if (warp == 0 && (!BY_STAGE || j >= 1) && j - BY_STAGE + NST < mine) issue(j - BY_STAGE + NST);
+        if (MODE != 3 && warp == 0 && (!BY_STAGE || j >= 1) && j - BY_STAGE + NST < mine) issue(j - BY_STAGE + NST);
         if (WPP > 1 && MODE != 1 && j > 0) wide_bounds(j - 1);
 
         // ---- scan of the 16 warp maps of channels 2 warp and 2 warp + 1 (one per half-warp) by 16 lanes
@@ -394,6 +407,7 @@ __global__ void __launch_bounds__(NT) scan_kernel(ScanArgs a, const __grid_const
         const int64_t pos = tile_start + row0;                   // a run lies inside one page
         T *dst = kv + (pos / S * 2 * S + pos % S) * D;
         float mn0 = INFINITY, mn1 = INFINITY, mx0 = -INFINITY, mx1 = -INFINITY;
+        if (!idle || (2 * warp * RT >= hi && 2 * warp * RT < fill_hi)) {
 #pragma unroll
         for (int r = 0; r < RT; ++r) {
             if (MAP || (row0 + r >= lo && row0 + r < hi)) {
@@ -413,6 +427,7 @@ __global__ void __launch_bounds__(NT) scan_kernel(ScanArgs a, const __grid_const
                 store2_cs(dst + r * D, make_float2(0.0f, 0.0f));
                 store2_cs(dst + (S + r) * D, make_float2(0.0f, 0.0f));
             }
+        }
         }
         if constexpr (MAP && BY_STAGE) {
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -445,7 +460,7 @@ __global__ void __launch_bounds__(NT) scan_kernel(ScanArgs a, const __grid_const
 #pragma unroll 1
     while (j < mine) {
 #pragma unroll 1
-        for (; j < mine && cr + j * CL >= full_from && cr + j * CL < full_to; ++j) {
+        for (; MODE != 3 && j < mine && cr + j * CL >= full_from && cr + j * CL < full_to; ++j) {
             if (MODE == 2) asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
             tile(BoolTag<true>(), j);
             if (MODE == 2) asm volatile("barrier.cluster.wait.aligned;" ::: "memory");
@@ -477,7 +492,7 @@ __global__ void __launch_bounds__(NT) scan_kernel(ScanArgs a, const __grid_const
     }
     if (!ok) {                                   // a wait ran out: no copy may still be on its way when the CTA exits
         atomicCAS(a.status, RQ_OK, RQ_ERR_TIMEOUT);
-        if (tid == 0)
+        if (MODE != 3 && tid == 0)
             for (int j = max(0, mine - NST); j < mine; ++j) mbar_wait(&full[j % NST], (uint32_t)((j / NST) & 1));
         __syncwarp();
     }
@@ -545,8 +560,14 @@ cudaError_t run(const ScanArgs &a, cudaStream_t s)
     p.ntiles = (int)(t1 - t0);
     p.units = (int)units;
     alignas(64) ScanMaps tm;
-    // tensor maps where there is a full tile and the strides can be described (a stride of zero cannot)
-    p.tma = a.T >= TT && a.T < ((int64_t)1 << 31) &&
+    const int sms = sm_count();
+    // A call inside one tile with more units than SMs: its CTAs follow one another, and what counts is how soon a CTA is done.
+    // 256 heads x 128, bf16, 16 / 100 / 255 tokens: one CTA per SM and tensor maps 25.3 / 26.6 / 30.8 us, two CTAs and plain
+    // loads 17.8 / 21.4 / 30.1 (copies of 16 bytes by all threads, before there were tensor maps, 22.0 / 23.9 / 31.9).  With
+    // fewer units the tensor maps win: 32 heads, 16 / 255 tokens 4.4 / 6.2 against 4.8 / 7.5.
+    const bool brief = p.ntiles == 1 && units > sms;
+    // tensor maps where the strides can be described (a stride of zero cannot)
+    p.tma = !brief && a.T < ((int64_t)1 << 31) &&
             prompt_tensor_map(&tm.k, a.k, sizeof(T), D, a.H, a.T, a.B, a.sh, a.st, a.sb, CG, TT) == cudaSuccess &&
             prompt_tensor_map(&tm.v, a.v, sizeof(T), D, a.H, a.T, a.B, a.sh, a.st, a.sb, CG, TT) == cudaSuccess &&
             prompt_tensor_map(&tm.g, a.g, sizeof(G), D, a.H, a.T, a.B, a.sh, a.st, a.sb, CG, TT) == cudaSuccess &&
@@ -556,7 +577,6 @@ cudaError_t run(const ScanArgs &a, cudaStream_t s)
     // by its hops of about 0.55 us, 290).  Otherwise as many CTAs per unit as leave every SM at most one, with at least four
     // tiles each (8 heads, 131072 tokens: 469 -> 283 us; 16 heads: 913 -> 543; clusters of eight find too little room: 386 for
     // the 4 heads).
-    const int sms = sm_count();
     int cl = 1, chunks = 1;
     if (a.chunk_scratch && 2 * units <= sms) {
         chunks = sms / p.units;
@@ -579,7 +599,9 @@ cudaError_t run(const ScanArgs &a, cudaStream_t s)
         if (e != cudaSuccess) return e;
         scan_chain_kernel<<<(unsigned)units, 2 * CG, 0, s>>>(a.state, D, D / CG, p.chunks, maps, entry);
     }
-    e = abreast ? start<T, G, D, S, 2>(a, tm, p, 1, maps, entry, DSM, s) : start<T, G, D, S, 0>(a, tm, p, cl, maps, entry, DSM, s);
+    e = brief     ? start<T, G, D, S, 3>(a, tm, p, 1, maps, entry, 0, s)
+        : abreast ? start<T, G, D, S, 2>(a, tm, p, 1, maps, entry, DSM, s)
+                  : start<T, G, D, S, 0>(a, tm, p, cl, maps, entry, DSM, s);
     return e != cudaSuccess ? e : cudaGetLastError();
 }
 

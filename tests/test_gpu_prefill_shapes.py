@@ -80,6 +80,18 @@ def test_states_cache_and_bounds(B, H, D, S, T, cuts, dtype, gdtype, layout):
         assert torch.equal(c.meta_view()[:, :, p, 0], rows.amin(2)) and torch.equal(c.meta_view()[:, :, p, 1], rows.amax(2))
 
 
+@pytest.mark.parametrize("layout", ["bthd", "shared"])
+@pytest.mark.parametrize("B,H,D,S,T,cuts,dtype,gdtype", [
+    (1, 40, 128, 16, 1, [], BF, BF), (2, 38, 64, 64, 16, [], BF, F32), (1, 38, 128, 64, 17, [16], F32, F32), (4, 20, 64, 16, 100, [7], BF, BF),
+    (1, 75, 64, 16, 255, [3, 17, 200], F32, BF), (1, 37, 128, 16, 256, [], BF, BF), (1, 40, 128, 64, 256, [1, 63, 64, 130], BF, BF),
+    (1, 40, 128, 64, 300, [250, 260], BF, F32), (1, 5, 128, 16, 1, [], BF, BF), (2, 3, 64, 64, 17, [], F32, F32),
+    (1, 5, 128, 64, 130, [64], BF, F32), (1, 6, 64, 16, 290, [256, 257], F32, BF)])
+def test_short_calls(B, H, D, S, T, cuts, dtype, gdtype, layout):
+    """Calls inside one tile, with more units than SMs (two CTAs per SM, plain loads) and with fewer (tensor maps longer than
+    the prompt)."""
+    test_states_cache_and_bounds(B, H, D, S, T, cuts, dtype, gdtype, layout)
+
+
 @pytest.mark.parametrize("H,D,S,T,dtype,gdtype", [(20, 128, 16, 16384, BF, BF), (32, 128, 64, 16500, BF, F32), (40, 64, 16, 16385, F32, BF),
                                                   (65, 64, 64, 16639, BF, BF)])
 def test_units_abreast(H, D, S, T, dtype, gdtype):
