@@ -145,7 +145,8 @@ RQ_API int rq_cache_reset(rq_cache *cache, void *stream);
  * The same call on the same inputs gives the same bits.  How a prompt is cut into calls, and how the
  * library cuts a very long prompt of a few heads into time chunks that run side by side, changes the
  * order of the fp32 operations: states agree within rounding (a few 1e-7 relative), not bit for bit.
- * Strides of zero and others that a tensor map cannot describe are taken, but read more slowly.
+ * A stride of zero shares the numbers: stride_h = 0 for all heads, stride_b = 0 for all batch items, stride_t = 0 for all
+ * positions (only the last one is read more slowly than a tensor of its own, by a tenth to a quarter).
  * Errors: INVALID_ARG (NULL, T < 0, misaligned), CAPACITY (len + T exceeds
  * capacity_tokens; nothing is enqueued), CUDA.  T == 0 is a no-op. */
 RQ_API int rq_build_cache(rq_cache *cache, const void *k, const void *v, const void *g,

@@ -191,19 +191,19 @@ __global__ void __launch_bounds__(NT, MODE == 3 ? 2 : 1) scan_kernel(ScanArgs a,
         const int i = cr + j * CL, st = j % NST;
         if (by_map(i)) {
             unsigned char *dst = dsm + (size_t)st * STAGE;
-            const int tok = (int)((tile0 + i) * TT - a.len0);
+            const int tok = (int)((tile0 + i) * TT - a.len0), mh = a.sh ? h : 0, mb = a.sb ? b : 0;
             mbar_expect_warp(&full[st], STAGE);
             // (rows of 128 bytes are whole lines that nobody else reads; of 64 bytes, half a line whose other half another CTA
             // reads at about the same time)
             if (sizeof(T) == 4) {
-                tma_load_4d_hint(dst, &tm.k, c0, h, tok, b, &full[st], once);
-                tma_load_4d_hint(dst + OFF_V, &tm.v, c0, h, tok, b, &full[st], once);
+                tma_load_4d_hint(dst, &tm.k, c0, mh, tok, mb, &full[st], once);
+                tma_load_4d_hint(dst + OFF_V, &tm.v, c0, mh, tok, mb, &full[st], once);
             } else {
-                tma_load_4d(dst, &tm.k, c0, h, tok, b, &full[st]);
-                tma_load_4d(dst + OFF_V, &tm.v, c0, h, tok, b, &full[st]);
+                tma_load_4d(dst, &tm.k, c0, mh, tok, mb, &full[st]);
+                tma_load_4d(dst + OFF_V, &tm.v, c0, mh, tok, mb, &full[st]);
             }
-            if (sizeof(G) == 4) tma_load_4d_hint(dst + OFF_G, &tm.g, c0, h, tok, b, &full[st], once);
-            else tma_load_4d(dst + OFF_G, &tm.g, c0, h, tok, b, &full[st]);
+            if (sizeof(G) == 4) tma_load_4d_hint(dst + OFF_G, &tm.g, c0, mh, tok, mb, &full[st], once);
+            else tma_load_4d(dst + OFF_G, &tm.g, c0, mh, tok, mb, &full[st]);
         } else if (lane == 0) {
             mbar_arrive(&full[st]);
         }
@@ -566,7 +566,7 @@ cudaError_t run(const ScanArgs &a, cudaStream_t s)
     // loads 17.8 / 21.4 / 30.1 (copies of 16 bytes by all threads, before there were tensor maps, 22.0 / 23.9 / 31.9).  With
     // fewer units the tensor maps win: 32 heads, 16 / 255 tokens 4.4 / 6.2 against 4.8 / 7.5.
     const bool brief = p.ntiles == 1 && units > sms;
-    // tensor maps where the strides can be described (a stride of zero cannot)
+    // tensor maps where the strides can be described (positions that are all the same, a stride of zero, cannot)
     p.tma = !brief && a.T < ((int64_t)1 << 31) &&
             prompt_tensor_map(&tm.k, a.k, sizeof(T), D, a.H, a.T, a.B, a.sh, a.st, a.sb, CG, TT) == cudaSuccess &&
             prompt_tensor_map(&tm.v, a.v, sizeof(T), D, a.H, a.T, a.B, a.sh, a.st, a.sb, CG, TT) == cudaSuccess &&

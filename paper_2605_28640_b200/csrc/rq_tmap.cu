@@ -73,8 +73,11 @@ cudaError_t prompt_tensor_map(CUtensorMap *out, const void *x, int es, int D, in
 {
     const TensorMapEncodeTiled encode = tensor_map_encoder();
     if (!encode) return cudaErrorNotSupported;
-    // (a dimension of one element has no stride of its own)
-    const int64_t bytes[3] = {(H > 1 ? sh : D) * es, st * es, (B > 1 ? sb : D) * es};
+    // heads or batch items that share their numbers (a stride of zero) are one element of that dimension; a dimension of one
+    // element has no stride of its own
+    if (sh == 0) H = 1;
+    if (sb == 0) B = 1;
+    const int64_t bytes[3] = {(H > 1 ? sh : D) * es, (T > 1 ? st : D) * es, (B > 1 ? sb : D) * es};
     for (int i = 0; i < 3; ++i)
         if (bytes[i] <= 0 || bytes[i] % 16 != 0 || bytes[i] >= ((int64_t)1 << 40)) return cudaErrorInvalidValue;
     const cuuint64_t dims[4] = {(cuuint64_t)D, (cuuint64_t)H, (cuuint64_t)T, (cuuint64_t)B};

@@ -15,7 +15,7 @@ cudaError_t cache_tensor_map(CUtensorMap *out, const void *kv, int D, int S, int
 
 // A prompt's keys, values or gates, element (b, t, h, d) at b * sb + t * st + h * sh + d (strides in elements of `es` bytes),
 // as a rank-4 tensor (channel, head, position, batch item); box = `channels` channels x one head x `positions` positions,
-// dense rows.  Fails where the strides cannot be described.
+// dense rows.  With sh = 0 the tensor has one head, with sb = 0 one batch item.  Fails where the strides cannot be described.
 cudaError_t prompt_tensor_map(CUtensorMap *out, const void *x, int es, int D, int H, int64_t T, int B, int64_t sh, int64_t st, int64_t sb,
                               int channels, int positions);
 
