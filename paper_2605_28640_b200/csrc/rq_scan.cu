@@ -130,6 +130,7 @@ struct ScanPlan {
 
 // MODE 0: the scan proper.  MODE 1: the affine map of a time chunk only (no output), for the time-chunked form.
 // MODE 2: MODE 0 with one CTA per unit and the CTAs of a head as a cluster that keeps them within a tile of each other.
+// MODE 4: MODE 0 where heads or batch items may share their numbers.
 // MODE 3: MODE 0 for a call inside one tile, with plain loads and without the ring, so that two CTAs share an SM.
 // Time chunks (chunks > 1; so few units that not even clusters fill the chip, and a long prompt): CTA x works on unit
 // x % units and the chunk_tiles tiles of chunk x / units.  First every chunk but the last is reduced to its map s -> A s + B
@@ -161,7 +162,7 @@ __global__ void __launch_bounds__(NT, MODE == 3 ? 2 : 1) scan_kernel(ScanArgs a,
     __shared__ __align__(8) uint64_t full[NST], carried[2]; // a stage has landed; the state entering a tile has arrived
 
     cg::cluster_group cl = cg::this_cluster();
-    const int CL = MODE >= 2 ? 1 : (int)cl.num_blocks(), cr = MODE >= 2 ? 0 : (int)cl.block_rank();
+    const int CL = MODE == 2 || MODE == 3 ? 1 : (int)cl.num_blocks(), cr = MODE == 2 || MODE == 3 ? 0 : (int)cl.block_rank();
     const int unit = blockIdx.x / CL % plan.units, chunk = blockIdx.x / CL / plan.units, chunks = plan.chunks;
     const int64_t tile0 = plan.tile0 + (int64_t)chunk * plan.chunk_tiles;
     const int ntiles = min(plan.chunk_tiles, plan.ntiles - chunk * plan.chunk_tiles);
@@ -173,7 +174,10 @@ __global__ void __launch_bounds__(NT, MODE == 3 ? 2 : 1) scan_kernel(ScanArgs a,
     const int ch2 = 2 * hl;                      // first of this lane's two channels inside the group
     constexpr int GPH = D / CG;                  // channel groups per head
     const int bh = unit / GPH, c0 = (unit % GPH) * CG;
-    const int b = bh / a.H, h = bh % a.H;
+    // coordinates in the inputs' tensor maps.  (Chosen only where numbers may be shared: the choice leaves the uniform
+    // registers, and each copy is started later: 32 heads x 128, 50000 tokens 348 -> 365 us)
+    constexpr bool SHARED = MODE == 1 || MODE == 4;
+    const int b = SHARED && a.sb == 0 ? 0 : bh / a.H, h = SHARED && a.sh == 0 ? 0 : bh % a.H;
     const int64_t end = a.len0 + a.T;
     const int64_t tail_end = (end + S - 1) / S * S;   // end of the last touched page
     const int64_t in_base = (int64_t)b * a.sb + (int64_t)h * a.sh + c0 + ch2;
@@ -191,19 +195,19 @@ __global__ void __launch_bounds__(NT, MODE == 3 ? 2 : 1) scan_kernel(ScanArgs a,
         const int i = cr + j * CL, st = j % NST;
         if (by_map(i)) {
             unsigned char *dst = dsm + (size_t)st * STAGE;
-            const int tok = (int)((tile0 + i) * TT - a.len0), mh = a.sh ? h : 0, mb = a.sb ? b : 0;
+            const int tok = (int)((tile0 + i) * TT - a.len0);
             mbar_expect_warp(&full[st], STAGE);
             // (rows of 128 bytes are whole lines that nobody else reads; of 64 bytes, half a line whose other half another CTA
             // reads at about the same time)
             if (sizeof(T) == 4) {
-                tma_load_4d_hint(dst, &tm.k, c0, mh, tok, mb, &full[st], once);
-                tma_load_4d_hint(dst + OFF_V, &tm.v, c0, mh, tok, mb, &full[st], once);
+                tma_load_4d_hint(dst, &tm.k, c0, h, tok, b, &full[st], once);
+                tma_load_4d_hint(dst + OFF_V, &tm.v, c0, h, tok, b, &full[st], once);
             } else {
-                tma_load_4d(dst, &tm.k, c0, mh, tok, mb, &full[st]);
-                tma_load_4d(dst + OFF_V, &tm.v, c0, mh, tok, mb, &full[st]);
+                tma_load_4d(dst, &tm.k, c0, h, tok, b, &full[st]);
+                tma_load_4d(dst + OFF_V, &tm.v, c0, h, tok, b, &full[st]);
             }
-            if (sizeof(G) == 4) tma_load_4d_hint(dst + OFF_G, &tm.g, c0, mh, tok, mb, &full[st], once);
-            else tma_load_4d(dst + OFF_G, &tm.g, c0, mh, tok, mb, &full[st]);
+            if (sizeof(G) == 4) tma_load_4d_hint(dst + OFF_G, &tm.g, c0, h, tok, b, &full[st], once);
+            else tma_load_4d(dst + OFF_G, &tm.g, c0, h, tok, b, &full[st]);
         } else if (lane == 0) {
             mbar_arrive(&full[st]);
         }
@@ -566,6 +570,7 @@ cudaError_t run(const ScanArgs &a, cudaStream_t s)
     // loads 17.8 / 21.4 / 30.1 (copies of 16 bytes by all threads, before there were tensor maps, 22.0 / 23.9 / 31.9).  With
     // fewer units the tensor maps win: 32 heads, 16 / 255 tokens 4.4 / 6.2 against 4.8 / 7.5.
     const bool brief = p.ntiles == 1 && units > sms;
+    const bool shared = !brief && ((a.H > 1 && a.sh == 0) || (a.B > 1 && a.sb == 0));
     // tensor maps where the strides can be described (positions that are all the same, a stride of zero, cannot)
     p.tma = !brief && a.T < ((int64_t)1 << 31) &&
             prompt_tensor_map(&tm.k, a.k, sizeof(T), D, a.H, a.T, a.B, a.sh, a.st, a.sb, CG, TT) == cudaSuccess &&
@@ -600,6 +605,7 @@ cudaError_t run(const ScanArgs &a, cudaStream_t s)
         scan_chain_kernel<<<(unsigned)units, 2 * CG, 0, s>>>(a.state, D, D / CG, p.chunks, maps, entry);
     }
     e = brief     ? start<T, G, D, S, 3>(a, tm, p, 1, maps, entry, 0, s)
+        : shared  ? start<T, G, D, S, 4>(a, tm, p, cl, maps, entry, DSM, s)
         : abreast ? start<T, G, D, S, 2>(a, tm, p, 1, maps, entry, DSM, s)
                   : start<T, G, D, S, 0>(a, tm, p, cl, maps, entry, DSM, s);
     return e != cudaSuccess ? e : cudaGetLastError();
