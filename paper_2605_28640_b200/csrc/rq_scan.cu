@@ -138,15 +138,14 @@ struct ScanPlan {
 // from its own entry state.  The inputs of all chunks but the last are read twice.  (Chunks and clusters exclude each other.)
 //   maps   [units][chunks][3][CG]   A, B of the keys, B of the values
 //   entry  [units][chunks][2][CG]   state entering a chunk (chunk 0: the cache's state)
-template <typename T, typename G, int D, int S, int MODE>
+template <typename T, typename G, int D, int S, int MODE, bool STAGED>
 __global__ void __launch_bounds__(NT, MODE == 3 ? 2 : 1) scan_kernel(ScanArgs a, const __grid_constant__ ScanMaps tm, ScanPlan plan, float *maps, const float *entry)
 {
     constexpr int NST = scan_stages<T, G>();
     constexpr int STAGE = scan_stage_bytes<T, G>();
     constexpr int OFF_V = TT * CG * (int)sizeof(T), OFF_G = 2 * OFF_V;
-    // 2-byte storage: a warp's rows go back into their stage and out with tensor-map stores (32 heads x 128, 131072 tokens:
-    // 973 -> 956 us); 4-byte storage: straight from registers (12 heads, 20000 tokens: 120 us, through the stage 138)
-    constexpr bool BY_STAGE = sizeof(T) == 2;
+    // a warp's rows go back into their stage and out with tensor-map stores, or out straight from registers (rule in run())
+    constexpr bool BY_STAGE = STAGED;
     constexpr int WPP = S / (2 * RT);                                          // warps that share a page
     constexpr unsigned FULLMASK = 0xffffffffu;
     static_assert(D % CG == 0, "a head is a whole number of channel groups");
@@ -198,15 +197,17 @@ __global__ void __launch_bounds__(NT, MODE == 3 ? 2 : 1) scan_kernel(ScanArgs a,
             const int tok = (int)((tile0 + i) * TT - a.len0);
             mbar_expect_warp(&full[st], STAGE);
             // (rows of 128 bytes are whole lines that nobody else reads; of 64 bytes, half a line whose other half another CTA
-            // reads at about the same time)
-            if (sizeof(T) == 4) {
+            // reads at about the same time.  fp32 rows that go out by their stage do better without: 32 heads x 128, 131072
+            // tokens 1861 -> 1780 us)
+            constexpr bool HINT_KV = sizeof(T) == 4 && !STAGED, HINT_G = sizeof(G) == 4 && (sizeof(T) == 2 || !STAGED);
+            if (HINT_KV) {
                 tma_load_4d_hint(dst, &tm.k, c0, h, tok, b, &full[st], once);
                 tma_load_4d_hint(dst + OFF_V, &tm.v, c0, h, tok, b, &full[st], once);
             } else {
                 tma_load_4d(dst, &tm.k, c0, h, tok, b, &full[st]);
                 tma_load_4d(dst + OFF_V, &tm.v, c0, h, tok, b, &full[st]);
             }
-            if (sizeof(G) == 4) tma_load_4d_hint(dst + OFF_G, &tm.g, c0, h, tok, b, &full[st], once);
+            if (HINT_G) tma_load_4d_hint(dst + OFF_G, &tm.g, c0, h, tok, b, &full[st], once);
             else tma_load_4d(dst + OFF_G, &tm.g, c0, h, tok, b, &full[st]);
         } else if (lane == 0) {
             mbar_arrive(&full[st]);
@@ -516,7 +517,7 @@ __global__ void scan_chain_kernel(const float *state, int D, int gph, int chunks
     }
 }
 
-template <typename T, typename G, int D, int S, int MODE>
+template <typename T, typename G, int D, int S, int MODE, bool STAGED>
 cudaError_t start(const ScanArgs &a, const ScanMaps &tm, const ScanPlan &p, int cl, float *maps, const float *entry, int smem, cudaStream_t s)
 {
     static bool ready[64];                                       // (set up form by form: the first use of a kernel loads it)
@@ -525,7 +526,7 @@ cudaError_t start(const ScanArgs &a, const ScanMaps &tm, const ScanPlan &p, int 
     if (e != cudaSuccess) return e;
     if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
     if (!ready[dev]) {
-        e = cudaFuncSetAttribute(scan_kernel<T, G, D, S, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        e = cudaFuncSetAttribute(scan_kernel<T, G, D, S, MODE, STAGED>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
         if (e != cudaSuccess) return e;
         ready[dev] = true;
     }
@@ -544,7 +545,7 @@ cudaError_t start(const ScanArgs &a, const ScanMaps &tm, const ScanPlan &p, int 
     const bool clusters = MODE == 2 || cl > 1;
     cfg.attrs = clusters ? at : at + 1;
     cfg.numAttrs = clusters ? 2 : 1;
-    return cudaLaunchKernelEx(&cfg, scan_kernel<T, G, D, S, MODE>, a, tm, p, maps, entry);
+    return cudaLaunchKernelEx(&cfg, scan_kernel<T, G, D, S, MODE, STAGED>, a, tm, p, maps, entry);
 }
 
 template <typename T, typename G, int D, int S>
@@ -598,16 +599,28 @@ cudaError_t run(const ScanArgs &a, cudaStream_t s)
     const bool abreast = cl == 1 && chunks == 1 && p.ntiles >= 64 && 9 * units <= 8 * sms;
     p.chunk_tiles = (p.ntiles + chunks - 1) / chunks;
     p.chunks = (p.ntiles + p.chunk_tiles - 1) / p.chunk_tiles;
+    // Rows of 2-byte elements go out by their stage (32 heads x 128, 131072 tokens: 973 -> 956 us).  Rows of 4 bytes, in stages of
+    // which only two find room, do so where enough CTAs with enough tiles wait for DRAM, which then has whole pages written
+    // side by side; elsewhere the refill would wait for them.  us, straight from registers / by their stage: fp32 gates, 32
+    // heads x 128, 50000 tokens 777 / 670 (by 16-byte pieces through shared memory, before, 675), 8 heads 201 / 172, 24 heads
+    // 537 / 578, 32 heads of 2000 tokens 31 / 33; bf16 gates, 32 heads, 60000 tokens 0.86 / 0.93 of the speed before, 64 heads
+    // of 64 pages 1.02 / 0.98.
+    const int64_t ctas = units * cl * p.chunks;
+    const bool staged = p.ntiles >= 12 * cl * p.chunks && 5 * ctas >= 4 * sms && (sizeof(G) == 4 || ctas <= sms);
     float *maps = a.chunk_scratch, *entry = a.chunk_scratch ? a.chunk_scratch + (size_t)units * p.chunks * 3 * CG : nullptr;
     if (p.chunks > 1) {
-        e = start<T, G, D, S, 1>(a, tm, p, 1, maps, entry, DSM, s);
+        e = start<T, G, D, S, 1, sizeof(T) == 2>(a, tm, p, 1, maps, entry, DSM, s);
         if (e != cudaSuccess) return e;
         scan_chain_kernel<<<(unsigned)units, 2 * CG, 0, s>>>(a.state, D, D / CG, p.chunks, maps, entry);
     }
-    e = brief     ? start<T, G, D, S, 3>(a, tm, p, 1, maps, entry, 0, s)
-        : shared  ? start<T, G, D, S, 4>(a, tm, p, cl, maps, entry, DSM, s)
-        : abreast ? start<T, G, D, S, 2>(a, tm, p, 1, maps, entry, DSM, s)
-                  : start<T, G, D, S, 0>(a, tm, p, cl, maps, entry, DSM, s);
+    auto go = [&](auto staged) {
+        constexpr bool ST = decltype(staged)::value;
+        return abreast ? start<T, G, D, S, 2, ST>(a, tm, p, 1, maps, entry, DSM, s) : start<T, G, D, S, 0, ST>(a, tm, p, cl, maps, entry, DSM, s);
+    };
+    if (brief) e = start<T, G, D, S, 3, false>(a, tm, p, 1, maps, entry, 0, s);
+    else if (shared) e = start<T, G, D, S, 4, sizeof(T) == 2>(a, tm, p, cl, maps, entry, DSM, s);
+    else if constexpr (sizeof(T) == 2) e = go(BoolTag<true>());
+    else e = staged ? go(BoolTag<true>()) : go(BoolTag<false>());
     return e != cudaSuccess ? e : cudaGetLastError();
 }
 
