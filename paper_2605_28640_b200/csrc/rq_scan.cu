@@ -137,7 +137,7 @@ struct ScanPlan {
 // (MODE 1), a small kernel chains the maps into the state that enters every chunk, then every chunk runs the scan proper
 // from its own entry state.  The inputs of all chunks but the last are read twice.  (Chunks and clusters exclude each other.)
 //   maps   [units][chunks][3][CG]   A, B of the keys, B of the values
-//   entry  [units][chunks][2][CG]   state entering a chunk (chunk 0: the cache's state)
+//   entry  [units][chunks][2][CG]   state entering a chunk
 template <typename T, typename G, int D, int S, int MODE, bool STAGED>
 __global__ void __launch_bounds__(NT, MODE == 3 ? 2 : 1) scan_kernel(ScanArgs a, const __grid_constant__ ScanMaps tm, ScanPlan plan, float *maps, const float *entry)
 {
@@ -242,10 +242,10 @@ __global__ void __launch_bounds__(NT, MODE == 3 ? 2 : 1) scan_kernel(ScanArgs a,
         } else if (MODE == 3) {
             first_k = a.state[(int64_t)bh * 2 * D + c0 + tid];
             first_v = a.state[(int64_t)bh * 2 * D + D + c0 + tid];
-        } else if (chunk == 0) {
+        } else if (chunks == 1) {
             carry[0][0][tid] = a.state[(int64_t)bh * 2 * D + c0 + tid];
             carry[0][1][tid] = a.state[(int64_t)bh * 2 * D + D + c0 + tid];
-        } else {
+        } else {                                 // (of the first chunk, too: the CTA of the last one overwrites the cache's state)
             const float *e = entry + ((int64_t)unit * chunks + chunk) * 2 * CG;
             carry[0][0][tid] = e[tid];
             carry[0][1][tid] = e[CG + tid];
@@ -510,6 +510,7 @@ __global__ void scan_chain_kernel(const float *state, int D, int gph, int chunks
     const int unit = blockIdx.x, kv = threadIdx.x / CG, ch = threadIdx.x % CG;
     const int bh = unit / gph, c0 = (unit % gph) * CG;
     float s = state[(int64_t)bh * 2 * D + kv * D + c0 + ch];
+    entry[((int64_t)unit * chunks * 2 + kv) * CG + ch] = s;
     for (int c = 0; c + 1 < chunks; ++c) {
         const float *mp = maps + ((int64_t)unit * chunks + c) * 3 * CG;
         s = fmaf(mp[ch], s, mp[(1 + kv) * CG + ch]);
