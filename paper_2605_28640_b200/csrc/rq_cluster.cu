@@ -466,18 +466,27 @@ int cluster_step_size(int BH, int64_t pages, int sms)
     return cl;
 }
 
-// Below 1024 pages one launch wins on every shape as long as the CTAs have little to read each (device time, 32 heads x 128,
-// separate launches / cluster, us: 4090 tokens in pages of 64, 16 kept 16.9 / 10.2; 1000 tokens 16.1 / 8.5; 8000 tokens, 125
-// of 500 pages 23.1 / 15.7; 4 heads, 1000 tokens 19.0 / 6.8; 256 heads, 8000 tokens, 31 of 500 47.6 / 33.4), and up to 2048
-// where the heads alone fill the chip (256 heads, 32000 tokens, 125 kept 107 / 102, 500 kept 224 / 215; 64 to 128 heads of
-// 2000 pages: 0.95 to 1.03).  Few heads with much to read leave most of the chip idle, and the separate kernels, which spread
-// a head over all of it, win: 4 heads, 2000 pages of 64 tokens, 500 kept (2 MB per CTA) 39 / 55.
-bool cluster_step_wins(int BH, int64_t pages, int64_t head_bytes, int sms)
+// With at most as many heads as SMs, one launch wins below 1024 pages as long as the CTAs have little to read each (device
+// time, 32 heads x 128, separate launches / cluster, us: 4090 tokens in pages of 64, 16 kept 16.9 / 10.2; 1000 tokens 16.1 /
+// 8.5; 8000 tokens, 125 of 500 pages 23.1 / 15.7; 4 heads, 1000 tokens 19.0 / 6.8).  Few heads with much to read leave most
+// of the chip idle, and the separate kernels, which spread a head over all of it, win: 4 heads, 2000 pages of 64 tokens, 500
+// kept (2 MB per CTA) 39 / 55.  (64 to 128 heads of 2000 pages: 0.95 to 1.03.)
+// More heads have a CTA each, and what counts is how evenly two to an SM they fill the chip.  From three quarters of one
+// round, or 85 % of several, the cluster form wins up to 2048 pages: 256 heads, 125 of 2000 pages 107 / 102, of 500 31 of them
+// 47 / 32; 512 heads, 127 of 2047 2 % less.  Otherwise a part of the SMs reads alone while the others are done, or in the last
+// round only a few read at all, and the separate kernels win what has much to read.  A page's bounds weigh more than its
+// rows (a CTA keeps fewer of them on their way), six times as much in the limits below, which lie where the measured
+// forms change places (bf16, pages of 16; us, separate / cluster): 160 heads, 31 of 500 pages 37 / 28, 56 of 900 44.6 / 44.3,
+// 127 of 2047 78 / 95; 200 heads, 43 of 700 35.9 / 38.3; 320 heads, 15 of 255 a
+// third more, 31 of 500 equal, 127 of 2047 138 / 183.
+bool cluster_step_wins(int BH, int64_t pages, int64_t bounds_bytes, int64_t rows_bytes, int sms)
 {
     const int cl = cluster_step_size(BH, pages, sms);
     if (cl == 0) return false;
-    if (BH >= sms) return true;
-    return pages < 1024 && head_bytes / cl <= (512 << 10);
+    if (BH <= sms) return pages < 1024 && (bounds_bytes + rows_bytes) / cl <= (512 << 10);
+    const int64_t round = 2 * (int64_t)sms, rounds = (BH + round - 1) / round;
+    if (rounds == 1 ? 4 * (int64_t)BH >= 3 * round : 20 * (int64_t)BH >= 17 * rounds * round) return true;
+    return 6 * bounds_bytes + rows_bytes <= (rounds == 1 ? 3200 << 10 : 1400 << 10);
 }
 
 cudaError_t launch_cluster_step(const DecodeArgs &a, const void *q, const void *k_t, const void *v_t, const void *g_t, float *scores,

@@ -212,3 +212,21 @@ def test_workload_generators_are_seeded_and_shaped():
         assert touched == sorted(pages[0, h].tolist())
     assert wl.CONFIGS[2].budget_pages(32769) == 257 and wl.CONFIGS[1].budget_pages() == 64
     assert wl.METRIC.budget_pages() == 512 and wl.CONFIGS[0].budget_pages() == 16
+
+
+@pytest.mark.skipif(not _no_gpu(), reason="the rule for 148 SMs, which is what the library plans for where it finds no device")
+@pytest.mark.parametrize("heads,S,pages,budget,one", [
+    (32, 16, 500, 125, True), (32, 16, 1024, 64, False), (4, 64, 900, 225, False), (148, 16, 900, 56, False),
+    (160, 16, 500, 31, True), (160, 16, 2047, 127, False), (200, 16, 1500, 93, False), (224, 16, 2047, 127, True),
+    (256, 16, 2047, 511, True), (256, 64, 2047, 2047, True), (320, 16, 200, 50, True), (320, 16, 900, 56, False),
+    (320, 64, 255, 255, False), (512, 16, 2047, 127, True), (256, 16, 2049, 127, False)])
+def test_shapes_of_the_cluster_step(lib, heads, S, pages, budget, one):
+    """Which decode steps run as one launch of a cluster per head: not those of more heads than SMs that fill the last round of
+    CTAs badly and have much to read (up to a third slower than separate kernels)."""
+    c = cfg(batch=1, heads=heads, page_size=S, capacity_tokens=4096 * S, max_budget_pages=4096)
+    cache = rq.rq_cache()
+    cache.cfg = c
+    cache.kv = cache.meta = cache.state = cache.workspace = 4096
+    cache.page_capacity = 4096
+    cache.len = pages * S - 5
+    assert (lib.rq_decode_step_launches(C.byref(cache), budget) == 1) == one
