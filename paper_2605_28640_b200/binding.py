@@ -136,8 +136,11 @@ def rq_build_cache(cache: rq_cache, k, v, g, stream=None):
 
 
 def rq_decode_step(cache: rq_cache, q, k_t, v_t, g_t, budget_pages, scale, o, sel_idx_out=None, stream=None):
-    status = (_lib or lib()).rq_decode_step(cache, q.data_ptr(), k_t.data_ptr(), v_t.data_ptr(), g_t.data_ptr(), budget_pages, scale,
-                                            o.data_ptr(), _ptr(sel_idx_out), _stream(stream))
+    try:                                    # (without five calls of _ptr)
+        status = (_lib or lib()).rq_decode_step(cache, q.data_ptr(), k_t.data_ptr(), v_t.data_ptr(), g_t.data_ptr(), budget_pages, scale,
+                                     o.data_ptr(), _ptr(sel_idx_out), _stream(stream))
+    except AttributeError:                  # None: the library refuses it
+        status = lib().rq_decode_step(cache, _ptr(q), _ptr(k_t), _ptr(v_t), _ptr(g_t), budget_pages, scale, _ptr(o), _ptr(sel_idx_out), _stream(stream))
     if status != RQ_OK:
         raise RqError(status, "rq_decode_step")
 
@@ -145,8 +148,11 @@ def rq_decode_step(cache: rq_cache, q, k_t, v_t, g_t, budget_pages, scale, o, se
 def rq_decode_step_host(cache: rq_cache, q, k_t, v_t, g_t, budget_pages, scale, o, sel_idx_out=None,
                         stream=None):
     """Same as rq_decode_step with HOST tensors (pinned for asynchronous copies)."""
-    status = (_lib or lib()).rq_decode_step_host(cache, q.data_ptr(), k_t.data_ptr(), v_t.data_ptr(), g_t.data_ptr(), budget_pages, scale,
-                                                 o.data_ptr(), _ptr(sel_idx_out), _stream(stream))
+    try:
+        status = (_lib or lib()).rq_decode_step_host(cache, q.data_ptr(), k_t.data_ptr(), v_t.data_ptr(), g_t.data_ptr(), budget_pages, scale,
+                                     o.data_ptr(), _ptr(sel_idx_out), _stream(stream))
+    except AttributeError:                  # None: the library refuses it
+        status = lib().rq_decode_step_host(cache, _ptr(q), _ptr(k_t), _ptr(v_t), _ptr(g_t), budget_pages, scale, _ptr(o), _ptr(sel_idx_out), _stream(stream))
     if status != RQ_OK:
         raise RqError(status, "rq_decode_step_host")
 

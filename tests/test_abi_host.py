@@ -230,3 +230,27 @@ def test_shapes_of_the_cluster_step(lib, heads, S, pages, budget, one):
     cache.page_capacity = 4096
     cache.len = pages * S - 5
     assert (lib.rq_decode_step_launches(C.byref(cache), budget) == 1) == one
+
+
+class _Stream:
+    cuda_stream = 0
+
+
+@pytest.mark.parametrize("call", [rq.rq_decode_step, rq.rq_decode_step_host])
+@pytest.mark.parametrize("missing", range(5))
+def test_a_missing_tensor_is_an_invalid_argument(lib, call, missing):
+    """None in the place of a tensor reaches the library as NULL and comes back as its error."""
+    import torch
+    cache = rq.rq_cache()
+    cache.cfg = cfg(capacity_tokens=64, max_budget_pages=2)
+    cache.kv = cache.meta = cache.state = cache.workspace = 4096
+    cache.page_capacity = 4
+    cache.len = 64                                                    # full: with all tensors there it would be CAPACITY
+    t = [torch.zeros(32 * 128) for _ in range(5)]
+    with pytest.raises(rq.RqError) as e:
+        call(cache, *t[:4], 1, 0.0, t[4], None, _Stream())
+    assert e.value.status == rq.RQ_ERR_CAPACITY
+    t[missing] = None
+    with pytest.raises(rq.RqError) as e:
+        call(cache, *t[:4], 1, 0.0, t[4], None, _Stream())
+    assert e.value.status == rq.RQ_ERR_INVALID_ARG
