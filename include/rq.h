@@ -255,13 +255,13 @@ RQ_API int rq_attend_pages_noalloc(const rq_config *cfg, const void *kv, int64_t
  * + i) seeing the positions up to its own; the `keep` most important entries are retained: the
  * window's own positions always (they count inside keep), then the most important earlier
  * positions, equal importance to the lower position.
- *   q_window       : [B][window][H][D] of cfg.dtype (device)
+ *   q_window       : [B][window][H][D] of cfg.dtype (device), 16-byte aligned if that is RQ_BF16
  *   idx_out        : int32 [B][H][keep] (device): retained positions, ascending; -1 beyond len
  *   importance_out : NULL or fp32 [B][H][len] (device)
  *   scratch        : device memory of rq_snapkv_scratch_bytes() bytes for the cache's current
  *                    length, 256-byte aligned, free again when the call's work has run
  *   scale          : softmax scale; <= 0 selects 1/sqrt(D)
- * Errors: INVALID_ARG (NULL, window outside 1..64 or longer than the cache, keep < 1), CUDA. */
+ * Errors: INVALID_ARG (NULL, misaligned, window outside 1..64 or longer than the cache, keep < 1), CUDA. */
 RQ_API int rq_snapkv_scratch_bytes(const rq_cache *cache, size_t *bytes);
 RQ_API int rq_snapkv_select(rq_cache *cache, const void *q_window, int32_t window, int32_t keep, float scale,
                             int32_t *idx_out, float *importance_out, void *scratch, void *stream);
@@ -285,9 +285,9 @@ RQ_API int rq_snapkv_compact(const rq_cache *src, const int32_t *idx, int32_t ke
  * block and the query's own block are always taken and count inside budget_blocks; with fewer
  * blocks than that before it, a query attends everything before it.  Attention is softmax over the
  * positions <= t of the chosen blocks, on the decayed keys and values as stored.
- *   q          : [B][T][H][D] of cfg.dtype (device), T = the cache's current length
+ *   q          : [B][T][H][D] of cfg.dtype (device), T = the cache's current length; 16-byte aligned
  *   block      : 64, 128, ... (a multiple of 64 and of the page size); at most 2048 blocks per prompt
- *   o          : [B][T][H][D] of cfg.dtype (device)
+ *   o          : [B][T][H][D] of cfg.dtype (device), 16-byte aligned
  *   blocks_out : NULL or int32 [B][H][T][budget_blocks] (device): chosen blocks, ascending, -1 beyond
  *   means_out  : NULL or fp32 [B][H][blocks][D] (device): the representatives
  *   scratch    : device memory of rq_moba_scratch_bytes() bytes, 256-byte aligned

@@ -621,6 +621,7 @@ int rq_snapkv_select(rq_cache *cache, const void *q_window, int32_t window, int3
     if (!q_window || !idx_out || !scratch || !aligned(scratch, 256)) return RQ_ERR_INVALID_ARG;
     if (window < 1 || window > 64 || keep < 1 || cache->len < window) return RQ_ERR_INVALID_ARG;
     const rq_config &c = cache->cfg;
+    if (c.dtype == RQ_BF16 && !aligned(q_window, 16)) return RQ_ERR_INVALID_ARG;      // read by tensor map
     cudaStream_t s = (cudaStream_t)stream;
     SnapArgs a;
     a.kv = cache->kv; a.page_cap = cache->page_capacity; a.len = cache->len;

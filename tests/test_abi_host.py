@@ -254,3 +254,14 @@ def test_a_missing_tensor_is_an_invalid_argument(lib, call, missing):
     with pytest.raises(rq.RqError) as e:
         call(cache, *t[:4], 1, 0.0, t[4], None, _Stream())
     assert e.value.status == rq.RQ_ERR_INVALID_ARG
+
+
+def test_misaligned_window_queries_are_refused(lib):
+    """The window's queries of a bf16 cache are read by tensor map, from a 16-byte aligned address."""
+    cache = rq.rq_cache()
+    cache.cfg = cfg(capacity_tokens=8192, max_budget_pages=8)
+    cache.kv = cache.meta = cache.state = cache.workspace = 4096
+    cache.page_capacity = 512
+    cache.len = 5000
+    for q in (258, 264):
+        assert lib.rq_snapkv_select(C.byref(cache), q, 64, 100, 0.0, 256, None, 256, None) == rq.RQ_ERR_INVALID_ARG
