@@ -304,12 +304,12 @@ RQ_API int64_t rq_cache_len(const rq_cache *cache);
  * sel_idx_out is NULL [no counterpart in the paper: bookkeeping for benchmarks]: ONE when the whole
  * step runs as one launch (chosen by the library for short contexts: fewer than 1024 pages per head
  * with up to a few MB to read per head, or up to 2048 pages when there are more (batch, head) pairs
- * than SMs; and for 64 to 128 (batch, head) pairs of 4096 to
+ * than SMs and they either keep all SMs equally busy or have little to read; and for 64 to 128 (batch, head) pairs of 4096 to
  * 12284 pages each that split into 4, 8 or 2 equal groups which keep the GPU's resident CTAs
  * busy, budget below the number of pages; cache.reserved[2] asks for it on other shapes);
- * otherwise three (update + scoring, selection, attention), or two when they are asked for on a
- * context short enough (at most 256 pages per head, at least 16 heads) for one CTA per head to do
- * the first two kernels' work in one launch.  A non-NULL sel_idx_out can add a launch that sorts the list.
+ * otherwise three (update + scoring, selection, attention), or two on a context short enough (at
+ * most 256 pages per head, at least 16 heads) for one CTA per head to do the first two kernels'
+ * work in one launch.  A non-NULL sel_idx_out can add a launch that sorts the list.
  * The first call on a device looks up launch parameters (occupancy).  -1 for an invalid cache. */
 RQ_API int rq_decode_step_launches(const rq_cache *cache, int32_t budget_pages);
 

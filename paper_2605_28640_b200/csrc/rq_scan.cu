@@ -1,12 +1,14 @@
 // Prefill: the gated decay recurrence (Eq. 1) over a whole sequence, fused with
 // the paged cache write and the per-page min/max of the stored keys
 // (Appendix A.1, "Sparse inference settings").  One launch, every input byte
-// read once, every output byte written once, no scratch in global memory.
+// read once, every output byte written once, no scratch in global memory, but for very long
+// prompts of a few heads, which are cut into time chunks (three launches, the inputs of all
+// chunks but the last read twice, the chunks' maps and entry states in the workspace).
 //
 // The recurrence x~_t = g_t x~_{t-1} + (1-g_t) x_t runs along time and is
 // independent per (batch, head, channel).  Work decomposition: a unit is one
 // (batch, head) pair and 32 neighbouring channels; it belongs to one CTA, or, when
-// there are few units and many positions, to a cluster of up to eight CTAs that take
+// there are few units and many positions, to a cluster of up to four CTAs that take
 // its tiles in turn.
 //
 // Time is cut into tiles of 256 positions that move through a ring of shared-memory
@@ -35,8 +37,9 @@
 // Bound: the phases of a tile between its two barriers, with DRAM close behind (131072 tokens of 32 heads x 128, bf16: 5.5
 // GB in 0.90 to 0.99 ms, 5.6 to 6.1 TB/s; the copies alone run at 5.8 TB/s).  Before (copies started and rows stored in
 // 16-byte pieces by all threads, one CTA per unit, three barriers, the inputs read twice for few heads) / now, us: 32 heads,
-// 131072 tokens 1120 / 900; 4001 tokens and the clearing before them 50 / 40; 8 heads, 50003 tokens, fp32 gates 195 / 110; 8 heads, 8000 tokens 76 / 33; 4 heads, 8000 tokens
-// 75 / 31; fp32, 12 heads, 20000 tokens 176 / 120; fp32, 32 heads, 8000 tokens, pages of 16 120 / 126.
+// 131072 tokens 1120 / 900; 4001 tokens and the clearing before them 50 / 40; 8 heads, 50003 tokens, fp32 gates 195 / 111; 8
+// heads, 8000 tokens 76 / 33; 4 heads, 8000 tokens 75 / 31; 256 heads, 16 tokens 22 / 18; fp32, 12 heads, 20000 tokens 176 /
+// 120; fp32, 32 heads, 8000 tokens, pages of 16, 120 / 121.
 #include "rq_async.cuh"
 #include "rq_device.cuh"
 #include "rq_internal.h"

@@ -3,11 +3,11 @@
 // accumulator back into registers.  One CTA per product (cta_group::1), bf16 operands, fp32
 // accumulator.
 //
-// Operand tiles are K-major (a row's K elements are consecutive in the source) and stored without
-// swizzle as 8-row x 16-byte core matrices: element (row r, 16-byte piece c of the row's K extent)
-// lives at  (r / 8) * SBO + c * LBO + (r % 8) * 16  with LBO = 128 (the pieces of one 8-row group
-// follow each other) and SBO = pieces * 128 (then the next 8 rows).  One instruction consumes
-// K = 16 elements = two pieces; the descriptor of the k-th step starts 256 bytes further on.
+// Operand tiles are K-major (a row's K elements are consecutive in the source) in the layout with the 128-byte swizzle, which is
+// what a tiled bulk-tensor copy (TMA) with CU_TENSOR_MAP_SWIZZLE_128B writes: the K extent is cut into halves of 64 elements
+// (128 bytes); a half holds its rows 128 bytes apart, groups of 8 rows 1024 bytes apart, and inside a row the 16-byte piece p
+// sits at ((p ^ (row % 8)) * 16).  Tile bases are 1024-byte aligned.  One instruction consumes K = 16 elements; the next K
+// step is 32 bytes further on inside the half.
 #pragma once
 #include <stdint.h>
 
@@ -15,31 +15,12 @@
 
 namespace rq {
 
-constexpr uint32_t kUmmaLbo = 128;             // bytes between the two 16-byte pieces of one K step
-
-// byte offset of piece (row, piece) in a tile whose rows hold `pieces` 16-byte pieces
-__device__ __forceinline__ uint32_t umma_tile_offset(int row, int piece, int pieces)
-{
-    return (uint32_t)(row >> 3) * (uint32_t)(pieces * 128) + (uint32_t)piece * kUmmaLbo + (uint32_t)(row & 7) * 16u;
-}
-
-// shared-memory matrix descriptor: start address, leading and stride byte offsets (all without
-// their 4 low bits), descriptor version 1, no swizzle
-__device__ __forceinline__ uint64_t umma_desc(uint32_t saddr, uint32_t sbo_bytes)
-{
-    return (uint64_t)((saddr & 0x3FFFFu) >> 4) | ((uint64_t)(kUmmaLbo >> 4) << 16) | ((uint64_t)(sbo_bytes >> 4) << 32) |
-           (1ull << 46);
-}
-
-// The same tiles with the 128-byte swizzle, which is what a tiled bulk-tensor copy (TMA) with
-// CU_TENSOR_MAP_SWIZZLE_128B writes: the K extent is cut into halves of 64 elements (128 bytes); a half
-// holds its rows 128 bytes apart, groups of 8 rows 1024 bytes apart, and inside a row the 16-byte piece p
-// sits at ((p ^ (row % 8)) * 16).  Tile bases are 1024-byte aligned.  A K step of 16 elements is 32 bytes
-// further on inside the half.
 __device__ __forceinline__ uint32_t umma_sw128_offset(int row, int piece)   // piece: 0..7 inside the half
 {
     return (uint32_t)(row >> 3) * 1024u + (uint32_t)(row & 7) * 128u + (uint32_t)((piece ^ (row & 7)) * 16);
 }
+// shared-memory matrix descriptor: start address, leading and stride byte offsets (all without their 4 low bits), descriptor
+// version 1, 128-byte swizzle
 __device__ __forceinline__ uint64_t umma_desc_sw128(uint32_t saddr)
 {
     return (uint64_t)((saddr & 0x3FFFFu) >> 4) | (1ull << 16) | ((uint64_t)(1024u >> 4) << 32) | (1ull << 46) | (2ull << 61);
