@@ -51,6 +51,17 @@ __device__ __forceinline__ float max_nan(float a, float b)
     return y;
 }
 
+// two bf16 added to a sum each (their values are exact in fp32)
+__device__ __forceinline__ void add_bf16(float2 &sum, uint32_t pair)
+{
+    asm("{\n\t.reg .b16 lo, hi;\n\t"
+        "mov.b32 {lo, hi}, %2;\n\t"
+        "add.rn.f32.bf16 %0, lo, %0;\n\t"
+        "add.rn.f32.bf16 %1, hi, %1;\n\t}"
+        : "+f"(sum.x), "+f"(sum.y)
+        : "r"(pair));
+}
+
 // The walk over the chunks of the listed blocks: (entry of the list, chunk inside the block).
 struct Walk {
     int bi = 0, r = 0;
@@ -75,8 +86,9 @@ struct Walk {
 // by their sum at the end, so that O is hardly ever touched between the products.  The sum is that of the rounded weights:
 // relative to a lagging maximum the largest weight is not 1 exactly, and its rounding would be an error of the whole output;
 // so it cancels.  Error against fp64 (2-norm; 4096 positions, 16 of 64 blocks, logits of 1.5 / 5): 1.670e-3 / 1.656e-3; with
-// the sum of the weights before rounding 1.699e-3 / 1.731e-3, relative to the final maximum 1.694e-3 / 1.712e-3.  It costs two
-// operations a pair of weights, 2 % of the time.
+// the sum of the weights before rounding 1.699e-3 / 1.731e-3, relative to the final maximum 1.694e-3 / 1.712e-3.  The sum of
+// the rounded weights, an addition of a bf16 value to an fp32 one each, costs 1 % of the time, keeping infinite scores where
+// they belong another.
 // Warps 0..7 read scores, warp 8 starts the tensor-map copies, warps 9 and 10 the score products of an accumulator each,
 // warp 11 the output products; they meet through mbarriers only, every wait bounded.  One warp for all products was the
 // limit: 24 products, six commits and as many waits a chunk.  256 queries per CTA because keys and values come from L2 for
@@ -353,7 +365,7 @@ __global__ void __launch_bounds__(kThreads, 1) moba_mma_kernel(const __grid_cons
                 }
                 // a block the query did not choose: 2^-3e38 = 0; nor do scores of -inf weigh anything while there is no other
                 const float nm = nv > 0 ? fminf(-m, 3.0e38f) : -3.0e38f;
-                const float2 nm2 = make_float2(nm, nm), one2 = make_float2(1.0f, 1.0f);
+                const float2 nm2 = make_float2(nm, nm);
 #pragma unroll
                 for (int hf = 0; hf < 2; ++hf) {
                     uint32_t w[16];
@@ -362,7 +374,7 @@ __global__ void __launch_bounds__(kThreads, 1) moba_mma_kernel(const __grid_cons
                         const float2 x = fma2(make_float2(v[hf * 32 + 2 * k], v[hf * 32 + 2 * k + 1]), sc2, nm2);
                         const float2 p = make_float2(exp2_fast(x.x), exp2_fast(x.y));
                         w[k] = pack_bf16(p.x, p.y);
-                        l2 = fma2(make_float2(bf16lo(w[k]), bf16hi(w[k])), one2, l2);
+                        add_bf16(l2, w[k]);
                     }
                     tmem_st16(ts + hf * 16, w);
                 }
