@@ -633,7 +633,7 @@ int rq_snapkv_select(rq_cache *cache, const void *q_window, int32_t window, int3
     if (importance_out) a.imp = importance_out;              // (no copy: the selection reads it where the caller wants it)
     a.status = (int32_t *)((char *)cache->workspace + workspace_layout(c).status);
     if (launch_snap_scores(a, s) != cudaSuccess) return RQ_ERR_CUDA;
-    if (launch_snap_select(a.imp, BH, cache->len, window, keep, idx_out, s) != cudaSuccess) return RQ_ERR_CUDA;
+    if (launch_snap_select(a.imp, BH, cache->len, window, keep, a.dtype == RQ_BF16 && a.D == 128, idx_out, s) != cudaSuccess) return RQ_ERR_CUDA;
     return RQ_OK;
 }
 

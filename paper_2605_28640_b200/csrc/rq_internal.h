@@ -164,7 +164,8 @@ struct SnapArgs {
 size_t snap_scratch_bytes(int BH, int64_t len);
 void snap_carve(void *scratch, int BH, int64_t len, float **imp, float2 **stats, float2 **rowstat);
 cudaError_t launch_snap_scores(const SnapArgs &a, cudaStream_t s);
-cudaError_t launch_snap_select(const float *imp, int BH, int64_t len, int window, int keep, int32_t *idx, cudaStream_t s);
+// beside: the importances come from the tensor-core kernels for 128 channels, beside which the selection may start
+cudaError_t launch_snap_select(const float *imp, int BH, int64_t len, int window, int keep, bool beside, int32_t *idx, cudaStream_t s);
 struct SnapCompactArgs {
     const void *skv;    // the source cache
     int64_t s_page_cap;

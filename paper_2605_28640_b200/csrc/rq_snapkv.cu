@@ -1313,7 +1313,7 @@ static cudaError_t select_run(const float *imp, int BH, int64_t len, int w, int 
     return cudaLaunchKernelEx(&cfg, snap_select_kernel<EPT, NT>, imp, len, w, keep, per_warp, idx);
 }
 
-cudaError_t launch_snap_select(const float *imp, int BH, int64_t len, int window, int keep, int32_t *idx, cudaStream_t s)
+cudaError_t launch_snap_select(const float *imp, int BH, int64_t len, int window, int keep, bool beside, int32_t *idx, cudaStream_t s)
 {
     int w = window < keep ? window : keep;
     if ((int64_t)w > len) w = (int)len;
@@ -1345,6 +1345,10 @@ cudaError_t launch_snap_select(const float *imp, int BH, int64_t len, int window
     // four of these, or where there is room for two only, 1024 threads with up to 32 keys
     int64_t cl = C <= 4096 ? 1 : C <= 2 * 512 * 16 ? 2 : 4;
     if (cl > most) cl = most;
+    // (between four and eight of them few heads take eight where they may start beside the kernel ahead, which 1024 threads find
+    // no room for: a call for 12 heads x 128, 44560 positions 141 -> 137 us, 8 heads, 50000 positions 72 -> 66; with 64 channels
+    // the larger CTAs stay ahead, 8 heads 62 against 69, but for one or two heads, 36 against 34)
+    if (C > 4 * 512 * 16 && C <= 8 * 512 * 16 && (beside ? 11 : 64) * (int64_t)BH <= sms) cl = 8;
     const bool wide = C > cl * 512 * 16;
     if (wide)
         while (cl < most && C > cl * 512 * kSelMaxEpt) cl *= 2;

@@ -15,8 +15,8 @@ DEV = "cuda"
 @pytest.mark.parametrize("BH,T,keeps", [(1, 100, (64, 65, 99)), (2, 1063, (64, 700)), (2, 1089, (65, 70)), (40, 2112, (130,)),
                                         (3, 4096, (66, 1024)), (3, 16449, (300, 16448)), (160, 5000, (1000,)),
                                         (2, 131136, (8192,)), (1, 140001, (70, 9000)), (310, 9000, (64, 2000))])
-def test_index_for_index(BH, T, keeps, kinds):
-    D, W = 64, 64
+def test_index_for_index(BH, T, keeps, kinds, D=64):
+    W = 64
     g = torch.Generator(device=DEV)
     g.manual_seed(T + kinds)
     cache = rq.Cache(1, BH, D, 64, T, torch.bfloat16)
@@ -50,3 +50,9 @@ def test_index_for_index(BH, T, keeps, kinds):
 def test_forms_by_heads(BH, T, keeps, kinds):
     """At the edges of the rule that gives a head one CTA, a cluster of two, four or eight, or the one-CTA form by digits."""
     test_index_for_index(BH, T, keeps, kinds)
+
+
+@pytest.mark.parametrize("BH,T,keeps", [(5, 32833, (1000,)), (13, 65600, (64, 5000)), (14, 40000, (2000,))])
+def test_clusters_of_eight(BH, T, keeps):
+    """128 channels, few heads, keys that fill four to eight CTAs of 512 threads."""
+    test_index_for_index(BH, T, keeps, 0, D=128)
