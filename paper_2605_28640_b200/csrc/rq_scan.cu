@@ -140,7 +140,7 @@ struct ScanPlan {
 // (MODE 1), a small kernel chains the maps into the state that enters every chunk, then every chunk runs the scan proper
 // from its own entry state.  The inputs of all chunks but the last are read twice.  (Chunks and clusters exclude each other.)
 //   maps   [units][chunks][3][CG]   A, B of the keys, B of the values
-//   entry  [units][chunks][2][CG]   state entering a chunk
+//   entry  [units][chunks][2][CG]   state entering a chunk (not chunk 0), and the state before the call
 template <typename T, typename G, int D, int S, int MODE, bool STAGED>
 __global__ void __launch_bounds__(NT, MODE == 3 ? 2 : 1) scan_kernel(ScanArgs a, const __grid_constant__ ScanMaps tm, ScanPlan plan, float *maps, const float *entry)
 {
@@ -245,10 +245,15 @@ __global__ void __launch_bounds__(NT, MODE == 3 ? 2 : 1) scan_kernel(ScanArgs a,
         } else if (MODE == 3) {
             first_k = a.state[(int64_t)bh * 2 * D + c0 + tid];
             first_v = a.state[(int64_t)bh * 2 * D + D + c0 + tid];
-        } else if (chunks == 1) {
+        } else if (MODE == 2 && chunks == 1) {   // (of its own: read like below, the copies start later, 32 heads x 128, 50000 tokens 361 -> 391 us)
             carry[0][0][tid] = a.state[(int64_t)bh * 2 * D + c0 + tid];
             carry[0][1][tid] = a.state[(int64_t)bh * 2 * D + D + c0 + tid];
-        } else {                                 // (of the first chunk, too: the CTA of the last one overwrites the cache's state)
+        } else if (MODE != 2 && chunk == 0) {
+            // (with several chunks a copy behind the entry states: the CTA of the last chunk overwrites the cache's state meanwhile)
+            const float *from = chunks == 1 ? a.state : entry + (int64_t)plan.units * chunks * 2 * CG;
+            carry[0][0][tid] = from[(int64_t)bh * 2 * D + c0 + tid];
+            carry[0][1][tid] = from[(int64_t)bh * 2 * D + D + c0 + tid];
+        } else {
             const float *e = entry + ((int64_t)unit * chunks + chunk) * 2 * CG;
             carry[0][0][tid] = e[tid];
             carry[0][1][tid] = e[CG + tid];
@@ -508,12 +513,12 @@ __global__ void __launch_bounds__(NT, MODE == 3 ? 2 : 1) scan_kernel(ScanArgs a,
 }
 
 // The state entering every chunk from the chunks' maps, in order.  Grid: channel groups; a thread per (k or v, channel).
-__global__ void scan_chain_kernel(const float *state, int D, int gph, int chunks, const float *maps, float *entry)
+__global__ void scan_chain_kernel(const float *state, int D, int gph, int chunks, const float *maps, float *entry, float *state_copy)
 {
     const int unit = blockIdx.x, kv = threadIdx.x / CG, ch = threadIdx.x % CG;
     const int bh = unit / gph, c0 = (unit % gph) * CG;
     float s = state[(int64_t)bh * 2 * D + kv * D + c0 + ch];
-    entry[((int64_t)unit * chunks * 2 + kv) * CG + ch] = s;
+    state_copy[(int64_t)bh * 2 * D + kv * D + c0 + ch] = s;
     for (int c = 0; c + 1 < chunks; ++c) {
         const float *mp = maps + ((int64_t)unit * chunks + c) * 3 * CG;
         s = fmaf(mp[ch], s, mp[(1 + kv) * CG + ch]);
@@ -591,7 +596,7 @@ cudaError_t run(const ScanArgs &a, cudaStream_t s)
     if (a.chunk_scratch && 2 * units <= sms) {
         chunks = sms / p.units;
         if (chunks > p.ntiles / 16) chunks = p.ntiles / 16;
-        while (chunks > 1 && (size_t)p.units * chunks * 5 * CG * sizeof(float) > kScanScratchBytes) --chunks;
+        while (chunks > 1 && (size_t)p.units * (chunks * 5 + 2) * CG * sizeof(float) > kScanScratchBytes) --chunks;
     }
     if (chunks < 7) {
         chunks = 1;
@@ -615,7 +620,7 @@ cudaError_t run(const ScanArgs &a, cudaStream_t s)
     if (p.chunks > 1) {
         e = start<T, G, D, S, 1, sizeof(T) == 2>(a, tm, p, 1, maps, entry, DSM, s);
         if (e != cudaSuccess) return e;
-        scan_chain_kernel<<<(unsigned)units, 2 * CG, 0, s>>>(a.state, D, D / CG, p.chunks, maps, entry);
+        scan_chain_kernel<<<(unsigned)units, 2 * CG, 0, s>>>(a.state, D, D / CG, p.chunks, maps, entry, entry + (size_t)units * p.chunks * 2 * CG);
     }
     auto go = [&](auto staged) {
         constexpr bool ST = decltype(staged)::value;
