@@ -2,6 +2,8 @@
 // position over the positions up to its own of the blocks it chose, both contractions on the tensor cores (tcgen05).
 #include <math_constants.h>
 
+#include <algorithm>
+
 #include "rq_async.cuh"
 #include "rq_device.cuh"
 #include "rq_internal.h"
@@ -19,7 +21,12 @@ constexpr int kTiles = 2;                      // accumulators of a CTA: 256 con
 constexpr int kStages = 4;                     // chunks of keys, and of values, in shared memory
 constexpr int kReadWarps = 4 * kTiles;         // warps that turn scores into weights: a thread per query
 constexpr int kThreads = (kReadWarps + kTiles + 2) * 32;   // and one for the copies, two for the score products, one for the output products
-constexpr float kRaise = 8.0f;                 // powers of two a query's maximum may grow before its output is rescaled
+// Prompts whose keys and values, all heads together, take more than kSetFrom are worked on in sets of heads of kSetBytes, which
+// stay in L2 while the set's CTAs walk over them; below, all heads side by side balance better (32 heads x 30011 x 128, 492 MB:
+// 7.43 -> 7.18 ms; 32 x 9001 x 64, 74 MB: 799 -> 883 us in sets)
+constexpr int64_t kSetBytes = 64 << 20, kSetFrom = 256 << 20;
+constexpr float kLimit = 4294967296.0f;        // sum of a chunk's weights that is taken as it is (2^32)
+constexpr float kRaise = 8.0f;                 // powers of two by which a query's own chunk may exceed m
 
 template <int D> struct AttGeom {
     static constexpr int HALVES = D / 64;
@@ -43,14 +50,6 @@ __device__ __forceinline__ float exp2_fast(float x)
     return y;
 }
 
-// the larger one; NaN if one is NaN
-__device__ __forceinline__ float max_nan(float a, float b)
-{
-    float y;
-    asm("max.NaN.f32 %0, %1, %2;" : "=f"(y) : "f"(a), "f"(b));
-    return y;
-}
-
 // two bf16 added to a sum each (their values are exact in fp32)
 __device__ __forceinline__ void add_bf16(float2 &sum, uint32_t pair)
 {
@@ -71,39 +70,39 @@ struct Walk {
     }
 };
 
-// Grid (heads, tiles of 256 queries; the last queries of a head first: their work is the largest).  A CTA owns 256
-// consecutive queries as two accumulators of 128 lanes; everything per query (choice of blocks, causal cut, running
-// maximum, sum, weights) belongs to one thread.  The 64-position chunks of the blocks that any of the 256 queries chose
-// are walked once:
+// Grid: tiles of 256 queries of all heads, the last queries of a head first (their work is the largest).  A CTA owns 256
+// consecutive queries as two accumulators of 128 lanes; everything per query (choice of blocks, causal cut, what its weights
+// are relative to, their sum, the weights) belongs to one thread.  The 64-position chunks of the blocks that any of the 256
+// queries chose are walked once:
 //   S = Q K^T        128 x 64 per accumulator, fp32 in tensor memory, two score buffers per accumulator, so that the
 //                    product of the next chunk runs while the weights of this one are computed
 //   weights          2^(s - m) for the chosen blocks' positions up to the query's own, rounded to bf16, written over
 //                    the first half of their scores as the A operand of the second product; the rounded weights are
 //                    summed in fp32
 //   O += P V         accumulated in tensor memory over all chunks
-// m is the query's largest score so far, but it is raised (and the query's row of O multiplied down) only when a score
-// exceeds it by more than 8 powers of two: weights of up to 256 lose nothing in bf16 and fp32, and the output is divided
-// by their sum at the end, so that O is hardly ever touched between the products.  The sum is that of the rounded weights:
-// relative to a lagging maximum the largest weight is not 1 exactly, and its rounding would be an error of the whole output;
-// so it cancels.  Error against fp64 (2-norm; 4096 positions, 16 of 64 blocks, logits of 1.5 / 5): 1.670e-3 / 1.656e-3; with
-// the sum of the weights before rounding 1.699e-3 / 1.731e-3, relative to the final maximum 1.694e-3 / 1.712e-3.  The sum of
-// the rounded weights, an addition of a bf16 value to an fp32 one each, costs 1 % of the time, keeping infinite scores where
-// they belong another.
+// m is the largest score of the first chunk, which every query attends: bf16 and fp32 carry weights of any size equally well,
+// so m need not be the largest of all, and the other chunks' weights are taken as their scores come in, 32 at a time, without
+// looking for a maximum first.  Only where a chunk's weights add up to more than 2^32 (or to nothing that can be compared), and
+// in the query's own chunk, whose scores have to be cut anyway, the scores are looked through, m is raised and the query's row
+// of O multiplied down.  The output is divided by the sum of the rounded weights: relative to an m that is not the maximum the
+// largest weight is not 1 exactly, and its rounding would be an error of the whole output; so it cancels.  Error against fp64
+// (2-norm; 4096 positions, 16 of 64 blocks, decayed keys, logits of 0.64): 1.66603e-3, as with every chunk's maximum looked for.
+// (A limit of 2^10 is reached all the time, as the first keys of a prompt have hardly been accumulated and score low: 213 -> 262 us.)
 // Warps 0..7 read scores, warp 8 starts the tensor-map copies, warps 9 and 10 the score products of an accumulator each,
-// warp 11 the output products; they meet through mbarriers only, every wait bounded.  One warp for all products was the
-// limit: 24 products, six commits and as many waits a chunk.  256 queries per CTA because keys and values come from L2 for
-// every CTA.  A CTA's queries come by tensor map, and it may start before the routing kernel has ended: at 4096 positions
-// a CTA lives 50 us only, and the 20 us before its first product were a third of that.
-// Measured, 32 heads x 128 channels, 30011 positions (30 of 469 blocks) / 4096 (16 of 64): a warp per kind of product 7.61 ->
-// 6.13 ms / 234 -> 206 us; queries by tensor map, early start 206 -> 186 us; list by a lane per block, outputs through shared
-// memory 186 -> 181 us.  Bound: the readers' chain per chunk (about 1900 cycles, of which ex2 alone takes 1024, against 1280
-// for the products).  Slower were a quarter of the exponentials by polynomial, 16 reading warps, and pairs of chunks as one
-// product of 128 columns.
+// warp 11 the output products; they meet through mbarriers only, every wait bounded.  256 queries per CTA because keys and
+// values come from L2 for every CTA.  A CTA's queries come by tensor map, and it may start before the routing kernel has ended.
+// Measured, call, 32 heads x 128 channels, 30011 positions (30 of 469 blocks) / 4096 (16 of 64): with the maximum of every chunk
+// 7.49 ms / 227 us, as it is 6.46 ms / 213 us.  Bound: the readers' chain per chunk (about 1800 cycles at 4096 positions, of which
+// ex2 alone takes 1024, against 1280 for the products, whose operands take shared memory's bandwidth); at 30011 the power limit as
+// well.  Slower on this form: the next chunk's scores loaded while the weights are handed over (223 us, 162 registers); queries
+// as columns, so that weights are taken only for eights or sixteens of queries some of which chose the chunk (236 us / 7.1 ms;
+// 1.9 of the 2.0 us a pair of chunks takes are shared memory's and the readers' instructions); and only the queries that chose a
+// chunk gathered for it (377 us / 9.6 ms: lists, gathers and scattered weights cost more than the products they save).
 template <int D>
 __global__ void __launch_bounds__(kThreads, 1) moba_mma_kernel(const __grid_constant__ CUtensorMap tmap,
                                                                const __grid_constant__ CUtensorMap qmap,
                                                                const __grid_constant__ CUtensorMap omap, int64_t page_cap, int S,
-                                                               int64_t len, int H, int block, int nb,
+                                                               int64_t len, int H, int BH, int set, int tiles, int block, int nb,
                                                                const uint32_t *masks, const int32_t *lists, int K, float scale_log2, int32_t *status)
 {
     using G = AttGeom<D>;
@@ -123,8 +122,10 @@ __global__ void __launch_bounds__(kThreads, 1) moba_mma_kernel(const __grid_cons
     const int words = (nb + 31) / 32;
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int bh = blockIdx.x, b = bh / H, h = bh % H;
-    const int64_t t0 = (int64_t)(gridDim.y - 1 - blockIdx.y) * (kTile * kTiles);
+    const int first = (int)(blockIdx.x / (unsigned)(set * tiles)) * set, in_set = min(set, BH - first);
+    const int rest = (int)(blockIdx.x % (unsigned)(set * tiles));
+    const int bh = first + rest % in_set, b = bh / H, h = bh % H;
+    const int64_t t0 = (int64_t)(tiles - 1 - rest / in_set) * (kTile * kTiles);
     const int n_chunks_all = (int)((min(t0 + kTile * kTiles, len) + kChunk - 1) / kChunk);
     const int cpb = block / kChunk;                              // chunks of a block
     const int ppc = kChunk / S;                                  // pages of a chunk
@@ -295,7 +296,8 @@ __global__ void __launch_bounds__(kThreads, 1) moba_mma_kernel(const __grid_cons
         int w_at = -1;
         const int32_t *mine = lists + ((int64_t)bh * len + (in ? tq : 0)) * K;
         int at = 0;                                              // without masks: the query's first list entry that is not behind the walk
-        float m = -CUDART_INF_F;                                 // what the weights are relative to (scaled, log2)
+        const int own = (int)((t0 + s * kTile + (warp & 3) * 32) / kChunk);    // the chunk of the warp's queries
+        float m = -3.0e38f;                                      // what the weights are relative to (scaled, log2)
         float2 l2 = make_float2(0.0f, 0.0f);                     // sums of the weights (even and odd positions)
         const float2 sc2 = make_float2(scale_log2, scale_log2);
         int u = 0;
@@ -328,23 +330,48 @@ __global__ void __launch_bounds__(kThreads, 1) moba_mma_kernel(const __grid_cons
             tcgen05_after_sync();
             const uint32_t ts = tl + (uint32_t)(u & 1) * kChunk;
             if (__any_sync(FULL, nv > 0)) {
-                float v[kChunk];
-                tmem_ld64(ts, v);
-                const bool cut = __any_sync(FULL, nv > 0 && nv < kChunk);
-                if (cut) {
+                uint32_t p[kChunk / 2];
+                // a block the query did not choose: 2^-3e38 = 0
+                float nm = nv > 0 ? -m : -3.0e38f;
+                float2 part = make_float2(0.0f, 0.0f);
+                auto weigh = [&](const float (&v)[32], int hf) {
+                    const float2 nm2 = make_float2(nm, nm);
 #pragma unroll
-                    for (int k = 0; k < kChunk; ++k) v[k] = k < nv ? v[k] : -CUDART_INF_F;
+                    for (int k = 0; k < 16; ++k) {
+                        const float2 x = fma2(make_float2(v[2 * k], v[2 * k + 1]), sc2, nm2);
+                        p[hf * 16 + k] = pack_bf16(exp2_fast(x.x), exp2_fast(x.y));
+                        add_bf16(part, p[hf * 16 + k]);
+                    }
+                };
+                const bool whole = c != 0 && c != own;           // its weights are taken as the scores come in
+                if (whole) {
+                    float v[2][32];
+                    tmem_ld32_start(ts, v[0]);
+                    tmem_ld32_wait(v[0]);
+                    tmem_ld32_start(ts + 32, v[1]);
+                    weigh(v[0], 0);
+                    tmem_ld32_wait(v[1]);
+                    weigh(v[1], 1);
                 }
-                float tm[4] = {v[0], v[1], v[2], v[3]};
+                const bool off = !(part.x + part.y <= kLimit);
+                if (!whole || __any_sync(FULL, off)) {
+                    // the first chunk, the query's own one, and weights that are too large, or that are none (infinite or NaN
+                    // scores, of a block that the query did not choose, too)
+                    float v[kChunk];
+                    tmem_ld64(ts, v);
+                    if (c == own) {
 #pragma unroll
-                for (int k = 4; k < kChunk; ++k) tm[k & 3] = max_nan(tm[k & 3], v[k]);
-                const float top = max_nan(max_nan(tm[0], tm[1]), max_nan(tm[2], tm[3])) * scale_log2;
-                const bool raise = nv > 0 && top > m + kRaise;
-                const bool stray = nv == 0 && !(top < CUDART_INF_F);       // infinite or NaN scores of a block the query did not choose
-                if (__any_sync(FULL, raise || stray)) {
+                        for (int k = 0; k < kChunk; ++k) v[k] = k < nv ? v[k] : -CUDART_INF_F;
+                    }
+                    const bool stray = nv == 0 && off;
 #pragma unroll
                     for (int k = 0; k < kChunk; ++k) v[k] = stray ? -CUDART_INF_F : v[k];
-                    const bool touch = raise && m > -CUDART_INF_F;         // (otherwise the query's row of O is still zero)
+                    float tm[4] = {v[0], v[1], v[2], v[3]};
+#pragma unroll
+                    for (int k = 4; k < kChunk; ++k) tm[k & 3] = fmaxf(tm[k & 3], v[k]);
+                    const float top = fmaxf(fmaxf(tm[0], tm[1]), fmaxf(tm[2], tm[3])) * scale_log2;
+                    const bool raise = nv > 0 && top > (c == 0 || off ? m : m + kRaise);
+                    const bool touch = raise && c != 0;                    // (otherwise there is no O yet)
                     const float f = touch ? exp2_fast(m - top) : 1.0f;
                     if (raise) m = top;
                     if (__any_sync(FULL, touch)) {
@@ -362,20 +389,23 @@ __global__ void __launch_bounds__(kThreads, 1) moba_mma_kernel(const __grid_cons
                             tmem_st16(tl + OFF_O + cb, x);
                         }
                     }
+                    nm = nv > 0 ? -m : -3.0e38f;
+                    part = make_float2(0.0f, 0.0f);
+#pragma unroll
+                    for (int hf = 0; hf < 2; ++hf) {
+                        float y[32];
+#pragma unroll
+                        for (int k = 0; k < 32; ++k) y[k] = v[hf * 32 + k];
+                        weigh(y, hf);
+                    }
                 }
-                // a block the query did not choose: 2^-3e38 = 0; nor do scores of -inf weigh anything while there is no other
-                const float nm = nv > 0 ? fminf(-m, 3.0e38f) : -3.0e38f;
-                const float2 nm2 = make_float2(nm, nm);
+                l2.x += part.x;
+                l2.y += part.y;
 #pragma unroll
                 for (int hf = 0; hf < 2; ++hf) {
                     uint32_t w[16];
 #pragma unroll
-                    for (int k = 0; k < 16; ++k) {
-                        const float2 x = fma2(make_float2(v[hf * 32 + 2 * k], v[hf * 32 + 2 * k + 1]), sc2, nm2);
-                        const float2 p = make_float2(exp2_fast(x.x), exp2_fast(x.y));
-                        w[k] = pack_bf16(p.x, p.y);
-                        add_bf16(l2, w[k]);
-                    }
+                    for (int k = 0; k < 16; ++k) w[k] = p[hf * 16 + k];
                     tmem_st16(ts + hf * 16, w);
                 }
             } else {                                             // none of the warp's queries chose the block
@@ -460,18 +490,20 @@ template <int D> cudaError_t attend_run(const MobaArgs &a, cudaStream_t s)
     if (e != cudaSuccess) return e;
     e = query_tensor_map(&omap, a.o, D, a.H, a.len, a.B, 32);
     if (e != cudaSuccess) return e;
-    const unsigned tiles = (unsigned)((a.len + kTile * kTiles - 1) / (kTile * kTiles));
+    const int tiles = (int)((a.len + kTile * kTiles - 1) / (kTile * kTiles));
+    const int64_t head_bytes = a.len * D * 4;
+    const int set = BH * head_bytes > kSetFrom ? (int)std::max<int64_t>(1, std::min<int64_t>(BH, kSetBytes / head_bytes)) : BH;
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute at = {};
     at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at.val.programmaticStreamSerializationAllowed = 1;
-    cfg.gridDim = dim3((unsigned)BH, tiles);
+    cfg.gridDim = dim3((unsigned)BH * (unsigned)tiles);
     cfg.blockDim = dim3(kThreads);
     cfg.dynamicSmemBytes = G::SMEM_BYTES;
     cfg.stream = s;
     cfg.attrs = &at;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, moba_mma_kernel<D>, tmap, qmap, omap, a.page_cap, a.S, a.len, a.H, a.block, nb, (const uint32_t *)a.masks,
+    return cudaLaunchKernelEx(&cfg, moba_mma_kernel<D>, tmap, qmap, omap, a.page_cap, a.S, a.len, a.H, BH, set, tiles, a.block, nb, (const uint32_t *)a.masks,
                               (const int32_t *)a.list, a.K, a.scale * 1.4426950408889634f, a.status);
 }
 
