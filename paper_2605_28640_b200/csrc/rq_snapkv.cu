@@ -232,29 +232,39 @@ __global__ void __launch_bounds__(kMmaThreads) snap_mma_kernel(const __grid_cons
     unsigned char *qs = dsm, *ks = dsm + G::Q_BYTES;
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int bh = blockIdx.y, b = bh / H, h = bh % H;
-    const int t0 = blockIdx.x * tiles_per_cta, n = min(tiles_per_cta, ntiles - t0);
+    // The second pass goes backwards, heads, runs and tiles: what the first pass read last is in L2 still, and the second pass's
+    // own reads are the first to be replaced.  Select, compact and one step, us: 12 heads x 50000 109.1 -> 103.4, 32 x 33000 177.4 ->
+    // 176.2, 32 x 131000 505 -> 495 (lowest 488 -> 477).  Of 64 channels, whose passes the readers bound, forwards (32 x 65536 197.3,
+    // backwards 199.3).  Asking the last 32 to 96 MB of the first pass to stay in L2 as well won less.
+    constexpr bool BACK = PASS == 2 && D == 128;
+    const int run = BACK ? gridDim.x - 1 - blockIdx.x : blockIdx.x;
+    const int bh = BACK ? gridDim.y - 1 - blockIdx.y : blockIdx.y, b = bh / H, h = bh % H;
+    const int t0 = run * tiles_per_cta, n = min(tiles_per_cta, ntiles - t0);
+    auto tile = [&](int i) { return BACK ? t0 + n - 1 - i : t0 + i; };
     const int64_t first_q = len - W;                           // position of query 0
     const int ppt = kMmaKeys / S;                              // pages per tile
     int n_issued = 0, n_landed = 0;                            // the producing warp: tiles whose copies were started / seen complete
 
     if (warp == 0) tmem_alloc(&tbase, TCOLS);
-    // the keys of tile t (relative to t0) into its stage: position j lives in page j / S, slot j % S of the
+    // the keys of the CTA's i-th tile into its stage: position j lives in page j / S, slot j % S of the
     // head's cache; pages past the head's last one hold somebody else's rows or nothing, and every key at
     // or beyond `len` is masked where the scores are used.  One warp.
     auto issue = [&](int i) {
         const int stage = i % NST;
         unsigned char *dst = ks + (size_t)stage * G::TILE_BYTES;
-        const int page = (int)((int64_t)bh * page_cap + (int64_t)(t0 + i) * ppt);
+        const int page = (int)((int64_t)bh * page_cap + (int64_t)tile(i) * ppt);
         mbar_expect_warp(&full[stage], G::TILE_BYTES);
 #pragma unroll
-        for (int hh = 0; hh < G::HALVES; ++hh) tma_load_4d(dst + hh * G::HALF_BYTES, &tmap, hh * 64, 0, 0, page, &full[stage]);
+        for (int hh = 0; hh < G::HALVES; ++hh) {
+            if (BACK) tma_load_4d_hint(dst + hh * G::HALF_BYTES, &tmap, hh * 64, 0, 0, page, &full[stage], l2_evict_first_policy());
+            else tma_load_4d(dst + hh * G::HALF_BYTES, &tmap, hh * 64, 0, 0, page, &full[stage]);
+        }
         n_issued = i + 1;
         // two stages keep too few bytes on their way from DRAM for its latency: the keys of a later tile of this
         // CTA are asked into L2 now, so that their copy is short when its turn comes
         if (i + kMmaAhead < n) {
 #pragma unroll
-            for (int hh = 0; hh < G::HALVES; ++hh) tma_prefetch_4d(&tmap, hh * 64, 0, 0, page + kMmaAhead * ppt);
+            for (int hh = 0; hh < G::HALVES; ++hh) tma_prefetch_4d(&tmap, hh * 64, 0, 0, page + (BACK ? -kMmaAhead : kMmaAhead) * ppt);
         }
     };
     if (warp == kMmaWarps) {                                   // copies start before anything else
@@ -277,7 +287,7 @@ __global__ void __launch_bounds__(kMmaThreads) snap_mma_kernel(const __grid_cons
         }
         for (int s = 0; s < NST && s < n; ++s) issue(s);
         for (int t = NST; t < kMmaAhead && t < n; ++t) {       // the tiles between the first copies and the first prefetch
-            const int page = (int)((int64_t)bh * page_cap + (int64_t)(t0 + t) * ppt);
+            const int page = (int)((int64_t)bh * page_cap + (int64_t)tile(t) * ppt);
 #pragma unroll
             for (int hh = 0; hh < G::HALVES; ++hh) tma_prefetch_4d(&tmap, hh * 64, 0, 0, page);
         }
@@ -337,7 +347,7 @@ __global__ void __launch_bounds__(kMmaThreads) snap_mma_kernel(const __grid_cons
         ok = mbar_wait(&bar[i & 1], (uint32_t)((i >> 1) & 1));
         if (!__all_sync(0xffffffffu, ok)) break;               // (a warp's lanes stay together: the accumulator loads are warp-wide)
         tcgen05_after_sync();
-        const int64_t j0 = (int64_t)(t0 + i) * kMmaKeys;
+        const int64_t j0 = (int64_t)tile(i) * kMmaKeys;
         const uint32_t tl = tb + (uint32_t)(i & 1) * ACC + ((uint32_t)(warp * 32) << 16);    // this warp's lanes of the accumulator
         if (PASS == 1) {
             // lane = query (both halves of the lanes hold the same 64 queries), column = key
@@ -395,7 +405,7 @@ __global__ void __launch_bounds__(kMmaThreads) snap_mma_kernel(const __grid_cons
             const float mn = fmaxf(m, o.x);
             float lt = 0.0f;
             if (mn > -CUDART_INF_F) lt = l * exp2f(m - mn) + o.y * exp2f(o.x - mn);
-            stats[((int64_t)bh * gridDim.x + blockIdx.x) * kSnapRows + row] = make_float2(mn, lt);
+            stats[((int64_t)bh * gridDim.x + run) * kSnapRows + row] = make_float2(mn, lt);
         }
     }
     tcgen05_before_sync();
