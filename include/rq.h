@@ -284,7 +284,9 @@ RQ_API int rq_snapkv_compact(const rq_cache *src, const int32_t *idx, int32_t ke
  * block's stored decayed keys) and the best are taken, equal scores to the lower block; the first
  * block and the query's own block are always taken and count inside budget_blocks; with fewer
  * blocks than that before it, a query attends everything before it.  Attention is softmax over the
- * positions <= t of the chosen blocks, on the decayed keys and values as stored.
+ * positions <= t of the chosen blocks, on the decayed keys and values as stored.  Values are summed in
+ * fp32 under weights of up to 2^8 before the sum is divided by theirs: they stay finite as long as
+ * 2^8 * attended positions * largest magnitude does (2^100 for any prompt of up to 2^19 positions).
  *   q          : [B][T][H][D] of cfg.dtype (device), T = the cache's current length; 16-byte aligned
  *   block      : 64, 128, ... (a multiple of 64 and of the page size); at most 2048 blocks per prompt
  *   o          : [B][T][H][D] of cfg.dtype (device), 16-byte aligned

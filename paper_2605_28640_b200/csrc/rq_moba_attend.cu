@@ -25,8 +25,7 @@ constexpr int kThreads = (kReadWarps + kTiles + 2) * 32;   // and one for the co
 // stay in L2 while the set's CTAs walk over them; below, all heads side by side balance better (32 heads x 30011 x 128, 492 MB:
 // 7.43 -> 7.18 ms; 32 x 9001 x 64, 74 MB: 799 -> 883 us in sets)
 constexpr int64_t kSetBytes = 64 << 20, kSetFrom = 256 << 20;
-constexpr float kLimit = 4294967296.0f;        // sum of a chunk's weights that is taken as it is (2^32)
-constexpr float kRaise = 8.0f;                 // powers of two by which a query's own chunk may exceed m
+constexpr float kRaise = 8.0f;                 // powers of two a query's maximum may grow before its output is rescaled
 
 template <int D> struct AttGeom {
     static constexpr int HALVES = D / 64;
@@ -47,6 +46,14 @@ __device__ __forceinline__ float exp2_fast(float x)
 {
     float y;
     asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+
+// the larger one; NaN if one is NaN
+__device__ __forceinline__ float max_nan(float a, float b)
+{
+    float y;
+    asm("max.NaN.f32 %0, %1, %2;" : "=f"(y) : "f"(a), "f"(b));
     return y;
 }
 
@@ -80,24 +87,26 @@ struct Walk {
 //                    the first half of their scores as the A operand of the second product; the rounded weights are
 //                    summed in fp32
 //   O += P V         accumulated in tensor memory over all chunks
-// m is the largest score of the first chunk, which every query attends: bf16 and fp32 carry weights of any size equally well,
-// so m need not be the largest of all, and the other chunks' weights are taken as their scores come in, 32 at a time, without
-// looking for a maximum first.  Only where a chunk's weights add up to more than 2^32 (or to nothing that can be compared), and
-// in the query's own chunk, whose scores have to be cut anyway, the scores are looked through, m is raised and the query's row
-// of O multiplied down.  The output is divided by the sum of the rounded weights: relative to an m that is not the maximum the
-// largest weight is not 1 exactly, and its rounding would be an error of the whole output; so it cancels.  Error against fp64
-// (2-norm; 4096 positions, 16 of 64 blocks, decayed keys, logits of 0.64): 1.66603e-3, as with every chunk's maximum looked for.
-// (A limit of 2^10 is reached all the time, as the first keys of a prompt have hardly been accumulated and score low: 213 -> 262 us.)
+// m is the query's largest score so far, but it is raised (and the query's row of O multiplied down) only when a score
+// exceeds it by more than 8 powers of two: weights of up to 256 lose nothing in bf16 and fp32, and the output is divided
+// by their sum at the end.  The sum is that of the rounded weights: relative to a lagging maximum the largest weight is not 1
+// exactly, and its rounding would be an error of the whole output; so it cancels.  Error against fp64 (2-norm; 4096 positions,
+// 16 of 64 blocks, plain keys, logits of 1.5 / 5 / 15): 2.142e-3 / 1.799e-3 / 1.509e-3.  The more queries end with an m that is not
+// their maximum, the larger it is: with the first chunk's maximum kept until a chunk's weights add up to more than 2^32, 0 / 1.4 /
+// 0.8 % more, and values above 2^92 overflow.  The first keys of a prompt have hardly been accumulated and score low, so that a fifth
+// to a half of a warp's chunks raise one of its queries; the row of O is therefore multiplied down after the chunk's weights have
+// been written, when the product before is mostly over, 32 columns at a time with the next 32 on their way.
 // Warps 0..7 read scores, warp 8 starts the tensor-map copies, warps 9 and 10 the score products of an accumulator each,
 // warp 11 the output products; they meet through mbarriers only, every wait bounded.  256 queries per CTA because keys and
 // values come from L2 for every CTA.  A CTA's queries come by tensor map, and it may start before the routing kernel has ended.
-// Measured, call, 32 heads x 128 channels, 30011 positions (30 of 469 blocks) / 4096 (16 of 64): with the maximum of every chunk
-// 7.49 ms / 227 us, as it is 6.46 ms / 213 us.  Bound: the readers' chain per chunk (about 1800 cycles at 4096 positions, of which
-// ex2 alone takes 1024, against 1280 for the products, whose operands take shared memory's bandwidth); at 30011 the power limit as
-// well.  Slower on this form: the next chunk's scores loaded while the weights are handed over (223 us, 162 registers); queries
-// as columns, so that weights are taken only for eights or sixteens of queries some of which chose the chunk (236 us / 7.1 ms;
-// 1.9 of the 2.0 us a pair of chunks takes are shared memory's and the readers' instructions); and only the queries that chose a
-// chunk gathered for it (377 us / 9.6 ms: lists, gathers and scattered weights cost more than the products they save).
+// Measured, call, 32 heads x 128 channels, 4096 positions (16 of 64 blocks) at logits of 1.4 / 5 / 11: rows multiplied down before
+// the weights, 16 columns at a time, 223.5 / 238 / 243 us; after them 217 / 227 / 231 (without ever doing it 214).  Bound: the
+// readers' chain per chunk (about 1850 cycles at 4096 positions, of which ex2 alone takes 1024, against 1280 for the products, whose
+// operands take shared memory's bandwidth); at 30011 positions the power limit as well.  Slower: weights taken before the maximum is known and again where it
+// was too far off (251 us; by halves of a chunk 240); the next chunk's scores loaded while the weights are handed over; queries as
+// columns, so that weights are taken only for eights or sixteens of queries some of which chose the chunk (236 us / 7.1 ms at 30011);
+// and only the queries that chose a chunk gathered for it (377 us / 9.6 ms: lists, gathers and scattered weights cost more than
+// the products they save).
 template <int D>
 __global__ void __launch_bounds__(kThreads, 1) moba_mma_kernel(const __grid_constant__ CUtensorMap tmap,
                                                                const __grid_constant__ CUtensorMap qmap,
@@ -296,8 +305,7 @@ __global__ void __launch_bounds__(kThreads, 1) moba_mma_kernel(const __grid_cons
         int w_at = -1;
         const int32_t *mine = lists + ((int64_t)bh * len + (in ? tq : 0)) * K;
         int at = 0;                                              // without masks: the query's first list entry that is not behind the walk
-        const int own = (int)((t0 + s * kTile + (warp & 3) * 32) / kChunk);    // the chunk of the warp's queries
-        float m = -3.0e38f;                                      // what the weights are relative to (scaled, log2)
+        float m = -CUDART_INF_F;                                 // what the weights are relative to (scaled, log2)
         float2 l2 = make_float2(0.0f, 0.0f);                     // sums of the weights (even and odd positions)
         const float2 sc2 = make_float2(scale_log2, scale_log2);
         int u = 0;
@@ -330,83 +338,64 @@ __global__ void __launch_bounds__(kThreads, 1) moba_mma_kernel(const __grid_cons
             tcgen05_after_sync();
             const uint32_t ts = tl + (uint32_t)(u & 1) * kChunk;
             if (__any_sync(FULL, nv > 0)) {
-                uint32_t p[kChunk / 2];
-                // a block the query did not choose: 2^-3e38 = 0
-                float nm = nv > 0 ? -m : -3.0e38f;
-                float2 part = make_float2(0.0f, 0.0f);
-                auto weigh = [&](const float (&v)[32], int hf) {
-                    const float2 nm2 = make_float2(nm, nm);
+                float v[kChunk];
+                tmem_ld64(ts, v);
+                const bool cut = __any_sync(FULL, nv > 0 && nv < kChunk);
+                if (cut) {
 #pragma unroll
-                    for (int k = 0; k < 16; ++k) {
-                        const float2 x = fma2(make_float2(v[2 * k], v[2 * k + 1]), sc2, nm2);
-                        p[hf * 16 + k] = pack_bf16(exp2_fast(x.x), exp2_fast(x.y));
-                        add_bf16(part, p[hf * 16 + k]);
-                    }
-                };
-                const bool whole = c != 0 && c != own;           // its weights are taken as the scores come in
-                if (whole) {
-                    float v[2][32];
-                    tmem_ld32_start(ts, v[0]);
-                    tmem_ld32_wait(v[0]);
-                    tmem_ld32_start(ts + 32, v[1]);
-                    weigh(v[0], 0);
-                    tmem_ld32_wait(v[1]);
-                    weigh(v[1], 1);
+                    for (int k = 0; k < kChunk; ++k) v[k] = k < nv ? v[k] : -CUDART_INF_F;
                 }
-                const bool off = !(part.x + part.y <= kLimit);
-                if (!whole || __any_sync(FULL, off)) {
-                    // the first chunk, the query's own one, and weights that are too large, or that are none (infinite or NaN
-                    // scores, of a block that the query did not choose, too)
-                    float v[kChunk];
-                    tmem_ld64(ts, v);
-                    if (c == own) {
+                float tm[4] = {v[0], v[1], v[2], v[3]};
 #pragma unroll
-                        for (int k = 0; k < kChunk; ++k) v[k] = k < nv ? v[k] : -CUDART_INF_F;
-                    }
-                    const bool stray = nv == 0 && off;
+                for (int k = 4; k < kChunk; ++k) tm[k & 3] = max_nan(tm[k & 3], v[k]);
+                const float top = max_nan(max_nan(tm[0], tm[1]), max_nan(tm[2], tm[3])) * scale_log2;
+                const bool raise = nv > 0 && top > m + kRaise;
+                const bool stray = nv == 0 && !(top < CUDART_INF_F);       // infinite or NaN scores of a block the query did not choose
+                bool touch = false;
+                float f = 1.0f;                                            // what the sum and the query's row of O are multiplied by
+                if (__any_sync(FULL, raise || stray)) {
 #pragma unroll
                     for (int k = 0; k < kChunk; ++k) v[k] = stray ? -CUDART_INF_F : v[k];
-                    float tm[4] = {v[0], v[1], v[2], v[3]};
-#pragma unroll
-                    for (int k = 4; k < kChunk; ++k) tm[k & 3] = fmaxf(tm[k & 3], v[k]);
-                    const float top = fmaxf(fmaxf(tm[0], tm[1]), fmaxf(tm[2], tm[3])) * scale_log2;
-                    const bool raise = nv > 0 && top > (c == 0 || off ? m : m + kRaise);
-                    const bool touch = raise && c != 0;                    // (otherwise there is no O yet)
-                    const float f = touch ? exp2_fast(m - top) : 1.0f;
+                    touch = raise && m > -CUDART_INF_F;                    // (otherwise the query's row of O is still zero)
+                    f = touch ? exp2_fast(m - top) : 1.0f;
                     if (raise) m = top;
-                    if (__any_sync(FULL, touch)) {
-                        l2.x *= f;
-                        l2.y *= f;
-                        ok = mbar_wait(&pv_done[s][(u - 1) & 1], (uint32_t)(((u - 1) >> 1) & 1));   // nothing is being added to O
-                        if (!__all_sync(FULL, ok)) break;
-                        tcgen05_after_sync();
-#pragma unroll 1
-                        for (int cb = 0; cb < D; cb += 16) {
-                            uint32_t x[16];
-                            tmem_ld16(tl + OFF_O + cb, x);
-#pragma unroll
-                            for (int k = 0; k < 16; ++k) x[k] = __float_as_uint(__uint_as_float(x[k]) * f);
-                            tmem_st16(tl + OFF_O + cb, x);
-                        }
-                    }
-                    nm = nv > 0 ? -m : -3.0e38f;
-                    part = make_float2(0.0f, 0.0f);
-#pragma unroll
-                    for (int hf = 0; hf < 2; ++hf) {
-                        float y[32];
-#pragma unroll
-                        for (int k = 0; k < 32; ++k) y[k] = v[hf * 32 + k];
-                        weigh(y, hf);
-                    }
+                    l2.x *= f;
+                    l2.y *= f;
                 }
-                l2.x += part.x;
-                l2.y += part.y;
+                // a block the query did not choose: 2^-3e38 = 0; nor do scores of -inf weigh anything while there is no other
+                const float nm = nv > 0 ? fminf(-m, 3.0e38f) : -3.0e38f;
+                const float2 nm2 = make_float2(nm, nm);
 #pragma unroll
                 for (int hf = 0; hf < 2; ++hf) {
                     uint32_t w[16];
 #pragma unroll
-                    for (int k = 0; k < 16; ++k) w[k] = p[hf * 16 + k];
+                    for (int k = 0; k < 16; ++k) {
+                        const float2 x = fma2(make_float2(v[hf * 32 + 2 * k], v[hf * 32 + 2 * k + 1]), sc2, nm2);
+                        const float2 p = make_float2(exp2_fast(x.x), exp2_fast(x.y));
+                        w[k] = pack_bf16(p.x, p.y);
+                        add_bf16(l2, w[k]);
+                    }
                     tmem_st16(ts + hf * 16, w);
+                }
+                if (__any_sync(FULL, touch)) {
+                    ok = mbar_wait(&pv_done[s][(u - 1) & 1], (uint32_t)(((u - 1) >> 1) & 1));   // nothing is being added to O
+                    if (!__all_sync(FULL, ok)) break;
+                    tcgen05_after_sync();
+                    float x[2][32];
+                    tmem_ld32_start(tl + OFF_O, x[0]);
+#pragma unroll
+                    for (int cb = 0; cb < D / 32; ++cb) {
+                        float (&y)[32] = x[cb & 1];
+                        tmem_ld32_wait(y);
+                        if (cb + 1 < D / 32) tmem_ld32_start(tl + OFF_O + (cb + 1) * 32, x[(cb + 1) & 1]);
+#pragma unroll
+                        for (int hf = 0; hf < 2; ++hf) {
+                            uint32_t w[16];
+#pragma unroll
+                            for (int k = 0; k < 16; ++k) w[k] = __float_as_uint(y[hf * 16 + k] * f);
+                            tmem_st16(tl + OFF_O + cb * 32 + hf * 16, w);
+                        }
+                    }
                 }
             } else {                                             // none of the warp's queries chose the block
                 const uint32_t z[16] = {0u, 0u, 0u, 0u, 0u, 0u, 0u, 0u, 0u, 0u, 0u, 0u, 0u, 0u, 0u, 0u};
