@@ -21,10 +21,14 @@ constexpr int kTiles = 2;                      // accumulators of a CTA: 256 con
 constexpr int kStages = 4;                     // chunks of keys, and of values, in shared memory
 constexpr int kReadWarps = 4 * kTiles;         // warps that turn scores into weights: a thread per query
 constexpr int kThreads = (kReadWarps + kTiles + 2) * 32;   // and one for the copies, two for the score products, one for the output products
-// Prompts whose keys and values, all heads together, take more than kSetFrom are worked on in sets of heads of kSetBytes, which
-// stay in L2 while the set's CTAs walk over them; below, all heads side by side balance better (32 heads x 30011 x 128, 492 MB:
-// 7.43 -> 7.18 ms; 32 x 9001 x 64, 74 MB: 799 -> 883 us in sets)
-constexpr int64_t kSetBytes = 64 << 20, kSetFrom = 256 << 20;
+// Heads are worked on in sets of up to kSetBytes of keys and values, which stay in L2 while the set's CTAs walk over them; the set
+// that is not full comes first, so that no few heads' longest walks are left for the end.  Call, us, one set / sets, 128 channels:
+// 32 heads x 30011 positions (492 MB) 7457 / 7027, 33 heads 7628 / 7251 (the smaller set last 7689), 27 x 20000 (276 MB) 2768 / 2711,
+// 17 x 30011 (261 MB) 3800 / 3703, 320 x 9486 (1.55 GB) 10266 / 9212, 320 x 3001 (492 MB) 1335 / 1275, 20 x 20000 (205 MB) 2052 / 1997,
+// 30 x 9001 (138 MB) 682 / 678; just above one set 14 x 14500 709 / 717, 7 x 30000 1498 / 1497, 50 x 4096 336 / 334.  Of 64
+// channels, whose walks the readers bound, within 1 % of each other from 102 to 737 MB.  Sets of 32 MB win less (33 heads 7224 when
+// sets of 64 and of 96 MB take 7198 and 7176; 16 x 14001 827, 764, 770).
+constexpr int64_t kSetBytes = 96 << 20;
 constexpr float kRaise = 8.0f;                 // powers of two a query's maximum may grow before its output is rescaled
 
 template <int D> struct AttGeom {
@@ -131,8 +135,10 @@ __global__ void __launch_bounds__(kThreads, 1) moba_mma_kernel(const __grid_cons
     const int words = (nb + 31) / 32;
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int first = (int)(blockIdx.x / (unsigned)(set * tiles)) * set, in_set = min(set, BH - first);
-    const int rest = (int)(blockIdx.x % (unsigned)(set * tiles));
+    const int part = BH % set;                                   // heads of the first set, if it is not full
+    const int at_tile = (int)blockIdx.x - part * tiles;
+    const int first = at_tile < 0 ? 0 : part + at_tile / (set * tiles) * set, in_set = at_tile < 0 ? part : set;
+    const int rest = at_tile < 0 ? (int)blockIdx.x : at_tile % (set * tiles);
     const int bh = first + rest % in_set, b = bh / H, h = bh % H;
     const int64_t t0 = (int64_t)(tiles - 1 - rest / in_set) * (kTile * kTiles);
     const int n_chunks_all = (int)((min(t0 + kTile * kTiles, len) + kChunk - 1) / kChunk);
@@ -481,7 +487,7 @@ template <int D> cudaError_t attend_run(const MobaArgs &a, cudaStream_t s)
     if (e != cudaSuccess) return e;
     const int tiles = (int)((a.len + kTile * kTiles - 1) / (kTile * kTiles));
     const int64_t head_bytes = a.len * D * 4;
-    const int set = BH * head_bytes > kSetFrom ? (int)std::max<int64_t>(1, std::min<int64_t>(BH, kSetBytes / head_bytes)) : BH;
+    const int set = (int)std::max<int64_t>(1, std::min<int64_t>(BH, kSetBytes / head_bytes));
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute at = {};
     at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
