@@ -232,10 +232,11 @@ __global__ void __launch_bounds__(kMmaThreads) snap_mma_kernel(const __grid_cons
     unsigned char *qs = dsm, *ks = dsm + G::Q_BYTES;
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    // The second pass goes backwards, heads, runs and tiles: what the first pass read last is in L2 still, and the second pass's
-    // own reads are the first to be replaced.  Select, compact and one step, us: 12 heads x 50000 109.1 -> 103.4, 32 x 33000 177.4 ->
-    // 176.2, 32 x 131000 505 -> 495 (lowest 488 -> 477).  Of 64 channels, whose passes the readers bound, forwards (32 x 65536 197.3,
-    // backwards 199.3).  Asking the last 32 to 96 MB of the first pass to stay in L2 as well won less.
+    // The second pass goes backwards, heads, runs and tiles: what the first pass read last is in L2 still.  Its copies mark their
+    // lines as the first to be replaced (the prefetches in front of them do not).  Select, us, forwards / backwards: 32 heads x 16384
+    // 70.3 / 61.8, x 33000 139.7 / 129.3, x 65536 233 / 221.5, x 131000 423 / 417; 12 x 50000 90.7 / 80.5; 256 x 6000 175 / 167.5; up
+    // to 50 MB of keys the same.  Of 64 channels, whose passes the readers bound, forwards (select, compact and one step, 32 x 65536:
+    // 197.3, backwards 199.3).  Asking the last 32 to 96 MB of the first pass to stay in L2 as well won less.
     constexpr bool BACK = PASS == 2 && D == 128;
     const int run = BACK ? gridDim.x - 1 - blockIdx.x : blockIdx.x;
     const int bh = BACK ? gridDim.y - 1 - blockIdx.y : blockIdx.y, b = bh / H, h = bh % H;

@@ -1,7 +1,7 @@
 """Importance of prompts that take two passes, the second from the last head, run and tile to the first: numbers of tiles that do
-not fill the last run, heads and runs in one round of CTAs and (the last case: 1920) in several, a window of fewer than 64 queries, pages of
-both sizes; against softmax in fp64.  The bound is that of the short prompts: a score of D terms carries at most D 2^-24 of its terms'
-absolute values, ex2 2^-22, the sums less; 2e-5 of the largest importance."""
+not fill the last run, heads and runs in one round of CTAs and (the last case: 1920) in several, a window of fewer than 64
+queries, pages of both sizes; against softmax in fp64. The bound is that of the short prompts: a score of D terms carries at
+most D 2^-24 of its terms' absolute values, ex2 2^-22, the sums less; 2e-5 of the largest importance."""
 import pytest
 import torch
 
