@@ -43,6 +43,12 @@ __device__ __forceinline__ float2 mul2(float2 a, float2 b)
     asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(rd) : "l"(ra), "l"(rb));
     return *reinterpret_cast<float2 *>(&rd);
 }
+__device__ __forceinline__ float2 add2(float2 a, float2 b)
+{
+    unsigned long long ra = *reinterpret_cast<unsigned long long *>(&a), rb = *reinterpret_cast<unsigned long long *>(&b), rd;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(rd) : "l"(ra), "l"(rb));
+    return *reinterpret_cast<float2 *>(&rd);
+}
 
 template <typename T> __device__ __forceinline__ void unpack16(const uint4 &r, float *out);
 template <> __device__ __forceinline__ void unpack16<bf16>(const uint4 &r, float *out)

@@ -211,8 +211,12 @@ __device__ __forceinline__ float exp2_fast(float x)
 // tmap: the cache as a rank-4 tensor (channel, slot, key / value, page over all heads), box = 64 channels
 // x the slots of a page x keys only x the pages of 128 positions, 128-byte swizzle: one copy brings one
 // 64-channel half of a tile's keys into shared memory in the layout the tensor core reads.
+// Bound: HBM (128 channels), the readers' chain per tile (64): the maxima, sums and weights of a thread run in several chains on
+// packed pairs, and what the window masks is asked for only in tiles that it cuts.  One chain each, masks everywhere / now, a call of
+// rq_snapkv_select, us: 32 heads x 131000 430 / 392, 256 x 16384 437 / 396, 32 x 16384 60.6 / 56.6, 12 x 50000 81 / 78; 64 channels,
+// 32 x 65536 176 / 149, 256 x 10000 211 / 179.
 template <int D, int PASS>
-__global__ void __launch_bounds__(kMmaThreads) snap_mma_kernel(const __grid_constant__ CUtensorMap tmap,
+__global__ void __launch_bounds__(kMmaThreads, D == 128 ? 6 : 4) snap_mma_kernel(const __grid_constant__ CUtensorMap tmap,
                                                                const __grid_constant__ CUtensorMap qmap, int64_t page_cap, int S,
                                                                int64_t len, int W, int H, float scale_log2,
                                                                float2 *stats, const float2 *rowstat, float *imp,
@@ -222,12 +226,16 @@ __global__ void __launch_bounds__(kMmaThreads) snap_mma_kernel(const __grid_cons
     constexpr int NST = kMmaStages;
     constexpr uint32_t ACC = PASS == 1 ? 128 : 64;             // columns of one accumulator
     constexpr uint32_t TCOLS = 2 * ACC;                        // two accumulators: one is filled while the other is read
+    // scores a reader takes at a time.  Of 128 channels HBM is the bound, and the registers left over let the kernel behind start
+    // beside this one (12 heads x 50000, a call 89 us with 64 at a time, 77 with 32); of 64 channels the readers are (32 x 65536 149 / 158)
+    constexpr int N = D == 128 ? 32 : 64;
     extern __shared__ __align__(1024) unsigned char dsm_raw[];
     __shared__ __align__(8) uint64_t bar[2];                   // an accumulator's product is complete
     __shared__ __align__(8) uint64_t full[NST], full_q;        // a stage's keys, the queries have landed
     __shared__ __align__(8) uint64_t acc_free[2];              // an accumulator has been read by all four warps
     __shared__ uint32_t tbase;
-    __shared__ float2 qst[kSnapRows];                          // pass 1: merge of the two halves; pass 2: (max, 1 / sum) per query
+    __shared__ float2 qst[kSnapRows];                          // pass 1: merge of the two halves
+    __shared__ __align__(16) float q_nm[kSnapRows], q_il[kSnapRows];   // pass 2: -maximum and 1 / sum of every query
     unsigned char *dsm = dsm_raw + ((1024u - (smem_addr(dsm_raw) & 1023u)) & 1023u);
     unsigned char *qs = dsm, *ks = dsm + G::Q_BYTES;
 
@@ -339,7 +347,8 @@ __global__ void __launch_bounds__(kMmaThreads) snap_mma_kernel(const __grid_cons
         grid_dependency_wait();                                // the statistics come from the kernel before, the keys do not
         if (tid < kSnapRows) {
             const float2 f = tid < W ? __ldcg(rowstat + (int64_t)bh * kSnapRows + tid) : make_float2(0.0f, 1.0f);
-            qst[tid] = make_float2(f.x, 1.0f / f.y);
+            q_nm[tid] = -f.x;
+            q_il[tid] = 1.0f / f.y;
         }
         asm volatile("bar.sync 1, %0;" ::"n"(kMmaWarps * 32) : "memory");
     }
@@ -350,47 +359,68 @@ __global__ void __launch_bounds__(kMmaThreads) snap_mma_kernel(const __grid_cons
         tcgen05_after_sync();
         const int64_t j0 = (int64_t)tile(i) * kMmaKeys;
         const uint32_t tl = tb + (uint32_t)(i & 1) * ACC + ((uint32_t)(warp * 32) << 16);    // this warp's lanes of the accumulator
+        const bool cut = W < kSnapRows || j0 + kMmaKeys - 1 > first_q;     // some key of the tile is not seen by all 64 queries
+        const float2 sc2 = make_float2(scale_log2, scale_log2);
+        float v[N];
+        auto load = [&](int c0) {
+            if constexpr (N == 32) tmem_ld32(tl + (uint32_t)c0, v);
+            else tmem_ld64(tl + (uint32_t)c0, v);
+        };
         if (PASS == 1) {
             // lane = query (both halves of the lanes hold the same 64 queries), column = key
-            const int64_t pq = first_q + row;                  // query `row` sees keys up to its own position
 #pragma unroll 1
-            for (int cb = 0; cb < 64; cb += 32) {
-                float v[32];
-                tmem_ld32(tl + (uint32_t)(half * 64 + cb), v);
-                const int64_t jb = j0 + half * 64 + cb;
-                if (row < W && jb <= pq) {
-                    const int nv = (int)min((int64_t)32, pq - jb + 1);   // visible keys among these 32
-                    float tm = -CUDART_INF_F;
+            for (int cb = 0; cb < 64; cb += N) {
+                load(half * 64 + cb);
+                int nv = N;                                    // visible keys among these: up to the query's own position
+                if (cut) {
+                    nv = row < W ? (int)max((int64_t)0, min((int64_t)N, first_q + row - (j0 + half * 64 + cb) + 1)) : 0;
 #pragma unroll
-                    for (int c = 0; c < 32; ++c) {
-                        v[c] = c < nv ? v[c] * scale_log2 : -CUDART_INF_F;
-                        tm = fmaxf(tm, v[c]);
+                    for (int c = 0; c < N; ++c) v[c] = c < nv ? v[c] : -CUDART_INF_F;
+                }
+                float tm[4] = {v[0], v[1], v[2], v[3]};
+#pragma unroll
+                for (int c = 4; c < N; ++c) tm[c & 3] = fmaxf(tm[c & 3], v[c]);
+                if (nv > 0) {                                  // (so that the maximum is that of a key)
+                    const float mn = fmaxf(m, fmaxf(fmaxf(tm[0], tm[1]), fmaxf(tm[2], tm[3])) * scale_log2);   // (the scale is positive)
+                    const float2 nm2 = make_float2(-mn, -mn);
+                    float2 sum[2] = {make_float2(0.0f, 0.0f), make_float2(0.0f, 0.0f)};
+#pragma unroll
+                    for (int c = 0; c < N; c += 2) {
+                        const float2 x = fma2(make_float2(v[c], v[c + 1]), sc2, nm2);
+                        sum[(c >> 1) & 1] = add2(sum[(c >> 1) & 1], make_float2(exp2_fast(x.x), exp2_fast(x.y)));
                     }
-                    const float mn = fmaxf(m, tm);             // finite: at least one key is visible
-                    float sum = 0.0f;
-#pragma unroll
-                    for (int c = 0; c < 32; ++c) sum += exp2_fast(v[c] - mn);
-                    l = l * exp2_fast(m - mn) + sum;           // 2^(-inf) = 0 the first time
+                    const float2 both = add2(sum[0], sum[1]);
+                    l = l * exp2_fast(m - mn) + (both.x + both.y);         // 2^(-inf) = 0 the first time
                     m = mn;
                 }
             }
         } else {
-            // lane = key, column = query: the key's weights summed over the queries that see it
+            // lane = key, column = query: the key's weights summed over the queries that see it, in the same order for every key
             const int64_t j = j0 + tid;
-            const int q_lo = (int)max((int64_t)0, j - first_q);
-            float acc = 0.0f;
+            const int q_lo = (int)min((int64_t)64, max((int64_t)0, j - first_q));
+            float2 acc[2] = {make_float2(0.0f, 0.0f), make_float2(0.0f, 0.0f)};
 #pragma unroll 1
-            for (int cb = 0; cb < kSnapRows; cb += 32) {
-                float v[32];
-                tmem_ld32(tl + (uint32_t)cb, v);
+            for (int cb = 0; cb < kSnapRows; cb += N) {
+                load(cb);
 #pragma unroll
-                for (int c = 0; c < 32; ++c) {
+                for (int c = 0; c < N; c += 4) {
                     const int q = cb + c;
-                    const float2 st = qst[q];
-                    if (q < W && q >= q_lo) acc = fmaf(exp2_fast(fmaf(v[c], scale_log2, -st.x)), st.y, acc);
+                    const float4 nm = *reinterpret_cast<const float4 *>(&q_nm[q]), il = *reinterpret_cast<const float4 *>(&q_il[q]);
+                    const float2 x = fma2(make_float2(v[c], v[c + 1]), sc2, make_float2(nm.x, nm.y));
+                    const float2 y = fma2(make_float2(v[c + 2], v[c + 3]), sc2, make_float2(nm.z, nm.w));
+                    float2 e = make_float2(exp2_fast(x.x), exp2_fast(x.y)), f = make_float2(exp2_fast(y.x), exp2_fast(y.y));
+                    if (cut) {
+                        e.x = q < W && q >= q_lo ? e.x : 0.0f;
+                        e.y = q + 1 < W && q + 1 >= q_lo ? e.y : 0.0f;
+                        f.x = q + 2 < W && q + 2 >= q_lo ? f.x : 0.0f;
+                        f.y = q + 3 < W && q + 3 >= q_lo ? f.y : 0.0f;
+                    }
+                    acc[0] = fma2(e, make_float2(il.x, il.y), acc[0]);
+                    acc[1] = fma2(f, make_float2(il.z, il.w), acc[1]);
                 }
             }
-            if (j < len) imp[(int64_t)bh * len + j] = acc;
+            const float2 both = add2(acc[0], acc[1]);
+            if (j < len) imp[(int64_t)bh * len + j] = both.x + both.y;
         }
         tcgen05_before_sync();
         mbar_arrive(&acc_free[i & 1]);                         // this thread has read the accumulator

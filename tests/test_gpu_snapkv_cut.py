@@ -1,0 +1,36 @@
+"""Importance of prompts that take two passes, where keys the whole window sees share a tile with keys it does not: equal keys have
+equal importance, bit for bit, whichever of the two kinds of tile they lie in; against softmax in fp64 within
+2e-5 of the largest importance (a score of D terms carries at most D 2^-24 of its terms' absolute values, ex2 2^-22)."""
+import pytest
+import torch
+
+import paper_2605_28640_b200 as rq
+
+pytestmark = pytest.mark.gpu
+DEV = "cuda"
+
+
+@pytest.mark.parametrize("scale", [0.0, 0.4])
+@pytest.mark.parametrize("BH,T,D", [(2, 4224, 128), (3, 4300, 64), (2, 8191, 128), (1, 40001, 64)])
+def test_equal_keys_in_both_kinds_of_tile(BH, T, D, scale, W=64, S=16):
+    g = torch.Generator(device=DEV)
+    g.manual_seed(T)
+    cache = rq.Cache(1, BH, D, S, T, torch.bfloat16)
+    k = torch.randn(1, T, BH, D, generator=g, device=DEV, dtype=torch.bfloat16)
+    k[:, T - W - 1] = k[:, 0]                                     # the last position before the window
+    z = torch.zeros_like(k)
+    rq.rq_build_cache(cache.handle, k, z, z)                      # zero gates: the cache holds the keys themselves
+    qw = torch.randn(1, W, BH, D, generator=g, device=DEV, dtype=torch.bfloat16)
+    scratch = torch.empty(rq.rq_snapkv_scratch_bytes(cache.handle), dtype=torch.uint8, device=DEV)
+    idx = torch.empty(1, BH, W, dtype=torch.int32, device=DEV)
+    imp = torch.full((1, BH, T), float("nan"), dtype=torch.float32, device=DEV)
+    rq.rq_snapkv_select(cache.handle, qw, W, W, scale, idx, imp, scratch)
+    torch.cuda.synchronize()
+    assert rq.rq_device_status(cache.handle) == rq.RQ_OK
+    pos = torch.arange(T, device=DEV)
+    for h in range(BH):
+        s = qw[0, :, h].double() @ k[0, :, h].double().T * (scale or D ** -0.5)
+        s[pos[None, :] > (T - W + torch.arange(W, device=DEV))[:, None]] = float("-inf")
+        want = torch.softmax(s, -1).sum(0)
+        assert (imp[0, h].double() - want).abs().max().item() <= 2e-5 * want.max().item()
+    assert torch.equal(imp[0, :, 0], imp[0, :, T - W - 1])
