@@ -454,7 +454,9 @@ __global__ void __launch_bounds__(kMmaThreads, D == 128 ? 6 : 4) snap_mma_kernel
 // Warps 0..7 read the accumulators (a lane per key, a warp per half of the queries), warp 8 copies and multiplies.  The
 // maximum is the head's before a weight is taken, as in the two-pass kernels: equal keys get equal importance wherever they
 // lie.  Bound by the chain of a CTA (copies, two exchanges over the cluster, three walks over the scores: 11 us for 512
-// keys), which two CTAs per SM overlap.  256 heads x 4096 keys x 128 channels: 124 (two passes and the merge) -> 95 us.
+// keys), which two CTAs per SM overlap.  256 heads x 4096 keys x 128 channels: 124 (two passes and the merge) -> 95 us.  Walks on packed
+// pairs, scaled after the maximum, a call of rq_snapkv_select, us, before / now: 256 heads x 4096 110.6 / 108.5, 64 channels 100.9 /
+// 98.5, 128 x 2000 30.1 / 28.7.
 // Eight tiles per CTA, for up to 8192 positions, fill tensor memory with one CTA per SM and were slower than two passes at
 // every number of heads (8192 positions, a call, us: 4 heads 24 / 20, 32 heads 55 / 40, 256 heads 266 / 229).
 // CTAs wait for one another with their tensor memory in hand, so a CTA must never stand in tcgen05.alloc behind another
@@ -511,7 +513,7 @@ __global__ void __launch_bounds__(kOnceThreads, 2) snap_once_kernel(const __grid
     __shared__ uint32_t tbase;
     __shared__ float red[4][kSnapRows];                        // per quarter of the keys and query
     __shared__ float xch[2][kOnceCluster][kSnapRows];          // what every CTA of the cluster found: maxima, sums
-    __shared__ __align__(16) float ref[kSnapRows];             // per query: the maximum, then 1 / sum
+    __shared__ __align__(16) float ref[kSnapRows];             // per query: -maximum, then 1 / sum
     __shared__ float part[RT][kMmaKeys];                       // importance of a key from the upper half of the queries
     cg::cluster_group cl = cg::this_cluster();
     cg::cluster_group::arrival_token started = cl.barrier_arrive();
@@ -603,10 +605,10 @@ __global__ void __launch_bounds__(kOnceThreads, 2) snap_once_kernel(const __grid
             if (cut(i)) {
                 const int c_lo = first_seen(i);
 #pragma unroll
-                for (int c = 0; c < 32; ++c) a[c] = c >= c_lo && c < c_end ? fmaxf(a[c], v[c] * scale_log2) : a[c];
+                for (int c = 0; c < 32; ++c) a[c] = c >= c_lo && c < c_end ? fmaxf(a[c], v[c]) : a[c];
             } else {
 #pragma unroll
-                for (int c = 0; c < 32; ++c) a[c] = fmaxf(a[c], v[c] * scale_log2);
+                for (int c = 0; c < 32; ++c) a[c] = fmaxf(a[c], v[c]);
             }
         }
         red[quad][half * 32 + lane] = lanes_reduce<true>(a, lane);
@@ -624,10 +626,11 @@ __global__ void __launch_bounds__(kOnceThreads, 2) snap_once_kernel(const __grid
         return x;
     };
     cl.barrier_wait(std::move(started));                       // every CTA of the cluster runs: its shared memory may be written
-    const float top = exchange(0, [](float x, float y) { return fmaxf(x, y); });
-    if (tid < kSnapRows) ref[tid] = top > -CUDART_INF_F ? top : 0.0f;
+    const float top = exchange(0, [](float x, float y) { return fmaxf(x, y); }) * scale_log2;         // (the scale is positive)
+    if (tid < kSnapRows) ref[tid] = top > -CUDART_INF_F ? -top : 0.0f;
     __syncthreads();
     if (reader) {
+        const float2 sc2 = make_float2(scale_log2, scale_log2);
 #pragma unroll
         for (int c = 0; c < 32; ++c) a[c] = 0.0f;
         if (ok) {
@@ -636,11 +639,13 @@ __global__ void __launch_bounds__(kOnceThreads, 2) snap_once_kernel(const __grid
                 tmem_ld32(tl + (uint32_t)i * kSnapRows, v);
 #pragma unroll
                 for (int c = 0; c < 32; c += 4) {
-                    const float4 m = *reinterpret_cast<const float4 *>(&ref[half * 32 + c]);
-                    v[c] = exp2_fast(fmaf(v[c], scale_log2, -m.x));
-                    v[c + 1] = exp2_fast(fmaf(v[c + 1], scale_log2, -m.y));
-                    v[c + 2] = exp2_fast(fmaf(v[c + 2], scale_log2, -m.z));
-                    v[c + 3] = exp2_fast(fmaf(v[c + 3], scale_log2, -m.w));
+                    const float4 nm = *reinterpret_cast<const float4 *>(&ref[half * 32 + c]);
+                    const float2 x = fma2(make_float2(v[c], v[c + 1]), sc2, make_float2(nm.x, nm.y));
+                    const float2 y = fma2(make_float2(v[c + 2], v[c + 3]), sc2, make_float2(nm.z, nm.w));
+                    v[c] = exp2_fast(x.x);
+                    v[c + 1] = exp2_fast(x.y);
+                    v[c + 2] = exp2_fast(y.x);
+                    v[c + 3] = exp2_fast(y.y);
                 }
                 if (cut(i)) {
                     const int c_lo = first_seen(i);
@@ -651,9 +656,13 @@ __global__ void __launch_bounds__(kOnceThreads, 2) snap_once_kernel(const __grid
                 for (int hf = 0; hf < 2; ++hf) {
                     uint32_t w[16];
 #pragma unroll
-                    for (int c = 0; c < 16; ++c) {
-                        a[hf * 16 + c] += v[hf * 16 + c];
-                        w[c] = __float_as_uint(v[hf * 16 + c]);
+                    for (int c = 0; c < 16; c += 2) {
+                        const int k = hf * 16 + c;
+                        const float2 x = add2(make_float2(a[k], a[k + 1]), make_float2(v[k], v[k + 1]));
+                        a[k] = x.x;
+                        a[k + 1] = x.y;
+                        w[c] = __float_as_uint(v[k]);
+                        w[c + 1] = __float_as_uint(v[k + 1]);
                     }
                     tmem_st16(tl + (uint32_t)i * kSnapRows + hf * 16, w);
                 }
@@ -671,15 +680,15 @@ __global__ void __launch_bounds__(kOnceThreads, 2) snap_once_kernel(const __grid
         for (int i = 0; i < RT; ++i) {
             if (i >= n) break;
             tmem_ld32(tl + (uint32_t)i * kSnapRows, v);
-            float s = 0.0f;
+            float2 s2[2] = {make_float2(0.0f, 0.0f), make_float2(0.0f, 0.0f)};
 #pragma unroll
             for (int c = 0; c < 32; c += 4) {
                 const float4 f = *reinterpret_cast<const float4 *>(&ref[half * 32 + c]);
-                s = fmaf(v[c], f.x, s);
-                s = fmaf(v[c + 1], f.y, s);
-                s = fmaf(v[c + 2], f.z, s);
-                s = fmaf(v[c + 3], f.w, s);
+                s2[0] = fma2(make_float2(v[c], v[c + 1]), make_float2(f.x, f.y), s2[0]);
+                s2[1] = fma2(make_float2(v[c + 2], v[c + 3]), make_float2(f.z, f.w), s2[1]);
             }
+            const float2 both = add2(s2[0], s2[1]);
+            const float s = both.x + both.y;
             acc[i] = s;
             if (half) part[i][row] = s;
         }
