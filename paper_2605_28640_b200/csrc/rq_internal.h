@@ -192,12 +192,15 @@ struct MobaArgs {
     // room than the lists), and as lists [BH][len][K], ascending, -1 beyond.  One of the two may be NULL for bf16 caches
     uint32_t *masks;
     int32_t *list;
+    // bf16 caches: the representatives as three bf16 terms, 64 blocks of a head at a time as the routing's tensor core reads them,
+    // in what the scratch has left; NULL where that is too little
+    void *terms;
     void *o;            // [B][len][H][D]
     int32_t *status;    // the cache's device status word
 };
 constexpr int kMobaMaxBlocks = 2048;           // blocks of a prompt at most
 size_t moba_scratch_bytes(int BH, int64_t len, int D, int block, int K);
-// means, masks and list of `a` (its shape filled in) from the scratch and, if not NULL, the caller's lists
+// means, masks, list and terms of `a` (its shape filled in) from the scratch and, if not NULL, the caller's lists
 void moba_carve(void *scratch, int32_t *blocks_out, MobaArgs &a);
 cudaError_t launch_moba(const MobaArgs &a, cudaStream_t s);
 // bf16 caches: representatives and routing (rq_moba_route.cu)

@@ -25,14 +25,20 @@ constexpr int kRouteQueries = 128;             // queries of a CTA: the lanes of
 constexpr int kRouteThreads = 512;             // four threads per query, each a quarter of the score words
 constexpr int kRouteGroup = 64;                // blocks of one product (N)
 constexpr int kPanelGroups = 8;                // groups whose scores fit in tensor memory at once (512 columns)
-constexpr int kRouteBins = 64;                 // value buckets of the threshold search
 constexpr int kRouteCap = 16;                  // blocks of the threshold's bucket that are ranked directly
+constexpr int kRoutePitch = kRouteQueries + 1; // words between the mask words of a query: read by word and by query without conflicts
+// value buckets of the threshold search: by form (up to 64 blocks; up to 512, one panel; more)
+constexpr int route_bins(int form) { return form == 2 ? 64 : 128; }
+
+// what a term leaves of a number for the next ones: exact; of an infinite mean, nothing
+__device__ __forceinline__ float term_rest(float x, float term) { return fabsf(term) == CUDART_INF_F ? 0.0f : x - term; }
 
 // ---------------------------------------------------------------- block representatives
 // Grid (ceil(blocks / R), heads), R = 256 / (D / 2) blocks per CTA, a thread per two channels of a block.  The sum
 // runs over the block's valid positions in order.
+// terms: the same numbers as three bf16 terms each, for 64 blocks at a time in the layout the tensor core reads (NULL: not wanted).
 __global__ void __launch_bounds__(256) moba_means_bf16_kernel(const bf16 *kv, int64_t page_cap, int S, int D, int64_t len, int block,
-                                                             float *means, int nb)
+                                                             float *means, int nb, unsigned char *terms)
 {
     const int per = D / 2, r = threadIdx.x / per, c = 2 * (threadIdx.x % per);
     const int j = blockIdx.x * (256 / per) + r, bh = blockIdx.y;
@@ -58,26 +64,35 @@ __global__ void __launch_bounds__(256) moba_means_bf16_kernel(const bf16 *kv, in
     }
     const float n = (float)(hi - lo), m0 = s0 / n, m1 = s1 / n;
     *reinterpret_cast<float2 *>(means + ((int64_t)bh * nb + j) * D + c) = make_float2(m0, m1);
+    if (terms) {
+        const int plane = D / 64 * kRouteGroup * 128, groups = (nb + kRouteGroup - 1) / kRouteGroup;
+        unsigned char *dst = terms + ((int64_t)bh * groups + j / kRouteGroup) * 3 * plane + (c >> 6) * (kRouteGroup * 128) +
+                             umma_sw128_offset(j % kRouteGroup, (c & 63) >> 3) + (c & 7) * 2;
+        float x = m0, y = m1;
+#pragma unroll
+        for (int t = 0; t < 3; ++t) {
+            const uint32_t w = pack_bf16(x, y);
+            *reinterpret_cast<uint32_t *>(dst + t * plane) = w;
+            x = term_rest(x, bf16lo(w));
+            y = term_rest(y, bf16hi(w));
+        }
+    }
 }
 
 // ---------------------------------------------------------------- routing
-template <int D> struct RouteGeom {
+template <int D, int FORM> struct RouteGeom {
     static constexpr int HALVES = D / 64;
     static constexpr int Q_BYTES = HALVES * kRouteQueries * 128;
     static constexpr int PLANE_BYTES = HALVES * kRouteGroup * 128;
     static constexpr int GROUP_BYTES = 3 * PLANE_BYTES;
-    static constexpr int WORK_BYTES = kRouteBins * kRouteQueries * 4 + kRouteCap * kRouteQueries * 6;   // buckets, ranked blocks
-    static constexpr int SMALL_BYTES = (12 + 6) * kRouteQueries * 4;
+    static constexpr int BINS = route_bins(FORM);
+    static constexpr int WORK_BYTES = (BINS + 1) * kRouteQueries * 4 + kRouteCap * kRouteQueries * 8;   // buckets, ranked blocks
+    static constexpr int SMALL_BYTES = (12 + 7) * kRouteQueries * 4;
     // a prompt of one panel is done with queries and representatives when the buckets are needed, so these share the space
-    static __host__ __device__ int front_bytes(bool one_panel)
-    {
-        const int qb = Q_BYTES + GROUP_BYTES;
-        return one_panel ? (qb > WORK_BYTES ? qb : WORK_BYTES) : qb + WORK_BYTES;
-    }
-    static int smem_bytes(bool one_panel, int words)
-    {
-        return 1024 + front_bytes(one_panel) + 2 * words * kRouteQueries * 4 + SMALL_BYTES;
-    }
+    static constexpr int QB_BYTES = Q_BYTES + GROUP_BYTES;
+    static constexpr int OFF_WORK = FORM < 2 ? 0 : QB_BYTES;
+    static constexpr int FRONT_BYTES = ((FORM < 2 ? (QB_BYTES > WORK_BYTES ? QB_BYTES : WORK_BYTES) : QB_BYTES + WORK_BYTES) + 15) & ~15;
+    static __host__ __device__ int smem_bytes(int words) { return 1024 + FRONT_BYTES + 2 * words * kRoutePitch * 4 + SMALL_BYTES; }
 };
 
 // order-preserving image of a score; -0 counts as +0
@@ -86,60 +101,66 @@ __device__ __forceinline__ uint32_t score_key(float v)
     const uint32_t b = __float_as_uint(v + 0.0f);
     return b ^ ((b >> 31) ? 0xffffffffu : 0x80000000u);
 }
-// Value bucket of a score between the query's smallest and largest: monotone in v, 0 .. kRouteBins - 1.
-__device__ __forceinline__ uint32_t score_bin(float v, float lo, float inv)
+// Value bucket of a score between the query's smallest and largest: monotone in v, 0 .. NB - 1; as a float, 2^23 + bucket
+// (scores that are not finite may exceed the last one).
+__device__ __forceinline__ float score_place(float v, float lo, float inv) { return fmaf(v - lo, inv, 8388609.0f); }
+template <int NB> __device__ __forceinline__ uint32_t score_bin(float v, float lo, float inv)
 {
-    return min(__float_as_uint(fmaf(v - lo, inv, 8388609.0f)) - 0x4B000000u, (uint32_t)(kRouteBins - 1));
+    return min(__float_as_uint(score_place(v, lo, inv)) - 0x4B000000u, (uint32_t)(NB - 1));
 }
 
 // Grid (heads, tiles of 128 queries; the tiles of the last queries first: their work is the largest).  Bound by the
-// instructions of the three passes over the scores (smallest and largest, buckets, mask; about a dozen per score and
-// 32 queries), which is why a pass that ranks every candidate, or one that takes one block per round, is so much
-// slower.  Per query:
+// instructions of the three passes over the scores (smallest and largest, buckets, mask) and the chain of copies, products and
+// barriers in between, which two CTAs per SM overlap (up to 256 blocks; beyond, tensor memory holds one CTA's scores).  Per query:
 //   1. smallest and largest score of its candidates (the complete blocks between the first and the query's own);
-//   2. 64 value buckets between them: the bucket that holds the last block taken, and how many of it are wanted;
+//   2. value buckets between them: the bucket that holds the last block taken, and how many of it are wanted;
 //   3. blocks of higher buckets into the mask; those of the threshold's bucket are ranked against each other by
 //      (score, lower block first).
 // A threshold bucket of more than 16 blocks is cut further by buckets on the scores' integer images until at most 16
 // are left or all left are equal (equal scores: the lowest blocks).  More than 512 blocks are taken in panels of 512,
 // whose scores are computed again for each pass (the tensor cores have nothing else to do here).
-// Measured, 32 heads x 128 channels: 4096 queries, 16 of 64 blocks each, 158 -> 42 us; 30011 queries, 30 of 469 blocks
-// each, 28.9 -> 1.0 ms.  (Before: fp32 FMA scores, a lane per block, then a bit-wise vote search up to 128 blocks and one
-// round per taken block beyond.  Of the former: queries by tensor map and four product steps per election 58 -> 52 us,
-// candidates noted by one atomic per word instead of one each 52 -> 47 us, half words for up to 64 blocks 47 -> 42 us.)
-// HALF: prompts of at most 64 blocks, whose two words of scores are taken by half words, so that all four threads of a query
-// have some.
-template <int D, bool HALF>
-__global__ void __launch_bounds__(kRouteThreads, 2) moba_route_mma_kernel(const __grid_constant__ CUtensorMap qmap, const float *means, int64_t len, int H,
+// The representatives' terms come by bulk copies as the means' kernel laid them out, where the scratch had room for them behind
+// the masks; cutting them for every tile of queries again took a sixth of the kernel's instructions and its longest chain.
+// FORM: 0 for prompts of at most 64 blocks, whose two words of scores are taken by half words, so that all four threads of a query
+// have some; 1 for up to 512, one panel; 2 beyond.
+// Measured, 32 heads x 128 channels, before / now: 4096 queries, 16 of 64 blocks each, 42.5 -> 32 us; 30011 queries, 30 of 469 blocks
+// each, 1020 -> 650 us.  In steps: counting without branches and one comparison less per score 940 us; terms by copies, 128 buckets
+// instead of 64 (fewer blocks to rank), mask words without bank conflicts 690 us; blocks to rank read again by column instead of
+// picked from registers, divisions out of the stores of the masks 650 us.  The threshold by rounds of counting three keys at a time in
+// the registers of a query's four threads instead of buckets: 49.7 us for the 4096 queries.
+template <int D, int FORM>
+__global__ void __launch_bounds__(kRouteThreads, 2) moba_route_mma_kernel(const __grid_constant__ CUtensorMap qmap, const float *means, const unsigned char *terms, int64_t len, int H,
                                                                       int block, int nb, int K, int words, uint32_t *masks,
                                                                       int32_t *list, int32_t *status)
 {
-    using G = RouteGeom<D>;
-    constexpr int NQ = kRouteQueries, NB = kRouteBins, CAP = kRouteCap;
+    using G = RouteGeom<D, FORM>;
+    constexpr bool HALF = FORM == 0;
+    constexpr int NQ = kRouteQueries, NB = G::BINS, CAP = kRouteCap, MP = kRoutePitch;
     extern __shared__ __align__(1024) unsigned char rsm_raw[];
-    __shared__ __align__(8) uint64_t full_q, done;                                    // a product is complete
+    __shared__ __align__(8) uint64_t full_q, done[kPanelGroups];                      // the queries have landed, a group's products are complete
+    __shared__ __align__(8) uint64_t full_t[3], free_t[3];                            // a plane of terms has landed, has been read
     __shared__ uint32_t tbase;
     unsigned char *sm = rsm_raw + ((1024u - (smem_addr(rsm_raw) & 1023u)) & 1023u);
     const int groups_all = (nb + kRouteGroup - 1) / kRouteGroup;
-    const bool one_panel_launch = groups_all <= kPanelGroups;
     unsigned char *qs = sm, *bs = sm + G::Q_BYTES;
-    uint32_t *hist = reinterpret_cast<uint32_t *>(one_panel_launch ? sm : sm + G::Q_BYTES + G::GROUP_BYTES);   // [NB][NQ]
-    uint32_t *ckey = hist + NB * NQ;                                           // [CAP][NQ]
-    uint16_t *cidx = reinterpret_cast<uint16_t *>(ckey + CAP * NQ);            // [CAP][NQ]
-    uint32_t *mk = reinterpret_cast<uint32_t *>(sm + G::front_bytes(one_panel_launch));   // [words][NQ] chosen blocks
-    uint32_t *tie = mk + words * NQ;                                           // [words][NQ] equal scores at the threshold
-    uint32_t *part_a = tie + words * NQ, *part_b = part_a + 4 * NQ, *part_c = part_b + 4 * NQ;    // [4][NQ] each
+    uint32_t *hist = reinterpret_cast<uint32_t *>(sm + G::OFF_WORK);              // [NB + 1][NQ]: the last for what does not count
+    uint2 *ranked = reinterpret_cast<uint2 *>(hist + (NB + 1) * NQ);           // [CAP][NQ] blocks of the threshold's bucket: key, block
+    uint32_t *mk = reinterpret_cast<uint32_t *>(sm + G::FRONT_BYTES);          // [words][MP] chosen blocks
+    uint32_t *tie = mk + words * MP;                                           // [words][MP] equal scores at the threshold
+    uint32_t *part_a = tie + words * MP, *part_b = part_a + 4 * NQ, *part_c = part_b + 4 * NQ;    // [4][NQ] each
     int32_t *s_tb = reinterpret_cast<int32_t *>(part_c + 4 * NQ), *s_need = s_tb + NQ, *s_cnt = s_need + NQ;
     uint32_t *s_klo = reinterpret_cast<uint32_t *>(s_cnt + NQ), *s_khi = s_klo + NQ, *s_n = s_khi + NQ;
+    int32_t *s_own = reinterpret_cast<int32_t *>(s_n + NQ);
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int ql = (warp & 3) * 32 + lane, part = warp >> 2;                   // this thread's query and quarter of the words
     const int bh = blockIdx.x, b = bh / H, h = bh % H;
     const int64_t t0 = (int64_t)(gridDim.y - 1 - blockIdx.y) * NQ, t = t0 + ql;
-    const int own = (int)(t / block), own_last = (int)((min(t0 + NQ, len) - 1) / block), own_first = (int)(t0 / block);
+    const int own = (int)t / block, own_last = ((int)min(t0 + NQ, len) - 1) / block, own_first = (int)t0 / block;
     const int want = K - 2;                                                    // beside the first block and the query's own
     const bool active = t < len && K < own + 1;                                // otherwise everything up to the query is taken
     const int c_hi = active ? own : 0;                                         // candidates: blocks 1 .. c_hi - 1
+    const int c_all = own_first >= K ? own_first : 0;                          // every query of the CTA has blocks 1 .. c_all - 1
     const bool any = K < own_last + 1;                                         // some query of the CTA has to choose
     const int groups = any ? (own_last + kRouteGroup - 1) / kRouteGroup : 0;   // groups that hold blocks 0 .. own_last - 1
     const int panels = (groups + kPanelGroups - 1) / kPanelGroups;
@@ -147,37 +168,97 @@ __global__ void __launch_bounds__(kRouteThreads, 2) moba_route_mma_kernel(const 
     uint32_t tcols = kRouteGroup;
     while ((int)tcols < min(groups, kPanelGroups) * kRouteGroup) tcols *= 2;
 
-    for (int i = tid; i < 2 * words * NQ; i += kRouteThreads) mk[i] = 0u;      // mk and tie
+    for (int i = tid; i < 2 * words * MP; i += kRouteThreads) mk[i] = 0u;      // mk and tie
     if (part == 0) {
-        s_tb[ql] = NB; s_need[ql] = 0; s_cnt[ql] = 0;
+        s_tb[ql] = NB; s_need[ql] = 0; s_cnt[ql] = 0; s_own[ql] = own;
         s_klo[ql] = 0u; s_khi[ql] = 0xffffffffu; s_n[ql] = 0u;
     }
     bool ok = true;
     if (any) {
-        if (tid == 0) {
-            mbar_init(&done, 1);
-            mbar_init(&full_q, 1);
-            mbar_init_fence();
+        // the i-th plane of terms of the panel that starts with group g0 (a whole warp; stage i % 3, the smallest terms first)
+        auto issue = [&](int g0, int i) {
+            const int st = i % 3, off = (i / 3) * G::GROUP_BYTES + (2 - st) * G::PLANE_BYTES;
+            mbar_expect_warp(&full_t[st], G::PLANE_BYTES);
+            if (lane == 0) bulk_g2s(bs + (2 - st) * G::PLANE_BYTES, terms + ((int64_t)bh * groups_all + g0) * G::GROUP_BYTES + off, G::PLANE_BYTES, &full_t[st]);
+        };
+        if (warp == 0) {                                                       // copies start before anything else
+            if (lane == 0) {
+                for (int i = 0; i < kPanelGroups; ++i) mbar_init(&done[i], 1);
+                for (int i = 0; i < 3; ++i) { mbar_init(&full_t[i], 1); mbar_init(&free_t[i], 1); }
+                mbar_init(&full_q, 1);
+                mbar_init_fence();
+            }
+            __syncwarp();
+            mbar_expect_warp(&full_q, G::Q_BYTES);                             // the queries; rows past the prompt come as zeros
+#pragma unroll
+            for (int hf = 0; hf < G::HALVES; ++hf) tma_load_4d(qs + hf * (NQ * 128), &qmap, hf * 64, h, (int)t0, b, &full_q);
+            grid_dependency_wait();                                            // the representatives come from the kernel before
+            if (terms)
+                for (int i = 0; i < 3; ++i) issue(0, i);
         }
-        if (warp == 0) tmem_alloc(&tbase, tcols);
+        if (warp == 1) tmem_alloc(&tbase, tcols);
         tcgen05_before_sync();
         __syncthreads();
         tcgen05_after_sync();
-        if (warp == 0) {                                                       // the queries; rows past the prompt come as zeros
-            mbar_expect_warp(&full_q, G::Q_BYTES);
-#pragma unroll
-            for (int hf = 0; hf < G::HALVES; ++hf) tma_load_4d(qs + hf * (NQ * 128), &qmap, hf * 64, h, (int)t0, b, &full_q);
-        }
-        grid_dependency_wait();                                                // the representatives come from the kernel before
+        grid_dependency_wait();
         const uint32_t tb = __shfl_sync(FULL, tbase, 0), tl = tb + ((uint32_t)((warp & 3) * 32) << 16);
-        int used = 0;                                                          // products started
-
-        // the scores of panel p into tensor memory, 64 blocks at a time: all threads cut representatives into terms, the
-        // first warp starts the products (the whole warp, see rq_umma.cuh)
-        constexpr int PER = kRouteGroup * D / 4 / kRouteThreads;               // float4 of a thread
-        auto rest = [](float x, float term) { return fabsf(term) == CUDART_INF_F ? 0.0f : x - term; };     // of an infinite mean: nothing
+        int w_first = 0;                                                       // first word of the panel in tensor memory
+        int seq = 0, fills = 0;                                                // panels computed, fillings of a stage before
+        constexpr uint32_t idesc = umma_idesc_bf16(NQ, kRouteGroup);
+        const uint64_t qd = umma_desc_sw128(smem_addr(qs)), bd = umma_desc_sw128(smem_addr(bs));
+        // the products of one term of group g of a panel
+        auto product = [&](int g, int pl) {
+#pragma unroll
+            for (int hf = 0; hf < G::HALVES; ++hf)
+                umma_bf16_x4<2, 2>(tb + (uint32_t)g * kRouteGroup, qd + (uint64_t)((hf * (NQ * 128)) >> 4),
+                                   bd + (uint64_t)((pl * G::PLANE_BYTES + hf * (kRouteGroup * 128)) >> 4), idesc, !(pl == 2 && hf == 0));
+        };
+        // the groups that a shorter panel has not: told all the same, so that every barrier counts panels
+        auto finish = [&](int gn) {
+            for (int g = gn; g < kPanelGroups; ++g) umma_commit(&done[g]);
+        };
+        // the scores of panel p into tensor memory, 64 blocks at a time, the smallest terms first; done[g] is told of each group.
+        // The terms come by bulk copies, each plane's as soon as the products before have read its room: the first warp (the whole
+        // warp, see rq_umma.cuh) starts copies and products, the others go on.  Where the scratch had no room for the terms all
+        // threads cut the representatives
         auto panel = [&](int p) {
             const int g0 = p * kPanelGroups, gn = min(kPanelGroups, groups - g0);
+            if (terms) {
+                if (warp != 0) return;
+                int landed = 0, issued = 3;
+                const int u0 = fills;
+                if (seq > 0)
+                    for (int i = 0; i < 3; ++i) issue(g0, i);
+                if (seq == 0) ok = __all_sync(FULL, mbar_wait(&full_q, 0u) || mbar_wait(&full_q, 0u));
+#pragma unroll 1
+                for (int g = 0; g < gn && ok; ++g) {
+#pragma unroll
+                    for (int st = 0; st < 3; ++st) {
+                        ok = ok && __all_sync(FULL, mbar_wait(&full_t[st], (uint32_t)((u0 + g) & 1)));
+                        if (!ok) break;
+                        landed = 3 * g + st + 1;
+                        tcgen05_after_sync();
+                        product(g, 2 - st);
+                        umma_commit(&free_t[st]);
+                    }
+                    if (!ok) break;
+                    umma_commit(&done[g]);
+                    if (g + 1 < gn)
+#pragma unroll
+                        for (int st = 0; st < 3; ++st) {                       //
+                            ok = ok && __all_sync(FULL, mbar_wait(&free_t[st], (uint32_t)((u0 + g) & 1)));
+                            if (!ok) break;
+                            issue(g0, 3 * (g + 1) + st);
+                            issued = 3 * (g + 1) + st + 1;
+                        }
+                }
+                fills += gn;
+                if (FORM == 2) finish(gn);
+                // after a wait that ran out: no copy may still be on its way into this CTA's shared memory when it exits
+                for (int i = landed; i < issued; ++i) mbar_wait(&full_t[i % 3], (uint32_t)((u0 + i / 3) & 1));
+                return;
+            }
+            constexpr int PER = kRouteGroup * D / 4 / kRouteThreads;           // float4 of a thread
             float4 f[PER];
             auto load = [&](int g) {
 #pragma unroll
@@ -190,7 +271,7 @@ __global__ void __launch_bounds__(kRouteThreads, 2) moba_route_mma_kernel(const 
             load(g0);
 #pragma unroll 1
             for (int g = 0; g < gn; ++g) {
-                if (used > 0) ok = ok && mbar_wait(&done, (uint32_t)((used - 1) & 1));     // the product before has read its terms
+                if (g > 0) ok = ok && mbar_wait(&done[g - 1], (uint32_t)(seq & 1));        // the products before have read their terms
 #pragma unroll
                 for (int i = 0; i < PER; ++i) {
                     const int e = tid + i * kRouteThreads, r = e / (D / 4), c = 4 * (e % (D / 4));
@@ -200,7 +281,7 @@ __global__ void __launch_bounds__(kRouteThreads, 2) moba_route_mma_kernel(const 
                     for (int t = 0; t < 3; ++t) {                              // the remainders are exact: each term takes the next 8 bits
                         const uint2 w = make_uint2(pack_bf16(x.x, x.y), pack_bf16(x.z, x.w));
                         *reinterpret_cast<uint2 *>(dst + t * G::PLANE_BYTES) = w;
-                        x = make_float4(rest(x.x, bf16lo(w.x)), rest(x.y, bf16hi(w.x)), rest(x.z, bf16lo(w.y)), rest(x.w, bf16hi(w.y)));
+                        x = make_float4(term_rest(x.x, bf16lo(w.x)), term_rest(x.y, bf16hi(w.x)), term_rest(x.z, bf16lo(w.y)), term_rest(x.w, bf16hi(w.y)));
                     }
                 }
                 asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // ordinary stores, read by the tensor core
@@ -208,31 +289,27 @@ __global__ void __launch_bounds__(kRouteThreads, 2) moba_route_mma_kernel(const 
                 ok = __syncthreads_and(ok);
                 if (!ok) break;
                 if (warp == 0) {
-                    constexpr uint32_t idesc = umma_idesc_bf16(NQ, kRouteGroup);
-                    const uint64_t qd = umma_desc_sw128(smem_addr(qs)), bd = umma_desc_sw128(smem_addr(bs));
-                    if (used == 0) ok = __all_sync(FULL, mbar_wait(&full_q, 0u) || mbar_wait(&full_q, 0u));
+                    if (g == 0 && seq == 0) ok = __all_sync(FULL, mbar_wait(&full_q, 0u) || mbar_wait(&full_q, 0u));
                     tcgen05_after_sync();
 #pragma unroll
-                    for (int pl = 2; pl >= 0; --pl)                            // the smallest terms first
-#pragma unroll
-                        for (int hf = 0; hf < G::HALVES; ++hf)
-                            umma_bf16_x4<2, 2>(tb + (uint32_t)g * kRouteGroup, qd + (uint64_t)((hf * (NQ * 128)) >> 4),
-                                               bd + (uint64_t)((pl * G::PLANE_BYTES + hf * (kRouteGroup * 128)) >> 4), idesc, !(pl == 2 && hf == 0));
-                    umma_commit(&done);
+                    for (int pl = 2; pl >= 0; --pl) product(g, pl);
+                    umma_commit(&done[g]);
                 }
-                ++used;
             }
-            ok = ok && mbar_wait(&done, (uint32_t)((used - 1) & 1));
-            ok = __syncthreads_and(ok);
-            tcgen05_after_sync();
+            if (FORM == 2 && warp == 0) finish(gn);
         };
-        // body(word, its first column taken, scores, candidates among them as bits) for this thread's words of every panel
+        // body(word, its first column taken, scores, candidates among them as bits, every score is a candidate of every query) for this
+        // thread's words of every panel
         auto for_scores = [&](bool first, auto body) {
             for (int p = 0; p < panels && ok; ++p) {
-                if (first || panels > 1) panel(p);
-                if (!ok) break;
+                const bool fresh = first || FORM == 2;
+                if (fresh) panel(p);
+                w_first = p * 2 * kPanelGroups;
+                // group g of the panel is there (a wait that has to be done once only, and costs little then)
+                auto there = [&](int g) { return ok = __all_sync(FULL, ok && (!fresh || mbar_wait(&done[g], (uint32_t)(seq & 1)))); };
                 if constexpr (HALF) {
-                    if ((part >> 1) < words_cta) {
+                    if ((part >> 1) < words_cta && there(0)) {
+                        tcgen05_after_sync();
                         uint32_t x[16];
                         float v[16];
                         tmem_ld16(tl + (uint32_t)part * 16u, x);
@@ -241,31 +318,41 @@ __global__ void __launch_bounds__(kRouteThreads, 2) moba_route_mma_kernel(const 
                         const int hi = c_hi - 16 * part;
                         uint32_t cand = hi >= 16 ? 0xffffu : hi <= 0 ? 0u : (1u << hi) - 1u;
                         if (part == 0) cand &= ~1u;
-                        body(part >> 1, (part & 1) * 16, v, cand);
+                        body(part >> 1, (part & 1) * 16, v, cand, part > 0 && 16 * part + 16 <= c_all);
                     }
                 } else
 #pragma unroll 1
                 for (int wl = part; wl < 2 * kPanelGroups; wl += 4) {
                     const int w = p * 2 * kPanelGroups + wl;
-                    if (w >= words_cta) break;
+                    if (w >= words_cta || !there(wl >> 1)) break;
+                    tcgen05_after_sync();
                     float v[32];
                     __syncwarp();
                     tmem_ld32(tl + (uint32_t)wl * 32u, v);
                     const int hi = c_hi - 32 * w;
                     uint32_t cand = hi >= 32 ? 0xffffffffu : hi <= 0 ? 0u : (1u << hi) - 1u;
                     if (w == 0) cand &= ~1u;
-                    body(w, 0, v, cand);
+                    body(w, 0, v, cand, w > 0 && 32 * w + 32 <= c_all);
                 }
                 tcgen05_before_sync();
-                if (panels > 1) __syncthreads();                               // the scores may be overwritten
+                if (fresh) {                                                   // (of several panels: the scores may be overwritten)
+                    ok = __syncthreads_and(ok);
+                    ++seq;
+                }
             }
         };
         // the bucket that holds the want-th largest of a query's counted scores: thread `part` of the query adds up a
-        // quarter of the buckets, the one whose quarter holds the threshold walks it
+        // quarter of the buckets, the one whose quarter holds the threshold looks for it, eighths of the quarter first
         auto find_bin = [&](bool mine, int wanted, int &bin, int &need, int &cnt) -> bool {
-            uint32_t s = 0u;
+            constexpr int Q4 = NB / 4, E = Q4 / 8;
+            uint32_t es[8], s = 0u;
 #pragma unroll
-            for (int i = 0; i < NB / 4; ++i) s += hist[(part * (NB / 4) + i) * NQ + ql];
+            for (int j = 0; j < 8; ++j) {
+                es[j] = 0u;
+#pragma unroll
+                for (int i = 0; i < E; ++i) es[j] += hist[(part * Q4 + j * E + i) * NQ + ql];
+                s += es[j];
+            }
             part_c[part * NQ + ql] = s;
             __syncthreads();
             int cum = 0, pt = 3;
@@ -275,23 +362,34 @@ __global__ void __launch_bounds__(kRouteThreads, 2) moba_route_mma_kernel(const 
                 cum += c;
             }
             if (!mine || part != pt) return false;
-            int i = NB / 4 - 1;
+            int j = 0;
+            bool found = false;
+#pragma unroll
+            for (int k = 7; k > 0; --k)
+                if (!found) {
+                    if (cum + (int)es[k] >= wanted) { j = k; found = true; }
+                    else cum += (int)es[k];
+                }
+            int i = E - 1;
             for (; i > 0; --i) {
-                const int c = (int)hist[(pt * (NB / 4) + i) * NQ + ql];
+                const int c = (int)hist[(pt * Q4 + j * E + i) * NQ + ql];
                 if (cum + c >= wanted) break;
                 cum += c;
             }
-            bin = pt * (NB / 4) + i;
+            bin = pt * Q4 + j * E + i;
             cnt = (int)hist[bin * NQ + ql];
             need = wanted - cum;
             return true;
+        };
+        auto clear_bins = [&]() {
+            for (int i = tid; i < NB * NQ / 4; i += kRouteThreads) reinterpret_cast<uint4 *>(hist)[i] = make_uint4(0u, 0u, 0u, 0u);
         };
 
         // ---- 1. smallest and largest
         float mn = CUDART_INF_F, mx = -CUDART_INF_F;
         constexpr int N = HALF ? 16 : 32;                                      // scores taken at a time
-        for_scores(true, [&](int w, int c0, float (&v)[N], uint32_t cand) {
-            if (w + c0 > 0 && 32 * w + c0 + N <= own_first && own_first >= K) {         // every score is a candidate of every query
+        for_scores(true, [&](int, int, float (&v)[N], uint32_t cand, bool all) {
+            if (all) {
 #pragma unroll
                 for (int c = 0; c < N; ++c) { mn = fminf(mn, v[c]); mx = fmaxf(mx, v[c]); }
             } else {
@@ -303,7 +401,7 @@ __global__ void __launch_bounds__(kRouteThreads, 2) moba_route_mma_kernel(const 
         if (ok) {
             part_a[part * NQ + ql] = __float_as_uint(mn);
             part_b[part * NQ + ql] = __float_as_uint(mx);
-            for (int i = tid; i < NB * NQ; i += kRouteThreads) hist[i] = 0u;
+            clear_bins();
             __syncthreads();
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
@@ -315,10 +413,14 @@ __global__ void __launch_bounds__(kRouteThreads, 2) moba_route_mma_kernel(const 
         const float inv = range > 0.0f ? fminf((float)(NB - 3) / range, 3.0e38f) : 0.0f;
 
         // ---- 2. buckets
-        for_scores(false, [&](int, int, float (&v)[N], uint32_t cand) {
+        for_scores(false, [&](int, int, float (&v)[N], uint32_t cand, bool all) {
+            if (all) {
 #pragma unroll
-            for (int c = 0; c < N; ++c)
-                if ((cand >> c) & 1u) atomicAdd(&hist[score_bin(v[c], mn, inv) * NQ + ql], 1u);
+                for (int c = 0; c < N; ++c) atomicAdd(&hist[score_bin<NB>(v[c], mn, inv) * NQ + ql], 1u);
+            } else {
+#pragma unroll
+                for (int c = 0; c < N; ++c) atomicAdd(&hist[((cand >> c) & 1u ? score_bin<NB>(v[c], mn, inv) : (uint32_t)NB) * NQ + ql], 1u);
+            }
         });
         if (ok) {
             __syncthreads();
@@ -338,11 +440,11 @@ __global__ void __launch_bounds__(kRouteThreads, 2) moba_route_mma_kernel(const 
             if (over && klo == khi) { tied = true; over = false; }             // all equal: the lowest blocks are taken below
             if (!__syncthreads_or(over)) break;
             uint32_t kmin = 0xffffffffu, kmax = 0u;
-            for_scores(false, [&](int, int, float (&v)[N], uint32_t cand) {
+            for_scores(false, [&](int, int, float (&v)[N], uint32_t cand, bool all) {
 #pragma unroll
                 for (int c = 0; c < N; ++c) {
                     const uint32_t k = score_key(v[c]);
-                    if (over && ((cand >> c) & 1u) && (int)score_bin(v[c], mn, inv) == tbin && k >= klo && k <= khi) {
+                    if (over && ((cand >> c) & 1u) && (int)score_bin<NB>(v[c], mn, inv) == tbin && k >= klo && k <= khi) {
                         kmin = min(kmin, k);
                         kmax = max(kmax, k);
                     }
@@ -351,7 +453,7 @@ __global__ void __launch_bounds__(kRouteThreads, 2) moba_route_mma_kernel(const 
             if (!ok) break;
             part_a[part * NQ + ql] = kmin;
             part_b[part * NQ + ql] = kmax;
-            for (int i = tid; i < NB * NQ; i += kRouteThreads) hist[i] = 0u;
+            clear_bins();
             __syncthreads();
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
@@ -359,12 +461,12 @@ __global__ void __launch_bounds__(kRouteThreads, 2) moba_route_mma_kernel(const 
                 kmax = max(kmax, part_b[i * NQ + ql]);
             }
             const uint32_t span = over ? kmax - kmin : 0u;
-            const int sh = max(0, 26 - __clz((int)span));                      // (span >> sh) < 64
-            for_scores(false, [&](int, int, float (&v)[N], uint32_t cand) {
+            const int sh = max(0, (NB == 128 ? 25 : 26) - __clz((int)span));   // (span >> sh) < NB
+            for_scores(false, [&](int, int, float (&v)[N], uint32_t cand, bool all) {
 #pragma unroll
                 for (int c = 0; c < N; ++c) {
                     const uint32_t k = score_key(v[c]);
-                    if (over && ((cand >> c) & 1u) && (int)score_bin(v[c], mn, inv) == tbin && k >= kmin && k <= kmax)
+                    if (over && ((cand >> c) & 1u) && (int)score_bin<NB>(v[c], mn, inv) == tbin && k >= kmin && k <= kmax)
                         atomicAdd(&hist[((k - kmin) >> sh) * NQ + ql], 1u);
                 }
             });
@@ -387,36 +489,59 @@ __global__ void __launch_bounds__(kRouteThreads, 2) moba_route_mma_kernel(const 
             const uint32_t klo = s_klo[ql], khi = s_khi[ql];
             const bool refined = klo != 0u || khi != 0xffffffffu || tied;
             auto put = [&](uint32_t *words_of, int w, int c0, uint32_t x) {
-                if constexpr (HALF) reinterpret_cast<uint16_t *>(words_of)[(w * NQ + ql) * 2 + (c0 >> 4)] = (uint16_t)x;
-                else words_of[w * NQ + ql] = x;
+                if constexpr (HALF) reinterpret_cast<uint16_t *>(words_of)[(w * MP + ql) * 2 + (c0 >> 4)] = (uint16_t)x;
+                else words_of[w * MP + ql] = x;
             };
-            for_scores(false, [&](int w, int c0, float (&v)[N], uint32_t cand) {
+            // bounds of the threshold's bucket (the last bucket holds nothing finite: refined, too)
+            const bool slow = __any_sync(FULL, refined || tbin == NB - 1);
+            const float above = 8388608.0f + (float)tbin, from = need > 0 ? above : CUDART_INF_F;
+            for_scores(false, [&](int w, int c0, float (&v)[N], uint32_t cand, bool) {
                 uint32_t bits = 0u, eq = 0u;
-                if (!__any_sync(FULL, refined)) {
+                if (!slow) {
                     // one atomic per thread and word: one per candidate, each waited for while most lanes had none, took
                     // half of a CTA's time
 #pragma unroll
                     for (int c = 0; c < N; ++c) {
-                        const int bin = (int)score_bin(v[c], mn, inv);
-                        if (bin > tbin) bits |= 1u << c;
-                        if (bin == tbin) eq |= 1u << c;
+                        const float x = score_place(v[c], mn, inv);
+                        if (!(x <= above)) bits |= 1u << c;                    // (a NaN: the highest)
+                        if (!(x < from)) eq |= 1u << c;
                     }
+                    eq &= cand & ~bits;
                     put(mk, w, c0, bits & cand);
-                    eq = need > 0 ? eq & cand : 0u;
-                    if (!__any_sync(FULL, eq != 0u)) return;
-                    uint32_t at = eq ? atomicAdd(&s_n[ql], (uint32_t)__popc(eq)) : (uint32_t)CAP;
+                    uint32_t cols = __reduce_or_sync(FULL, eq);          // columns that are of the threshold's bucket for some query
+                    if (cols == 0u) return;
+                    const uint32_t n = (uint32_t)__popc(eq), at = eq ? atomicAdd(&s_n[ql], n) : 0u;
+                    if (at + n > (uint32_t)CAP) eq = 0u;                       // (cannot be: the bucket holds no more)
+                    uint2 *to = ranked + at * NQ + ql;
+                    __syncwarp();
+                    // these columns once more, up to eight loads in flight (picking registers by number took a branch per column)
+                    const uint32_t col0 = tl + (uint32_t)(HALF ? part * 16 : (w - w_first) * 32);
+                    int c = 0;
+                    while (cols) {
+                        uint32_t x[8];
+                        int at_c[8];
 #pragma unroll
-                    for (int c = 0; c < N; ++c)
-                        if (((eq >> c) & 1u) && at < (uint32_t)CAP) {
-                            ckey[at * NQ + ql] = score_key(v[c]);
-                            cidx[at * NQ + ql] = (uint16_t)(32 * w + c0 + c);
-                            ++at;
+                        for (int u = 0; u < 8; ++u) {
+                            if (cols) c = __ffs(cols) - 1;                     // (none left: the last one again, which counts no more)
+                            cols &= cols - 1u;
+                            at_c[u] = c;
+                            tmem_ld1_start(col0 + (uint32_t)c, x[u]);
                         }
+                        tmem_ld1_wait(x);
+#pragma unroll
+                        for (int u = 0; u < 8; ++u) {
+                            if ((eq >> at_c[u]) & 1u) {
+                                *to = make_uint2(x[u], (uint32_t)(32 * w + c0 + at_c[u]));
+                                to += NQ;
+                            }
+                            eq &= ~(1u << at_c[u]);
+                        }
+                    }
                     return;
                 }
 #pragma unroll
                 for (int c = 0; c < N; ++c) {
-                    const int bin = (int)score_bin(v[c], mn, inv);
+                    const int bin = (int)score_bin<NB>(v[c], mn, inv);
                     if (bin > tbin) bits |= 1u << c;
                     if (bin == tbin && ((cand >> c) & 1u)) {
                         const uint32_t k = score_key(v[c]);
@@ -427,10 +552,8 @@ __global__ void __launch_bounds__(kRouteThreads, 2) moba_route_mma_kernel(const 
                                 eq |= 1u << c;
                             } else {
                                 const uint32_t at = atomicAdd(&s_n[ql], 1u);
-                                if (at < (uint32_t)CAP) {
-                                    ckey[at * NQ + ql] = k;
-                                    cidx[at * NQ + ql] = (uint16_t)(32 * w + c0 + c);
-                                }
+                                if (at < (uint32_t)CAP)
+                                    ranked[at * NQ + ql] = make_uint2(__float_as_uint(v[c]), (uint32_t)(32 * w + c0 + c));
                             }
                         }
                     }
@@ -444,45 +567,48 @@ __global__ void __launch_bounds__(kRouteThreads, 2) moba_route_mma_kernel(const 
                     if (part == 0) {
                         int left = need;
                         for (int w = 0; w < words_cta && left > 0; ++w) {
-                            uint32_t e = tie[w * NQ + ql], take = 0u;
+                            uint32_t e = tie[w * MP + ql], take = 0u;
                             while (e && left > 0) { take |= e & (0u - e); e &= e - 1u; --left; }
-                            mk[w * NQ + ql] |= take;
+                            mk[w * MP + ql] |= take;
                         }
                     }
                 } else {
                     const int n = min((int)s_n[ql], CAP);
                     for (int i = part; i < n; i += 4) {
-                        const uint32_t k = ckey[i * NQ + ql];
-                        const int j = cidx[i * NQ + ql];
+                        const uint2 e = ranked[i * NQ + ql];
+                        const uint32_t k = score_key(__uint_as_float(e.x));
+                        const int j = (int)e.y;
                         int rank = 0;
+#pragma unroll 4
                         for (int u = 0; u < n; ++u) {
-                            const uint32_t ku = ckey[u * NQ + ql];
-                            rank += (ku > k || (ku == k && (int)cidx[u * NQ + ql] < j)) ? 1 : 0;
+                            const uint2 f = ranked[u * NQ + ql];
+                            const uint32_t ku = score_key(__uint_as_float(f.x));
+                            rank += (ku > k || (ku == k && (int)f.y < j)) ? 1 : 0;
                         }
-                        if (rank < need) atomicOr(&mk[(j >> 5) * NQ + ql], 1u << (j & 31));
+                        if (rank < need) atomicOr(&mk[(j >> 5) * MP + ql], 1u << (j & 31));
                     }
                 }
             }
         }
         tcgen05_before_sync();
         __syncthreads();
-        if (warp == 0) tmem_dealloc(tbase, tcols);
+        if (warp == 1) tmem_dealloc(tbase, tcols);
     }
     if (!ok && tid == 0) atomicCAS(status, RQ_OK, RQ_ERR_TIMEOUT);
     grid_dependency_wait();
     grid_launch_dependents();
     __syncthreads();
-    // the masks go out, with the first block and the query's own
+    // the masks go out, with the first block and the query's own; a word after the other of the CTA's, so that the stores fill lines
+    const float per_word = 1.0f / (float)words;
     for (int i = tid; i < NQ * words; i += kRouteThreads) {
-        const int r = i / words, w = i % words;
-        const int64_t tq = t0 + r;
-        if (tq >= len) continue;
-        const int o = (int)(tq / block), hi = o + 1 - 32 * w;
+        const int r = (int)(((float)i + 0.5f) * per_word), w = i - r * words;  // (exact: i < 2^18, and half a word is never within rounding)
+        if (t0 + r >= len) continue;
+        const int o = s_own[r], hi = o + 1 - 32 * w;
         uint32_t m;
         if (K >= o + 1) m = hi >= 32 ? 0xffffffffu : hi <= 0 ? 0u : (1u << hi) - 1u;
-        else m = mk[w * NQ + r] | (w == 0 ? 1u : 0u) | (w == (o >> 5) ? 1u << (o & 31) : 0u);
+        else m = mk[w * MP + r] | (w == 0 ? 1u : 0u) | (w == (o >> 5) ? 1u << (o & 31) : 0u);
         if (masks) masks[((int64_t)bh * len + t0) * words + i] = m;
-        if (list) mk[w * NQ + r] = m;
+        if (list) mk[w * MP + r] = m;
     }
     if (!list) return;
     __syncthreads();
@@ -491,7 +617,7 @@ __global__ void __launch_bounds__(kRouteThreads, 2) moba_route_mma_kernel(const 
         int32_t *out = list + ((int64_t)bh * len + t0 + r) * K;
         int base = 0;
         for (int w0 = 0; w0 < words; w0 += 32) {
-            const uint32_t m = w0 + lane < words ? mk[(w0 + lane) * NQ + r] : 0u;
+            const uint32_t m = w0 + lane < words ? mk[(w0 + lane) * MP + r] : 0u;
             const int cnt = __popc(m);
             int inc = cnt;
 #pragma unroll
@@ -508,30 +634,21 @@ __global__ void __launch_bounds__(kRouteThreads, 2) moba_route_mma_kernel(const 
     }
 }
 
-template <int D> cudaError_t route_run(const MobaArgs &a, cudaStream_t s)
+template <int D, int FORM> cudaError_t route_launch(const MobaArgs &a, int nb, int words, cudaStream_t s)
 {
-    using G = RouteGeom<D>;
-    const int BH = a.B * a.H, nb = (int)((a.len + a.block - 1) / a.block), words = (nb + 31) / 32;
-    const int groups = (nb + kRouteGroup - 1) / kRouteGroup;
-    const bool one_panel = groups <= kPanelGroups;
-    const bool half = words <= 2;
-    static bool ready[2][64];
+    using G = RouteGeom<D, FORM>;
+    const int BH = a.B * a.H;
+    static bool ready[64];
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
-    const auto kernel = half ? moba_route_mma_kernel<D, true> : moba_route_mma_kernel<D, false>;
-    if (!ready[half][dev]) {
-        const int one = G::smem_bytes(true, kPanelGroups * kRouteGroup / 32), more = G::smem_bytes(false, kMobaMaxBlocks / 32);
-        e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, half ? G::smem_bytes(true, 2) : one > more ? one : more);
+    if (!ready[dev]) {
+        e = cudaFuncSetAttribute(moba_route_mma_kernel<D, FORM>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 G::smem_bytes(FORM == 0 ? 2 : FORM == 1 ? kPanelGroups * kRouteGroup / 32 : kMobaMaxBlocks / 32));
         if (e != cudaSuccess) return e;
-        ready[half][dev] = true;
+        ready[dev] = true;
     }
-    const int per = 256 / (D / 2);
-    moba_means_bf16_kernel<<<dim3((unsigned)((nb + per - 1) / per), (unsigned)BH), 256, 0, s>>>(
-        (const bf16 *)a.kv, a.page_cap, a.S, D, a.len, a.block, a.means, nb);
-    e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
     alignas(64) CUtensorMap qmap;
     e = query_tensor_map(&qmap, a.q, D, a.H, a.len, a.B, kRouteQueries);
     if (e != cudaSuccess) return e;
@@ -541,12 +658,24 @@ template <int D> cudaError_t route_run(const MobaArgs &a, cudaStream_t s)
     at.val.programmaticStreamSerializationAllowed = 1;
     cfg.gridDim = dim3((unsigned)BH, (unsigned)((a.len + kRouteQueries - 1) / kRouteQueries));
     cfg.blockDim = dim3(kRouteThreads);
-    cfg.dynamicSmemBytes = (size_t)G::smem_bytes(one_panel, words);
+    cfg.dynamicSmemBytes = (size_t)G::smem_bytes(words);
     cfg.stream = s;
     cfg.attrs = &at;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kernel, qmap, (const float *)a.means, a.len, a.H, a.block, nb, a.K, words, a.masks,
-                              a.list, a.status);
+    return cudaLaunchKernelEx(&cfg, moba_route_mma_kernel<D, FORM>, qmap, (const float *)a.means, (const unsigned char *)a.terms, a.len, a.H, a.block,
+                              nb, a.K, words, a.masks, a.list, a.status);
+}
+
+template <int D> cudaError_t route_run(const MobaArgs &a, cudaStream_t s)
+{
+    const int BH = a.B * a.H, nb = (int)((a.len + a.block - 1) / a.block), words = (nb + 31) / 32;
+    const int per = 256 / (D / 2);
+    moba_means_bf16_kernel<<<dim3((unsigned)((nb + per - 1) / per), (unsigned)BH), 256, 0, s>>>(
+        (const bf16 *)a.kv, a.page_cap, a.S, D, a.len, a.block, a.means, nb, (unsigned char *)a.terms);
+    const cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    if (words <= 2) return route_launch<D, 0>(a, nb, words, s);
+    return nb <= kPanelGroups * kRouteGroup ? route_launch<D, 1>(a, nb, words, s) : route_launch<D, 2>(a, nb, words, s);
 }
 
 }  // namespace
