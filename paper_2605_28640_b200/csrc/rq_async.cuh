@@ -77,6 +77,31 @@ __device__ __forceinline__ void bulk_g2s(void *dst_smem, const void *src_gmem, u
         : "memory");
 }
 
+// Cluster launch control: asks for a CTA of this grid that has not been launched yet, to be worked on here in its stead.  The answer
+// (16 bytes) is counted on the barrier; one thread, once at a time, and not again after an answer of "none".
+__device__ __forceinline__ void next_cta_ask(void *answer, uint64_t *bar)
+{
+    asm volatile("fence.proxy.async.shared::cta;\n\t"
+                 "mbarrier.arrive.expect_tx.shared::cta.b64 _, [%1], 16;\n\t"
+                 "clusterlaunchcontrol.try_cancel.async.shared::cta.mbarrier::complete_tx::bytes.b128 [%0], [%1];" ::"r"(smem_addr(answer)),
+                 "r"(smem_addr(bar))
+                 : "memory");
+}
+// its x index, or -1: none
+__device__ __forceinline__ int next_cta(const void *answer)
+{
+    int x;
+    asm volatile("{\n\t.reg .pred p;\n\t.reg .b128 r;\n\t"
+                 "ld.shared.b128 r, [%1];\n\t"
+                 "clusterlaunchcontrol.query_cancel.is_canceled.pred.b128 p, r;\n\t"
+                 "mov.b32 %0, -1;\n\t"
+                 "@p clusterlaunchcontrol.query_cancel.get_first_ctaid.v4.b32.b128 {%0, _, _, _}, r;\n\t}"
+                 : "=r"(x)
+                 : "r"(smem_addr(answer))
+                 : "memory");
+    return x;
+}
+
 // L2 policy for data that is read once: its lines are the first to be replaced, so that a long
 // stream does not push the step's small intermediate results (scores, page lists, partial
 // outputs) out of L2 before the next kernel reads them.

@@ -195,12 +195,13 @@ struct MobaArgs {
     // bf16 caches: the representatives as three bf16 terms, 64 blocks of a head at a time as the routing's tensor core reads them,
     // in what the scratch has left; NULL where that is too little
     void *terms;
+    uint32_t *unions;   // bf16 caches: blocks that any of 128 consecutive queries chose, [BH][tiles of 128][words]; NULL as above
     void *o;            // [B][len][H][D]
     int32_t *status;    // the cache's device status word
 };
 constexpr int kMobaMaxBlocks = 2048;           // blocks of a prompt at most
 size_t moba_scratch_bytes(int BH, int64_t len, int D, int block, int K);
-// means, masks, list and terms of `a` (its shape filled in) from the scratch and, if not NULL, the caller's lists
+// means, masks, list, terms and unions of `a` (its shape filled in) from the scratch and, if not NULL, the caller's lists
 void moba_carve(void *scratch, int32_t *blocks_out, MobaArgs &a);
 cudaError_t launch_moba(const MobaArgs &a, cudaStream_t s);
 // bf16 caches: representatives and routing (rq_moba_route.cu)

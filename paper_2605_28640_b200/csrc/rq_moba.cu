@@ -458,12 +458,17 @@ void moba_carve(void *scratch, int32_t *blocks_out, MobaArgs &a)
     void *rest = (char *)scratch + round256((size_t)a.B * a.H * nb * a.D * sizeof(float));     // room for the lists
     a.masks = a.dtype == RQ_BF16 && (nb + 31) / 32 <= (size_t)a.K ? (uint32_t *)rest : nullptr;
     a.list = blocks_out ? blocks_out : a.masks ? nullptr : (int32_t *)rest;
-    // the terms of 64 blocks take 6 bytes a channel; the lists' room, where they are not in it, holds them behind the masks
-    // but for the smallest budgets of short prompts
-    const size_t room = round256((size_t)a.B * a.H * (size_t)a.len * a.K * sizeof(int32_t));
-    const size_t used = a.masks ? round256((size_t)a.B * a.H * (size_t)a.len * ((nb + 31) / 32) * sizeof(uint32_t)) : 0;
-    const size_t need = (size_t)a.B * a.H * ((nb + 63) / 64) * 64 * a.D * 6;
-    a.terms = a.dtype == RQ_BF16 && (void *)a.list != rest && used + need <= room ? (char *)rest + used : nullptr;
+    // what the lists would take, where they are not in it, holds more behind the masks, but for the smallest budgets of short prompts
+    const size_t BH = (size_t)a.B * a.H, words = (nb + 31) / 32, room = a.list == (int32_t *)rest ? 0 : round256(BH * (size_t)a.len * a.K * sizeof(int32_t));
+    size_t used = a.masks ? round256(BH * (size_t)a.len * words * sizeof(uint32_t)) : 0;
+    auto take = [&](size_t bytes) -> void * {
+        if (a.dtype != RQ_BF16 || used + round256(bytes) > room) return nullptr;
+        void *p = (char *)rest + used;
+        used += round256(bytes);
+        return p;
+    };
+    a.unions = (uint32_t *)take(BH * (((size_t)a.len + 127) / 128) * words * sizeof(uint32_t));
+    a.terms = take(BH * ((nb + 63) / 64) * 64 * a.D * 6);      // 64 blocks' terms: 6 bytes a channel
 }
 
 cudaError_t launch_moba(const MobaArgs &a, cudaStream_t s)

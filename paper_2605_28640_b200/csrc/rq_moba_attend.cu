@@ -29,6 +29,9 @@ constexpr int kThreads = (kReadWarps + kTiles + 2) * 32;   // and one for the co
 // channels, whose walks the readers bound, within 1 % of each other from 102 to 737 MB.  Sets of 32 MB win less (33 heads 7224 when
 // sets of 64 and of 96 MB take 7198 and 7176; 16 x 14001 827, 764, 770).
 constexpr int64_t kSetBytes = 96 << 20;
+// steps before the last one at which a CTA asks for its next tile: the answer takes one, the tile's choices another, and the copies run
+// up to four steps ahead
+constexpr int kAskSteps = 6;
 constexpr float kRaise = 8.0f;                 // powers of two a query's maximum may grow before its output is rescaled
 
 template <int D> struct AttGeom {
@@ -37,8 +40,8 @@ template <int D> struct AttGeom {
     static constexpr int C_BYTES = HALVES * kChunk * 128;          // the keys (or the values) of a chunk
     static constexpr int OFF_K = kTiles * Q_BYTES;
     static constexpr int OFF_V = OFF_K + kStages * C_BYTES;
-    static constexpr int OFF_LIST = OFF_V + kStages * C_BYTES;     // blocks to walk
-    static constexpr int SMEM_BYTES = OFF_LIST + kMobaMaxBlocks * 2 + 1024;   // + room to align the base to 1024 bytes
+    static constexpr int OFF_O = OFF_V + kStages * C_BYTES;        // 32 rows of 64 channels of the output, for every reading warp
+    static constexpr int SMEM_BYTES = OFF_O + kReadWarps * 32 * 128 + 1024;   // + room to align the base to 1024 bytes
 };
 
 __device__ __forceinline__ uint64_t desc_sw128_mn(uint32_t saddr, uint32_t lbo_bytes)
@@ -72,17 +75,50 @@ __device__ __forceinline__ void add_bf16(float2 &sum, uint32_t pair)
         : "r"(pair));
 }
 
-// The walk over the chunks of the listed blocks: (entry of the list, chunk inside the block).
+// What any query of a tile's two accumulators chose, by words of 32 blocks.
+struct Chosen {
+    uint32_t by[kTiles][kMobaMaxBlocks / 32];
+};
+// The walk over the chunks of the blocks that are chosen: block j, chunk r of it, ascending.
 struct Walk {
-    int bi = 0, r = 0;
-    __device__ __forceinline__ void next(int cpb)
+    int w = -1, r = 0;
+    uint32_t bits = 0u;                                          // blocks of word w that are still to come, the present one first
+    __device__ __forceinline__ void block(const Chosen &c)
     {
-        if (++r == cpb) { r = 0; ++bi; }
+        bits &= bits - 1u;
+        while (!bits) {
+            ++w;
+            bits = c.by[0][w] | c.by[1][w];
+        }
     }
+    // to the first step, and from step to step; not beyond the last one
+    __device__ __forceinline__ void start(const Chosen &c)
+    {
+        w = -1;
+        r = 0;
+        bits = 0u;
+        block(c);
+    }
+    __device__ __forceinline__ void next(const Chosen &c, int cpb)
+    {
+        if (++r == cpb) {
+            r = 0;
+            block(c);
+        }
+    }
+    __device__ __forceinline__ int j() const { return w * 32 + __ffs(bits) - 1; }
+    __device__ __forceinline__ bool in(const Chosen &c, int s) const { return c.by[s][w] & bits & (0u - bits); }
 };
 
-// Grid: tiles of 256 queries of all heads, the last queries of a head first (their work is the largest).  A CTA owns 256
-// consecutive queries as two accumulators of 128 lanes; everything per query (choice of blocks, causal cut, what its weights
+// Grid: tiles of 256 queries of all heads, the last queries of a head first (their work is the largest).  A CTA that is done with
+// its tile asks for one whose CTA has not been launched yet (cluster launch control) and goes on with it, in the same order: the
+// rings of keys, values, scores and weights run on from tile to tile, the next tile's choices, queries and first products come while
+// the last weights of this one are taken and its output goes.  A CTA per tile spent 0.6 us on its set-up, 2 on the list of blocks,
+// 1.5 up to the first product and 3 at the end.  Launch, us, a CTA per tile / this: 32 heads x 4096 positions 185 / 174.5, x 30011
+// 5760 / 5570 (three stages of keys and values and all of the output's rows in shared memory at once instead of four and halves:
+// 174.5 / 5680; a next tile taken at once instead of six steps before the end would pair the longest tiles).  What any query of a tile
+// chose comes from the routing as a word per 32 blocks, 128 queries together; the walk goes by its bits.
+// A tile's 256 consecutive queries are two accumulators of 128 lanes; everything per query (choice of blocks, causal cut, what its weights
 // are relative to, their sum, the weights) belongs to one thread.  The 64-position chunks of the blocks that any of the 256
 // queries chose are walked once:
 //   S = Q K^T        128 x 64 per accumulator, fp32 in tensor memory, two score buffers per accumulator, so that the
@@ -100,9 +136,9 @@ struct Walk {
 // 0.8 % more, and values above 2^92 overflow.  The first keys of a prompt have hardly been accumulated and score low, so that a fifth
 // to a half of a warp's chunks raise one of its queries; the row of O is therefore multiplied down after the chunk's weights have
 // been written, when the product before is mostly over, 32 columns at a time with the next 32 on their way.
-// Warps 0..7 read scores, warp 8 starts the tensor-map copies, warps 9 and 10 the score products of an accumulator each,
-// warp 11 the output products; they meet through mbarriers only, every wait bounded.  256 queries per CTA because keys and
-// values come from L2 for every CTA.  A CTA's queries come by tensor map, and it may start before the routing kernel has ended.
+// Warps 0..7 read scores, warp 8 looks after tiles and copies, warps 9 and 10 after the queries and score products of an accumulator
+// each, warp 11 after the output products; they meet through mbarriers only, every wait bounded.  256 queries per CTA because keys and
+// values come from L2 for every tile.  A CTA may start before the routing kernel has ended.
 // Measured, call, 32 heads x 128 channels, 4096 positions (16 of 64 blocks) at logits of 1.4 / 5 / 11: rows multiplied down before
 // the weights, 16 columns at a time, 223.5 / 238 / 243 us; after them 217 / 227 / 231 (without ever doing it 214).  Bound: the
 // readers' chain per chunk (about 1850 cycles at 4096 positions, of which ex2 alone takes 1024, against 1280 for the products, whose
@@ -116,7 +152,8 @@ __global__ void __launch_bounds__(kThreads, 1) moba_mma_kernel(const __grid_cons
                                                                const __grid_constant__ CUtensorMap qmap,
                                                                const __grid_constant__ CUtensorMap omap, int64_t page_cap, int S,
                                                                int64_t len, int H, int BH, int set, int tiles, int block, int nb,
-                                                               const uint32_t *masks, const int32_t *lists, int K, float scale_log2, int32_t *status)
+                                                               const uint32_t *masks, const uint32_t *unions, const int32_t *lists, int K,
+                                                               float scale_log2, int32_t *status)
 {
     using G = AttGeom<D>;
     constexpr int NST = kStages;
@@ -124,111 +161,154 @@ __global__ void __launch_bounds__(kThreads, 1) moba_mma_kernel(const __grid_cons
     // afterwards), then the output
     constexpr uint32_t ACC = 256, OFF_O = 128;
     extern __shared__ __align__(1024) unsigned char asm_raw[];
-    __shared__ __align__(8) uint64_t full_k[NST], full_v[NST], free_k[NST], free_v[NST], full_q;
+    __shared__ __align__(8) uint64_t full_k[NST], full_v[NST], free_k[NST], free_v[NST], full_q[kTiles], free_q[kTiles];
     __shared__ __align__(8) uint64_t s_ready[kTiles][2], p_ready[kTiles][2], pv_done[kTiles][2];
-    __shared__ uint32_t um[kTiles][kMobaMaxBlocks / 32];         // blocks chosen by any query of an accumulator
+    __shared__ __align__(8) uint64_t known[2], left[2], answered;    // a tile's choices are in shared memory, all warps are done with them
+    __shared__ Chosen chosen_of[2];                              // by parity of the CTA's tiles
+    __shared__ int head_of[2], row_of[2], steps_of[2];           // its head (-1: there is no more), first query and steps of the walk
+    __shared__ __align__(16) uint4 answer;
     __shared__ uint32_t tbase;
-    __shared__ int n_list;
     unsigned char *sm = asm_raw + ((1024u - (smem_addr(asm_raw) & 1023u)) & 1023u);
     unsigned char *qs = sm, *kst = sm + G::OFF_K, *vst = sm + G::OFF_V;
-    uint16_t *list = reinterpret_cast<uint16_t *>(sm + G::OFF_LIST);   // block | 0x4000 (first accumulator) | 0x8000 (second)
     const int words = (nb + 31) / 32;
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int part = BH % set;                                   // heads of the first set, if it is not full
-    const int at_tile = (int)blockIdx.x - part * tiles;
-    const int first = at_tile < 0 ? 0 : part + at_tile / (set * tiles) * set, in_set = at_tile < 0 ? part : set;
-    const int rest = at_tile < 0 ? (int)blockIdx.x : at_tile % (set * tiles);
-    const int bh = first + rest % in_set, b = bh / H, h = bh % H;
-    const int64_t t0 = (int64_t)(tiles - 1 - rest / in_set) * (kTile * kTiles);
-    const int n_chunks_all = (int)((min(t0 + kTile * kTiles, len) + kChunk - 1) / kChunk);
     const int cpb = block / kChunk;                              // chunks of a block
     const int ppc = kChunk / S;                                  // pages of a chunk
+    // head and first query of a tile
+    auto place = [&](int tile, int &bh, int64_t &t0) {
+        const int part = BH % set;                               // heads of the first set, if it is not full
+        const int at_tile = tile - part * tiles;
+        const int first = at_tile < 0 ? 0 : part + at_tile / (set * tiles) * set, in_set = at_tile < 0 ? part : set;
+        const int rest = at_tile < 0 ? tile : at_tile % (set * tiles);
+        bh = first + rest % in_set;
+        t0 = (int64_t)(tiles - 1 - rest / in_set) * (kTile * kTiles);
+    };
 
     if (tid == 0) {
         for (int i = 0; i < NST; ++i) {
             mbar_init(&full_k[i], 1); mbar_init(&full_v[i], 1);
             mbar_init(&free_k[i], kTiles); mbar_init(&free_v[i], 1);
         }
-        mbar_init(&full_q, 1);
-        for (int s = 0; s < kTiles; ++s)
+        for (int s = 0; s < kTiles; ++s) {
+            mbar_init(&full_q[s], 1);
+            mbar_init(&free_q[s], 1);
             for (int i = 0; i < 2; ++i) {
                 mbar_init(&s_ready[s][i], 1);
                 mbar_init(&p_ready[s][i], kTile);
                 mbar_init(&pv_done[s][i], 1);
             }
+        }
+        for (int i = 0; i < 2; ++i) { mbar_init(&known[i], 1); mbar_init(&left[i], kReadWarps + kTiles + 1); }
+        mbar_init(&answered, 1);
         mbar_init_fence();
     }
     if (warp == kReadWarps) tmem_alloc(&tbase, 512);
-    for (int i = tid; i < kTiles * words; i += kThreads) um[i / words][i % words] = 0u;
-    __syncthreads();
-    if (warp == kReadWarps) {                                    // the queries; rows past the prompt come as zeros
-        mbar_expect_warp(&full_q, kTiles * G::Q_BYTES);
-#pragma unroll
-        for (int s = 0; s < kTiles; ++s)
-#pragma unroll
-            for (int hf = 0; hf < G::HALVES; ++hf)
-                tma_load_4d(qs + s * G::Q_BYTES + hf * (kTile * 128), &qmap, hf * 64, h, (int)t0 + s * kTile, b, &full_q);
-    }
-    grid_dependency_wait();                                      // the choices of blocks come from the kernel before
-    if (warp < kReadWarps) {
-        const bool in = t0 + tid < len;
-        if (masks) {
-            const uint32_t *row = masks + ((int64_t)bh * len + (in ? t0 + tid : 0)) * words;
-            for (int w0 = 0; w0 < words; w0 += 8) {              // eight loads in flight
-                uint32_t m[8];
-#pragma unroll
-                for (int u = 0; u < 8; ++u) m[u] = in && w0 + u < words ? __ldcg(row + w0 + u) : 0u;
-#pragma unroll
-                for (int u = 0; u < 8; ++u) {
-                    m[u] = __reduce_or_sync(FULL, m[u]);
-                    if (lane == 0 && m[u]) atomicOr(&um[warp >> 2][w0 + u], m[u]);
-                }
-            }
-        } else if (in) {
-            const int32_t *mine = lists + ((int64_t)bh * len + t0 + tid) * K;
-            for (int i = 0; i < K; ++i) {
-                const int j = __ldcg(mine + i);
-                if (j >= 0) atomicOr(&um[warp >> 2][j >> 5], 1u << (j & 31));
-            }
-        }
-    }
-    __syncthreads();
-    if (warp == 0) {                                             // the list of blocks, ascending
-        int base = 0;
-#pragma unroll 4
-        for (int w = 0; w < words; ++w) {                        // a lane per block
-            const uint32_t m0 = um[0][w], m1 = um[1][w], m = m0 | m1;
-            if ((m >> lane) & 1u)
-                list[base + __popc(m & ((1u << lane) - 1u))] =
-                    (uint16_t)((w * 32 + lane) | (((m0 >> lane) & 1u) << 14) | (((m1 >> lane) & 1u) << 15));
-            base += __popc(m);
-        }
-        if (lane == 0) n_list = base;
-    }
     tcgen05_before_sync();
     __syncthreads();
     tcgen05_after_sync();
     const uint32_t tb = __shfl_sync(FULL, tbase, 0);             // (the shuffle tells the compiler that it is uniform)
-    // steps of the walk: whole blocks, the last one (the last query's own) up to the CTA's last chunk
-    const int nl = n_list, n = (nl - 1) * cpb + min(cpb, n_chunks_all - (list[nl - 1] & 0x3fff) * cpb);
     bool ok = true;
+    auto wait_all = [&](uint64_t *x, int phase) -> bool { return ok = __all_sync(FULL, mbar_wait(x, (uint32_t)(phase & 1))); };
+    // the CTA's k-th tile, for the warps that work on it; false: there is none
+    int n = 0, bh = 0;
+    int64_t t0 = 0;
+    auto take = [&](int k) -> bool {
+        if (!wait_all(&known[k & 1], k >> 1)) return false;
+        bh = __shfl_sync(FULL, head_of[k & 1], 0);
+        t0 = __shfl_sync(FULL, row_of[k & 1], 0);
+        n = __shfl_sync(FULL, steps_of[k & 1], 0);
+        return bh >= 0;
+    };
+    auto leave = [&](int k) {
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&left[k & 1]);
+    };
+    int g = 0;                                                   // steps of all tiles together, before the present one
 
     if (warp == kReadWarps) {
-        // ---- copies (the whole warp, like the products below: see rq_umma.cuh)
-        {
-            Walk w;
-            int issued = 0;
+        // ---- what is to be walked over, and the copies (the whole warp, like the products below: see rq_umma.cuh).  The stages
+        // of keys and values go on from tile to tile: this warp is up to four steps ahead of the products
+        int asked = 0, issued = 0;
+        int tile = (int)blockIdx.x;
+        // a lane's words of what the tile's accumulators chose: lane and lane + 32; where the routing left them they come early
+        uint32_t mine[kTiles][2];
+        auto load = [&]() {
+            const uint32_t *x = unions + ((int64_t)bh * ((len + kTile - 1) / kTile) + t0 / kTile) * words;
+#pragma unroll
+            for (int s = 0; s < kTiles; ++s)
+#pragma unroll
+                for (int i = 0; i < 2; ++i)
+                    mine[s][i] = lane + 32 * i < words && t0 + s * kTile < len ? __ldcg(x + s * words + lane + 32 * i) : 0u;
+        };
+        grid_dependency_wait();                                  // the choices of blocks come from the kernel before
+        place(tile, bh, t0);
+        if (unions) load();
 #pragma unroll 1
-            for (int i = 0; i < n; ++i, w.next(cpb)) {
-                const int st = i % NST;
-                if (i >= NST) {
-                    const uint32_t ph = (uint32_t)((i / NST - 1) & 1);
+        for (int k = 0;; ++k) {
+            Chosen &c = chosen_of[k & 1];
+            if (k >= 2 && !wait_all(&left[k & 1], (k >> 1) - 1)) break;
+            if (tile >= 0) {
+                if (unions) {
+#pragma unroll
+                    for (int s = 0; s < kTiles; ++s)
+#pragma unroll
+                        for (int i = 0; i < 2; ++i)
+                            if (lane + 32 * i < words) c.by[s][lane + 32 * i] = mine[s][i];
+                } else {
+                    for (int w = lane; w < words; w += 32) c.by[0][w] = c.by[1][w] = 0u;
+                    __syncwarp();
+                    for (int r = lane; r < kTile * kTiles; r += 32) {
+                        if (t0 + r >= len) continue;
+                        uint32_t *by = c.by[r / kTile];
+                        if (masks) {
+                            const uint32_t *row = masks + ((int64_t)bh * len + t0 + r) * words;
+                            for (int w0 = 0; w0 < words; w0 += 8) {                // eight loads in flight
+                                uint32_t m[8];
+#pragma unroll
+                                for (int x = 0; x < 8; ++x) m[x] = w0 + x < words ? __ldcg(row + w0 + x) : 0u;
+#pragma unroll
+                                for (int x = 0; x < 8; ++x)
+                                    if (m[x]) atomicOr(&by[w0 + x], m[x]);
+                            }
+                        } else {
+                            const int32_t *list = lists + ((int64_t)bh * len + t0 + r) * K;
+                            for (int x = 0; x < K; ++x) {
+                                const int j = __ldcg(list + x);
+                                if (j >= 0) atomicOr(&by[j >> 5], 1u << (j & 31));
+                            }
+                        }
+                    }
+                }
+                __syncwarp();
+                int count = 0;
+                for (int w = lane; w < words; w += 32) count += __popc(c.by[0][w] | c.by[1][w]);
+                count = __reduce_add_sync(FULL, count);
+                // steps of the walk: whole blocks, the last one (the last query's own) up to the tile's last chunk
+                const int end = (int)min(t0 + kTile * kTiles, len);
+                n = (count - 1) * cpb + min(cpb, (end + kChunk - 1) / kChunk - (end - 1) / block * cpb);
+            }
+            if (lane == 0) {
+                head_of[k & 1] = tile >= 0 ? bh : -1;
+                row_of[k & 1] = (int)t0;
+                steps_of[k & 1] = n;
+            }
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&known[k & 1]);
+            if (tile < 0) break;
+            Walk w;
+            w.start(c);
+            const int head = bh;
+#pragma unroll 1
+            for (int i = 0; i < n; ++i, ++g) {
+                const int st = g % NST;
+                if (g >= NST) {
+                    const uint32_t ph = (uint32_t)((g / NST - 1) & 1);
                     ok = mbar_wait(&free_k[st], ph) && mbar_wait(&free_v[st], ph);
                     ok = __all_sync(FULL, ok);
                     if (!ok) break;
                 }
-                const int page = (int)((int64_t)bh * page_cap + (int64_t)(__shfl_sync(FULL, list[w.bi] & 0x3fff, 0) * cpb + w.r) * ppc);
+                const int page = (int)((int64_t)head * page_cap + (int64_t)(__shfl_sync(FULL, w.j(), 0) * cpb + w.r) * ppc);
                 mbar_expect_warp(&full_k[st], G::C_BYTES);
 #pragma unroll
                 for (int hf = 0; hf < G::HALVES; ++hf)
@@ -237,104 +317,165 @@ __global__ void __launch_bounds__(kThreads, 1) moba_mma_kernel(const __grid_cons
 #pragma unroll
                 for (int hf = 0; hf < G::HALVES; ++hf)
                     tma_load_4d(vst + (size_t)st * G::C_BYTES + hf * (kChunk * 128), &tmap, hf * 64, 0, 1, page, &full_v[st]);
-                issued = i + 1;
-            }
-            // no copy may still be on its way into this CTA's shared memory when it exits, after a wait that ran out either
-            ok = mbar_wait(&full_q, 0u) && ok;
-            if (!ok)
-                for (int k = max(0, issued - NST); k < issued; ++k) {
-                    mbar_wait(&full_k[k % NST], (uint32_t)((k / NST) & 1));
-                    mbar_wait(&full_v[k % NST], (uint32_t)((k / NST) & 1));
+                issued = g + 1;
+                if (i + 1 < n) w.next(c, cpb);
+                // the next tile, a CTA that need not be launched any more: asked for shortly before the end only, so that the tiles,
+                // longest first, go to who is done first; known in time for its first copies to follow this tile's last
+                if (i == max(0, n - kAskSteps)) {
+                    if (lane == 0) next_cta_ask(&answer, &answered);
+                    ++asked;
                 }
+                if (i == max(0, n - kAskSteps + 3)) {
+                    if (!wait_all(&answered, asked - 1)) break;
+                    tile = __shfl_sync(FULL, next_cta(&answer), 0);
+                    if (tile >= 0) place(tile, bh, t0);
+                    if (tile >= 0 && unions) load();
+                }
+            }
+            if (!ok) break;
+        }
+        // no copy may still be on its way into this CTA's shared memory when it exits, after a wait that ran out either
+        if (!ok) {
+            for (int x = max(0, issued - NST); x < issued; ++x) {
+                mbar_wait(&full_k[x % NST], (uint32_t)((x / NST) & 1));
+                mbar_wait(&full_v[x % NST], (uint32_t)((x / NST) & 1));
+            }
+            if (asked > 0) mbar_wait(&answered, (uint32_t)((asked - 1) & 1));
         }
     } else if (warp > kReadWarps && warp <= kReadWarps + kTiles) {
-        // ---- score products, a warp per accumulator
+        // ---- queries and score products, a warp per accumulator
         const int s = warp - kReadWarps - 1;
         constexpr uint32_t idesc_s = umma_idesc_bf16(kTile, kChunk);
         const uint64_t qd = umma_desc_sw128(smem_addr(qs) + s * G::Q_BYTES), kd = umma_desc_sw128(smem_addr(kst));
         const uint32_t ts = tb + s * ACC;
         int u = 0;                                               // products started
-        Walk w;
-        ok = __all_sync(FULL, mbar_wait(&full_q, 0u));
-#pragma unroll 1
-        for (int i = 0; i < n && ok; ++i, w.next(cpb)) {
-            const int st = i % NST;
-            // (waited for even if not used: the stage's release counts one arrival of each of the two warps per filling)
-            ok = __all_sync(FULL, mbar_wait(&full_k[st], (uint32_t)((i / NST) & 1)));
-            if (!ok) break;
-            if ((__shfl_sync(FULL, (uint32_t)list[w.bi], 0) >> (14 + s)) & 1u) {
-                if (u >= 2) ok = mbar_wait(&pv_done[s][u & 1], (uint32_t)(((u >> 1) - 1) & 1));   // the buffer's weights were used
-                ok = __all_sync(FULL, ok);
-                if (!ok) break;
-                tcgen05_after_sync();
+        auto ask = [&]() {                                       // the queries of the tile; rows past the prompt come as zeros
+            mbar_expect_warp(&full_q[s], G::Q_BYTES);
 #pragma unroll
-                for (int hf = 0; hf < G::HALVES; ++hf)
-                    umma_bf16_x4<2, 2>(ts + (uint32_t)(u & 1) * kChunk, qd + (uint64_t)((hf * (kTile * 128)) >> 4),
-                                       kd + (uint64_t)((st * G::C_BYTES + hf * (kChunk * 128)) >> 4), idesc_s, hf > 0);
-                umma_commit(&s_ready[s][u & 1]);
-                ++u;
+            for (int hf = 0; hf < G::HALVES; ++hf)
+                tma_load_4d(qs + s * G::Q_BYTES + hf * (kTile * 128), &qmap, hf * 64, bh % H, (int)t0 + s * kTile, bh / H, &full_q[s]);
+        };
+        place((int)blockIdx.x, bh, t0);
+        ask();                                                   // (the first tile's before its choices are known)
+#pragma unroll 1
+        for (int k = 0; take(k); ++k) {
+            if (k > 0) {
+                if (!wait_all(&free_q[s], k - 1)) break;         // the tile before has read its queries
+                ask();
             }
-            umma_commit(&free_k[st]);
+            ok = __all_sync(FULL, mbar_wait(&full_q[s], (uint32_t)(k & 1)) || mbar_wait(&full_q[s], (uint32_t)(k & 1)));
+            if (!ok) break;
+            const Chosen &c = chosen_of[k & 1];
+            Walk w;
+            w.start(c);
+#pragma unroll 1
+            for (int i = 0; i < n; ++i, ++g) {
+                const int st = g % NST;
+                // (waited for even if not used: the stage's release counts one arrival of each of the two warps per filling)
+                if (!wait_all(&full_k[st], g / NST)) break;
+                if (__shfl_sync(FULL, (uint32_t)w.in(c, s), 0)) {
+                    if (u >= 2 && !wait_all(&pv_done[s][u & 1], (u >> 1) - 1)) break;      // the buffer's weights were used
+                    tcgen05_after_sync();
+#pragma unroll
+                    for (int hf = 0; hf < G::HALVES; ++hf)
+                        umma_bf16_x4<2, 2>(ts + (uint32_t)(u & 1) * kChunk, qd + (uint64_t)((hf * (kTile * 128)) >> 4),
+                                           kd + (uint64_t)((st * G::C_BYTES + hf * (kChunk * 128)) >> 4), idesc_s, hf > 0);
+                    umma_commit(&s_ready[s][u & 1]);
+                    ++u;
+                }
+                umma_commit(&free_k[st]);
+                if (i + 1 < n) w.next(c, cpb);
+            }
+            if (!ok) break;
+            umma_commit(&free_q[s]);
+            leave(k);
         }
+        if (!ok) mbar_wait(&full_q[s], 0u), mbar_wait(&full_q[s], 1u);       // (a copy of queries may be on its way)
     } else if (warp == kReadWarps + kTiles + 1) {
         // ---- output products
         constexpr uint32_t idesc_o = umma_idesc_bf16(kTile, D) | (1u << 16);       // the values are MN-major
         const uint64_t vd = desc_sw128_mn(smem_addr(vst), kChunk * 128);
         int up[kTiles] = {0, 0};                                 // products started
-        Walk w;
 #pragma unroll 1
-        for (int i = 0; i < n && ok; ++i, w.next(cpb)) {
-            const int st = i % NST;
-            const uint32_t e = __shfl_sync(FULL, (uint32_t)list[w.bi], 0);
-            ok = __all_sync(FULL, mbar_wait(&full_v[st], (uint32_t)((i / NST) & 1)));
+        for (int k = 0; take(k); ++k) {
+            const Chosen &c = chosen_of[k & 1];
+            const int u0[kTiles] = {up[0], up[1]};
+            Walk w;
+            w.start(c);
+#pragma unroll 1
+            for (int i = 0; i < n && ok; ++i, ++g) {
+                const int st = g % NST;
+                if (!wait_all(&full_v[st], g / NST)) break;
 #pragma unroll
-            for (int s = 0; s < kTiles; ++s) {
-                if (!ok || !((e >> (14 + s)) & 1u)) continue;
-                const int u = up[s]++;
-                ok = __all_sync(FULL, mbar_wait(&p_ready[s][u & 1], (uint32_t)((u >> 1) & 1)));
-                if (!ok) continue;
-                tcgen05_after_sync();
-                umma_bf16_ta_x4<8, 128>(tb + s * ACC + OFF_O, tb + s * ACC + (uint32_t)(u & 1) * kChunk, vd + (uint64_t)((st * G::C_BYTES) >> 4),
-                                        idesc_o, u > 0);
-                umma_commit(&pv_done[s][u & 1]);
+                for (int s = 0; s < kTiles; ++s) {
+                    if (!ok || !__shfl_sync(FULL, (uint32_t)w.in(c, s), 0)) continue;
+                    const int u = up[s]++;
+                    if (!wait_all(&p_ready[s][u & 1], u >> 1)) continue;
+                    tcgen05_after_sync();
+                    umma_bf16_ta_x4<8, 128>(tb + s * ACC + OFF_O, tb + s * ACC + (uint32_t)(u & 1) * kChunk, vd + (uint64_t)((st * G::C_BYTES) >> 4),
+                                            idesc_o, u > u0[s]);
+                    umma_commit(&pv_done[s][u & 1]);
+                }
+                if (ok) umma_commit(&free_v[st]);
+                if (i + 1 < n) w.next(c, cpb);
             }
-            if (ok) umma_commit(&free_v[st]);
+            if (!ok) break;
+            leave(k);
         }
     } else {
         // ---- weights: a thread per query
         const int s = warp >> 2, lq = (warp & 3) * 32 + lane;
+        const uint32_t tl = tb + s * ACC + ((uint32_t)((warp & 3) * 32) << 16);
+        const float2 sc2 = make_float2(scale_log2, scale_log2);
+        unsigned char *os = sm + G::OFF_O + warp * (32 * 128);
+        int u = 0;
+        uint32_t w_first = 0u;                                   // the query's choice of the first 32 blocks, asked for early
+        auto first_word = [&]() {
+            const int64_t t = t0 + s * kTile + lq;
+            w_first = masks && t < len ? __ldcg(masks + ((int64_t)bh * len + t) * words) : 0u;
+        };
+        grid_dependency_wait();
+        bool more = take(0);
+        if (more) first_word();
+#pragma unroll 1
+        for (int k = 0; more; ++k) {
+        const Chosen &c_of = chosen_of[k & 1];
         const int64_t tq = t0 + s * kTile + lq;
         const bool in = tq < len;
-        const uint32_t tl = tb + s * ACC + ((uint32_t)((warp & 3) * 32) << 16);
         const uint32_t *row = masks + ((int64_t)bh * len + (in ? tq : 0)) * words;
-        uint32_t w_cur = 0u, w_next = 0u;                        // the query's choice of the 32 blocks around the walk, and of the next 32
-        int w_at = -1;
+        // the walk of this warp's accumulator, by words of 32 blocks: the blocks of the word that are still to come, the present
+        // one's bit, those of the accumulator's queries, the query's own and its next 32
+        uint32_t bits = 0u, low = 0u, ours = 0u, w_cur = 0u, w_next = w_first;
+        int w = -1, r = cpb - 1;
         const int32_t *mine = lists + ((int64_t)bh * len + (in ? tq : 0)) * K;
         int at = 0;                                              // without masks: the query's first list entry that is not behind the walk
         float m = -CUDART_INF_F;                                 // what the weights are relative to (scaled, log2)
         float2 l2 = make_float2(0.0f, 0.0f);                     // sums of the weights (even and odd positions)
-        const float2 sc2 = make_float2(scale_log2, scale_log2);
-        int u = 0;
-        Walk wk;
+        const int u0 = u;
 #pragma unroll 1
-        for (int i = 0; i < n; ++i, wk.next(cpb)) {
-            const uint32_t e = list[wk.bi];
-            if (!((e >> (14 + s)) & 1u)) continue;
-            const int j = e & 0x3fff;
+        for (int i = 0; i < n; ++i, ++g) {
+            if (++r == cpb) {
+                r = 0;
+                bits ^= low;
+                while (!bits) {
+                    ++w;
+                    ours = c_of.by[s][w];
+                    bits = c_of.by[0][w] | c_of.by[1][w];
+                    w_cur = w_next;
+                    w_next = in && masks && w + 1 < words ? __ldcg(row + w + 1) : 0u;
+                }
+                low = bits & (0u - bits);
+            }
+            if (!(ours & low)) continue;
+            const int j = w * 32 + 31 - __clz((int)low);
             bool chosen;
             if (masks) {
-                if ((j >> 5) != w_at) {
-                    const int w = j >> 5;
-                    w_cur = w_at >= 0 && w == w_at + 1 ? w_next : in ? __ldcg(row + w) : 0u;
-                    w_next = in && w + 1 < words ? __ldcg(row + w + 1) : 0u;
-                    w_at = w;
-                }
-                chosen = (w_cur >> (j & 31)) & 1u;
+                chosen = w_cur & low;
             } else {
                 while (in && at < K && (uint32_t)__ldcg(mine + at) < (uint32_t)j) ++at;    // (-1: beyond every block)
                 chosen = in && at < K && __ldcg(mine + at) == j;
             }
-            const int c = j * cpb + wk.r;
+            const int c = j * cpb + r;
             const int64_t p0 = (int64_t)c * kChunk;
             // positions this query attends among the chunk's: none if it did not choose the block, else those up to its own
             int nv = 0;
@@ -411,11 +552,11 @@ __global__ void __launch_bounds__(kThreads, 1) moba_mma_kernel(const __grid_cons
             if (p0 + kChunk > len) {
                 // the prompt ends inside this chunk: the value rows past its end hold whatever the cache's memory held; a
                 // weight of zero would not stop a NaN there, so those rows are cleared once they have landed
-                ok = mbar_wait(&full_v[i % NST], (uint32_t)((i / NST) & 1));
+                ok = mbar_wait(&full_v[g % NST], (uint32_t)((g / NST) & 1));
                 if (!__all_sync(FULL, ok)) break;
                 const int r = lq & (kChunk - 1), hf = lq >> 6;
                 if (hf < G::HALVES && p0 + r >= len) {
-                    uint4 *vrow = reinterpret_cast<uint4 *>(vst + (size_t)(i % NST) * G::C_BYTES + hf * (kChunk * 128) + (r >> 3) * 1024 +
+                    uint4 *vrow = reinterpret_cast<uint4 *>(vst + (size_t)(g % NST) * G::C_BYTES + hf * (kChunk * 128) + (r >> 3) * 1024 +
                                                             (r & 7) * 128);
 #pragma unroll
                     for (int k = 0; k < 8; ++k) vrow[k] = make_uint4(0u, 0u, 0u, 0u);
@@ -427,36 +568,53 @@ __global__ void __launch_bounds__(kThreads, 1) moba_mma_kernel(const __grid_cons
             mbar_arrive(&p_ready[s][u & 1]);
             ++u;
         }
+        ok = __all_sync(FULL, ok);
+        if (!ok) break;
+        // the next tile, whose first choices come while this one's output goes
+        const int h = bh % H, b = bh / H;
+        more = take(k + 1);
+        if (!ok) break;
+        if (more) first_word();
         // the output once the last product is complete, divided by the sum of the query's weights
-        if (__all_sync(FULL, ok) && u > 0) {
-            ok = mbar_wait(&pv_done[s][(u - 1) & 1], (uint32_t)(((u - 1) >> 1) & 1));
-            if (__all_sync(FULL, ok)) {
-                tcgen05_after_sync();
-                const float inv = 1.0f / (l2.x + l2.y);          // (nothing but scores of -inf: NaN; rows past the prompt are not stored)
-                // (the accumulator's queries are not read any more: its rows go out through their room, a store per warp and
-                // 64 channels; rows past the prompt are cut off by the map)
-                unsigned char *os = qs + s * G::Q_BYTES + (warp & 3) * 32 * 128;
-#pragma unroll 1
-                for (int cb = 0; cb < D; cb += 32) {
-                    float v[32];
-                    tmem_ld32(tl + OFF_O + cb, v);
+        if (u > u0) {
+            if (!wait_all(&pv_done[s][(u - 1) & 1], (u - 1) >> 1)) break;
+            tcgen05_after_sync();
+            const float inv = 1.0f / (l2.x + l2.y);              // (nothing but scores of -inf: NaN; rows past the prompt are not stored)
+            // (the rows go out through room of their own, a store per warp and 64 channels; rows past the prompt are cut off by the map)
+            const float2 inv2 = make_float2(inv, inv);
+            auto pair = [&](float x, float y) {
+                const float2 z = mul2(make_float2(x, y), inv2);
+                return pack_bf16(z.x, z.y);
+            };
+            float v[2][32];
+            tmem_ld32_start(tl + OFF_O, v[0]);
 #pragma unroll
-                    for (int k = 0; k < 32; k += 8)
-                        *reinterpret_cast<uint4 *>(os + (cb >> 6) * (kTile * 128) + umma_sw128_offset(lane, ((cb & 63) + k) >> 3)) =
-                            make_uint4(pack_bf16(v[k] * inv, v[k + 1] * inv), pack_bf16(v[k + 2] * inv, v[k + 3] * inv),
-                                       pack_bf16(v[k + 4] * inv, v[k + 5] * inv), pack_bf16(v[k + 6] * inv, v[k + 7] * inv));
+            for (int cb = 0; cb < D / 32; ++cb) {
+                float (&y)[32] = v[cb & 1];
+                tmem_ld32_wait(y);
+                if (cb + 1 < D / 32) tmem_ld32_start(tl + OFF_O + (cb + 1) * 32, v[(cb + 1) & 1]);
+                if ((cb & 1) == 0) {
+                    tma_store_wait_read();                       // what was there before has gone
+                    __syncwarp();
                 }
-                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-                __syncwarp();
-                if (tq - lane < len) {
 #pragma unroll
-                    for (int hf = 0; hf < G::HALVES; ++hf)
-                        tma_store_4d(os + hf * (kTile * 128), &omap, hf * 64, h, (int)(tq - lane), b);
-                    tma_store_commit();
-                    tma_store_wait_read();
+                for (int x = 0; x < 32; x += 8)
+                    *reinterpret_cast<uint4 *>(os + umma_sw128_offset(lane, ((cb & 1) * 32 + x) >> 3)) =
+                        make_uint4(pair(y[x], y[x + 1]), pair(y[x + 2], y[x + 3]), pair(y[x + 4], y[x + 5]), pair(y[x + 6], y[x + 7]));
+                if (cb & 1) {
+                    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                    __syncwarp();
+                    if (tq - lane < len) {
+                        tma_store_4d(os, &omap, (cb >> 1) * 64, h, (int)(tq - lane), b);
+                        tma_store_commit();
+                    }
                 }
             }
+            tcgen05_before_sync();
         }
+        leave(k);
+        }
+        tma_store_wait_read();                                   // nothing leaves this CTA's shared memory after it
     }
     if (__any_sync(FULL, !ok) && lane == 0) atomicCAS(status, RQ_OK, RQ_ERR_TIMEOUT);
     tcgen05_before_sync();
@@ -499,7 +657,7 @@ template <int D> cudaError_t attend_run(const MobaArgs &a, cudaStream_t s)
     cfg.attrs = &at;
     cfg.numAttrs = 1;
     return cudaLaunchKernelEx(&cfg, moba_mma_kernel<D>, tmap, qmap, omap, a.page_cap, a.S, a.len, a.H, BH, set, tiles, a.block, nb, (const uint32_t *)a.masks,
-                              (const int32_t *)a.list, a.K, a.scale * 1.4426950408889634f, a.status);
+                              (const uint32_t *)a.unions, (const int32_t *)a.list, a.K, a.scale * 1.4426950408889634f, a.status);
 }
 
 }  // namespace

@@ -130,7 +130,7 @@ template <int NB> __device__ __forceinline__ uint32_t score_bin(float v, float l
 // the registers of a query's four threads instead of buckets: 49.7 us for the 4096 queries.
 template <int D, int FORM>
 __global__ void __launch_bounds__(kRouteThreads, 2) moba_route_mma_kernel(const __grid_constant__ CUtensorMap qmap, const float *means, const unsigned char *terms, int64_t len, int H,
-                                                                      int block, int nb, int K, int words, uint32_t *masks,
+                                                                      int block, int nb, int K, int words, uint32_t *masks, uint32_t *unions,
                                                                       int32_t *list, int32_t *status)
 {
     using G = RouteGeom<D, FORM>;
@@ -598,15 +598,29 @@ __global__ void __launch_bounds__(kRouteThreads, 2) moba_route_mma_kernel(const 
     grid_dependency_wait();
     grid_launch_dependents();
     __syncthreads();
-    // the masks go out, with the first block and the query's own; a word after the other of the CTA's, so that the stores fill lines
+    // a query's choice among the 32 blocks of a word, with the first block and the query's own
+    auto chosen = [&](int r, int w) -> uint32_t {
+        const int o = s_own[r], hi = o + 1 - 32 * w;
+        if (K >= o + 1) return hi >= 32 ? 0xffffffffu : hi <= 0 ? 0u : (1u << hi) - 1u;
+        return mk[w * MP + r] | (w == 0 ? 1u : 0u) | (w == (o >> 5) ? 1u << (o & 31) : 0u);
+    };
+    if (unions) {                                                              // what any of the queries chose, a warp per word
+        for (int w = warp; w < words; w += kRouteThreads / 32) {
+            uint32_t m = 0u;
+#pragma unroll
+            for (int i = 0; i < NQ / 32; ++i)
+                if (t0 + i * 32 + lane < len) m |= chosen(i * 32 + lane, w);
+            m = __reduce_or_sync(FULL, m);
+            if (lane == 0) unions[((int64_t)bh * gridDim.y + (t0 / NQ)) * words + w] = m;
+        }
+        if (list) __syncthreads();                                             // (mk changes below)
+    }
+    // the masks go out; a word after the other of the CTA's, so that the stores fill lines
     const float per_word = 1.0f / (float)words;
     for (int i = tid; i < NQ * words; i += kRouteThreads) {
         const int r = (int)(((float)i + 0.5f) * per_word), w = i - r * words;  // (exact: i < 2^18, and half a word is never within rounding)
         if (t0 + r >= len) continue;
-        const int o = s_own[r], hi = o + 1 - 32 * w;
-        uint32_t m;
-        if (K >= o + 1) m = hi >= 32 ? 0xffffffffu : hi <= 0 ? 0u : (1u << hi) - 1u;
-        else m = mk[w * MP + r] | (w == 0 ? 1u : 0u) | (w == (o >> 5) ? 1u << (o & 31) : 0u);
+        const uint32_t m = chosen(r, w);
         if (masks) masks[((int64_t)bh * len + t0) * words + i] = m;
         if (list) mk[w * MP + r] = m;
     }
@@ -663,7 +677,7 @@ template <int D, int FORM> cudaError_t route_launch(const MobaArgs &a, int nb, i
     cfg.attrs = &at;
     cfg.numAttrs = 1;
     return cudaLaunchKernelEx(&cfg, moba_route_mma_kernel<D, FORM>, qmap, (const float *)a.means, (const unsigned char *)a.terms, a.len, a.H, a.block,
-                              nb, a.K, words, a.masks, a.list, a.status);
+                              nb, a.K, words, a.masks, a.unions, a.list, a.status);
 }
 
 template <int D> cudaError_t route_run(const MobaArgs &a, cudaStream_t s)
