@@ -116,7 +116,8 @@ struct Walk {
 // the last weights of this one are taken and its output goes.  A CTA per tile spent 0.6 us on its set-up, 2 on the list of blocks,
 // 1.5 up to the first product and 3 at the end.  Launch, us, a CTA per tile / this: 32 heads x 4096 positions 185 / 174.5, x 30011
 // 5760 / 5570 (three stages of keys and values and all of the output's rows in shared memory at once instead of four and halves:
-// 174.5 / 5680; a next tile taken at once instead of six steps before the end would pair the longest tiles).  What any query of a tile
+// 174.5 / 5680; a next tile taken at once instead of six steps before the end would pair the longest tiles); with the readers' positions
+// in 32 bits 169.5 / 5420: every instruction between one score buffer and the next counts.  What any query of a tile
 // chose comes from the routing as a word per 32 blocks, 128 queries together; the walk goes by its bits.
 // A tile's 256 consecutive queries are two accumulators of 128 lanes; everything per query (choice of blocks, causal cut, what its weights
 // are relative to, their sum, the weights) belongs to one thread.  The 64-position chunks of the blocks that any of the 256
@@ -142,7 +143,10 @@ struct Walk {
 // Measured, call, 32 heads x 128 channels, 4096 positions (16 of 64 blocks) at logits of 1.4 / 5 / 11: rows multiplied down before
 // the weights, 16 columns at a time, 223.5 / 238 / 243 us; after them 217 / 227 / 231 (without ever doing it 214).  Bound: the
 // readers' chain per chunk (about 1850 cycles at 4096 positions, of which ex2 alone takes 1024, against 1280 for the products, whose
-// operands take shared memory's bandwidth); at 30011 positions the power limit as well.  Slower: weights taken before the maximum is known and again where it
+// operands take shared memory's bandwidth); at 30011 positions the power limit as well.  Of 174 us (5580) without exponentials 141
+// (4530), without raising 164 (5350), without maxima and sums 161 (5290), without output products 165 (5300).  Slower: two sets of
+// readers that take chunks in turn, a query's m handed on through shared memory (179 us / 5.70 ms: a buffer's way from product to product
+// is the bound then); scores in one buffer that is free once they are in registers, weights in two of their own (222 / 7.2); weights taken before the maximum is known and again where it
 // was too far off (251 us; by halves of a chunk 240); the next chunk's scores loaded while the weights are handed over; queries as
 // columns, so that weights are taken only for eights or sixteens of queries some of which chose the chunk (236 us / 7.1 ms at 30011);
 // and only the queries that chose a chunk gathered for it (377 us / 9.6 ms: lists, gathers and scattered weights cost more than
@@ -440,8 +444,9 @@ __global__ void __launch_bounds__(kThreads, 1) moba_mma_kernel(const __grid_cons
 #pragma unroll 1
         for (int k = 0; more; ++k) {
         const Chosen &c_of = chosen_of[k & 1];
-        const int64_t tq = t0 + s * kTile + lq;
+        const int tq = (int)t0 + s * kTile + lq;
         const bool in = tq < len;
+        const int seen = in ? tq + 1 : 0;                        // positions that the query may attend
         const uint32_t *row = masks + ((int64_t)bh * len + (in ? tq : 0)) * words;
         // the walk of this warp's accumulator, by words of 32 blocks: the blocks of the word that are still to come, the present
         // one's bit, those of the accumulator's queries, the query's own and its next 32
@@ -475,11 +480,9 @@ __global__ void __launch_bounds__(kThreads, 1) moba_mma_kernel(const __grid_cons
                 while (in && at < K && (uint32_t)__ldcg(mine + at) < (uint32_t)j) ++at;    // (-1: beyond every block)
                 chosen = in && at < K && __ldcg(mine + at) == j;
             }
-            const int c = j * cpb + r;
-            const int64_t p0 = (int64_t)c * kChunk;
+            const int p0 = j * block + r * kChunk;
             // positions this query attends among the chunk's: none if it did not choose the block, else those up to its own
-            int nv = 0;
-            if (in && chosen) nv = (int)max((int64_t)0, min((int64_t)kChunk, tq - p0 + 1));
+            const int nv = chosen ? max(0, min(kChunk, seen - p0)) : 0;
             ok = mbar_wait(&s_ready[s][u & 1], (uint32_t)((u >> 1) & 1));
             if (!__all_sync(FULL, ok)) break;
             tcgen05_after_sync();
@@ -605,7 +608,7 @@ __global__ void __launch_bounds__(kThreads, 1) moba_mma_kernel(const __grid_cons
                     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
                     __syncwarp();
                     if (tq - lane < len) {
-                        tma_store_4d(os, &omap, (cb >> 1) * 64, h, (int)(tq - lane), b);
+                        tma_store_4d(os, &omap, (cb >> 1) * 64, h, tq - lane, b);
                         tma_store_commit();
                     }
                 }
