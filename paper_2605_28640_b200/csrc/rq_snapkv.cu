@@ -12,6 +12,7 @@
 // weights.
 //   snap_once_kernel          bf16 caches, up to 4096 positions: the scores do fit in the tensor memory of a cluster of CTAs
 //                             and the keys are read once
+//   snap_stream_kernel        bf16 caches, many heads of up to 16384 positions: the two passes below side by side in one launch
 //   snap_mma_kernel<PASS 1>   longer bf16 caches.  Per (head, run of 128-key tiles): the scores of a tile on the
 //                             tensor cores (tcgen05.mma, operands in shared memory, fp32 accumulator
 //                             in tensor memory): D[query][key] with the window's queries as the M
@@ -35,6 +36,7 @@
 #include <math.h>
 #include <math_constants.h>
 
+#include <algorithm>
 #include <utility>
 
 #include "rq_async.cuh"
@@ -207,6 +209,59 @@ __device__ __forceinline__ float exp2_fast(float x)
     return y;
 }
 
+// (largest score, sum of exponentials relative to it) of two sets of keys together
+__device__ __forceinline__ float2 merge_stat(float2 a, float2 b)
+{
+    const float m = fmaxf(a.x, b.x);
+    const float fa = a.x > -CUDART_INF_F ? exp2f(a.x - m) : 0.0f, fb = b.x > -CUDART_INF_F ? exp2f(b.x - m) : 0.0f;
+    return make_float2(m, a.y * fa + b.y * fb);
+}
+
+// N scores of one query join its running statistics (maximum m and sum l of exponentials, log2 domain); not seen: -inf, but
+// at least one is seen.  Four chains for the maximum, packed pairs for the sum.  The scale is positive.
+template <int N> __device__ __forceinline__ void add_scores(const float (&v)[N], float scale_log2, float &m, float &l)
+{
+    float tm[4] = {v[0], v[1], v[2], v[3]};
+#pragma unroll
+    for (int c = 4; c < N; ++c) tm[c & 3] = fmaxf(tm[c & 3], v[c]);
+    const float mn = fmaxf(m, fmaxf(fmaxf(tm[0], tm[1]), fmaxf(tm[2], tm[3])) * scale_log2);
+    const float2 sc2 = make_float2(scale_log2, scale_log2), nm2 = make_float2(-mn, -mn);
+    float2 sum[2] = {make_float2(0.0f, 0.0f), make_float2(0.0f, 0.0f)};
+#pragma unroll
+    for (int c = 0; c < N; c += 2) {
+        const float2 x = fma2(make_float2(v[c], v[c + 1]), sc2, nm2);
+        sum[(c >> 1) & 1] = add2(sum[(c >> 1) & 1], make_float2(exp2_fast(x.x), exp2_fast(x.y)));
+    }
+    const float2 both = add2(sum[0], sum[1]);
+    l = l * exp2_fast(m - mn) + (both.x + both.y);             // 2^(-inf) = 0 the first time
+    m = mn;
+}
+
+// N queries' scores of one key: its weights under queries q0 .. q0 + N - 1 (nm: -maximum, il: 1 / sum of each) are added up, in
+// the same order for every key.  Cut: only queries q_lo .. W - 1 see the key.
+template <int N>
+__device__ __forceinline__ void add_weights(const float (&v)[N], int q0, bool cut, int q_lo, int W, float scale_log2, const float *q_nm,
+                                            const float *q_il, float2 (&acc)[2])
+{
+    const float2 sc2 = make_float2(scale_log2, scale_log2);
+#pragma unroll
+    for (int c = 0; c < N; c += 4) {
+        const int q = q0 + c;
+        const float4 nm = *reinterpret_cast<const float4 *>(&q_nm[q]), il = *reinterpret_cast<const float4 *>(&q_il[q]);
+        const float2 x = fma2(make_float2(v[c], v[c + 1]), sc2, make_float2(nm.x, nm.y));
+        const float2 y = fma2(make_float2(v[c + 2], v[c + 3]), sc2, make_float2(nm.z, nm.w));
+        float2 e = make_float2(exp2_fast(x.x), exp2_fast(x.y)), f = make_float2(exp2_fast(y.x), exp2_fast(y.y));
+        if (cut) {
+            e.x = q < W && q >= q_lo ? e.x : 0.0f;
+            e.y = q + 1 < W && q + 1 >= q_lo ? e.y : 0.0f;
+            f.x = q + 2 < W && q + 2 >= q_lo ? f.x : 0.0f;
+            f.y = q + 3 < W && q + 3 >= q_lo ? f.y : 0.0f;
+        }
+        acc[0] = fma2(e, make_float2(il.x, il.y), acc[0]);
+        acc[1] = fma2(f, make_float2(il.z, il.w), acc[1]);
+    }
+}
+
 // Grid (runs of tiles, heads).  stats: [bh][runs][64]; rowstat: [bh][64]; imp: [bh][len].
 // tmap: the cache as a rank-4 tensor (channel, slot, key / value, page over all heads), box = 64 channels
 // x the slots of a page x keys only x the pages of 128 positions, 128-byte swizzle: one copy brings one
@@ -360,7 +415,6 @@ __global__ void __launch_bounds__(kMmaThreads, D == 128 ? 6 : 4) snap_mma_kernel
         const int64_t j0 = (int64_t)tile(i) * kMmaKeys;
         const uint32_t tl = tb + (uint32_t)(i & 1) * ACC + ((uint32_t)(warp * 32) << 16);    // this warp's lanes of the accumulator
         const bool cut = W < kSnapRows || j0 + kMmaKeys - 1 > first_q;     // some key of the tile is not seen by all 64 queries
-        const float2 sc2 = make_float2(scale_log2, scale_log2);
         float v[N];
         auto load = [&](int c0) {
             if constexpr (N == 32) tmem_ld32(tl + (uint32_t)c0, v);
@@ -377,47 +431,17 @@ __global__ void __launch_bounds__(kMmaThreads, D == 128 ? 6 : 4) snap_mma_kernel
 #pragma unroll
                     for (int c = 0; c < N; ++c) v[c] = c < nv ? v[c] : -CUDART_INF_F;
                 }
-                float tm[4] = {v[0], v[1], v[2], v[3]};
-#pragma unroll
-                for (int c = 4; c < N; ++c) tm[c & 3] = fmaxf(tm[c & 3], v[c]);
-                if (nv > 0) {                                  // (so that the maximum is that of a key)
-                    const float mn = fmaxf(m, fmaxf(fmaxf(tm[0], tm[1]), fmaxf(tm[2], tm[3])) * scale_log2);   // (the scale is positive)
-                    const float2 nm2 = make_float2(-mn, -mn);
-                    float2 sum[2] = {make_float2(0.0f, 0.0f), make_float2(0.0f, 0.0f)};
-#pragma unroll
-                    for (int c = 0; c < N; c += 2) {
-                        const float2 x = fma2(make_float2(v[c], v[c + 1]), sc2, nm2);
-                        sum[(c >> 1) & 1] = add2(sum[(c >> 1) & 1], make_float2(exp2_fast(x.x), exp2_fast(x.y)));
-                    }
-                    const float2 both = add2(sum[0], sum[1]);
-                    l = l * exp2_fast(m - mn) + (both.x + both.y);         // 2^(-inf) = 0 the first time
-                    m = mn;
-                }
+                if (nv > 0) add_scores<N>(v, scale_log2, m, l);
             }
         } else {
-            // lane = key, column = query: the key's weights summed over the queries that see it, in the same order for every key
+            // lane = key, column = query: the key's weights summed over the queries that see it
             const int64_t j = j0 + tid;
             const int q_lo = (int)min((int64_t)64, max((int64_t)0, j - first_q));
             float2 acc[2] = {make_float2(0.0f, 0.0f), make_float2(0.0f, 0.0f)};
 #pragma unroll 1
             for (int cb = 0; cb < kSnapRows; cb += N) {
                 load(cb);
-#pragma unroll
-                for (int c = 0; c < N; c += 4) {
-                    const int q = cb + c;
-                    const float4 nm = *reinterpret_cast<const float4 *>(&q_nm[q]), il = *reinterpret_cast<const float4 *>(&q_il[q]);
-                    const float2 x = fma2(make_float2(v[c], v[c + 1]), sc2, make_float2(nm.x, nm.y));
-                    const float2 y = fma2(make_float2(v[c + 2], v[c + 3]), sc2, make_float2(nm.z, nm.w));
-                    float2 e = make_float2(exp2_fast(x.x), exp2_fast(x.y)), f = make_float2(exp2_fast(y.x), exp2_fast(y.y));
-                    if (cut) {
-                        e.x = q < W && q >= q_lo ? e.x : 0.0f;
-                        e.y = q + 1 < W && q + 1 >= q_lo ? e.y : 0.0f;
-                        f.x = q + 2 < W && q + 2 >= q_lo ? f.x : 0.0f;
-                        f.y = q + 3 < W && q + 3 >= q_lo ? f.y : 0.0f;
-                    }
-                    acc[0] = fma2(e, make_float2(il.x, il.y), acc[0]);
-                    acc[1] = fma2(f, make_float2(il.z, il.w), acc[1]);
-                }
+                add_weights<N>(v, cb, cut, q_lo, W, scale_log2, q_nm, q_il, acc);
             }
             const float2 both = add2(acc[0], acc[1]);
             if (j < len) imp[(int64_t)bh * len + j] = both.x + both.y;
@@ -442,6 +466,350 @@ __global__ void __launch_bounds__(kMmaThreads, D == 128 ? 6 : 4) snap_mma_kernel
     tcgen05_before_sync();
     __syncthreads();
     if (warp == 0) tmem_dealloc(tbase, TCOLS);
+}
+
+// ---------------------------------------------------------------- many heads: both passes in one launch, side by side
+// One CTA per SM runs both passes, each a pipeline of its own: the first takes items (a run of tiles of a head) in order of a
+// ticket counter, the second takes the same items in the same order from a counter of its own, as soon as the head's statistics are
+// known; its keys are mostly in L2 still.
+//   warps 0..7    read the first pass's accumulators, 8..15 the second's: two groups of four, which take tiles in turn
+//   warps 16, 17  tickets and copies of a pass, in pieces of 64 channels of a tile's keys
+//   warps 18, 19  queries and products of a pass
+//   warp 20       statistics: merges those of an item's four parts into a record; who brings a head's last record merges them
+//   warp 21       the head's statistics for the second pass's readers
+// The first pass waits for nothing but its own copies and products, and the second for items of the first whose tickets CTAs that run
+// have taken: nothing here depends on how many CTAs run at a time.  A query's statistics are there once its word is not zero (the
+// words are cleared before the launch, and the sum of a maximum and smaller terms is at least one).
+// Bound: the handshakes of a tile (without arithmetic, 64 channels, 256 heads x 4096: the first pass alone 0.7 us a tile, the second
+// 0.5, of which an SM has 55 each).  A call of rq_snapkv_select, us, cluster or two launches / this: 256 heads x 4096 113 / 96, 64 channels
+// 99 / 78; 320 x 3200 119 / 95; 160 x 3500 72 / 62; 256 x 5000 139.5 / 126.6; 256 x 8192 221 / 195; 256 x 16384 437 / 379; 96 x
+// 12000 126.5 / 124.  Items of 4 or 12 tiles: 256 x 4096 94 and 96 (8: 92, on one box).  Not for fewer tiles than thirty to an SM, which do
+// not outweigh its start and end (128 x 4096 60.4 / 61.2), nor for heads of more than 128 tiles, whose second pass is
+// so far behind that L2 has lost their keys (32 x 65536: 968 MB read from DRAM of 537; 96 x 40000 375 / 407, 64 channels 32 x 50000 121 /
+// 138; smaller items or a first pass held back lose more than they win).
+constexpr int kStreamStages = 5;               // pieces a pass has in shared memory
+constexpr int kStreamItems = 4;                // items a pass's warps know ahead
+constexpr int kStreamReaders = 8;              // per pass
+constexpr int kStreamThreads = (2 * kStreamReaders + 6) * 32;
+constexpr int kStreamTiles = 8;                // tiles of an item, about
+constexpr int kStreamMaxTiles = 128;           // of a head
+constexpr int kStreamMaxRuns = kStreamMaxTiles / kStreamTiles;
+// tiles per SM that it takes at least: where it stands for the cluster form or the readers of two launches are their bound; where it
+// stands for two launches of 128 channels, whose second pass finds smaller sets of keys in L2 as well (70 x 8192 65.6 / 69.7, 40 x 14500
+// 85.4 / 88.5, but 128 x 6000 82.4 / 79.8, 128 x 8192 109 / 96)
+constexpr int kStreamPerSm = 30, kStreamPerSmWide = 40;
+constexpr int kStreamAhead = 3;                // tiles between an L2 prefetch and the copy of the same keys
+
+template <int D>
+struct SnapStreamGeom {
+    static constexpr int HALVES = D / 64;
+    static constexpr int PIECE_BYTES = kMmaKeys * 128;
+    static constexpr int OFF_Q2 = HALVES * PIECE_BYTES;        // the first pass's queries, twice (128 rows); then the second's
+    static constexpr int OFF_K = OFF_Q2 + HALVES * PIECE_BYTES / 2;
+    static constexpr int SMEM_BYTES = OFF_K + 2 * kStreamStages * PIECE_BYTES + 1024;
+};
+struct SnapItem { int bh, t0, n, run; };                       // n = 0: the end
+
+// what the warps of a pass meet through
+struct SnapPipe {
+    uint64_t full_k[kStreamStages], free_k[kStreamStages], full_q, free_q, full_i[kStreamItems], free_i[kStreamItems];
+    uint64_t ready[4], acc_free[4], stat_full[2], stat_free[2];
+    SnapItem item[kStreamItems];
+};
+
+template <int D>
+__global__ void __launch_bounds__(kStreamThreads, 1) snap_stream_kernel(const __grid_constant__ CUtensorMap tmap,
+                                                                        const __grid_constant__ CUtensorMap qmap, int64_t page_cap, int S,
+                                                                        int64_t len, int W, int H, int BH, float scale_log2, float2 *stats,
+                                                                        float2 *rowstat, int32_t *counters, float *imp, int ntiles, int tpc,
+                                                                        int runs, int32_t *status)
+{
+    using G = SnapStreamGeom<D>;
+    constexpr unsigned FULL = 0xffffffffu;
+    constexpr int NST = kStreamStages, NI = kStreamItems;
+    extern __shared__ __align__(1024) unsigned char dsm_raw[];
+    __shared__ __align__(8) SnapPipe pipes[2];
+    __shared__ uint32_t tbase;
+    __shared__ __align__(16) float2 part[2][4][kSnapRows];     // first pass: an item's statistics by group and half of the tile's keys
+    __shared__ __align__(16) float q_nm[2][kSnapRows], q_il[2][kSnapRows];   // second pass: -maximum and 1 / sum of an item's queries
+    unsigned char *dsm = dsm_raw + ((1024u - (smem_addr(dsm_raw) & 1023u)) & 1023u);
+
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int64_t first_q = len - W;                           // position of query 0
+    if (warp == 0) tmem_alloc(&tbase, 512);
+    if (warp == 1 && lane < 2) {
+        SnapPipe &p = pipes[lane];
+        for (int i = 0; i < NST; ++i) { mbar_init(&p.full_k[i], 1); mbar_init(&p.free_k[i], 1); }
+        mbar_init(&p.full_q, 1);
+        mbar_init(&p.free_q, 1);
+        for (int i = 0; i < NI; ++i) { mbar_init(&p.full_i[i], 1); mbar_init(&p.free_i[i], kStreamReaders + 2); }
+        for (int i = 0; i < 4; ++i) { mbar_init(&p.ready[i], 1); mbar_init(&p.acc_free[i], 4); }
+        for (int i = 0; i < 2; ++i) {
+            mbar_init(&p.stat_full[i], lane == 0 ? kStreamReaders : 1);
+            mbar_init(&p.stat_free[i], lane == 0 ? 1 : kStreamReaders);
+        }
+        mbar_init_fence();
+    }
+    tcgen05_before_sync();
+    __syncthreads();
+    tcgen05_after_sync();
+    const uint32_t tb = __shfl_sync(FULL, tbase, 0);           // (the shuffle tells the compiler that it is uniform)
+    grid_dependency_wait();                                    // the counters are cleared by the kernel before
+    grid_launch_dependents();
+    bool ok = true;
+    auto wait_all = [&](uint64_t *x, int phase) -> bool { return ok = __all_sync(FULL, mbar_wait(x, (uint32_t)(phase & 1))); };
+    auto arrive = [&](uint64_t *x) {                           // of a warp
+        __syncwarp();
+        if (lane == 0) mbar_arrive(x);
+    };
+    // the q-th item of a pass; false: there is none, or a wait ran out
+    auto item_at = [&](SnapPipe &p, int q, SnapItem &it) -> bool {
+        if (!wait_all(&p.full_i[q % NI], q / NI)) return false;
+        const SnapItem &e = p.item[q % NI];
+        it.bh = __shfl_sync(FULL, e.bh, 0);
+        it.t0 = __shfl_sync(FULL, e.t0, 0);
+        it.n = __shfl_sync(FULL, e.n, 0);
+        it.run = __shfl_sync(FULL, e.run, 0);
+        arrive(&p.free_i[q % NI]);
+        return it.n != 0;
+    };
+
+    const int pass = warp < 2 * kStreamReaders ? warp / kStreamReaders : warp & 1;
+    SnapPipe &p = pipes[pass];
+    unsigned char *qs = dsm + (pass ? G::OFF_Q2 : 0), *ks = dsm + G::OFF_K + pass * NST * G::PIECE_BYTES;
+    const uint32_t q_half = pass ? G::PIECE_BYTES / 2 : G::PIECE_BYTES;      // 64 channels of the queries
+    const int n_acc = pass ? 4 : 2, acc_cols = pass ? 64 : 128;
+    const uint32_t tp = tb + (uint32_t)pass * 256u;
+    SnapItem it;
+    if (warp >= 2 * kStreamReaders && warp < 2 * kStreamReaders + 2) {
+        // ---- tickets and copies (the whole warp, like the products: see rq_umma.cuh)
+        const int ppt = kMmaKeys / S;
+        int32_t *ticket = counters + BH + pass;
+        int next = lane == 0 ? atomicAdd(ticket, 1) : 0;
+        int known = 0, pi = 0;                                 // items announced, pieces started
+        auto announce = [&]() -> SnapItem {
+            const int t = __shfl_sync(FULL, next, 0);
+            SnapItem e = {0, 0, 0, 0};
+            if (t < BH * runs) {
+                if (lane == 0) next = atomicAdd(ticket, 1);
+                e.bh = t / runs;
+                e.run = t % runs;
+                e.t0 = e.run * tpc;
+                e.n = min(tpc, ntiles - e.t0);
+            }
+            if (known >= NI && !wait_all(&p.free_i[known % NI], known / NI - 1)) return e;
+            if (lane == 0) p.item[known % NI] = e;
+            arrive(&p.full_i[known % NI]);
+            ++known;
+            return e;
+        };
+        auto page_of = [&](const SnapItem &e, int i) { return (int)((int64_t)e.bh * page_cap + (int64_t)(e.t0 + i) * ppt); };
+        const uint64_t drop = l2_evict_first_policy();
+        SnapItem cur = announce();
+        while (ok && cur.n) {
+            const SnapItem after = announce();                 // known an item ahead
+#pragma unroll 1
+            for (int i = 0; i < cur.n && ok; ++i) {
+#pragma unroll
+                for (int hf = 0; hf < G::HALVES; ++hf, ++pi) {
+                    const int st = pi % NST;
+                    if (pi >= NST && !wait_all(&p.free_k[st], pi / NST - 1)) break;
+                    mbar_expect_warp(&p.full_k[st], G::PIECE_BYTES);
+                    if (pass) tma_load_4d_hint(ks + st * G::PIECE_BYTES, &tmap, hf * 64, 0, 0, page_of(cur, i), &p.full_k[st], drop);
+                    else tma_load_4d(ks + st * G::PIECE_BYTES, &tmap, hf * 64, 0, 0, page_of(cur, i), &p.full_k[st]);
+                }
+                // the stages keep too few bytes on their way from DRAM: a later tile, of the next item too, goes into L2 now
+                if (pass == 0 && ok) {
+                    const bool here = i + kStreamAhead < cur.n;
+                    const SnapItem &e = here ? cur : after;
+                    const int at = here ? i + kStreamAhead : i + kStreamAhead - cur.n;
+                    if (at < e.n) {
+#pragma unroll
+                        for (int hf = 0; hf < G::HALVES; ++hf) tma_prefetch_4d(&tmap, hf * 64, 0, 0, page_of(e, at));
+                    }
+                }
+            }
+            cur = after;
+        }
+        // after a wait that ran out: no copy may still be on its way into this CTA's shared memory when it exits
+        if (!ok)
+            for (int k = max(0, pi - NST); k < pi; ++k) mbar_wait(&p.full_k[k % NST], (uint32_t)((k / NST) & 1));
+    } else if (warp >= 2 * kStreamReaders + 2 && warp < 2 * kStreamReaders + 4) {
+        // ---- queries and products
+        const uint64_t qd = umma_desc_sw128(smem_addr(qs)), kd = umma_desc_sw128(smem_addr(ks));
+        int gi = 0, pi = 0;
+#pragma unroll 1
+        for (int q = 0; item_at(p, q, it); ++q) {
+            if (q > 0 && !wait_all(&p.free_q, q - 1)) break;   // the products of the item before have read its queries
+            mbar_expect_warp(&p.full_q, G::HALVES * q_half);
+#pragma unroll
+            for (int hf = 0; hf < G::HALVES; ++hf) {           // rows beyond the window come as zeros
+                tma_load_4d(qs + hf * q_half, &qmap, hf * 64, it.bh % H, 0, it.bh / H, &p.full_q);
+                if (pass == 0) tma_load_4d(qs + hf * q_half + q_half / 2, &qmap, hf * 64, it.bh % H, 0, it.bh / H, &p.full_q);
+            }
+            ok = __all_sync(FULL, mbar_wait(&p.full_q, (uint32_t)(q & 1)) || mbar_wait(&p.full_q, (uint32_t)(q & 1)));
+            if (!ok) break;
+#pragma unroll 1
+            for (int i = 0; i < it.n && ok; ++i, ++gi) {
+                const int acc = gi % n_acc;
+                if (gi >= n_acc && !wait_all(&p.acc_free[acc], gi / n_acc - 1)) break;
+#pragma unroll
+                for (int hf = 0; hf < G::HALVES; ++hf, ++pi) {
+                    const int st = pi % NST;
+                    if (!wait_all(&p.full_k[st], pi / NST)) break;
+                    tcgen05_after_sync();
+                    const uint64_t dq = qd + (uint64_t)((hf * q_half) >> 4), dk = kd + (uint64_t)((st * G::PIECE_BYTES) >> 4);
+                    if (pass == 0) umma_bf16_x4<2, 2>(tp + (uint32_t)(acc * acc_cols), dq, dk, umma_idesc_bf16(128, kMmaKeys), hf > 0);
+                    else umma_bf16_x4<2, 2>(tp + (uint32_t)(acc * acc_cols), dk, dq, umma_idesc_bf16(kMmaKeys, kSnapRows), hf > 0);
+                    umma_commit(&p.free_k[st]);
+                }
+                if (ok) umma_commit(&p.ready[acc]);
+            }
+            if (!ok) break;
+            umma_commit(&p.free_q);
+        }
+    } else if (warp == 2 * kStreamReaders + 4) {
+        // ---- statistics of the first pass; a lane has queries 2 lane, 2 lane + 1
+        auto merge4 = [&](float4 a, float4 b) {
+            const float2 x = merge_stat(make_float2(a.x, a.y), make_float2(b.x, b.y)), y = merge_stat(make_float2(a.z, a.w), make_float2(b.z, b.w));
+            return make_float4(x.x, x.y, y.x, y.y);
+        };
+#pragma unroll 1
+        for (int q = 0; item_at(p, q, it); ++q) {
+            if (!wait_all(&p.stat_full[q & 1], q >> 1)) break;
+            const float4 *mine = reinterpret_cast<const float4 *>(&part[q & 1][0][0]) + lane;
+            float4 f = mine[0];
+#pragma unroll
+            for (int i = 1; i < 4; ++i) f = merge4(f, mine[i * (kSnapRows / 2)]);
+            arrive(&p.stat_free[q & 1]);
+            if (runs > 1) {
+                float2 *rec = stats + (int64_t)it.bh * runs * kSnapRows;
+                __stcg(reinterpret_cast<float4 *>(rec + (int64_t)it.run * kSnapRows) + lane, f);
+                __syncwarp();
+                int others = 0;
+                if (lane == 0) others = atom_add_acq_rel(counters + it.bh, 1);
+                others = __shfl_sync(FULL, others, 0);
+                if (others != runs - 1) continue;
+                __syncwarp();
+                float4 x[kStreamMaxRuns];                      // all loads in flight at once
+#pragma unroll
+                for (int i = 0; i < kStreamMaxRuns; ++i)
+                    x[i] = i < runs ? ld_cg_now(reinterpret_cast<const float4 *>(rec + (int64_t)i * kSnapRows) + lane) : f;
+                f = x[0];
+#pragma unroll
+                for (int i = 1; i < kStreamMaxRuns; ++i)
+                    if (i < runs) f = merge4(f, x[i]);
+            }
+            // (a query that sees nothing: a sum of one)
+            unsigned long long *out = reinterpret_cast<unsigned long long *>(rowstat + (int64_t)it.bh * kSnapRows + 2 * lane);
+            f.y = f.y > 0.0f ? f.y : 1.0f;
+            f.w = f.w > 0.0f ? f.w : 1.0f;
+            st_relaxed(out, (unsigned long long)__float_as_uint(f.x) | (unsigned long long)__float_as_uint(f.y) << 32);
+            st_relaxed(out + 1, (unsigned long long)__float_as_uint(f.z) | (unsigned long long)__float_as_uint(f.w) << 32);
+        }
+    } else if (warp == 2 * kStreamReaders + 5) {
+        // ---- statistics for the second pass
+#pragma unroll 1
+        for (int q = 0; item_at(p, q, it); ++q) {
+            if (q >= 2 && !wait_all(&p.stat_free[q & 1], (q >> 1) - 1)) break;
+            const unsigned long long *in = reinterpret_cast<const unsigned long long *>(rowstat + (int64_t)it.bh * kSnapRows + 2 * lane);
+            unsigned long long a = 0ull, b = 0ull;
+            bool here = false;
+            for (int n = 0; n < kFlagPollLimit && !here; ++n) {
+                a = ld_relaxed(in);
+                b = ld_relaxed(in + 1);
+                here = __all_sync(FULL, a != 0ull && b != 0ull);
+            }
+            if (!here) { ok = false; break; }
+            auto put = [&](int row, unsigned long long w) {
+                const float m = __uint_as_float((uint32_t)w), l = __uint_as_float((uint32_t)(w >> 32));
+                q_nm[q & 1][row] = row < W ? -m : 0.0f;
+                q_il[q & 1][row] = row < W ? 1.0f / l : 1.0f;
+            };
+            put(2 * lane, a);
+            put(2 * lane + 1, b);
+            arrive(&p.stat_full[q & 1]);
+        }
+    } else {
+        // ---- readers: group g takes every other tile
+        const int g = (warp >> 2) & 1, gt = tid & 127, w = warp & 3;
+        const uint32_t tl = tp + ((uint32_t)(w * 32) << 16);
+        int gi = 0;                                            // tiles before the item
+#pragma unroll 1
+        for (int q = 0; item_at(p, q, it); ++q) {
+            if (pass == 0) {
+                const int row = gt & (kSnapRows - 1), half = gt >> 6;          // this thread's query and half of the tile's keys
+                float m = -CUDART_INF_F, l = 0.0f;
+#pragma unroll 1
+                for (int i = (gi ^ g) & 1; i < it.n; i += 2) {
+                    const int acc = (gi + i) & 1;
+                    if (!wait_all(&p.ready[acc], (gi + i) >> 1)) break;
+                    tcgen05_after_sync();
+                    const int64_t jb = (int64_t)(it.t0 + i) * kMmaKeys + half * 64;
+                    const bool cut = W < kSnapRows || jb + 63 > first_q;
+#pragma unroll 1
+                    for (int cb = 0; cb < 64; cb += 32) {
+                        float v[32];
+                        tmem_ld32(tl + (uint32_t)(acc * 128 + half * 64 + cb), v);
+                        if (cb) {
+                            tcgen05_before_sync();
+                            arrive(&p.acc_free[acc]);
+                        }
+                        int nv = 32;                           // visible keys among these: up to the query's own position
+                        if (cut) {
+                            nv = row < W ? (int)max((int64_t)0, min((int64_t)32, first_q + row - (jb + cb) + 1)) : 0;
+#pragma unroll
+                            for (int c = 0; c < 32; ++c) v[c] = c < nv ? v[c] : -CUDART_INF_F;
+                        }
+                        if (nv > 0) add_scores<32>(v, scale_log2, m, l);
+                        __syncwarp();
+                    }
+                }
+                if (!ok) break;
+                if (q >= 2 && !wait_all(&p.stat_free[q & 1], (q >> 1) - 1)) break;
+                part[q & 1][g * 2 + half][row] = make_float2(m, l);
+                arrive(&p.stat_full[q & 1]);
+            } else {
+                if (!wait_all(&p.stat_full[q & 1], q >> 1)) break;
+#pragma unroll 1
+                for (int i = (gi ^ g) & 1; i < it.n; i += 2) {
+                    const int acc = (gi + i) & 3;
+                    if (!wait_all(&p.ready[acc], (gi + i) >> 2)) break;
+                    tcgen05_after_sync();
+                    const int64_t j0 = (int64_t)(it.t0 + i) * kMmaKeys, j = j0 + gt;       // lane = key
+                    const bool cut = W < kSnapRows || j0 + kMmaKeys - 1 > first_q;
+                    const int q_lo = (int)min((int64_t)64, max((int64_t)0, j - first_q));
+                    float2 a[2] = {make_float2(0.0f, 0.0f), make_float2(0.0f, 0.0f)};
+#pragma unroll 1
+                    for (int cb = 0; cb < kSnapRows; cb += 32) {
+                        float v[32];
+                        tmem_ld32(tl + (uint32_t)(acc * 64 + cb), v);
+                        if (cb) {
+                            tcgen05_before_sync();
+                            arrive(&p.acc_free[acc]);
+                        }
+                        add_weights<32>(v, cb, cut, q_lo, W, scale_log2, q_nm[q & 1], q_il[q & 1], a);
+                    }
+                    const float2 both = add2(a[0], a[1]);
+                    if (j < len) imp[(int64_t)it.bh * len + j] = both.x + both.y;
+                }
+                if (!ok) break;
+                arrive(&p.stat_free[q & 1]);
+            }
+            gi += it.n;
+        }
+    }
+    if (__any_sync(FULL, !ok) && lane == 0) atomicCAS(status, RQ_OK, RQ_ERR_TIMEOUT);
+    tcgen05_before_sync();
+    __syncthreads();
+    if (warp == 0) tmem_dealloc(tbase, 512);
+}
+
+// Clears the counters and the heads' statistics for the launch above.
+__global__ void __launch_bounds__(256) snap_stream_clear_kernel(uint4 *p, size_t n)
+{
+    grid_launch_dependents();
+    for (size_t i = (size_t)blockIdx.x * 256 + threadIdx.x; i < n; i += (size_t)gridDim.x * 256) p[i] = make_uint4(0u, 0u, 0u, 0u);
 }
 
 // ---------------------------------------------------------------- short prompts: the keys read once
@@ -1240,6 +1608,44 @@ cudaError_t snap_scores_once(const SnapArgs &a, const CUtensorMap &tmap, const C
                               ntiles, tpc, a.status);
 }
 
+size_t round256(size_t x) { return (x + 255) & ~(size_t)255; }
+
+// The same for many heads of up to kStreamMaxTiles tiles.
+template <int D>
+cudaError_t snap_scores_stream(const SnapArgs &a, const CUtensorMap &tmap, const CUtensorMap &qmap, int ntiles, cudaStream_t s)
+{
+    using G = SnapStreamGeom<D>;
+    static bool ready[64];
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
+    if (!ready[dev]) {
+        e = cudaFuncSetAttribute(snap_stream_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, G::SMEM_BYTES);
+        if (e != cudaSuccess) return e;
+        ready[dev] = true;
+    }
+    const int BH = a.B * a.H, items = (ntiles + kStreamTiles - 1) / kStreamTiles, tpc = (ntiles + items - 1) / items, runs = (ntiles + tpc - 1) / tpc;
+    // the counters lie in front of the heads' statistics: the records in front of them take less than half of their room
+    const size_t ctr = round256(((size_t)BH + 2) * sizeof(int32_t)), n = (ctr + (size_t)BH * kSnapRows * sizeof(float2)) / 16;
+    int32_t *counters = (int32_t *)((char *)a.rowstat - ctr);
+    snap_stream_clear_kernel<<<(unsigned)std::min<size_t>((n + 255) / 256, 64), 256, 0, s>>>((uint4 *)counters, n);
+    e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute at = {};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cfg.gridDim = dim3((unsigned)std::min<int64_t>(sm_count(), (int64_t)BH * runs));
+    cfg.blockDim = dim3(kStreamThreads);
+    cfg.dynamicSmemBytes = G::SMEM_BYTES;
+    cfg.stream = s;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, snap_stream_kernel<D>, tmap, qmap, a.page_cap, a.S, a.len, a.W, a.H, BH, a.scale * 1.4426950408889634f, a.stats,
+                              a.rowstat, counters, a.imp, ntiles, tpc, runs, a.status);
+}
+
 template <int D>
 cudaError_t snap_scores_mma(const SnapArgs &a, cudaStream_t s)
 {
@@ -1257,6 +1663,9 @@ cudaError_t snap_scores_mma(const SnapArgs &a, cudaStream_t s)
     e = query_tensor_map(&qmap, a.qw, D, a.H, a.W, a.B, kSnapRows);
     if (e != cudaSuccess) return e;
     const int ntiles = (int)((a.len + kMmaKeys - 1) / kMmaKeys);
+    const int per_sm = D == 128 && ntiles > kOnceTiles * kOnceCluster ? kStreamPerSmWide : kStreamPerSm;
+    if (ntiles >= kStreamTiles && ntiles <= kStreamMaxTiles && (int64_t)BH * ntiles > (int64_t)per_sm * sm_count())
+        return snap_scores_stream<D>(a, tmap, qmap, ntiles, s);
     if (ntiles <= kOnceTiles * kOnceCluster) return snap_scores_once<D>(a, tmap, qmap, ntiles, s);
     if (!ready[dev]) {
         e = cudaFuncSetAttribute(snap_mma_kernel<D, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, G::TWO_BYTES);
@@ -1307,8 +1716,6 @@ cudaError_t snap_scores_mma(const SnapArgs &a, cudaStream_t s)
     return cudaLaunchKernelEx(&cfg, snap_mma_kernel<D, 2>, tmap, qmap, a.page_cap, a.S, a.len, a.W, a.H, sl2, (float2 *)nullptr,
                               (const float2 *)a.rowstat, a.imp, ntiles, tpc, a.status);
 }
-
-size_t round256(size_t x) { return (x + 255) & ~(size_t)255; }
 
 }  // namespace
 

@@ -1,0 +1,47 @@
+"""Importance of many heads' prompts, both passes in one launch (more than thirty or forty tiles of 128 keys to an SM, heads of 8 to 128 tiles): at
+the edges of that range and of its items of eight tiles, a last tile of one key, windows of fewer than 64 queries, pages of both sizes,
+several calls on one scratch; against softmax in fp64.  The bound is that of the other forms: a score of D terms carries at most D 2^-24
+of its terms' absolute values, ex2 2^-22, the sums less; 2e-5 of the largest importance."""
+import pytest
+import torch
+
+import paper_2605_28640_b200 as rq
+
+pytestmark = pytest.mark.gpu
+DEV = "cuda"
+
+
+@pytest.mark.parametrize("BH,T,W,S,D", [(556, 1000, 64, 16, 64), (640, 897, 64, 64, 128), (500, 1025, 64, 16, 128), (139, 4096, 64, 64, 64), (139, 4096, 33, 16, 128),
+                                        (256, 4096, 64, 16, 128), (137, 4097, 64, 16, 64), (118, 6401, 1, 64, 128), (47, 16384, 64, 16, 128),
+                                        (35, 16257, 17, 64, 64), (47, 16385, 64, 16, 128)])
+def test_importance(BH, T, W, S, D):
+    g = torch.Generator(device=DEV)
+    g.manual_seed(T + W)
+    cache = rq.Cache(1, BH, D, S, T, torch.bfloat16)
+    k = torch.randn(1, T, BH, D, generator=g, device=DEV, dtype=torch.bfloat16)
+    k[:, T // 2] = k[:, 0]                                        # equal keys in different items,
+    k[:, T - W - 1] = k[:, 0]                                     # and in a tile that the window cuts
+    z = torch.zeros_like(k)
+    rq.rq_build_cache(cache.handle, k, z, z)                      # zero gates: the cache holds the keys themselves
+    n = rq.rq_snapkv_scratch_bytes(cache.handle)
+    scratch = torch.full((n + 4096,), 0x5A, dtype=torch.uint8, device=DEV)
+    idx = torch.empty(1, BH, W, dtype=torch.int32, device=DEV)
+    first = None
+    for gain in (1.0, 3.0, 1.0):                                  # what a call leaves in the scratch is not for the next one
+        qw = torch.randn(1, W, BH, D, generator=torch.Generator(device=DEV).manual_seed(int(gain)), device=DEV, dtype=torch.bfloat16) * gain
+        imp = torch.full((1, BH, T), float("nan"), dtype=torch.float32, device=DEV)
+        rq.rq_snapkv_select(cache.handle, qw, W, W, 0.0, idx, imp, scratch)
+        torch.cuda.synchronize()
+        assert rq.rq_device_status(cache.handle) == rq.RQ_OK
+        assert (scratch[n:] == 0x5A).all() and not imp.isnan().any()
+        for h in sorted({0, BH // 3, BH // 2, BH - 2, BH - 1}):
+            s = qw[0, :, h].double() @ k[0, :, h].double().T * D ** -0.5
+            pos = torch.arange(T, device=DEV)
+            s[pos[None, :] > (T - W + torch.arange(W, device=DEV))[:, None]] = float("-inf")
+            want = torch.softmax(s, -1).sum(0)
+            err = (imp[0, h].double() - want).abs().max().item()
+            assert err <= 2e-5 * want.max().item(), f"head {h}: {err} of {want.max().item()}"
+        assert torch.equal(imp[0, :, 0], imp[0, :, T // 2]) and torch.equal(imp[0, :, 0], imp[0, :, T - W - 1])
+        if gain == 1.0:
+            first = imp if first is None else first
+            assert torch.equal(first.view(torch.int32)[0, 0, :64], imp.view(torch.int32)[0, 0, :64])
