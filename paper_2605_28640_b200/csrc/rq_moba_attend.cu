@@ -117,7 +117,8 @@ struct Walk {
 // 1.5 up to the first product and 3 at the end.  Launch, us, a CTA per tile / this: 32 heads x 4096 positions 185 / 174.5, x 30011
 // 5760 / 5570 (three stages of keys and values and all of the output's rows in shared memory at once instead of four and halves:
 // 174.5 / 5680; a next tile taken at once instead of six steps before the end would pair the longest tiles); with the readers' positions
-// in 32 bits 169.5 / 5420: every instruction between one score buffer and the next counts.  What any query of a tile
+// in 32 bits 169.5 / 5420, barriers asked about before they are waited for 167 / 5370: every instruction between one score buffer and the
+// next counts.  What any query of a tile
 // chose comes from the routing as a word per 32 blocks, 128 queries together; the walk goes by its bits.
 // A tile's 256 consecutive queries are two accumulators of 128 lanes; everything per query (choice of blocks, causal cut, what its weights
 // are relative to, their sum, the weights) belongs to one thread.  The 64-position chunks of the blocks that any of the 256
@@ -213,7 +214,7 @@ __global__ void __launch_bounds__(kThreads, 1) moba_mma_kernel(const __grid_cons
     tcgen05_after_sync();
     const uint32_t tb = __shfl_sync(FULL, tbase, 0);             // (the shuffle tells the compiler that it is uniform)
     bool ok = true;
-    auto wait_all = [&](uint64_t *x, int phase) -> bool { return ok = __all_sync(FULL, mbar_wait(x, (uint32_t)(phase & 1))); };
+    auto wait_all = [&](uint64_t *x, int phase) -> bool { return ok = __all_sync(FULL, mbar_wait_soon(x, (uint32_t)(phase & 1))); };
     // the CTA's k-th tile, for the warps that work on it; false: there is none
     int n = 0, bh = 0;
     int64_t t0 = 0;
@@ -308,7 +309,7 @@ __global__ void __launch_bounds__(kThreads, 1) moba_mma_kernel(const __grid_cons
                 const int st = g % NST;
                 if (g >= NST) {
                     const uint32_t ph = (uint32_t)((g / NST - 1) & 1);
-                    ok = mbar_wait(&free_k[st], ph) && mbar_wait(&free_v[st], ph);
+                    ok = mbar_wait_soon(&free_k[st], ph) && mbar_wait_soon(&free_v[st], ph);
                     ok = __all_sync(FULL, ok);
                     if (!ok) break;
                 }
@@ -341,10 +342,10 @@ __global__ void __launch_bounds__(kThreads, 1) moba_mma_kernel(const __grid_cons
         // no copy may still be on its way into this CTA's shared memory when it exits, after a wait that ran out either
         if (!ok) {
             for (int x = max(0, issued - NST); x < issued; ++x) {
-                mbar_wait(&full_k[x % NST], (uint32_t)((x / NST) & 1));
-                mbar_wait(&full_v[x % NST], (uint32_t)((x / NST) & 1));
+                mbar_wait_soon(&full_k[x % NST], (uint32_t)((x / NST) & 1));
+                mbar_wait_soon(&full_v[x % NST], (uint32_t)((x / NST) & 1));
             }
-            if (asked > 0) mbar_wait(&answered, (uint32_t)((asked - 1) & 1));
+            if (asked > 0) mbar_wait_soon(&answered, (uint32_t)((asked - 1) & 1));
         }
     } else if (warp > kReadWarps && warp <= kReadWarps + kTiles) {
         // ---- queries and score products, a warp per accumulator
@@ -367,7 +368,7 @@ __global__ void __launch_bounds__(kThreads, 1) moba_mma_kernel(const __grid_cons
                 if (!wait_all(&free_q[s], k - 1)) break;         // the tile before has read its queries
                 ask();
             }
-            ok = __all_sync(FULL, mbar_wait(&full_q[s], (uint32_t)(k & 1)) || mbar_wait(&full_q[s], (uint32_t)(k & 1)));
+            ok = __all_sync(FULL, mbar_wait_soon(&full_q[s], (uint32_t)(k & 1)) || mbar_wait_soon(&full_q[s], (uint32_t)(k & 1)));
             if (!ok) break;
             const Chosen &c = chosen_of[k & 1];
             Walk w;
@@ -394,7 +395,7 @@ __global__ void __launch_bounds__(kThreads, 1) moba_mma_kernel(const __grid_cons
             umma_commit(&free_q[s]);
             leave(k);
         }
-        if (!ok) mbar_wait(&full_q[s], 0u), mbar_wait(&full_q[s], 1u);       // (a copy of queries may be on its way)
+        if (!ok) mbar_wait_soon(&full_q[s], 0u), mbar_wait_soon(&full_q[s], 1u);       // (a copy of queries may be on its way)
     } else if (warp == kReadWarps + kTiles + 1) {
         // ---- output products
         constexpr uint32_t idesc_o = umma_idesc_bf16(kTile, D) | (1u << 16);       // the values are MN-major
@@ -483,7 +484,7 @@ __global__ void __launch_bounds__(kThreads, 1) moba_mma_kernel(const __grid_cons
             const int p0 = j * block + r * kChunk;
             // positions this query attends among the chunk's: none if it did not choose the block, else those up to its own
             const int nv = chosen ? max(0, min(kChunk, seen - p0)) : 0;
-            ok = mbar_wait(&s_ready[s][u & 1], (uint32_t)((u >> 1) & 1));
+            ok = mbar_wait_soon(&s_ready[s][u & 1], (uint32_t)((u >> 1) & 1));
             if (!__all_sync(FULL, ok)) break;
             tcgen05_after_sync();
             const uint32_t ts = tl + (uint32_t)(u & 1) * kChunk;
@@ -528,7 +529,7 @@ __global__ void __launch_bounds__(kThreads, 1) moba_mma_kernel(const __grid_cons
                     tmem_st16(ts + hf * 16, w);
                 }
                 if (__any_sync(FULL, touch)) {
-                    ok = mbar_wait(&pv_done[s][(u - 1) & 1], (uint32_t)(((u - 1) >> 1) & 1));   // nothing is being added to O
+                    ok = mbar_wait_soon(&pv_done[s][(u - 1) & 1], (uint32_t)(((u - 1) >> 1) & 1));   // nothing is being added to O
                     if (!__all_sync(FULL, ok)) break;
                     tcgen05_after_sync();
                     float x[2][32];
@@ -555,7 +556,7 @@ __global__ void __launch_bounds__(kThreads, 1) moba_mma_kernel(const __grid_cons
             if (p0 + kChunk > len) {
                 // the prompt ends inside this chunk: the value rows past its end hold whatever the cache's memory held; a
                 // weight of zero would not stop a NaN there, so those rows are cleared once they have landed
-                ok = mbar_wait(&full_v[g % NST], (uint32_t)((g / NST) & 1));
+                ok = mbar_wait_soon(&full_v[g % NST], (uint32_t)((g / NST) & 1));
                 if (!__all_sync(FULL, ok)) break;
                 const int r = lq & (kChunk - 1), hf = lq >> 6;
                 if (hf < G::HALVES && p0 + r >= len) {

@@ -124,9 +124,9 @@ template <int NB> __device__ __forceinline__ uint32_t score_bin(float v, float l
 // FORM: 0 for prompts of at most 64 blocks, whose two words of scores are taken by half words, so that all four threads of a query
 // have some; 1 for up to 512, one panel; 2 beyond.
 // Measured, 32 heads x 128 channels, before / now: 4096 queries, 16 of 64 blocks each, 42.5 -> 32 us; 30011 queries, 30 of 469 blocks
-// each, 1020 -> 650 us.  In steps: counting without branches and one comparison less per score 940 us; terms by copies, 128 buckets
+// each, 1020 -> 610 us.  In steps: counting without branches and one comparison less per score 940 us; terms by copies, 128 buckets
 // instead of 64 (fewer blocks to rank), mask words without bank conflicts 690 us; blocks to rank read again by column instead of
-// picked from registers, divisions out of the stores of the masks 650 us.  The threshold by rounds of counting three keys at a time in
+// picked from registers, divisions out of the stores of the masks 650 us; a warp of its own for the copies 610 us.  The threshold by rounds of counting three keys at a time in
 // the registers of a query's four threads instead of buckets: 49.7 us for the 4096 queries.
 template <int D, int FORM>
 __global__ void __launch_bounds__(kRouteThreads, 2) moba_route_mma_kernel(const __grid_constant__ CUtensorMap qmap, const float *means, const unsigned char *terms, int64_t len, int H,
@@ -219,43 +219,41 @@ __global__ void __launch_bounds__(kRouteThreads, 2) moba_route_mma_kernel(const 
         };
         // the scores of panel p into tensor memory, 64 blocks at a time, the smallest terms first; done[g] is told of each group.
         // The terms come by bulk copies, each plane's as soon as the products before have read its room: the first warp (the whole
-        // warp, see rq_umma.cuh) starts copies and products, the others go on.  Where the scratch had no room for the terms all
+        // warp, see rq_umma.cuh) starts the products, the second the copies (one warp for both, which takes 600 cycles for a plane's
+        // barriers, product and copy, 660 us / 610), the others go on.  Where the scratch had no room for the terms all
         // threads cut the representatives
         auto panel = [&](int p) {
             const int g0 = p * kPanelGroups, gn = min(kPanelGroups, groups - g0);
             if (terms) {
+                const int planes = 3 * gn, u0 = fills;
+                fills += gn;
+                if (warp == 1) {                                               // (the first panel's first three are on their way)
+                    int issued = seq == 0 ? 3 : 0;
+#pragma unroll 1
+                    for (; issued < planes && ok; ++issued) {
+                        if (issued >= 3) ok = __all_sync(FULL, mbar_wait(&free_t[issued % 3], (uint32_t)((u0 + issued / 3 - 1) & 1)));
+                        if (ok) issue(g0, issued);
+                        else break;
+                    }
+                    // after a wait that ran out: no copy may still be on its way into this CTA's shared memory when it exits
+                    if (!ok)
+                        for (int i = max(0, issued - 3); i < issued; ++i) mbar_wait(&full_t[i % 3], (uint32_t)((u0 + i / 3) & 1));
+                }
                 if (warp != 0) return;
-                int landed = 0, issued = 3;
-                const int u0 = fills;
-                if (seq > 0)
-                    for (int i = 0; i < 3; ++i) issue(g0, i);
                 if (seq == 0) ok = __all_sync(FULL, mbar_wait(&full_q, 0u) || mbar_wait(&full_q, 0u));
 #pragma unroll 1
                 for (int g = 0; g < gn && ok; ++g) {
 #pragma unroll
                     for (int st = 0; st < 3; ++st) {
-                        ok = ok && __all_sync(FULL, mbar_wait(&full_t[st], (uint32_t)((u0 + g) & 1)));
+                        ok = ok && __all_sync(FULL, mbar_wait_soon(&full_t[st], (uint32_t)((u0 + g) & 1)));
                         if (!ok) break;
-                        landed = 3 * g + st + 1;
                         tcgen05_after_sync();
                         product(g, 2 - st);
                         umma_commit(&free_t[st]);
                     }
-                    if (!ok) break;
-                    umma_commit(&done[g]);
-                    if (g + 1 < gn)
-#pragma unroll
-                        for (int st = 0; st < 3; ++st) {                       //
-                            ok = ok && __all_sync(FULL, mbar_wait(&free_t[st], (uint32_t)((u0 + g) & 1)));
-                            if (!ok) break;
-                            issue(g0, 3 * (g + 1) + st);
-                            issued = 3 * (g + 1) + st + 1;
-                        }
+                    if (ok) umma_commit(&done[g]);
                 }
-                fills += gn;
                 if (FORM == 2) finish(gn);
-                // after a wait that ran out: no copy may still be on its way into this CTA's shared memory when it exits
-                for (int i = landed; i < issued; ++i) mbar_wait(&full_t[i % 3], (uint32_t)((u0 + i / 3) & 1));
                 return;
             }
             constexpr int PER = kRouteGroup * D / 4 / kRouteThreads;           // float4 of a thread
