@@ -284,6 +284,8 @@ __global__ void __launch_bounds__(kMmaThreads, D == 128 ? 6 : 4) snap_mma_kernel
     // scores a reader takes at a time.  Of 128 channels HBM is the bound, and the registers left over let the kernel behind start
     // beside this one (12 heads x 50000, a call 89 us with 64 at a time, 77 with 32); of 64 channels the readers are (32 x 65536 149 / 158)
     constexpr int N = D == 128 ? 32 : 64;
+    // (of 64 channels most phases are complete when they are waited for: 32 heads x 65536, a call 149.5 / 142.6 us; of 128 0.7 % slower)
+    auto wait_for = [](uint64_t *bar, uint32_t parity) { return D == 64 ? mbar_wait_soon(bar, parity) : mbar_wait(bar, parity); };
     extern __shared__ __align__(1024) unsigned char dsm_raw[];
     __shared__ __align__(8) uint64_t bar[2];                   // an accumulator's product is complete
     __shared__ __align__(8) uint64_t full[NST], full_q;        // a stage's keys, the queries have landed
@@ -369,14 +371,14 @@ __global__ void __launch_bounds__(kMmaThreads, D == 128 ? 6 : 4) snap_mma_kernel
         // ---- the producing warp starts the copies and the products (all its lanes run this, see rq_umma.cuh);
         // nobody else waits for it except through the barriers
         {
-            ok = __all_sync(0xffffffffu, mbar_wait(&full_q, 0u) || mbar_wait(&full_q, 0u));
+            ok = __all_sync(0xffffffffu, wait_for(&full_q, 0u) || wait_for(&full_q, 0u));
             constexpr uint32_t idesc = PASS == 1 ? umma_idesc_bf16(128, kMmaKeys) : umma_idesc_bf16(kMmaKeys, kSnapRows);
             const uint64_t qd = umma_desc_sw128(smem_addr(qs)), kd = umma_desc_sw128(smem_addr(ks));
 #pragma unroll 1
             for (int i = 0; i < n && ok; ++i) {
                 // accumulator i & 1 has been read (tile i - 2), the tile's keys have landed
-                if (i >= 2) ok = __all_sync(0xffffffffu, mbar_wait(&acc_free[i & 1], (uint32_t)(((i >> 1) - 1) & 1)));
-                ok = ok && __all_sync(0xffffffffu, mbar_wait(&full[i % NST], (uint32_t)((i / NST) & 1)));
+                if (i >= 2) ok = __all_sync(0xffffffffu, wait_for(&acc_free[i & 1], (uint32_t)(((i >> 1) - 1) & 1)));
+                ok = ok && __all_sync(0xffffffffu, wait_for(&full[i % NST], (uint32_t)((i / NST) & 1)));
                 if (!ok) break;
                 n_landed = i + 1;
                 tcgen05_after_sync();
@@ -390,12 +392,12 @@ __global__ void __launch_bounds__(kMmaThreads, D == 128 ? 6 : 4) snap_mma_kernel
                 umma_commit(&bar[i & 1]);
                 // the stage of tile i - 1 is free once its product has completed; it takes tile i - 1 + NST
                 if (i >= 1 && i - 1 + NST < n) {
-                    ok = __all_sync(0xffffffffu, mbar_wait(&bar[(i - 1) & 1], (uint32_t)(((i - 1) >> 1) & 1)));
+                    ok = __all_sync(0xffffffffu, wait_for(&bar[(i - 1) & 1], (uint32_t)(((i - 1) >> 1) & 1)));
                     if (ok) issue(i - 1 + NST);
                 }
             }
             // after a wait that ran out: no copy may still be on its way into this CTA's shared memory when it exits
-            for (int k = n_landed; k < n_issued; ++k) mbar_wait(&full[k % NST], (uint32_t)((k / NST) & 1));
+            for (int k = n_landed; k < n_issued; ++k) wait_for(&full[k % NST], (uint32_t)((k / NST) & 1));
         }
     } else {
     if (PASS == 2) {
@@ -409,7 +411,7 @@ __global__ void __launch_bounds__(kMmaThreads, D == 128 ? 6 : 4) snap_mma_kernel
     }
 #pragma unroll 1
     for (int i = 0; i < n; ++i) {
-        ok = mbar_wait(&bar[i & 1], (uint32_t)((i >> 1) & 1));
+        ok = wait_for(&bar[i & 1], (uint32_t)((i >> 1) & 1));
         if (!__all_sync(0xffffffffu, ok)) break;               // (a warp's lanes stay together: the accumulator loads are warp-wide)
         tcgen05_after_sync();
         const int64_t j0 = (int64_t)tile(i) * kMmaKeys;
