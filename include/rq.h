@@ -305,7 +305,7 @@ RQ_API int64_t rq_cache_len(const rq_cache *cache);
 /* Kernel launches the next rq_decode_step on this cache will enqueue for this budget when
  * sel_idx_out is NULL [no counterpart in the paper: bookkeeping for benchmarks]: ONE when the whole
  * step runs as one launch (chosen by the library for short contexts: fewer than 1024 pages per head
- * with up to a few MB to read per head, or up to 2048 pages when there are more (batch, head) pairs
+ * with up to a few MB to read per head, more where every page is kept, or up to 2048 pages when there are more (batch, head) pairs
  * than SMs and they either keep all SMs equally busy or have little to read; and for 64 to 128 (batch, head) pairs of 4096 to
  * 12284 pages each that split into 4, 8 or 2 equal groups which keep the GPU's resident CTAs
  * busy, budget below the number of pages; cache.reserved[2] asks for it on other shapes);

@@ -1,0 +1,35 @@
+"""Decode steps that keep every page, at both sides of where one launch of a cluster per head takes the place of separate kernels: as
+many launches as the rule gives, and the results of the two forms agree (states and stored rows bit for bit, the output to what the
+order of the fp32 sums moves, well inside one bf16 step)."""
+import pytest
+import torch
+
+import paper_2605_28640_b200 as rq
+
+pytestmark = pytest.mark.gpu
+DEV = "cuda"
+
+
+@pytest.mark.parametrize("H,D,S,T,launches", [(32, 128, 16, 8200, 1), (16, 128, 16, 16001, 1), (24, 128, 64, 30000, 1), (16, 128, 64, 30000, 3),
+                                              (128, 64, 16, 8200, 1), (74, 64, 16, 12001, 3), (32, 128, 16, 16400, 3)])
+def test_every_page_kept(H, D, S, T, launches):
+    g = torch.Generator(device=DEV)
+    g.manual_seed(T)
+    k = torch.randn(1, T, H, D, generator=g, device=DEV, dtype=torch.bfloat16)
+    q, kt, vt = (torch.randn(1, H, D, generator=g, device=DEV, dtype=torch.bfloat16) for _ in range(3))
+    gt = torch.rand(1, H, D, generator=g, device=DEV, dtype=torch.float32).to(torch.bfloat16)
+    P = -(-(T + 1) // S)
+    outs = []
+    for form in (0, 1):
+        cache = rq.Cache(1, H, D, S, T + 1, torch.bfloat16)
+        rq.rq_build_cache(cache.handle, k, k, torch.full_like(k, 0.9))
+        cache.handle.reserved[2] = form
+        if form == 0:
+            assert rq.rq_decode_step_launches(cache.handle, P) == launches
+        o = torch.empty(1, H, D, dtype=torch.bfloat16, device=DEV)
+        rq.rq_decode_step(cache.handle, q, kt, vt, gt, P, 0.0, o)
+        torch.cuda.synchronize()
+        assert rq.rq_device_status(cache.handle) == rq.RQ_OK
+        outs.append((o.float(), cache.state.clone(), cache.kv.clone()))
+    assert torch.equal(outs[0][1], outs[1][1]) and torch.equal(outs[0][2], outs[1][2])
+    assert (outs[0][0] - outs[1][0]).abs().max().item() <= 2 ** -8 * outs[1][0].abs().max().item()
