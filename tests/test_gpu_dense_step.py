@@ -11,7 +11,8 @@ DEV = "cuda"
 
 
 @pytest.mark.parametrize("H,D,S,T,launches", [(32, 128, 16, 8200, 1), (16, 128, 16, 16001, 1), (24, 128, 64, 30000, 1), (16, 128, 64, 30000, 3),
-                                              (128, 64, 16, 8200, 1), (74, 64, 16, 12001, 3), (32, 128, 16, 16400, 3)])
+                                              (128, 64, 16, 8200, 1), (74, 64, 16, 12001, 3), (140, 64, 16, 4001, 0), (9, 64, 64, 20000, 0), (9, 128, 16, 14000, 1),
+                                              (23, 64, 64, 60000, 0), (32, 128, 16, 16400, 3)])
 def test_every_page_kept(H, D, S, T, launches):
     g = torch.Generator(device=DEV)
     g.manual_seed(T)
@@ -25,7 +26,8 @@ def test_every_page_kept(H, D, S, T, launches):
         rq.rq_build_cache(cache.handle, k, k, torch.full_like(k, 0.9))
         cache.handle.reserved[2] = form
         if form == 0:
-            assert rq.rq_decode_step_launches(cache.handle, P) == launches
+            n = rq.rq_decode_step_launches(cache.handle, P)
+            assert n == launches if launches else n > 1      # 0: separate kernels, two or three
         o = torch.empty(1, H, D, dtype=torch.bfloat16, device=DEV)
         rq.rq_decode_step(cache.handle, q, kt, vt, gt, P, 0.0, o)
         torch.cuda.synchronize()
